@@ -17,9 +17,8 @@
  *     and never frees or writes caller inputs.
  *   - Streams.  `stream` is a cudaStream_t passed as void*.  Results are ordered
  *     on it: work enqueued on `stream` after a call sees that call's outputs.
- *     fc_score_layer runs power-of-two sequences of 1024..65536 tokens and long
- *     sequences of other lengths on the handle's internal streams (two by
- *     default), which wait for everything enqueued on `stream` before the call
+ *     fc_score_layer runs sequences of up to 65536 tokens on the handle's
+ *     internal streams (two by default), which wait for everything enqueued on `stream` before the call
  *     and which `stream` waits for before the call returns, through events; no
  *     host synchronisation is involved (see fc_set_score_overlap for the
  *     variant that defers the second wait).  Nothing uses the default stream.
@@ -90,9 +89,8 @@ typedef struct {
 /* Create a handle on `device`.  max_seqlen bounds every N_b later passed in
  * (1 <= max_seqlen <= 131072; lengths that are not a power of two, or below 16,
  * are limited to 65536).  Allocates the twiddle table (8 bytes * 4 * next power of two of
- * max_seqlen), room for eight chirp-kernel spectra with their per-row chirp factors (each 8 bytes *
- * (the power of two from 2*max_seqlen-1 up + 2*max_seqlen), at most 2 MiB; lengths that are not a
- * power of two reuse theirs from layer to layer) and a status word.  Returns FC_ERR_CUDA if the device cannot be
+ * max_seqlen), room for eight filter tables (16 bytes * the power of two from 2*max_seqlen-1 up each, at most
+ * 2 MiB; lengths that are not a power of two reuse theirs from layer to layer) and a status word.  Returns FC_ERR_CUDA if the device cannot be
  * used, FC_ERR_UNSUPPORTED if max_seqlen is out of range. */
 fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen);
 void fc_destroy(fc_handle *h);
@@ -161,12 +159,9 @@ fc_status fc_set_score_overlap(fc_handle *h, int32_t enabled);
  * call waits for the one before it. */
 fc_status fc_set_select_overlap(fc_handle *h, int32_t enabled);
 
-/* Sequences whose length is not a power of two are transformed by chirp convolutions of a padded
- * power-of-two length (>= 2N - 1).  enabled = 1 (default): where the cutoff index omega of Eq. 8
- * allows a shorter padded length (>= N + 2*omega + 1), only the bins -omega .. omega of the
- * spectrum are computed, the low-pass part (the Base KV of Eq. 9) is transformed back and the
- * score of Eq. 10 is taken against the input rows.  Same result to fp32 rounding; speed only.
- * enabled = 0: always the full-length form (all N bins, residual formed in the frequency domain). */
+/* Which chirp form fc_describe_plan counts for lengths that are not a power of two: enabled = 1 (default) the
+ * band form (only the bins -omega .. omega of the spectrum, padded length >= N + 2*omega + 1) where it is shorter than
+ * the full-length form (>= 2N - 1), enabled = 0 always the latter.  No effect on how such lengths are computed. */
 fc_status fc_set_chirp_band(fc_handle *h, int32_t enabled);
 
 /* Number of internal streams fc_score_layer spreads the head groups of a sequence over (1..4,
@@ -191,9 +186,10 @@ fc_status fc_reset_ordering(fc_handle *h);
  * Default 32 MiB.  Affects speed only. */
 fc_status fc_set_group_bytes(fc_handle *h, size_t bytes);
 
-/* How a sequence of length seqlen is transformed at cutoff ratio gamma (diagnostic, used for flop
- * accounting; head_dim a multiple of 64 assumed): out = { direct power-of-two path (0), chirp
- * convolutions in the full-length form (1) or in the band form (2, see fc_set_chirp_band),
+/* The transform of a sequence of length seqlen at cutoff ratio gamma that roofline figures are counted on
+ * (diagnostic; head_dim a multiple of 64 assumed): out = { power of two: the transform itself (0); other lengths: the
+ * shortest chirp convolutions in the full-length (1) or band form (2, see fc_set_chirp_band) -- a yardstick: the
+ * library computes such lengths as one padded convolution of at least 2N - 1 points --,
  * transform length, first factor N1, second factor N2 }. */
 fc_status fc_describe_plan(const fc_handle *h, int32_t seqlen, double gamma, int32_t out[4]);
 
@@ -396,6 +392,22 @@ fc_status fc_select_compact_layers(fc_handle *h, const fc_kv_view *shape, const 
                                    int32_t num_layers, const int32_t *budgets, const int64_t *out_offsets,
                                    const fc_select_options *opt, void *workspace, size_t workspace_bytes,
                                    fc_stream stream);
+
+/*
+ * fc_score_layer for several layers that share one layout, the same scores and energies bit for bit (Sec. 3.2.1).
+ * Launches run over the KV heads of consecutive layers, so short sequences fill the GPU, and the host enqueues a few
+ * launches per sequence instead of a few per sequence and layer.
+ *
+ *   shape        the layout all layers share (its k and v are not read)
+ *   layers       HOST array [num_layers]; k, v and scores are used, the outputs of the selection are not; the arrays
+ *                the scores point at are written although the type (shared with the selection) says const
+ *   energy       DEVICE double[num_layers][B][4]
+ *   workspace    DEVICE, 256-byte aligned, >= fc_score_layers_workspace_bytes()
+ * Errors and ordering: as fc_score_layer.
+ */
+size_t fc_score_layers_workspace_bytes(const fc_handle *h, const fc_kv_view *shape, int32_t num_layers);
+fc_status fc_score_layers(fc_handle *h, const fc_kv_view *shape, const fc_layer_buffers *layers, int32_t num_layers,
+                          double gamma, double *energy, void *workspace, size_t workspace_bytes, fc_stream stream);
 
 /* Rows one layer's compacted cache can receive at most: the sum over sequences of
  * min(N_b, B_tot(b)), B_tot = clamp(floor(rho*N*L + 1/2), L*lo, L*N) (Sec. 3.2.2; the total the

@@ -26,7 +26,7 @@ EXPORTS = (
     "fc_set_group_bytes", "fc_set_chirp_band", "fc_set_internal_streams", "fc_set_l2_persist", "fc_reset_ordering", "fc_set_score_overlap", "fc_set_select_overlap", "fc_profile_begin", "fc_profile_stride", "fc_profile_end", "fc_describe_plan",
     "fc_score_workspace_bytes", "fc_select_workspace_bytes",
     "fc_score_layer", "fc_allocate_budgets", "fc_select_compact", "fc_select_compact_ex",
-    "fc_select_compact_layers", "fc_layer_capacity_rows",
+    "fc_select_compact_layers", "fc_layer_capacity_rows", "fc_score_layers", "fc_score_layers_workspace_bytes",
     "fc_power_spectrum_workspace_bytes", "fc_power_spectrum", "fc_cutoff_from_spectrum",
     "fc_decode_workspace_bytes", "fc_decode_attention",
     "fc_static_scratch_bytes", "fc_score_layer_static", "fc_static_last_device_status",
@@ -138,6 +138,11 @@ def _load() -> ctypes.CDLL:
     lib.fc_score_layer.argtypes = [c_void_p, POINTER(fc_kv_view), c_double, c_void_p, c_void_p,
                                    c_void_p, c_size_t, c_void_p]
     lib.fc_score_layer.restype = c_int
+    lib.fc_score_layers_workspace_bytes.argtypes = [c_void_p, POINTER(fc_kv_view), c_int32]
+    lib.fc_score_layers_workspace_bytes.restype = c_size_t
+    lib.fc_score_layers.argtypes = [c_void_p, POINTER(fc_kv_view), POINTER(fc_layer_buffers), c_int32, c_double,
+                                    c_void_p, c_void_p, c_size_t, c_void_p]
+    lib.fc_score_layers.restype = c_int
     lib.fc_allocate_budgets.argtypes = [c_void_p, c_void_p, c_int32, c_int32, POINTER(c_int32),
                                         c_double, c_int32, c_void_p, c_void_p, c_void_p]
     lib.fc_allocate_budgets.restype = c_int
@@ -323,6 +328,25 @@ def fc_score_layer(handle, k, v, cu_seqlens, gamma: float, scores, energy, works
     _check(_lib.fc_score_layer(handle, byref(view), float(gamma), c_void_p(scores.data_ptr()),
                                c_void_p(energy.data_ptr()), c_void_p(workspace.data_ptr()),
                                workspace.numel() * workspace.element_size(), _stream()), "fc_score_layer")
+
+
+def fc_score_layers_workspace_bytes(handle, k, v, cu_seqlens, num_layers: int) -> int:
+    cu = _cu_array(cu_seqlens)
+    view = make_view(k, v, cu)
+    return int(_lib.fc_score_layers_workspace_bytes(handle, byref(view), int(num_layers)))
+
+
+def fc_score_layers(handle, K_layers, V_layers, cu_seqlens, gamma: float, scores, energy, workspace) -> None:
+    """fc_score_layer for all layers (one layout) in one call.  scores: float32 [L, H, T]; energy: float64 [L, B, 4]."""
+    L = len(K_layers)
+    cu = _cu_array(cu_seqlens)
+    view = make_view(K_layers[0], V_layers[0], cu)
+    tab = (fc_layer_buffers * L)()
+    for l in range(L):
+        tab[l].k, tab[l].v, tab[l].scores = K_layers[l].data_ptr(), V_layers[l].data_ptr(), scores[l].data_ptr()
+    _check(_lib.fc_score_layers(handle, byref(view), tab, L, float(gamma), c_void_p(energy.data_ptr()),
+                                c_void_p(workspace.data_ptr()), workspace.numel() * workspace.element_size(), _stream()),
+           "fc_score_layers")
 
 
 def fc_static_scratch_bytes() -> int:
@@ -528,7 +552,7 @@ class Compressor:
             pass
 
     def _workspace(self, k, v):
-        need = max(fc_score_workspace_bytes(self.handle, k, v, self.cu),
+        need = max(fc_score_layers_workspace_bytes(self.handle, k, v, self.cu, self.L),
                    fc_select_workspace_bytes(self.handle, k, v, self.cu))
         if need == 0:
             raise FlashCacheError(1, "fc_score_workspace_bytes")
@@ -572,12 +596,21 @@ class Compressor:
                                       self.out_k[l].data_ptr(), self.out_v[l].data_ptr(),
                                       self.out_idx[l].data_ptr(), m["cap"])
         m["layers"] = tab
+        # layers laid out alike are scored in one call
+        m["alike"] = all((k.stride(), v.stride(), k.dtype) == (K_layers[0].stride(), V_layers[0].stride(), K_layers[0].dtype)
+                         for k, v in zip(K_layers, V_layers))
         self._m, self._mkey, self._m_out = m, key, (id(self.out_k), id(self._ws))
         return m
 
     def score(self, K_layers, V_layers):
         m = self._marshal(K_layers, V_layers)
         st, h, gamma = _stream(), self.handle, c_double(self.gamma)
+        if m["alike"]:
+            rc = _lib.fc_score_layers(h, m["refs"][0], m["layers"], self.L, gamma, c_void_p(self.energy.data_ptr()),
+                                      m["ws"], m["ws_bytes"], st)
+            if rc != FC_OK:
+                raise FlashCacheError(rc, "fc_score_layers")
+            return
         call = _lib.fc_score_layer
         for l in range(self.L):
             rc = call(h, m["refs"][l], gamma, m["scores"][l], m["energy"][l], m["ws"], m["ws_bytes"], st)

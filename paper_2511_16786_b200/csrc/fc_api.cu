@@ -132,8 +132,6 @@ extern "C" fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen) 
   h->status_word = nullptr;
   h->done_counter = nullptr;
   h->group_bytes = (size_t)32 << 20;
-  h->tune_cpw = 32;        // tile widths of the specialised kernels in channel pairs (the measured best)
-  h->tune_cp = 8;
   h->launches = 0;
   h->num_aux = 2;
   h->ev_fork = nullptr;
@@ -149,7 +147,7 @@ extern "C" fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen) 
   h->score_overlap = 0;
   h->band_form = 1;
   h->step = 0;
-  h->last_sig = -1;
+  h->last_sig = 0;
   h->pending_join = false;
   for (int a = 0; a < 2; ++a) for (int b = 0; b < FC_MAX_AUX; ++b) h->ev_done[a][b] = nullptr;
   cudaDeviceProp prop;
@@ -163,24 +161,23 @@ extern "C" fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen) 
   if (cudaMalloc(&h->master, (size_t)h->master_len * sizeof(float2)) != cudaSuccess ||
       cudaMalloc(&h->status_word, sizeof(int)) != cudaSuccess ||
       cudaMemset(h->status_word, 0, sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&h->done_counter, 2 * sizeof(unsigned)) != cudaSuccess ||
-      cudaMemset(h->done_counter, 0, 2 * sizeof(unsigned)) != cudaSuccess ||
+      cudaMalloc(&h->done_counter, 2 * FC_LAYER_CHUNK * sizeof(unsigned)) != cudaSuccess ||
+      cudaMemset(h->done_counter, 0, 2 * FC_LAYER_CHUNK * sizeof(unsigned)) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
       !create_streams(h)) {
     fc_destroy(h);
     return FC_ERR_CUDA;
   }
   {
-    // room for the chirp kernel's spectrum of the longest sequence that is not a power of two (transform
-    // length: the power of two from 2N-1 up, at most 131072)
-    int m = 64;
+    // room for the filter tables of the longest padded sequence (transform length: at most the power of two from
+    // 2N-1 up, 131072)
+    int m = 1024;
     const int nmax = max_seqlen < 65536 ? max_seqlen : 65536;
     while (m < 2 * nmax - 1) m <<= 1;
-    h->hhat_cache_len = m;
-    h->hhat_slot_len = m + 2 * ((nmax + 31) / 32 * 32);
-    for (int i = 0; i < FC_HHAT_SLOTS; ++i) h->hhat_cache_n[i] = 0;
-    h->hhat_cache_next = 0;
-    if (cudaMalloc(&h->hhat_cache, (size_t)FC_HHAT_SLOTS * h->hhat_slot_len * sizeof(float2)) != cudaSuccess) {
+    h->tab_slot_len = m;
+    for (int i = 0; i < FC_TAB_SLOTS; ++i) h->tab_key[i] = 0;
+    h->tab_next = 0;
+    if (cudaMalloc(&h->tab_cache, (size_t)FC_TAB_SLOTS * h->tab_slot_len * sizeof(float4)) != cudaSuccess) {
       fc_destroy(h);
       return FC_ERR_CUDA;
     }
@@ -263,7 +260,7 @@ extern "C" void fc_destroy(fc_handle *h) {
   delete[] h->host_ev;
   if (h->ev_inputs_free) cudaEventDestroy(h->ev_inputs_free);
   if (h->ev_outputs_done) cudaEventDestroy(h->ev_outputs_done);
-  if (h->hhat_cache) cudaFree(h->hhat_cache);
+  if (h->tab_cache) cudaFree(h->tab_cache);
   if (h->master) cudaFree(h->master);
   if (h->status_word) cudaFree(h->status_word);
   if (h->done_counter) cudaFree(h->done_counter);
@@ -376,7 +373,7 @@ extern "C" fc_status fc_reset_ordering(fc_handle *h) {
   h->last_sig = 0;
   h->pending_join = false;
   h->host_last_arena = nullptr;
-  for (int i = 0; i < FC_HHAT_SLOTS; ++i) h->hhat_cache_n[i] = 0;
+  for (int i = 0; i < FC_TAB_SLOTS; ++i) h->tab_key[i] = 0;
   return FC_OK;
 }
 

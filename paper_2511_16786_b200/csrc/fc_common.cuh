@@ -14,7 +14,8 @@
 
 #define FC_MAX_STAGES 4
 #define FC_MAX_AUX 4     // internal streams a handle may use
-#define FC_HHAT_SLOTS 8  // chirp-kernel spectra a handle keeps (one per sequence length)
+#define FC_TAB_SLOTS 8   // filter tables a handle keeps (one per sequence length and cutoff)
+#define FC_LAYER_CHUNK 32  // layers one launch of the scoring kernels can span (kernel-argument table)
 
 // Bits of the device status word.
 #define FC_DEV_FLAG_INTERNAL 1
@@ -26,9 +27,8 @@ struct fc_handle {
   int master_len;          // power of two; master[i] = exp(-2*pi*i*j/master_len)
   float2 *master;          // DEVICE
   int *status_word;        // DEVICE
-  unsigned *done_counter;  // DEVICE, zero between calls (the last block of a sequence resets it)
+  unsigned *done_counter;  // DEVICE [2][FC_LAYER_CHUNK], zero between calls (the last block of a layer's sequence resets it)
   size_t group_bytes;
-  int tune_cpw, tune_cp;   // tile widths of the specialised kernels (channel pairs), see fc_create
   int num_sms;
   // L2 residency of the transform intermediates: the per-stream workspace buffers are declared a
   // persisting access window on the internal streams (0 switches it off, fc_set_l2_persist)
@@ -55,21 +55,19 @@ struct fc_handle {
   // fc_set_score_overlap: consecutive fc_score_layer calls keep running on the two internal streams
   // without rejoining the caller's stream; the join is made by the next call that consumes their results
   int score_overlap;
-  int band_form;           // 1: the chirp path may use its band form (fc_set_chirp_band)
+  int band_form;           // fc_set_chirp_band: which chirp form fc_describe_plan counts
   unsigned step;                 // specialised-path sequences scored so far (parity picks partial-sum buffers)
-  long long last_sig;            // (N, heads, head_dim) of the previous specialised-path step
+  size_t last_sig;               // how the previous call carved its workspace
   bool pending_join;             // internal streams hold work the caller's stream has not waited for
   cudaEvent_t ev_done[2][FC_MAX_AUX];   // [step parity][internal stream]: that stream finished that step
+  // filter tables of the last FC_TAB_SLOTS (length, cutoff) pairs that took the padded path (DEVICE, allocated by
+  // fc_create: FC_TAB_SLOTS x tab_slot_len entries; tab_key[i] = what slot i holds, 0 = nothing; round robin)
+  float4 *tab_cache;
+  int tab_slot_len, tab_next;
+  long long tab_key[FC_TAB_SLOTS];
   // fc_compress_host (created on its first call): the stream the host-to-device copies run on, one
   // event per layer (that layer's copies have landed), and the point of the previous job after
   // which the staged inputs of its arena may be overwritten
-  // spectra of the chirp kernel of the last FC_HHAT_SLOTS sequence lengths that took the chirp path (DEVICE,
-  // allocated by fc_create: FC_HHAT_SLOTS x hhat_cache_len points; hhat_cache_n[i] = length in slot i, 0 = none;
-  // slots are reused round robin)
-  float2 *hhat_cache;
-  int hhat_cache_len, hhat_cache_next;
-  int hhat_slot_len;       // points per slot: the spectrum (hhat_cache_len) and 2N per-row chirp factors behind it
-  long long hhat_cache_n[FC_HHAT_SLOTS];   // key of slot i: length + ((band + 1) << 32), 0 = none
   cudaStream_t host_copy;
   cudaEvent_t *host_ev;
   int host_ev_cap;
@@ -288,7 +286,8 @@ __device__ __forceinline__ void dft_coprime(float2 (&x)[R1 * R2]) {
 
 template <int R, int DIR>
 __device__ __forceinline__ void dft_small(float2 (&x)[R]) {
-  if constexpr (R == 2) dft2<DIR>(x[0], x[1]);
+  if constexpr (R == 6) dft_coprime<2, 3, DIR>(x);
+  else if constexpr (R == 2) dft2<DIR>(x[0], x[1]);
   else if constexpr (R == 3) dft3<DIR>(x[0], x[1], x[2]);
   else if constexpr (R == 4) dft4<DIR>(x[0], x[1], x[2], x[3]);
   else if constexpr (R == 5) dft5<DIR>(x);
@@ -301,6 +300,59 @@ __device__ __forceinline__ void dft_small(float2 (&x)[R]) {
     static_assert(R == 16, "unsupported small DFT length");
     dft16<DIR>(x);
   }
+}
+
+// cos and sin of 2*pi*i/R for the lengths below, folded at compile time (i < R/2)
+template <int R>
+__host__ __device__ constexpr float root_cos(int i) {
+  constexpr float c16[8] = {1.f, 0.92387953251128675613f, 0.70710678118654752440f, 0.38268343236508977173f,
+                            0.f, -0.38268343236508977173f, -0.70710678118654752440f, -0.92387953251128675613f};
+  constexpr float c14[7] = {1.f, 0.90096886790241912624f, 0.62348980185873353053f, 0.22252093395631440429f,
+                            -0.22252093395631440429f, -0.62348980185873353053f, -0.90096886790241912624f};
+  constexpr float c12[6] = {1.f, 0.86602540378443864676f, 0.5f, 0.f, -0.5f, -0.86602540378443864676f};
+  constexpr float c10[5] = {1.f, 0.80901699437494742410f, 0.30901699437494742410f, -0.30901699437494742410f,
+                            -0.80901699437494742410f};
+  return R == 16 ? c16[i % 8] : R == 14 ? c14[i % 7] : R == 12 ? c12[i % 6] : c10[i % 5];
+}
+template <int R>
+__host__ __device__ constexpr float root_sin(int i) {
+  constexpr float s16[8] = {0.f, 0.38268343236508977173f, 0.70710678118654752440f, 0.92387953251128675613f,
+                            1.f, 0.92387953251128675613f, 0.70710678118654752440f, 0.38268343236508977173f};
+  constexpr float s14[7] = {0.f, 0.43388373911755812048f, 0.78183148246802980871f, 0.97492791218182360702f,
+                            0.97492791218182360702f, 0.78183148246802980871f, 0.43388373911755812048f};
+  constexpr float s12[6] = {0.f, 0.5f, 0.86602540378443864676f, 1.f, 0.86602540378443864676f, 0.5f};
+  constexpr float s10[5] = {0.f, 0.58778525229247312917f, 0.95105651629515357212f, 0.95105651629515357212f,
+                            0.58778525229247312917f};
+  return R == 16 ? s16[i % 8] : R == 14 ? s14[i % 7] : R == 12 ? s12[i % 6] : s10[i % 5];
+}
+
+// R-point DFT of R/2 samples followed by R/2 zeros: even bins are the R/2-point DFT of the samples, odd bins that of
+// the samples times w_R^n.
+template <int R>
+__device__ __forceinline__ void dft_zero_tail(const float2 (&x)[R / 2], float2 (&y)[R]) {
+  float2 e[R / 2], o[R / 2];
+#pragma unroll
+  for (int n = 0; n < R / 2; ++n) {
+    e[n] = x[n];
+    o[n] = n == 0 ? x[n] : cmul(x[n], make_float2(root_cos<R>(n), -root_sin<R>(n)));
+  }
+  dft_small<R / 2, -1>(e);
+  dft_small<R / 2, -1>(o);
+#pragma unroll
+  for (int k = 0; k < R / 2; ++k) { y[2 * k] = e[k]; y[2 * k + 1] = o[k]; }
+}
+
+// The first R/2 samples of the inverse R-point DFT (the mirror of the above).
+template <int R>
+__device__ __forceinline__ void idft_first_half(const float2 (&y)[R], float2 (&x)[R / 2]) {
+  float2 e[R / 2], o[R / 2];
+#pragma unroll
+  for (int k = 0; k < R / 2; ++k) { e[k] = y[2 * k]; o[k] = y[2 * k + 1]; }
+  dft_small<R / 2, +1>(e);
+  dft_small<R / 2, +1>(o);
+#pragma unroll
+  for (int n = 0; n < R / 2; ++n)
+    x[n] = n == 0 ? cadd(e[n], o[n]) : cadd(e[n], cmul(o[n], make_float2(root_cos<R>(n), root_sin<R>(n))));
 }
 
 // ------------------------------------------------------------------ batched stages in shared memory

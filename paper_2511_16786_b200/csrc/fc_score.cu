@@ -20,8 +20,10 @@
 //   pass 2  for every k1 (with N1-k1, which holds the partner bins N-q):
 //           twiddle, DFT over n2, the filter above, inverse DFT over k2, twiddle -> B[k1][n2]
 //   pass 3  for every n2: inverse DFT over k1, |.|^2 summed over the channels -> scores
-// Lengths that are not a power of two (or are below 16) go through Bluestein's
-// chirp convolution on a power-of-two length M >= 2N-1 with the same three passes.
+// Every other length up to 65536 takes the same three passes on a longer transform with the residual written as one
+// padded convolution (fc_score_fast.cuh).  The generic kernels of this file serve the power of two 131072, the spectrum
+// diagnostics and the entry point without allocation; there, lengths that are not a power of two (or are below 16) go
+// through Bluestein's chirp convolution on a power-of-two length M >= 2N-1.
 #include "fc_common.cuh"
 #include "fc_score_fast.cuh"
 
@@ -29,6 +31,7 @@
 #include <mutex>
 #include <type_traits>
 #include <unordered_map>
+#include <vector>
 
 namespace {
 
@@ -148,22 +151,15 @@ struct FilterLoader {
 };
 
 // Bluestein convolution kernel h[p] = chirp(|p|) wrapped to length M, in column 0.
-// band >= 0: the kernel of the band form, g[j] = chirp(|j - band|) for j = -(N-1) .. 2*band, wrapped (outputs
-// 0 .. 2*band of the convolution are the bins -band .. band; needs M >= N + 2*band).
 struct ChirpKernelLoader {
   static constexpr int VEC = 2;
-  int N, M, band;
+  int N, M;
   __device__ void init() {}
   __device__ void load(int p, int gc, float2 (&out)[2]) {
     out[0] = out[1] = make_float2(0.f, 0.f);
     if (gc != 0) return;
-    if (band < 0) {
-      if (p < N) out[0] = chirp(p, N);
-      else if (p > M - N) out[0] = chirp(M - p, N);
-    } else {
-      if (p <= 2 * band) out[0] = chirp(p < band ? band - p : p - band, N);
-      else if (p > M - N) out[0] = chirp(band + (M - p), N);
-    }
+    if (p < N) out[0] = chirp(p, N);
+    else if (p > M - N) out[0] = chirp(M - p, N);
   }
 };
 
@@ -603,8 +599,9 @@ __global__ void k_power_accumulate(const float2 *__restrict__ partial, int ny, i
   spectrum[2 * m + 1] = b;
 }
 
-__global__ void k_zero_energy(double *energy) {
-  if (threadIdx.x < 4) energy[threadIdx.x] = 0.0;
+// energy[l*stride .. +3] = 0 for the n layers of an empty sequence
+__global__ void k_zero_energy(double *energy, int n, long long stride) {
+  if ((int)threadIdx.x < 4 * n) energy[(threadIdx.x >> 2) * stride + (threadIdx.x & 3)] = 0.0;
 }
 
 // ---------------------------------------------------------------------------
@@ -614,189 +611,256 @@ inline int ilog2(int x) { int b = 0; while ((1 << b) < x) ++b; return b; }
 inline bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// ---- generic kernels: the power of two 131072, the spectrum diagnostics and the no-allocation entry point ----
 struct SeqPlan {
   bool bluestein;
-  bool fast;                 // specialised kernels (power-of-two N in [1024, 65536])
   int N, Nfft, N1, N2;
   int cs, cs2;               // columns per tile in pass 1/3 and pass 2
 };
 
-// Factors and tile widths of the generic kernels for the transform length s.Nfft.
-void finish_plan(SeqPlan &s) {
+SeqPlan plan_sequence(int N) {
+  SeqPlan s;
+  s.N = N;
+  s.bluestein = !(is_pow2(N) && N >= 16);
+  s.Nfft = N;
+  if (s.bluestein) {
+    s.Nfft = 64;
+    while (s.Nfft < 2 * N - 1) s.Nfft <<= 1;
+  }
   const int bits = ilog2(s.Nfft);
   int b1 = bits / 2;
-  if (b1 > 7 && !s.fast) b1 = 7;
+  if (b1 > 7) b1 = 7;
   s.cs = 64;
   // 131072 points: 256 x 512 with 32-column tiles in passes 1 and 3 beats 128 x 1024, whose pass 2 has
-  // room for only 4 columns per block (measured on the chirp path: 461 against 488 ms per step)
+  // room for only 4 columns per block
   if (bits == 17) { b1 = 8; s.cs = 32; }
-  // 8192 points on the specialised kernels: 128 x 64 keeps every pass at 256-thread blocks (2 % over 64 x 128)
-  if (s.fast && bits == 13) b1 = 7;
   s.N1 = 1 << b1;
   s.N2 = s.Nfft / s.N1;
   int cs2 = 4096 / s.N2;      // 2*N2*cs2*8 bytes = 64 KiB
   if (cs2 > 64) cs2 = 64;
   if (cs2 < 4) cs2 = 4;
   s.cs2 = cs2;
-}
-
-SeqPlan plan_sequence(int N, bool allow_fast = true) {
-  SeqPlan s;
-  s.N = N;
-  s.bluestein = !(is_pow2(N) && N >= 16);
-  if (s.bluestein) {
-    int M = 64;
-    while (M < 2 * N - 1) M <<= 1;
-    s.Nfft = M;
-  } else {
-    s.Nfft = N;
-  }
-  s.fast = allow_fast && !s.bluestein && N >= 1024 && N <= 65536;
-  finish_plan(s);
   return s;
 }
 
-// Shape of a chirp transform on the specialised kernels: M = N1 * N2 with N1 = a * r1b (first-stage radix a of
-// passes 1 and 3, then radix r1b) and N2 = 16 * r2b, or 2 * 16 * r2b when pass 2 takes its rows in two halves (dbl).
-// Powers of two 1024..131072 have a = 16; 2^k * {5, 3, 7} have a = 10, 12, 14 with r1b = 8 or 16.  a == 0: no such
-// shape.
-// Channel pairs per block of passes 1 and 3 on the chirp path: with a radix-16 second stage and rows of 128 points
-// or more, 16 pairs (256-thread blocks, two or three per SM) instead of 32 (512 threads, one per SM): measured
-// 10..14 % on transforms of 57344..98304 points, 2 % at 28672, while 224 x 64 loses 4 % that way.
-constexpr int chirp_cpw(int r1b, int r2b, bool dbl) { return (r1b == 16 && (r2b >= 8 || dbl)) ? 16 : 32; }
-
-struct ChirpShape {
-  int a, r1b, r2b;
-  bool dbl;
-  int n1() const { return a * r1b; }
-  int n2() const { return (dbl ? 32 : 16) * r2b; }
-};
-
-inline ChirpShape chirp_shape(int M) {
-  ChirpShape c{0, 0, 0, false};
-  if (M == 131072) return ChirpShape{16, 16, 16, true};          // 256 x 512
-  if (is_pow2(M)) {
-    if (M < 1024 || M > 65536) return c;
-    const int bits = ilog2(M), b1 = bits / 2;
-    return ChirpShape{16, (1 << b1) / 16, (M >> b1) / 16, false};
-  }
-  const int a = (M % 5 == 0) ? 10 : (M % 3 == 0) ? 12 : (M % 7 == 0) ? 14 : 0;
-  if (a == 0 || M % (16 * a) != 0) return c;
-  // a = 10 and 12 with rows of 128 or 256 points run faster on a radix-8 second stage (80 or 96 x N2) than on
-  // 160 or 192 x N2/2: measured 3..10 % on the whole chirp path; a = 14 loses 8 % that way, and rows of 512 points
-  // (two halves per row in pass 2) lose 14 % against 160 or 192 x 256
-  const int n2w = M / (8 * a);
-  if (a != 14 && (n2w == 128 || n2w == 256)) return ChirpShape{a, 8, n2w / 16, false};
-  const int n2 = M / (16 * a);
-  if (!is_pow2(n2) || n2 < 32 || n2 > 512) return c;
-  return n2 == 512 ? ChirpShape{a, 16, 16, true} : ChirpShape{a, 16, n2 / 16, false};
-}
-
-// Smallest transform length >= need the specialised kernels take (0 if none up to 131072).
-inline int chirp_length(long long need) {
-  int best = 0;
-  for (int M = 1024; M <= 131072; M <<= 1)
-    if (M >= need) { best = M; break; }
-  for (int n1 = 160; n1 <= 224; n1 += 32)
-    for (int n2 = 32; n2 <= 512; n2 <<= 1) {
-      const int M = n1 * n2;
-      if (M >= need && (best == 0 || M < best)) best = M;
-    }
-  return best;
-}
-
-struct ScoreLayout {
+struct GenericLayout {
   size_t off_ws, off_spec, off_hhat, off_hcol, off_part_tot, off_part_hi, total;
-  size_t part_tot_bytes, part_hi_bytes;   // one copy; the specialised path keeps two and alternates (step parity)
-  size_t ws_buf_bytes;       // one group buffer; the fast path keeps two and alternates
   int heads_per_group;
-  int sub_cols;              // chirp path: columns of one head transformed together (head_dim = all of them)
-  int chirp_streams;         // chirp path: internal streams the head groups alternate over (1 = the caller's stream)
-  size_t spec_buf_bytes;     // chirp path: one group's N-point spectrum; one copy per stream
-  size_t layer_bytes;        // intermediates of all heads of the sequence together
+  int sub_cols;              // chirp form: columns of one head transformed together (head_dim = all of them)
 };
 
-// Workspace carve-up for one sequence plan (all sequences share the regions; the
-// query takes the maximum over the sequences of the view).
-ScoreLayout layout_for(const fc_handle *h, const SeqPlan &sp, int num_heads, int head_dim) {
-  ScoreLayout L;
+// Workspace carve-up for one sequence (all sequences share the regions; the query takes the maximum over the view).
+GenericLayout generic_layout(const fc_handle *h, const SeqPlan &sp, int num_heads, int head_dim) {
+  GenericLayout L;
   const size_t per_head = (size_t)sp.Nfft * head_dim * sizeof(float2);
-  L.layer_bytes = per_head * (size_t)num_heads;
   int hg = (int)(h->group_bytes / per_head);
   if (hg < 1) hg = 1;
   if (hg > num_heads) hg = num_heads;
-  int groups = (num_heads + hg - 1) / hg;
-  // Chirp transforms on the specialised kernels also alternate their head groups over the internal streams (two
-  // kernels in flight fill the GPU better; measured 20-25 % on 2500..15000 tokens and still 8 % where the two
-  // groups' intermediates no longer fit the L2 together).
-  const bool chirp_multi = sp.bluestein && !h->generic_only && h->aux[0] != nullptr && sp.Nfft >= 1024 &&
-                           sp.Nfft <= 131072 && num_heads >= h->num_aux && h->num_aux > 1;
-  // Power-of-two path, all heads fit one group: they stay one group (fuller launches) and consecutive calls alternate
-  // over the internal streams, where calls overlap (fc_set_score_overlap: 28 layers x 4 heads of 8192 tokens 1.31 ->
-  // 1.11 ms) or the whole layer is tiny (8 MiB: 44 -> 31 us per call at 4 heads of 1024 tokens); otherwise a call
-  // that has to finish before it returns is faster with its heads on both streams (49 against 56 us per layer).
-  const int hg_alloc = hg;                                     // the workspace does not depend on the mode
-  const bool one_group = sp.fast && groups == 1 && (h->score_overlap || L.layer_bytes <= ((size_t)8 << 20));
-  if ((sp.fast || chirp_multi) && groups < h->num_aux && num_heads >= h->num_aux && !one_group)
-    groups = h->num_aux;                                       // keep every internal stream busy
+  const int groups = (num_heads + hg - 1) / hg;
   hg = (num_heads + groups - 1) / groups;                      // balanced groups
   L.heads_per_group = hg;
-  L.chirp_streams = chirp_multi ? h->num_aux : 1;
-  // Chirp path, one head per group: the head is split into column groups only when its intermediates
-  // pass four times the budget.  Narrower tiles cost time (measured: +2 % at 64 columns, +8 % at 32 for
-  // 131072-point transforms) and the generic kernels do not wait on DRAM, so below that the split
-  // would only save workspace.
+  // A single head whose intermediates pass four times the budget is split into column groups: a workspace saving
+  // (narrower tiles cost 2..8 % of the time).
   int sub = head_dim;
   const size_t split_above = h->group_bytes > ((size_t)1 << 60) ? h->group_bytes : 4 * h->group_bytes;
-  if (sp.bluestein && hg == 1) {
-    // specialised kernels: the intermediates of the groups in flight (one per internal stream) should stay in the
-    // cache, so a head is halved down to 64 columns while they exceed three times the budget (measured on eight
-    // ragged sequences of 7k..54k tokens: 1.6 % of the step; the length is the full form's, the band form's is shorter)
-    const int Mf = h->generic_only ? 0 : chirp_length(2LL * sp.N - 1);
-    if (Mf != 0 && Mf <= sp.Nfft)
-      while (sub % 128 == 0 && (size_t)(chirp_multi ? h->num_aux : 1) * Mf * sub * sizeof(float2) > 3 * h->group_bytes)
-        sub /= 2;
+  if (sp.bluestein && hg == 1)
     while (sub % 64 == 0 && (size_t)sp.Nfft * sub * sizeof(float2) > split_above) sub /= 2;
-  }
   L.sub_cols = sub;
-  L.ws_buf_bytes = align_up((size_t)sp.Nfft * sub * (sp.fast ? hg_alloc : hg) * sizeof(float2), 256);
   size_t off = 0;
-  L.off_ws = off;       off += L.ws_buf_bytes * (sp.fast ? h->num_aux : L.chirp_streams);
-  L.spec_buf_bytes = sp.bluestein ? align_up((size_t)sp.N * sub * hg * sizeof(float2), 256) : 0;
-  L.off_spec = off;     off += L.spec_buf_bytes * L.chirp_streams;
+  L.off_ws = off;       off += align_up((size_t)sp.Nfft * sub * hg * sizeof(float2), 256);
+  L.off_spec = off;     off += sp.bluestein ? align_up((size_t)sp.N * sub * hg * sizeof(float2), 256) : 0;
   L.off_hhat = off;     off += sp.bluestein ? align_up((size_t)sp.Nfft * sizeof(float2), 256) : 0;
   L.off_hcol = off;     off += sp.bluestein ? align_up((size_t)sp.Nfft * 8 * sizeof(float2), 256) : 0;
   const size_t slices = (size_t)num_heads * head_dim / 32;   // finest slicing any kernel variant uses
-  L.part_tot_bytes = align_up(slices * sp.N2 * 2 * sizeof(double), 256);
-  L.part_hi_bytes = align_up((size_t)num_heads * (head_dim / sub) * sp.N2 * 2 * sizeof(double), 256);
-  L.off_part_tot = off; off += L.part_tot_bytes * (sp.fast ? 2 : 1);
-  L.off_part_hi = off;  off += L.part_hi_bytes * (sp.fast ? 2 : 1);
+  L.off_part_tot = off; off += align_up(slices * sp.N2 * 2 * sizeof(double), 256);
+  L.off_part_hi = off;  off += align_up((size_t)num_heads * (head_dim / sub) * sp.N2 * 2 * sizeof(double), 256);
   L.total = off;
   return L;
 }
 
-// The specialised path keeps each internal stream's intermediate buffer in the persisting part of L2.
+// ---- the specialised passes (fc_score_fast.cuh) ----
+struct PassPlan {
+  bool ok;                   // false: the length is left to the generic kernels
+  bool pad;                  // padded form (else direct: M == N)
+  int N, M, N1, N2;
+  int a, r1b, r2b;           // N1 = a * r1b, N2 = 16 * r2b (32 * r2b with dbl)
+  bool dbl;                  // pass 2 takes its rows in two halves
+  int cpw, cp;               // channel pairs per block of passes 1 and 3, per row tile of pass 2
+};
+
+// Shapes of the padded form: M = 2^k * {1, 5/4, 3/2, 7/4} from 1024 to 131072 (27 lengths, so that 2N-1 is padded by
+// 1.12 on average).  a = 10 and 12 with rows of 128 or 256 points run 3..10 % faster on a radix-8 second stage
+// (80 or 96 x N2) than on 160 or 192 x N2/2; a = 14 loses 8 % that way, and rows of 512 points lose 14 % against 160 or
+// 192 x 256.
+inline PassPlan pad_shape(int M) {
+  PassPlan p = {};
+  p.pad = true;
+  p.M = M;
+  p.a = is_pow2(M) ? 16 : (M % 5 == 0) ? 10 : (M % 3 == 0) ? 12 : 14;
+  if (p.a == 16) {
+    if (M < 1024 || M > 131072) return p;
+    const int bits = ilog2(M), b1 = bits / 2 > 8 ? 8 : bits / 2;
+    p.r1b = (1 << b1) / 16;
+  } else {
+    const int rest = M / p.a;                    // r1b * N2
+    if (M % (128 * p.a) != 0 || !is_pow2(rest)) return p;
+    if (rest <= 512) p.r1b = rest / 32;          // rows of 32 points
+    else if (p.a != 14 && (rest == 1024 || rest == 2048)) p.r1b = 8;
+    else p.r1b = 16;
+  }
+  p.N1 = p.a * p.r1b;
+  p.N2 = M / p.N1;
+  if (p.N2 < 32 || p.N2 > 512 || p.r1b < 2) return p;
+  p.dbl = p.N2 == 512;
+  p.r2b = p.dbl ? 16 : p.N2 / 16;
+  // radix-16 second stage and rows of 128 points or more: 16 pairs (256-thread blocks, two or three per SM) instead of
+  // 32 (512 threads, one per SM), 10..14 % on transforms of 57344..98304 points; shorter rows lose 4 % that way
+  p.cpw = (p.r1b == 16 && p.N2 >= 128) ? 16 : 32;
+  // 256-thread blocks in pass 2
+  p.cp = p.dbl ? 4 : p.r2b == 16 ? 8 : p.r2b == 8 ? 16 : 32;
+  p.ok = true;
+  return p;
+}
+
+// How a sequence of N tokens is transformed.
+PassPlan plan_passes(int N) {
+  PassPlan p = {};
+  if (is_pow2(N) && N >= 1024) {
+    if (N > 65536) return p;
+    const int bits = ilog2(N);
+    // 8192 points: 128 x 64 keeps every pass at 256-thread blocks (2 % over 64 x 128)
+    const int b1 = bits == 13 ? 7 : bits / 2;
+    p.N = p.M = N;
+    p.a = 16;
+    p.r1b = (1 << b1) / 16;
+    p.N1 = 1 << b1;
+    p.N2 = N / p.N1;
+    p.r2b = p.N2 / 16;
+    // every pass runs 256-thread blocks from 8192 points on, the measured optimum
+    p.cpw = p.N1 == 256 ? 16 : 32;
+    p.cp = (N == 8192) ? 32 : (N == 16384) ? 16 : 8;
+    p.ok = true;
+    return p;
+  }
+  if (N > 65536) return p;
+  // smallest padded length >= 2N - 1
+  int best = 0;
+  const int need = 2 * N - 1;
+  for (int k = 10; k <= 17; ++k)
+    for (int f = 4; f <= 7; ++f) {
+      const int M = (1 << k) / 4 * f;
+      if (M >= need && (best == 0 || M < best) && pad_shape(M).ok) best = M;
+    }
+  if (best == 0) return p;
+  p = pad_shape(best);
+  p.N = N;
+  return p;
+}
+
+// How one sequence's units (layer, head) are grouped into launches.
+struct GroupPlan {
+  int units;                 // units per launch
+  int sub, ngr;              // columns of a unit per launch and launches per unit (ngr > 1 only with units == 1)
+  size_t buf_bytes;          // intermediates of one launch (one copy per internal stream)
+  size_t layer_bytes;        // intermediates of all heads of one layer together
+};
+
+GroupPlan plan_groups(const fc_handle *h, const PassPlan &p, int num_units, int num_heads, int head_dim) {
+  GroupPlan g;
+  const size_t per_unit = (size_t)p.M * head_dim * sizeof(float2);
+  g.layer_bytes = per_unit * (size_t)num_heads;
+  int nu = (int)(h->group_bytes / per_unit);
+  if (nu < 1) nu = 1;
+  if (nu > num_units) nu = num_units;
+  int groups = (num_units + nu - 1) / nu;
+  const int nu_alloc = nu;                                     // the workspace does not depend on the mode
+  // All units fit one group: they stay one group (fuller launches) and consecutive calls alternate over the internal
+  // streams, where calls overlap (fc_set_score_overlap: 28 calls of 4 heads of 8192 tokens 1.31 -> 1.11 ms) or the
+  // whole call is tiny (8 MiB: 44 -> 31 us per call at 4 heads of 1024 tokens); otherwise a call that has to finish
+  // before it returns is faster with its units on both streams (49 against 56 us per layer of 4 heads of 8192 tokens).
+  const bool one_group = groups == 1 && (h->score_overlap || per_unit * (size_t)num_units <= ((size_t)8 << 20));
+  if (groups < h->num_aux && num_units >= h->num_aux && !one_group) groups = h->num_aux;
+  g.units = (num_units + groups - 1) / groups;                 // balanced groups
+  g.sub = head_dim;
+  if (p.pad && nu_alloc == 1) {
+    // the intermediates of the groups in flight (one per internal stream) should stay in the cache, so a unit is
+    // halved down to 64 columns while they exceed three times the budget
+    while (g.sub % 128 == 0 && (size_t)h->num_aux * p.M * g.sub * sizeof(float2) > 3 * h->group_bytes) g.sub /= 2;
+  }
+  g.ngr = head_dim / g.sub;
+  g.buf_bytes = align_up((size_t)p.M * g.sub * nu_alloc * sizeof(float2), 256);
+  return g;
+}
+
+// Workspace carve-up of one scoring call: the regions hold the largest sequence of the view.
+struct ScoreLayout {
+  size_t buf_bytes;          // intermediates, one buffer per internal stream
+  size_t off_buf, off_tab, off_tot, off_hi, total;
+  size_t tot_bytes, hi_bytes;   // per-block partial sums of one step; two copies, used in turn
+};
+
+inline bool first_of_its_length(const fc_kv_view *kv, int b) {
+  const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
+  for (int i = 0; i < b; ++i)
+    if (kv->cu_seqlens[i + 1] - kv->cu_seqlens[i] == N) return false;
+  return true;
+}
+
+ScoreLayout score_layout(const fc_handle *h, const fc_kv_view *kv, int num_layers) {
+  ScoreLayout L = {};
+  const int H = kv->num_heads, d = kv->head_dim, nl = num_layers < FC_LAYER_CHUNK ? num_layers : FC_LAYER_CHUNK;
+  size_t tab = 0, generic = 0;
+  for (int b = 0; b < kv->batch; ++b) {
+    const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
+    if (N == 0) continue;
+    const PassPlan p = plan_passes(N);
+    if (!p.ok || h->generic_only) {
+      const size_t t = generic_layout(h, plan_sequence(N), H, d).total;
+      if (t > generic) generic = t;
+      continue;
+    }
+    const GroupPlan g = plan_groups(h, p, nl * H, H, d);
+    const size_t tot = (size_t)nl * H * (d / (2 * p.cpw)) * p.N2 * 2 * sizeof(double);
+    const size_t hi = (size_t)nl * H * g.ngr * p.N2 * 2 * sizeof(double);
+    if (g.buf_bytes > L.buf_bytes) L.buf_bytes = g.buf_bytes;
+    if (tot > L.tot_bytes) L.tot_bytes = tot;
+    if (hi > L.hi_bytes) L.hi_bytes = hi;
+    if (p.pad && first_of_its_length(kv, b)) tab += (size_t)p.M * sizeof(float4);
+  }
+  L.tot_bytes = align_up(L.tot_bytes, 256);
+  L.hi_bytes = align_up(L.hi_bytes, 256);
+  size_t off = 0;
+  L.off_buf = off; off += L.buf_bytes * h->num_aux;
+  L.off_tab = off; off += align_up(tab, 256);
+  L.off_tot = off; off += 2 * L.tot_bytes;
+  L.off_hi = off;  off += 2 * L.hi_bytes;
+  L.total = off > generic ? off : generic;
+  if (L.total < 256) L.total = 256;
+  return L;
+}
+
+// Each internal stream's intermediate buffer is kept in the persisting part of L2, on the direct path only.
 // Not where the intermediates of all heads of the sequence are small against the cache (48 MiB: they stay
 // resident anyway and the set-aside only takes cache from the rows and scores; measured -2.5 % at 4 heads of 8192
 // tokens with the window, +1.6 % and +4 % at 2 and 4 heads of 32768, no difference at 64 MiB).
-bool window_fits(const fc_handle *h, const ScoreLayout &L) {
-  return h->l2_persist && L.layer_bytes > ((size_t)48 << 20) && L.ws_buf_bytes <= h->window_max &&
-         L.ws_buf_bytes * (size_t)h->num_aux <= h->persist_max;
+bool window_fits(const fc_handle *h, const PassPlan &p, const GroupPlan &g) {
+  return h->l2_persist && p.ok && !p.pad && g.layer_bytes > ((size_t)48 << 20) && g.buf_bytes <= h->window_max &&
+         g.buf_bytes * (size_t)h->num_aux <= h->persist_max;
 }
 
 // The persisting part of L2 is a limit of the whole context, shared by the handles of a device (fc_persist_acquire):
-// held while calls contain a sequence for the specialised path, let go when a call has none (the generic kernels
-// lose about a tenth of their speed to a set-aside they do not use).  Decided once per call; left as it is while
-// `st` is being captured into a graph, where device-wide settings cannot change.
-void claim_persisting_l2(fc_handle *h, const fc_kv_view *kv, cudaStream_t st) {
-  if (!h->l2_persist || h->generic_only) return;
+// held while calls contain a sequence that wants it, let go when a call has none.  Decided once per call; left as it is
+// while `st` is being captured into a graph, where device-wide settings cannot change.
+void claim_persisting_l2(fc_handle *h, const fc_kv_view *kv, int num_layers, cudaStream_t st) {
+  if (!h->l2_persist) return;
+  const int nl = num_layers < FC_LAYER_CHUNK ? num_layers : FC_LAYER_CHUNK;
   bool claim = false;
   for (int b = 0; b < kv->batch && !claim; ++b) {
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0) continue;
-    const SeqPlan sp = plan_sequence(N);
-    if (!sp.fast) continue;
-    claim = window_fits(h, layout_for(h, sp, kv->num_heads, kv->head_dim));
+    const PassPlan p = plan_passes(N);
+    if (!p.ok || p.pad) continue;
+    claim = window_fits(h, p, plan_groups(h, p, nl * kv->num_heads, kv->num_heads, kv->head_dim));
   }
   if (claim == (h->persist_on != 0)) return;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -809,8 +873,9 @@ void claim_persisting_l2(fc_handle *h, const fc_kv_view *kv, cudaStream_t st) {
   }
 }
 
-fc_status validate_view(const fc_handle *h, const fc_kv_view *kv) {
-  if (!h || !kv || !kv->k || !kv->v || !kv->cu_seqlens) return FC_ERR_INVALID_ARG;
+// `pointers`: the view's own k and v are checked too
+fc_status validate_view(const fc_handle *h, const fc_kv_view *kv, bool pointers) {
+  if (!h || !kv || !kv->cu_seqlens || (pointers && (!kv->k || !kv->v))) return FC_ERR_INVALID_ARG;
   if (kv->num_heads <= 0 || kv->head_dim <= 0 || kv->batch < 0) return FC_ERR_INVALID_ARG;
   if (kv->dtype != FC_F32 && kv->dtype != FC_F16 && kv->dtype != FC_BF16) return FC_ERR_UNSUPPORTED;
   if (kv->head_dim % 64 != 0) return FC_ERR_UNSUPPORTED;
@@ -824,7 +889,7 @@ fc_status validate_view(const fc_handle *h, const fc_kv_view *kv) {
   }
   if (kv->stride_token < (long long)kv->head_dim || kv->stride_head < (long long)kv->head_dim)
     return FC_ERR_INVALID_ARG;
-  if (((uintptr_t)kv->k & 15) || ((uintptr_t)kv->v & 15)) return FC_ERR_INVALID_ARG;
+  if (pointers && (((uintptr_t)kv->k & 15) || ((uintptr_t)kv->v & 15))) return FC_ERR_INVALID_ARG;
   if ((kv->stride_token * es) % 16 || (kv->stride_head * es) % 16) return FC_ERR_INVALID_ARG;
   return FC_OK;
 }
@@ -883,204 +948,127 @@ fc_status launch_pass2(fc_handle *h, cudaStream_t st, const SeqPlan &sp, int nco
   return fc_after_launch(h);
 }
 
-// The three specialised launches for one head group of a power-of-two sequence.
-// Channel pairs per block of passes 1 and 3 on the power-of-two path for a first factor n1.
-constexpr int fast_cpw(int n1, int cpw) { return n1 == 256 ? 16 : cpw; }
+// ---- launches of the specialised passes ----
+struct PassArgs {
+  fc_handle *h;
+  cudaStream_t st;
+  const PassPlan *p;
+  const fast::LayerPtrs *lp;
+  const fc_kv_view *kv;
+  int u0, nu, c0, cols;      // units of the launch; first channel and channels per unit
+  int omega;
+  float2 *ws;
+  const float4 *tab;
+};
 
-// CPW: channel pairs per block in passes 1 and 3; CP: channel pairs per half tile in pass 2.
-template <typename T, int R1B, int R2B, int CPW, int CP>
-fc_status launch_fast_impl(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const T *kp, const T *vp,
-                           const SeqPlan &sp, int h0, int hg, int omega, float2 *ws, double *ptot,
-                           double *phi, float *scores, long long total_tokens, const double *part_tot,
-                           const double *part_hi, double *energy_b) {
-  constexpr int N1 = 16 * R1B, N2 = 16 * R2B;
-  const int d = kv->head_dim, ncol_ws = hg * d;
-  const size_t sm1 = (size_t)N1 * CPW * sizeof(float4) + N1 * sizeof(float2);
-  const size_t sm2 = (size_t)2 * N2 * CP * sizeof(float4) + (5 * N2 + 16) * sizeof(float2);
-  fc_status s;
-  if ((s = set_smem(fast::k_p1<T, R1B, CPW>, sm1)) != FC_OK) return s;
-  {
-    ProfScope ps(h, FC_K_PASS1, st);
-    fast::k_p1<T, R1B, CPW><<<dim3(N2, ncol_ws / (2 * CPW)), CPW * R1B, sm1, st>>>(
-        kp, vp, kv->stride_token, kv->stride_head, h0, d, sp.N, N2, ncol_ws, ws, h->master, h->master_len, ptot);
-  }
-  if ((s = fc_after_launch(h)) != FC_OK) return s;
-  if ((s = set_smem(fast::k_p2<R2B, CP>, sm2)) != FC_OK) return s;
-  {
-    ProfScope ps(h, FC_K_PASS2, st);
-    fast::k_p2<R2B, CP><<<dim3(N1 / 2, ncol_ws / (2 * CP)), 2 * CP * R2B, sm2, st>>>(
-        N1, ncol_ws, ws, h->master, h->master_len, omega);
-  }
-  if ((s = fc_after_launch(h)) != FC_OK) return s;
-  if ((s = set_smem(fast::k_p3<R1B, CPW>, sm1)) != FC_OK) return s;
-  {
-    ProfScope ps(h, FC_K_PASS3, st);
-    const float inv = (float)(1.0 / ((double)sp.N * (double)sp.N * (double)d));
-    const int H = kv->num_heads;
-    fast::k_p3<R1B, CPW><<<dim3(N2, hg), CPW * R1B, sm1, st>>>(
-        sp.N, N2, ncol_ws, ws, h->master, h->master_len, scores, h0, d, total_tokens, inv, phi,
-        h->done_counter + (h->step & 1u), (unsigned)(N2 * H), part_tot, N2 * (H * d / (2 * CPW)), part_hi, N2 * H, energy_b);
-  }
-  return fc_after_launch(h);
+inline size_t smem_outer(const PassPlan &p) { return (size_t)p.N1 * p.cpw * sizeof(float4) + p.N1 * sizeof(float2); }
+
+template <typename T, int A, int R1B, int CPW, int LD>
+fc_status launch_p1(const PassArgs &x, double *part_tot, int layer_slots) {
+  const PassPlan &p = *x.p;
+  const size_t sm = smem_outer(p);
+  const int ncol = LD == fast::LD_TABLE ? 2 * CPW : x.nu * x.cols;
+  fc_status s = set_smem(fast::k_p1<T, R1B, CPW, LD, A>, sm);
+  if (s != FC_OK) return s;
+  ProfScope ps(x.h, FC_K_PASS1, x.st);
+  fast::k_p1<T, R1B, CPW, LD, A><<<dim3(p.N2, ncol / (2 * CPW)), CPW * R1B, sm, x.st>>>(
+      *x.lp, x.kv->stride_token, x.kv->stride_head, x.kv->num_heads, x.kv->head_dim, x.u0, x.c0, x.cols, p.N, p.N2, ncol,
+      x.ws, x.h->master, x.h->master_len, part_tot, layer_slots, x.omega);
+  return fc_after_launch(x.h);
 }
 
-template <typename T, int CPW, int CP>
-fc_status launch_fast_tuned(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const T *kp, const T *vp,
-                            const SeqPlan &sp, int h0, int hg, int omega, float2 *ws, double *ptot, double *phi,
-                            float *scores, long long total_tokens, const double *part_tot,
-                            const double *part_hi, double *energy_b) {
-  // Every pass runs 256-thread blocks, the measured optimum: CPWV channel pairs per block in passes 1 and 3 and CPV
-  // per half tile in pass 2 follow from the factors (CPW and CP are the widths for 128 x 256).
-#define FC_FAST_CASE(A, B, CPWV, CPV)                                                                     \
-  if (sp.N1 == 16 * A && sp.N2 == 16 * B)                                                                 \
-    return launch_fast_impl<T, A, B, CPWV, CPV>(h, st, kv, kp, vp, sp, h0, hg, omega, ws, ptot, phi, scores, \
-                                                total_tokens, part_tot, part_hi, energy_b);
-  FC_FAST_CASE(2, 2, CPW, CP) FC_FAST_CASE(2, 4, CPW, CP) FC_FAST_CASE(4, 4, CPW, CP) FC_FAST_CASE(4, 8, CPW, CP)
-  FC_FAST_CASE(8, 4, CPW, 4 * CP)                 // 8192 = 128 x 64
-  FC_FAST_CASE(8, 8, CPW, 2 * CP)                 // 16384 = 128 x 128
-  FC_FAST_CASE(8, 16, CPW, CP)                    // 32768 = 128 x 256
-  FC_FAST_CASE(16, 16, fast_cpw(256, CPW), CP)    // 65536 = 256 x 256
-#undef FC_FAST_CASE
+// first-stage radix, second-stage radix and channel pairs of passes 1 and 3: the shapes plan_passes gives
+#define FC_OUTER_PAD_SHAPES(X)                                                                                \
+  X(16, 2, 32) X(16, 4, 32) X(16, 8, 32) X(16, 16, 16) X(14, 4, 32) X(14, 8, 32) X(14, 16, 32) X(14, 16, 16) \
+  X(12, 4, 32) X(12, 8, 32) X(12, 16, 32) X(12, 16, 16) X(10, 4, 32) X(10, 8, 32) X(10, 16, 32) X(10, 16, 16)
+#define FC_OUTER_DIRECT_SHAPES(X) X(16, 2, 32) X(16, 4, 32) X(16, 8, 32) X(16, 16, 16)
+
+template <typename T>
+fc_status run_p1(const PassArgs &x, double *part_tot, int layer_slots) {
+  const PassPlan &p = *x.p;
+#define FC_P1(A_, R_, C_)                                                  \
+  if (p.pad && p.a == A_ && p.r1b == R_ && p.cpw == C_)                    \
+    return launch_p1<T, A_, R_, C_, fast::LD_PAD>(x, part_tot, layer_slots);
+  FC_OUTER_PAD_SHAPES(FC_P1)
+#undef FC_P1
+#define FC_P1(A_, R_, C_)                                                  \
+  if (!p.pad && p.a == A_ && p.r1b == R_ && p.cpw == C_)                   \
+    return launch_p1<T, A_, R_, C_, fast::LD_KV>(x, part_tot, layer_slots);
+  FC_OUTER_DIRECT_SHAPES(FC_P1)
+#undef FC_P1
   return FC_ERR_INTERNAL;
 }
 
-template <typename T>
-fc_status launch_fast(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const T *kp, const T *vp,
-                      const SeqPlan &sp, int h0, int hg, int omega, float2 *ws, double *ptot, double *phi,
-                      float *scores, long long total_tokens, const double *part_tot, const double *part_hi,
-                      double *energy_b) {
-#define FC_TUNE_CASE(W, C)                                                                              \
-  if (h->tune_cpw == W && h->tune_cp == C)                                                              \
-    return launch_fast_tuned<T, W, C>(h, st, kv, kp, vp, sp, h0, hg, omega, ws, ptot, phi, scores,       \
-                                      total_tokens, part_tot, part_hi, energy_b);
-  FC_TUNE_CASE(32, 8)
-#undef FC_TUNE_CASE
+fc_status run_p1_table(const PassArgs &x) {
+  const PassPlan &p = *x.p;
+#define FC_P1(A_, R_, C_) \
+  if (p.a == A_ && p.r1b == R_ && p.cpw == C_) return launch_p1<float, A_, R_, C_, fast::LD_TABLE>(x, nullptr, 0);
+  FC_OUTER_PAD_SHAPES(FC_P1)
+#undef FC_P1
   return FC_ERR_INTERNAL;
 }
 
-// The chirp path on the specialised kernels: two circular convolutions with the chirp kernel, each
-// pass 1 -> pass 2 (multiply by the kernel's spectrum) -> pass 3, on one stream.  Tile widths fixed.
-// DOUBLE: rows of 2 * 16 * R2B points, pass 2 joins two half-length transforms per row.
-// hout != nullptr: only the spectrum of the convolution kernel itself is computed (pass 1 with the kernel in column
-// 0 of a 64-column tile, the forward half of pass 2) and written to hout[0 .. M).
-template <typename T, int A, int R1B, int R2B, bool DOUBLE>
-fc_status launch_chirp_impl(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const T *kp, const T *vp, int Nseq,
-                            int h0, int hg, int omega, float2 *ws, float2 *spec, const float2 *hhat, double *ptot,
-                            double *phi, float *scores, long long total_tokens, int dcols, int accumulate, int band,
-                            float2 *hout, const float2 *ctab) {
-  constexpr int CPW = chirp_cpw(R1B, R2B, DOUBLE), CP = 8, N1 = A * R1B, N2 = (DOUBLE ? 32 : 16) * R2B;
-  constexpr int MIDV = DOUBLE ? fast::MID_CONV2 : fast::MID_CONV;
-  const size_t sm1 = (size_t)N1 * CPW * sizeof(float4) + N1 * sizeof(float2);
-  const size_t sm2 = (size_t)2 * (16 * R2B) * CP * sizeof(float4) + (7 * (16 * R2B) + 16) * sizeof(float2);
-  // band form's last pass, 16-bit inputs: staging slots for the K/V rows it reads again
-  const size_t sm3b = sm1 + (sizeof(T) == 2 ? (size_t)2 * A * CPW * R1B * sizeof(unsigned) : 0);
-  fc_status s;
-  if ((s = set_smem(fast::k_p2<R2B, CP, MIDV>, sm2)) != FC_OK) return s;
-  if (hout != nullptr) {
-    if ((s = set_smem(fast::k_p1<float, R1B, CPW, fast::LD_KERNEL, A>, sm1)) != FC_OK) return s;
-    {
-      ProfScope ps(h, FC_K_PASS1, st);
-      fast::k_p1<float, R1B, CPW, fast::LD_KERNEL, A><<<dim3(N2, 1), CPW * R1B, sm1, st>>>(
-          nullptr, nullptr, 0, 0, 0, 2 * CPW, Nseq, N2, 2 * CPW, ws, h->master, h->master_len, nullptr, nullptr, band);
-    }
-    if ((s = fc_after_launch(h)) != FC_OK) return s;
-    {
-      ProfScope ps(h, FC_K_PASS2, st);
-      fast::k_p2<R2B, CP, MIDV><<<dim3(DOUBLE ? N1 : N1 / 2, 1), 2 * CP * R2B, sm2, st>>>(
-          N1, 2 * CPW, ws, h->master, h->master_len, 0, nullptr, 1.f, 0, hout);
-    }
-    return fc_after_launch(h);
-  }
-  // dcols: columns of a head in this launch (head_dim, or a column group of one head: kp/vp point at its
-  // first channel and hg is 1)
-  const int d = kv->head_dim, ncol = hg * dcols;
-  const float invM = 1.f / (float)(N1 * N2);
-  const dim3 g1(N2, ncol / (2 * CPW)), g2(DOUBLE ? N1 : N1 / 2, ncol / (2 * CP)), g3(N2, hg);
-  if ((s = set_smem(fast::k_p1<T, R1B, CPW, fast::LD_CHIRP, A>, sm1)) != FC_OK) return s;
-  if ((s = set_smem(fast::k_p3<R1B, CPW, fast::OUT_SPEC, float, A>, sm1)) != FC_OK) return s;
-  if (band >= 0) {
-    if ((s = set_smem(fast::k_p1<float, R1B, CPW, fast::LD_BAND, A>, sm1)) != FC_OK) return s;
-    if ((s = set_smem(fast::k_p3<R1B, CPW, fast::OUT_SCORE_BAND, T, A>, sm3b)) != FC_OK) return s;
-  } else {
-    if ((s = set_smem(fast::k_p1<float, R1B, CPW, fast::LD_FILTER, A>, sm1)) != FC_OK) return s;
-    if ((s = set_smem(fast::k_p3<R1B, CPW, fast::OUT_SCORE_CHIRP, float, A>, sm1)) != FC_OK) return s;
-  }
-  {
-    ProfScope ps(h, FC_K_PASS1, st);
-    fast::k_p1<T, R1B, CPW, fast::LD_CHIRP, A><<<g1, CPW * R1B, sm1, st>>>(
-        kp, vp, kv->stride_token, kv->stride_head, h0, dcols, Nseq, N2, ncol, ws, h->master, h->master_len, ptot,
-        nullptr, 0, ctab);
-  }
-  if ((s = fc_after_launch(h)) != FC_OK) return s;
-  {
-    ProfScope ps(h, FC_K_PASS2, st);
-    fast::k_p2<R2B, CP, MIDV><<<g2, 2 * CP * R2B, sm2, st>>>(N1, ncol, ws, h->master, h->master_len, 0, hhat, invM);
-  }
-  if ((s = fc_after_launch(h)) != FC_OK) return s;
-  {
-    ProfScope ps(h, FC_K_PASS3, st);
-    fast::k_p3<R1B, CPW, fast::OUT_SPEC, float, A><<<g3, CPW * R1B, sm1, st>>>(
-        Nseq, N2, ncol, ws, h->master, h->master_len, nullptr, h0, dcols, 0, 0.f, nullptr, nullptr, 0u, nullptr, 0, nullptr, 0,
-        nullptr, spec, 0.f, 0, band, nullptr, nullptr, 0, 0, ctab);
-  }
-  if ((s = fc_after_launch(h)) != FC_OK) return s;
-  {
-    ProfScope ps(h, FC_K_PASS1, st);
-    if (band >= 0)
-      fast::k_p1<float, R1B, CPW, fast::LD_BAND, A><<<g1, CPW * R1B, sm1, st>>>(
-          nullptr, nullptr, 0, 0, 0, ncol, Nseq, N2, ncol, ws, h->master, h->master_len, nullptr, spec, band, ctab);
-    else
-      fast::k_p1<float, R1B, CPW, fast::LD_FILTER, A><<<g1, CPW * R1B, sm1, st>>>(
-          nullptr, nullptr, 0, 0, 0, ncol, Nseq, N2, ncol, ws, h->master, h->master_len, nullptr, spec, omega, ctab);
-  }
-  if ((s = fc_after_launch(h)) != FC_OK) return s;
-  {
-    // band form: the second convolution's kernel is the first one's read backwards, whose spectrum is hhat read
-    // backwards
-    ProfScope ps(h, FC_K_PASS2, st);
-    fast::k_p2<R2B, CP, MIDV><<<g2, 2 * CP * R2B, sm2, st>>>(N1, ncol, ws, h->master, h->master_len, 0, hhat, invM,
-                                                             band >= 0 ? 1 : 0);
-  }
-  if ((s = fc_after_launch(h)) != FC_OK) return s;
-  {
-    ProfScope ps(h, FC_K_PASS3, st);
-    if (band >= 0) {
-      fast::k_p3<R1B, CPW, fast::OUT_SCORE_BAND, T, A><<<g3, CPW * R1B, sm3b, st>>>(
-          Nseq, N2, ncol, ws, h->master, h->master_len, scores, h0, dcols, total_tokens, (float)(1.0 / (double)d), phi,
-          nullptr, 0u, nullptr, 0, nullptr, 0, nullptr, nullptr, (float)d, accumulate, band, kp, vp, kv->stride_token,
-          kv->stride_head, ctab);
-    } else {
-      const float inv = (float)(1.0 / ((double)Nseq * (double)Nseq * (double)d));
-      fast::k_p3<R1B, CPW, fast::OUT_SCORE_CHIRP, float, A><<<g3, CPW * R1B, sm1, st>>>(
-          Nseq, N2, ncol, ws, h->master, h->master_len, scores, h0, dcols, total_tokens, inv, phi, nullptr, 0u, nullptr, 0,
-          nullptr, 0, nullptr, nullptr, (float)d, accumulate, -1, nullptr, nullptr, 0, 0, ctab);
-    }
-  }
-  return fc_after_launch(h);
+// tab_out != nullptr: the forward half on the two kernel columns, `ncol` columns wide (run_p1_table)
+template <int R2B, int CP, bool PAD>
+fc_status launch_p2(const PassArgs &x, int ncol, float4 *tab_out) {
+  const PassPlan &p = *x.p;
+  const size_t sm = (size_t)2 * (16 * R2B) * CP * sizeof(float4) + (4 * R2B + 4) * sizeof(float2) +
+                    (PAD ? 2 * (16 * R2B) * sizeof(float4) : (2 * (16 * R2B) + 4) * sizeof(float2));
+  fc_status s = set_smem(fast::k_p2<R2B, CP, PAD>, sm);
+  if (s != FC_OK) return s;
+  ProfScope ps(x.h, FC_K_PASS2, x.st);
+  fast::k_p2<R2B, CP, PAD><<<dim3(p.N1 / 2, tab_out ? 1 : ncol / (2 * CP)), 2 * CP * R2B, sm, x.st>>>(
+      p.N1, ncol, x.ws, x.h->master, x.h->master_len, x.omega, x.tab, tab_out);
+  return fc_after_launch(x.h);
 }
 
-template <typename T>
-fc_status launch_chirp(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const T *kp, const T *vp, int Nseq, int M,
-                       int h0, int hg, int omega, float2 *ws, float2 *spec, const float2 *hhat, double *ptot,
-                       double *phi, float *scores, long long total_tokens, int dcols, int accumulate, int band,
-                       const float2 *ctab, float2 *hout = nullptr) {
-  const ChirpShape c = chirp_shape(M);
-#define FC_CHIRP_CASE(A, B, C, D)                                                                               \
-  if (c.a == A && c.r1b == B && c.r2b == C && c.dbl == D)                                                       \
-    return launch_chirp_impl<T, A, B, C, D>(h, st, kv, kp, vp, Nseq, h0, hg, omega, ws, spec, hhat, ptot, phi, \
-                                            scores, total_tokens, dcols, accumulate, band, hout, ctab);
-  FC_CHIRP_CASE(16, 2, 2, false) FC_CHIRP_CASE(16, 2, 4, false) FC_CHIRP_CASE(16, 4, 4, false)
-  FC_CHIRP_CASE(16, 4, 8, false) FC_CHIRP_CASE(16, 8, 8, false) FC_CHIRP_CASE(16, 8, 16, false)
-  FC_CHIRP_CASE(16, 16, 16, false) FC_CHIRP_CASE(16, 16, 16, true)
-  // a = 14: 224 x {32 .. 512}
-  FC_CHIRP_CASE(14, 16, 2, false) FC_CHIRP_CASE(14, 16, 4, false) FC_CHIRP_CASE(14, 16, 8, false)
-  FC_CHIRP_CASE(14, 16, 16, false) FC_CHIRP_CASE(14, 16, 16, true)
-  // a = 10, 12: {160, 192} x 32, {80, 96} x {128, 256}, {160, 192} x {256, 512}
-  FC_CHIRP_CASE(10, 16, 2, false) FC_CHIRP_CASE(10, 8, 8, false) FC_CHIRP_CASE(10, 8, 16, false)
-  FC_CHIRP_CASE(10, 16, 16, false) FC_CHIRP_CASE(10, 16, 16, true)
-  FC_CHIRP_CASE(12, 16, 2, false) FC_CHIRP_CASE(12, 8, 8, false) FC_CHIRP_CASE(12, 8, 16, false)
-  FC_CHIRP_CASE(12, 16, 16, false) FC_CHIRP_CASE(12, 16, 16, true)
-#undef FC_CHIRP_CASE
+fc_status run_p2(const PassArgs &x, int ncol, float4 *tab_out) {
+  const PassPlan &p = *x.p;
+  if (p.dbl) {
+    constexpr int CP = 4;
+    const size_t sm = (size_t)4 * (256 * CP + 16 * CP) * sizeof(float4) + 1024 * sizeof(float4) +
+                      (256 + 32 + 72) * sizeof(float2);
+    fc_status s = set_smem(fast::k_p2_double<CP>, sm);
+    if (s != FC_OK) return s;
+    ProfScope ps(x.h, FC_K_PASS2, x.st);
+    fast::k_p2_double<CP><<<dim3(p.N1 / 2, tab_out ? 1 : ncol / (2 * CP)), 64 * CP, sm, x.st>>>(
+        p.N1, ncol, x.ws, x.h->master, x.h->master_len, x.tab, tab_out);
+    return fc_after_launch(x.h);
+  }
+#define FC_P2(R_, C_, P_) \
+  if (p.pad == P_ && p.r2b == R_ && p.cp == C_) return launch_p2<R_, C_, P_>(x, ncol, tab_out);
+  FC_P2(2, 32, true) FC_P2(4, 32, true) FC_P2(8, 16, true) FC_P2(16, 8, true)
+  FC_P2(2, 8, false) FC_P2(4, 8, false) FC_P2(4, 32, false) FC_P2(8, 16, false) FC_P2(16, 8, false)
+#undef FC_P2
+  return FC_ERR_INTERNAL;
+}
+
+template <int A, int R1B, int CPW, bool PAD>
+fc_status launch_p3(const PassArgs &x, long long score_stride, int accumulate, int hi_base, const fast::EnergyOut &eo) {
+  const PassPlan &p = *x.p;
+  const size_t sm = smem_outer(p);
+  fc_status s = set_smem(fast::k_p3<R1B, CPW, PAD, A>, sm);
+  if (s != FC_OK) return s;
+  const float inv = (float)(1.0 / ((double)p.M * (double)p.M * (double)x.kv->head_dim));
+  ProfScope ps(x.h, FC_K_PASS3, x.st);
+  fast::k_p3<R1B, CPW, PAD, A><<<dim3(p.N2, x.nu), CPW * R1B, sm, x.st>>>(
+      *x.lp, x.kv->num_heads, x.kv->head_dim, x.u0, x.cols, p.N, p.N2, x.nu * x.cols, x.ws, x.h->master, x.h->master_len,
+      score_stride, inv, accumulate, hi_base, eo);
+  return fc_after_launch(x.h);
+}
+
+fc_status run_p3(const PassArgs &x, long long score_stride, int accumulate, int hi_base, const fast::EnergyOut &eo) {
+  const PassPlan &p = *x.p;
+#define FC_P3(A_, R_, C_)                               \
+  if (p.pad && p.a == A_ && p.r1b == R_ && p.cpw == C_) \
+    return launch_p3<A_, R_, C_, true>(x, score_stride, accumulate, hi_base, eo);
+  FC_OUTER_PAD_SHAPES(FC_P3)
+#undef FC_P3
+#define FC_P3(A_, R_, C_)                                \
+  if (!p.pad && p.a == A_ && p.r1b == R_ && p.cpw == C_) \
+    return launch_p3<A_, R_, C_, false>(x, score_stride, accumulate, hi_base, eo);
+  FC_OUTER_DIRECT_SHAPES(FC_P3)
+#undef FC_P3
   return FC_ERR_INTERNAL;
 }
 
@@ -1092,130 +1080,94 @@ inline int cutoff_index(double gamma, int N) {
   return (int)om;
 }
 
-// Convolution length of the chirp path.  Full form: M >= 2N - 1.  Band form: only the bins -omega .. omega of the
-// spectrum are needed (the low-pass part; the score is taken against the input rows), M >= N + 2*omega + 1.  The
-// specialised kernels take powers of two and 2^k * {3, 5, 7}; whichever form gives the shorter M runs, and the
-// generic kernels (M = sp.Nfft, a power of two, full form) remain for what the specialised ones do not take
-// (cols_ok: the column groups are multiples of 64 channels).
-struct ChirpChoice {
-  int band;      // omega when the band form runs, else -1
-  int M;         // convolution length
-  bool fast;     // specialised kernels
-};
-
-inline ChirpChoice choose_chirp(const fc_handle *h, const SeqPlan &sp, int N, int omega, bool cols_ok) {
-  ChirpChoice c{-1, sp.Nfft, false};
-  if (!sp.bluestein || h->generic_only || !cols_ok) return c;
-  const int Mf = chirp_length(2LL * N - 1);
-  if (Mf != 0 && Mf <= sp.Nfft) { c.M = Mf; c.fast = true; }
-  if (h->band_form && 2LL * omega + 1 < N) {
-    const int Mb = chirp_length((long long)N + 2LL * omega + 1);
-    if (Mb != 0 && Mb < c.M) { c.band = omega; c.M = Mb; c.fast = true; }
-  }
-  return c;
-}
-
-template <typename T>
-fc_status score_sequence(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, int b, double gamma,
-                         float *scores, double *energy, char *wsb) {
-  const int start = kv->cu_seqlens[b];
-  const int N = kv->cu_seqlens[b + 1] - start;
-  const long long total_tokens = kv->cu_seqlens[kv->batch];
-  double *energy_b = energy + 4 * (size_t)b;
-  if (N == 0) {
-    k_zero_energy<<<1, 32, 0, st>>>(energy_b);
-    return fc_after_launch(h);
-  }
-  const int d = kv->head_dim, H = kv->num_heads;
-  const SeqPlan sp = plan_sequence(N, !h->generic_only);
-  const ScoreLayout L = layout_for(h, sp, H, d);
-  const int omega = cutoff_index(gamma, N);
-
-  fc_status s0 = FC_OK;
-  float2 *ws = reinterpret_cast<float2 *>(wsb + L.off_ws);
-  float2 *spec = reinterpret_cast<float2 *>(wsb + L.off_spec);
-  float2 *hhat = reinterpret_cast<float2 *>(wsb + L.off_hhat);
-  float2 *hcol = reinterpret_cast<float2 *>(wsb + L.off_hcol);
-  double *part_tot = reinterpret_cast<double *>(wsb + L.off_part_tot);
-  double *part_hi = reinterpret_cast<double *>(wsb + L.off_part_hi);
-  const bool separate_fast = sp.fast;
-  if (separate_fast) {                 // consecutive steps alternate between two copies of the partial sums
-    part_tot = reinterpret_cast<double *>(wsb + L.off_part_tot + (h->step & 1u) * L.part_tot_bytes);
-    part_hi = reinterpret_cast<double *>(wsb + L.off_part_hi + (h->step & 1u) * L.part_hi_bytes);
-  } else {
-    if ((s0 = fc_flush_pending(h, st)) != FC_OK) return s0;   // this path works on the caller's stream
-  }
-  const T *kp = static_cast<const T *>(kv->k) + (long long)start * kv->stride_token;
-  const T *vp = static_cast<const T *>(kv->v) + (long long)start * kv->stride_token;
-  const FftPlan p1 = make_plan(sp.N1);
-  fc_status s;
-
-  const ChirpChoice cc = choose_chirp(h, sp, N, omega, L.sub_cols % 64 == 0);
-  const int band = cc.band, Mc = cc.M;
-  const bool chirp_fast = cc.fast;
-  SeqPlan spc = sp;                      // plan of the convolution length, for the generic kernels
-  if (is_pow2(Mc)) { spc.Nfft = Mc; finish_plan(spc); }
-
-  const float2 *ctab = nullptr;
-  if (sp.bluestein) {
-    // Spectrum of the chirp kernel.  It depends on the sequence length only, so the handle keeps the last few
-    // (layers of a prefill share their lengths).  While the stream is being captured the spectrum goes to the
-    // workspace instead, every time: a graph must not depend on what the handle holds when it is replayed.
-    bool cached = false;
-    if (h->hhat_cache && !h->generic_only && sp.Nfft <= h->hhat_cache_len) {
+// Filter tables of the padded form for every such sequence of the view, tabs[b].  A table depends on the length and the
+// cutoff only, so the handle keeps the last FC_TAB_SLOTS (the layers of a prefill share theirs).  While the stream is
+// being captured, and for lengths beyond the slots, tables go to the workspace, every call: a graph must not depend on
+// what the handle holds when it is replayed.
+fc_status prepare_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, double gamma, const ScoreLayout &L, char *wsb,
+                         const float4 **tabs) {
+  bool cached = true, any = false, flushed = false;
+  bool used[FC_TAB_SLOTS] = {};
+  auto key_of = [&](int b) {
+    const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
+    return (long long)N + ((long long)(cutoff_index(gamma, N) + 1) << 32);
+  };
+  for (int b = 0; b < kv->batch; ++b) {
+    tabs[b] = nullptr;
+    const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
+    if (N == 0) continue;
+    const PassPlan p = plan_passes(N);
+    if (!p.ok || !p.pad) continue;
+    if (!any) {
+      any = true;
       cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
       if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { cudaGetLastError(); cap = cudaStreamCaptureStatusActive; }
-      cached = (cap == cudaStreamCaptureStatusNone);
+      cached = cap == cudaStreamCaptureStatusNone;
     }
-    bool have = false;
-    int slot = 0;
-    const long long hkey = (long long)N + ((long long)(band + 1) << 32);
-    if (cached) {
-      for (int i = 0; i < FC_HHAT_SLOTS && !have; ++i)
-        if (h->hhat_cache_n[i] == hkey) { have = true; slot = i; }
-      if (!have) {
-        // the slot taken over was last read by a sequence that has been joined to `st` since (the chirp path
-        // joins the internal streams before it returns), so stream order protects it
-        slot = h->hhat_cache_next;
-        h->hhat_cache_next = (slot + 1) % FC_HHAT_SLOTS;
-        h->hhat_cache_n[slot] = 0;                          // not valid until both launches are in the stream
-      }
-      hhat = h->hhat_cache + (size_t)slot * h->hhat_slot_len;
-    }
-    if (!have) {
-      if (is_pow2(Mc)) {
-        ChirpKernelLoader cl{N, Mc, band};
-        if ((s = launch_pass1(h, st, cl, spc, 8, 8, hcol, nullptr)) != FC_OK) return s;
-        if ((s = launch_pass2<MID_SPEC>(h, st, spc, 8, 8, hcol, 0, hhat, 1.f)) != FC_OK) return s;
-      } else {
-        // lengths with an odd factor: the specialised kernels transform the kernel themselves (64 columns of the
-        // workspace, which no head group uses yet)
-        if ((s = launch_chirp<T>(h, st, kv, nullptr, nullptr, N, Mc, 0, 1, 0, ws, nullptr, nullptr, nullptr, nullptr,
-                                 nullptr, 0, 64, 0, band, nullptr, hhat)) != FC_OK) return s;
-      }
-      if (cached) h->hhat_cache_n[slot] = hkey;
-    }
-    // per-row factors of the chirp modes (2N values): behind the spectrum in its cache slot, else in the column
-    // buffer of the workspace, which the spectrum's transform no longer needs
-    ctab = cached ? hhat + h->hhat_cache_len : hcol;
-    if (!have && chirp_fast) {
-      ProfScope ps(h, FC_K_OTHER, st);
-      fast::k_chirp_tables<<<(N + 255) / 256, 256, 0, st>>>(const_cast<float2 *>(ctab), N);
-      if ((s = fc_after_launch(h)) != FC_OK) return s;
-    }
+    if (cached)
+      for (int i = 0; i < FC_TAB_SLOTS; ++i)
+        if (h->tab_key[i] == key_of(b)) { tabs[b] = h->tab_cache + (size_t)i * h->tab_slot_len; used[i] = true; }
   }
+  if (!any) return FC_OK;
+  float4 *spare = reinterpret_cast<float4 *>(wsb + L.off_tab);
+  for (int b = 0; b < kv->batch; ++b) {
+    const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
+    if (N == 0 || tabs[b]) continue;
+    const PassPlan p = plan_passes(N);
+    if (!p.ok || !p.pad) continue;
+    if (!first_of_its_length(kv, b)) {
+      for (int i = 0; i < b && !tabs[b]; ++i)
+        if (kv->cu_seqlens[i + 1] - kv->cu_seqlens[i] == N) tabs[b] = tabs[i];
+      continue;
+    }
+    fc_status s;
+    // the table's place and the intermediate buffer may still be in use on the internal streams
+    if (!flushed && (s = fc_flush_pending(h, st)) != FC_OK) return s;
+    flushed = true;
+    float4 *dst = nullptr;
+    int slot = -1;
+    for (int i = 0; cached && i < FC_TAB_SLOTS && slot < 0; ++i) {
+      const int c = (h->tab_next + i) % FC_TAB_SLOTS;
+      if (!used[c]) slot = c;
+    }
+    if (slot >= 0) {
+      h->tab_next = (slot + 1) % FC_TAB_SLOTS;
+      h->tab_key[slot] = 0;                                  // not valid until both launches are in the stream
+      used[slot] = true;
+      dst = h->tab_cache + (size_t)slot * h->tab_slot_len;
+    } else {
+      dst = spare;
+      spare += p.M;
+    }
+    static const fast::LayerPtrs none = {};
+    const PassArgs x{h, st, &p, &none, kv, 0, 1, 0, 2 * p.cpw, cutoff_index(gamma, N), reinterpret_cast<float2 *>(wsb + L.off_buf), nullptr};
+    if ((s = run_p1_table(x)) != FC_OK) return s;
+    if ((s = run_p2(x, 2 * p.cpw, dst)) != FC_OK) return s;
+    if (slot >= 0) h->tab_key[slot] = key_of(b);
+    tabs[b] = dst;
+  }
+  return FC_OK;
+}
 
-  // fc_score_layer has claimed the persisting part of L2 if any sequence of the call takes this path
-  const bool want_persist = separate_fast && window_fits(h, L);
-  if (want_persist && h->persist_on) {
+// One sequence on the specialised passes, for a chunk of layers.  `lp` points at the sequence's first token.
+template <typename T>
+fc_status score_sequence(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const PassPlan &p, int nl,
+                         const fast::LayerPtrs &lp, double gamma, double *energy, long long energy_stride,
+                         const ScoreLayout &L, char *wsb, const float4 *tab) {
+  const int d = kv->head_dim, H = kv->num_heads, U = nl * H;
+  const long long total_tokens = kv->cu_seqlens[kv->batch];
+  const GroupPlan g = plan_groups(h, p, U, H, d);
+  const unsigned par = h->step & 1u;               // consecutive steps alternate between two copies of the partial sums
+  fc_status s;
+  if (window_fits(h, p, g) && h->persist_on) {
     // keep each stream's intermediate in the persisting part of L2; everything else these streams touch
     // (the K/V rows, the scores) streams through
     for (int i = 0; i < h->num_aux; ++i) {
-      const char *base = wsb + L.off_ws + (size_t)i * L.ws_buf_bytes;
-      if (h->window_base[i] == base && h->window_bytes[i] == L.ws_buf_bytes) continue;
+      const char *base = wsb + L.off_buf + (size_t)i * L.buf_bytes;
+      if (h->window_base[i] == base && h->window_bytes[i] == g.buf_bytes) continue;
       cudaStreamAttrValue av = {};
       av.accessPolicyWindow.base_ptr = const_cast<char *>(base);
-      av.accessPolicyWindow.num_bytes = L.ws_buf_bytes;
+      av.accessPolicyWindow.num_bytes = g.buf_bytes;
       av.accessPolicyWindow.hitRatio = 1.0f;
       av.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
       av.accessPolicyWindow.missProp = cudaAccessPropertyStreaming;
@@ -1225,45 +1177,78 @@ fc_status score_sequence(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, in
         break;
       }
       h->window_base[i] = base;
-      h->window_bytes[i] = L.ws_buf_bytes;
+      h->window_bytes[i] = g.buf_bytes;
     }
   }
-  if (sp.fast) {
-    const long long sig = (long long)N + ((long long)H << 20) + ((long long)d << 40);
-    FC_CUDA_TRY(cudaEventRecord(h->ev_fork, st));
-    for (int i = 0; i < h->num_aux; ++i) {
-      FC_CUDA_TRY(cudaStreamWaitEvent(h->aux[i], h->ev_fork, 0));
-      for (int o = 0; o < h->num_aux; ++o) {
-        if (o == i) continue;
-        // the partial sums and the block counter of this parity were last used two steps ago: the other
-        // streams must be through with that step (this one is, by stream order)
-        if (h->step >= 2) FC_CUDA_TRY(cudaStreamWaitEvent(h->aux[i], h->ev_done[h->step & 1u][o], 0));
-        // a different shape carves the workspace differently: nothing of the previous step may be in flight
-        if (h->step >= 1 && sig != h->last_sig)
-          FC_CUDA_TRY(cudaStreamWaitEvent(h->aux[i], h->ev_done[(h->step - 1) & 1u][o], 0));
-      }
+  // the partial sums and the block counters of this parity were last used two steps ago: the other streams must be
+  // through with that step (this one is, by stream order)
+  if (h->step >= 2)
+    for (int i = 0; i < h->num_aux; ++i)
+      for (int o = 0; o < h->num_aux; ++o)
+        if (o != i) FC_CUDA_TRY(cudaStreamWaitEvent(h->aux[i], h->ev_done[par][o], 0));
+  double *part_tot = reinterpret_cast<double *>(wsb + L.off_tot + par * L.tot_bytes);
+  fast::EnergyOut eo;
+  eo.part_hi = reinterpret_cast<double *>(wsb + L.off_hi + par * L.hi_bytes);
+  eo.part_tot = part_tot;
+  eo.hi_slots = H * g.ngr * p.N2;
+  eo.tot_slots = H * (d / (2 * p.cpw)) * p.N2;
+  eo.done = h->done_counter + par * FC_LAYER_CHUNK;
+  eo.total_blocks = (unsigned)(H * g.ngr * p.N2);
+  eo.energy = energy;
+  eo.energy_stride = energy_stride;
+  int group = 0;
+  for (int u0 = 0; u0 < U; u0 += g.units, ++group) {
+    const int nu = U - u0 < g.units ? U - u0 : g.units;
+    const int si = (int)((group + h->step) % (unsigned)h->num_aux);   // a single group: steps alternate
+    PassArgs x{h, h->aux[si], &p, &lp, kv, u0, nu, 0, g.sub, cutoff_index(gamma, p.N),
+               reinterpret_cast<float2 *>(wsb + L.off_buf + (size_t)si * L.buf_bytes), tab};
+    for (int cg = 0; cg < g.ngr; ++cg) {                      // column groups of one unit, in stream order
+      x.c0 = cg * g.sub;
+      if ((s = run_p1<T>(x, part_tot, eo.tot_slots)) != FC_OK) return s;
+      if ((s = run_p2(x, nu * g.sub, nullptr)) != FC_OK) return s;
+      if ((s = run_p3(x, total_tokens, cg > 0 ? 1 : 0, cg * H * p.N2, eo)) != FC_OK) return s;
     }
-    h->last_sig = sig;
   }
-  const bool chirp_fork = sp.bluestein && L.chirp_streams > 1;
-  if (chirp_fork) {                     // the internal streams start after the chirp kernel's spectrum is ready
-    FC_CUDA_TRY(cudaEventRecord(h->ev_fork, st));
-    for (int i = 0; i < L.chirp_streams; ++i) FC_CUDA_TRY(cudaStreamWaitEvent(h->aux[i], h->ev_fork, 0));
+  for (int i = 0; i < h->num_aux; ++i) FC_CUDA_TRY(cudaEventRecord(h->ev_done[par][i], h->aux[i]));
+  h->step++;
+  h->pending_join = true;
+  return FC_OK;
+}
+
+// One sequence of one layer on the generic kernels, on the caller's stream.
+template <typename T>
+fc_status score_generic(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, int b, double gamma, float *scores,
+                        double *energy_b, char *wsb) {
+  const int start = kv->cu_seqlens[b];
+  const int N = kv->cu_seqlens[b + 1] - start;
+  const long long total_tokens = kv->cu_seqlens[kv->batch];
+  const int d = kv->head_dim, H = kv->num_heads;
+  const SeqPlan sp = plan_sequence(N);
+  const GenericLayout L = generic_layout(h, sp, H, d);
+  const int omega = cutoff_index(gamma, N);
+  float2 *ws = reinterpret_cast<float2 *>(wsb + L.off_ws);
+  float2 *spec = reinterpret_cast<float2 *>(wsb + L.off_spec);
+  float2 *hhat = reinterpret_cast<float2 *>(wsb + L.off_hhat);
+  float2 *hcol = reinterpret_cast<float2 *>(wsb + L.off_hcol);
+  double *part_tot = reinterpret_cast<double *>(wsb + L.off_part_tot);
+  double *part_hi = reinterpret_cast<double *>(wsb + L.off_part_hi);
+  const T *kp = static_cast<const T *>(kv->k) + (long long)start * kv->stride_token;
+  const T *vp = static_cast<const T *>(kv->v) + (long long)start * kv->stride_token;
+  const FftPlan p1 = make_plan(sp.N1);
+  fc_status s;
+  if (sp.bluestein) {
+    ChirpKernelLoader cl{N, sp.Nfft};
+    if ((s = launch_pass1(h, st, cl, sp, 8, 8, hcol, nullptr)) != FC_OK) return s;
+    if ((s = launch_pass2<MID_SPEC>(h, st, sp, 8, 8, hcol, 0, hhat, 1.f)) != FC_OK) return s;
   }
   size_t tot_slots = 0, hi_slots = 0;
-  int group = 0;
-  for (int h0 = 0; h0 < H; h0 += L.heads_per_group, ++group) {
+  for (int h0 = 0; h0 < H; h0 += L.heads_per_group) {
     const int hg = (H - h0 < L.heads_per_group) ? H - h0 : L.heads_per_group;
-    const int ncol_ws = hg * d;
     double *ptot = part_tot + 2 * tot_slots;
     double *phi = part_hi + 2 * hi_slots;
-    const size_t sm3 = smem_pass13(sp, sp.cs);
-    if (sp.fast) {
-      const int si = (int)((group + h->step) % (unsigned)h->num_aux);   // a single group: steps alternate
-      float2 *wsg = reinterpret_cast<float2 *>(wsb + L.off_ws + (size_t)si * L.ws_buf_bytes);
-      if ((s = launch_fast<T>(h, h->aux[si], kv, kp, vp, sp, h0, hg, omega, wsg, ptot, phi,
-                              scores + start, total_tokens, part_tot, part_hi, energy_b)) != FC_OK) return s;
-    } else if (!sp.bluestein) {
+    if (!sp.bluestein) {
+      const int ncol_ws = hg * d;
+      const size_t sm3 = smem_pass13(sp, sp.cs);
       KvLoader<T, false> ld{kp, vp, kv->stride_token, kv->stride_head, h0, d, N, 0.f, 0.f};
       if ((s = launch_pass1(h, st, ld, sp, ncol_ws, sp.cs, ws, ptot)) != FC_OK) return s;
       if ((s = launch_pass2<MID_DCT>(h, st, sp, ncol_ws, sp.cs2, ws, omega, nullptr, 1.f / (float)N)) != FC_OK) return s;
@@ -1275,92 +1260,134 @@ fc_status score_sequence(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, in
             total_tokens, 1.f / (float)d, phi, (float)d, 0);
       }
       if ((s = fc_after_launch(h)) != FC_OK) return s;
-    } else {
-      // One head may be transformed in several column groups (sub < d) so that the padded
-      // length-Nfft intermediates of a group stay within the cache budget; the groups run in
-      // stream order and the last pass adds their contributions to the score in that order.
-      if (chirp_fast) {                         // a length and a width the specialised kernels take
-        const int sub = L.sub_cols, ngr = (hg == 1) ? d / sub : 1, n2f = chirp_shape(Mc).n2();
-        const ChirpShape shp = chirp_shape(Mc);
-        const int tilew = 2 * chirp_cpw(shp.r1b, shp.r2b, shp.dbl);     // columns per block of passes 1 and 3
-        const int ncol = (hg == 1) ? sub : ncol_ws;
-        const int si = group % L.chirp_streams;                   // head groups alternate over the internal streams
-        cudaStream_t sx = L.chirp_streams > 1 ? h->aux[si] : st;
-        float2 *ws_s = reinterpret_cast<float2 *>(wsb + L.off_ws + (size_t)si * L.ws_buf_bytes);
-        float2 *spec_s = reinterpret_cast<float2 *>(wsb + L.off_spec + (size_t)si * L.spec_buf_bytes);
-        for (int cg = 0; cg < ngr; ++cg) {                        // column groups of one head, else one pass
-          if ((s = launch_chirp<T>(h, sx, kv, kp + cg * sub, vp + cg * sub, N, Mc, h0, hg, omega, ws_s, spec_s, hhat,
-                                   ptot + 2 * (size_t)cg * n2f * (ncol / tilew), phi + 2 * (size_t)cg * n2f * hg,
-                                   scores + start, total_tokens, (hg == 1) ? sub : d, cg > 0 ? 1 : 0, band, ctab)) != FC_OK)
-            return s;
-        }
-        tot_slots += (size_t)n2f * (ncol / tilew) * ngr;
-        hi_slots += (size_t)n2f * hg * ngr;
-        continue;
-      }
-      const float invM = 1.f / (float)sp.Nfft;
-      const float inv = (float)(1.0 / ((double)N * (double)N * (double)d));
-      const int sub = L.sub_cols, cs = (sub % 64 == 0) ? sp.cs : 32;
-      const int ngroups = (hg == 1) ? d / sub : 1;
-      const int ncol = (hg == 1) ? sub : ncol_ws;
-      int cs2 = 2 * sp.cs2 > 64 ? 64 : 2 * sp.cs2;       // the convolution pass holds single rows: twice the columns fit
-      while (ncol % cs2) cs2 >>= 1;
-      const size_t sm3c = smem_pass13(sp, cs);
-      for (int cg = 0; cg < ngroups; ++cg) {
-        const int c0 = cg * sub;
-        double *ptot_c = ptot + 2 * (size_t)cg * sp.N2 * (ncol / cs);
-        double *phi_c = phi + 2 * (size_t)cg * sp.N2 * hg;
-        const int dd = (hg == 1) ? sub : d;           // columns the loader and the last pass see per head
-        KvLoader<T, true> ld{kp + c0, vp + c0, kv->stride_token, kv->stride_head, h0, dd, N, 0.f, 0.f};
-        if ((s = launch_pass1(h, st, ld, sp, ncol, cs, ws, ptot_c)) != FC_OK) return s;
-        if ((s = launch_pass2<MID_MULH>(h, st, sp, ncol, cs2, ws, 0, hhat, invM)) != FC_OK) return s;
-        if ((s = set_smem(k_pass3<EPI_SPEC, true>, sm3c)) != FC_OK) return s;
-        {
-          ProfScope ps(h, FC_K_PASS3, st);
-          k_pass3<EPI_SPEC, true><<<dim3(sp.N2, ncol / cs), kThreads, sm3c, st>>>(
-              p1, sp.N2, N, ncol, ilog2(cs), ws, h->master, h->master_len, spec, nullptr, 0, dd, 0, 0.f, nullptr,
-              0.f, 0);
-        }
-        if ((s = fc_after_launch(h)) != FC_OK) return s;
-        FilterLoader fl{spec, ncol, N, omega};
-        if ((s = launch_pass1(h, st, fl, sp, ncol, cs, ws, nullptr)) != FC_OK) return s;
-        if ((s = launch_pass2<MID_MULH>(h, st, sp, ncol, cs2, ws, 0, hhat, invM)) != FC_OK) return s;
-        if ((s = set_smem(k_pass3<EPI_SCORE, true>, sm3c)) != FC_OK) return s;
-        {
-          ProfScope ps(h, FC_K_PASS3, st);
-          k_pass3<EPI_SCORE, true><<<dim3(sp.N2, hg), kThreads, sm3c, st>>>(
-              p1, sp.N2, N, ncol, ilog2(cs), ws, h->master, h->master_len, nullptr, scores + start, h0, dd,
-              total_tokens, inv, phi_c, (float)d, cg > 0 ? 1 : 0);
-        }
-        if ((s = fc_after_launch(h)) != FC_OK) return s;
-      }
-      tot_slots += (size_t)sp.N2 * (ncol / cs) * ngroups;
-      hi_slots += (size_t)sp.N2 * hg * ngroups;
+      tot_slots += (size_t)sp.N2 * (ncol_ws / sp.cs);
+      hi_slots += (size_t)sp.N2 * hg;
       continue;
     }
-    tot_slots += (size_t)sp.N2 * (ncol_ws / (sp.fast ? 2 * fast_cpw(sp.N1, h->tune_cpw) : sp.cs));
-    hi_slots += (size_t)sp.N2 * hg;
-  }
-  if (sp.fast) {
-    for (int i = 0; i < h->num_aux; ++i) FC_CUDA_TRY(cudaEventRecord(h->ev_done[h->step & 1u][i], h->aux[i]));
-    h->step++;
-    h->pending_join = true;
-    if (!h->score_overlap) {           // default: the caller's stream waits for this call's work right away
-      if ((s = fc_flush_pending(h, st)) != FC_OK) return s;
+    // One head may be transformed in several column groups (sub < d) so that the padded length-Nfft intermediates of a
+    // group stay within the budget; the groups run in stream order and the last pass adds their contributions to the
+    // score in that order.
+    const float invM = 1.f / (float)sp.Nfft;
+    const float inv = (float)(1.0 / ((double)N * (double)N * (double)d));
+    const int sub = L.sub_cols, cs = (sub % 64 == 0) ? sp.cs : 32;
+    const int ngroups = (hg == 1) ? d / sub : 1;
+    const int ncol = (hg == 1) ? sub : hg * d;
+    int cs2 = 2 * sp.cs2 > 64 ? 64 : 2 * sp.cs2;       // the convolution pass holds single rows: twice the columns fit
+    while (ncol % cs2) cs2 >>= 1;
+    const size_t sm3c = smem_pass13(sp, cs);
+    for (int cg = 0; cg < ngroups; ++cg) {
+      const int c0 = cg * sub;
+      double *ptot_c = ptot + 2 * (size_t)cg * sp.N2 * (ncol / cs);
+      double *phi_c = phi + 2 * (size_t)cg * sp.N2 * hg;
+      const int dd = (hg == 1) ? sub : d;           // columns the loader and the last pass see per head
+      KvLoader<T, true> ld{kp + c0, vp + c0, kv->stride_token, kv->stride_head, h0, dd, N, 0.f, 0.f};
+      if ((s = launch_pass1(h, st, ld, sp, ncol, cs, ws, ptot_c)) != FC_OK) return s;
+      if ((s = launch_pass2<MID_MULH>(h, st, sp, ncol, cs2, ws, 0, hhat, invM)) != FC_OK) return s;
+      if ((s = set_smem(k_pass3<EPI_SPEC, true>, sm3c)) != FC_OK) return s;
+      {
+        ProfScope ps(h, FC_K_PASS3, st);
+        k_pass3<EPI_SPEC, true><<<dim3(sp.N2, ncol / cs), kThreads, sm3c, st>>>(
+            p1, sp.N2, N, ncol, ilog2(cs), ws, h->master, h->master_len, spec, nullptr, 0, dd, 0, 0.f, nullptr, 0.f, 0);
+      }
+      if ((s = fc_after_launch(h)) != FC_OK) return s;
+      FilterLoader fl{spec, ncol, N, omega};
+      if ((s = launch_pass1(h, st, fl, sp, ncol, cs, ws, nullptr)) != FC_OK) return s;
+      if ((s = launch_pass2<MID_MULH>(h, st, sp, ncol, cs2, ws, 0, hhat, invM)) != FC_OK) return s;
+      if ((s = set_smem(k_pass3<EPI_SCORE, true>, sm3c)) != FC_OK) return s;
+      {
+        ProfScope ps(h, FC_K_PASS3, st);
+        k_pass3<EPI_SCORE, true><<<dim3(sp.N2, hg), kThreads, sm3c, st>>>(
+            p1, sp.N2, N, ncol, ilog2(cs), ws, h->master, h->master_len, nullptr, scores + start, h0, dd,
+            total_tokens, inv, phi_c, (float)d, cg > 0 ? 1 : 0);
+      }
+      if ((s = fc_after_launch(h)) != FC_OK) return s;
     }
-  }
-  if (sp.fast) return FC_OK;          // the last pass-3 block of the sequence has written the energy sums
-  if (chirp_fork) {                     // the caller's stream takes over again for the energy sums
-    for (int i = 0; i < L.chirp_streams; ++i) {
-      FC_CUDA_TRY(cudaEventRecord(h->ev_join[i], h->aux[i]));
-      FC_CUDA_TRY(cudaStreamWaitEvent(st, h->ev_join[i], 0));
-    }
+    tot_slots += (size_t)sp.N2 * (ncol / cs) * ngroups;
+    hi_slots += (size_t)sp.N2 * hg * ngroups;
   }
   {
     ProfScope ps(h, FC_K_OTHER, st);
     k_energy_finalize<<<1, 256, 0, st>>>(part_tot, (int)tot_slots, part_hi, (int)hi_slots, energy_b);
   }
   return fc_after_launch(h);
+}
+
+// All sequences of `num_layers` layers that share the view's layout; energy[l][B][4].
+template <typename T>
+fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const fc_layer_buffers *layers, int num_layers,
+                     double gamma, double *energy, char *wsb) {
+  const int B = kv->batch, H = kv->num_heads;
+  const ScoreLayout L = score_layout(h, kv, num_layers);
+  fc_status s;
+  bool fork = true, direct_only = true, any_fast = false;
+  std::vector<PassPlan> plans(B);
+  std::vector<const float4 *> tabs(B, nullptr);
+  for (int b = 0; b < B; ++b) {
+    const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
+    if (N == 0) continue;
+    if (!h->generic_only) plans[b] = plan_passes(N);
+    any_fast = any_fast || plans[b].ok;
+    if (!plans[b].ok || plans[b].pad) direct_only = false;
+  }
+  if (any_fast && (s = prepare_tables(h, st, kv, gamma, L, wsb, tabs.data())) != FC_OK) return s;
+  // a call that carves the workspace differently: nothing of the previous call may be in flight on the other streams
+  const size_t sig = reinterpret_cast<size_t>(wsb) ^ (L.buf_bytes << 20) ^ (L.tot_bytes << 8) ^ L.hi_bytes ^ (L.off_tot << 12);
+  if (any_fast && h->step >= 1 && sig != h->last_sig) {
+    for (int i = 0; i < h->num_aux; ++i)
+      for (int o = 0; o < h->num_aux; ++o)
+        if (o != i) FC_CUDA_TRY(cudaStreamWaitEvent(h->aux[i], h->ev_done[(h->step - 1) & 1u][o], 0));
+  }
+  if (any_fast) h->last_sig = sig;
+  for (int l0 = 0; l0 < num_layers; l0 += FC_LAYER_CHUNK) {
+    const int nl = num_layers - l0 < FC_LAYER_CHUNK ? num_layers - l0 : FC_LAYER_CHUNK;
+    for (int b = 0; b < B; ++b) {
+      const int start = kv->cu_seqlens[b];
+      double *en = energy + 4 * ((size_t)l0 * B + b);
+      if (kv->cu_seqlens[b + 1] == start) {
+        k_zero_energy<<<1, 128, 0, st>>>(en, nl, 4ll * B);
+        if ((s = fc_after_launch(h)) != FC_OK) return s;
+        continue;
+      }
+      if (!plans[b].ok) {                       // generic kernels: they share the workspace and run on `st`
+        if ((s = fc_flush_pending(h, st)) != FC_OK) return s;
+        fork = true;
+        for (int l = 0; l < nl; ++l) {
+          fc_kv_view one = *kv;
+          one.k = layers[l0 + l].k;
+          one.v = layers[l0 + l].v;
+          s = score_generic<T>(h, st, &one, b, gamma, const_cast<float *>(layers[l0 + l].scores), en + 4ll * B * l, wsb);
+          if (s != FC_OK) return s;
+        }
+        continue;
+      }
+      if (fork) {
+        FC_CUDA_TRY(cudaEventRecord(h->ev_fork, st));
+        for (int i = 0; i < h->num_aux; ++i) FC_CUDA_TRY(cudaStreamWaitEvent(h->aux[i], h->ev_fork, 0));
+        fork = false;
+      }
+      fast::LayerPtrs lp = {};
+      for (int l = 0; l < nl; ++l) {
+        lp.k[l] = static_cast<const T *>(layers[l0 + l].k) + (long long)start * kv->stride_token;
+        lp.v[l] = static_cast<const T *>(layers[l0 + l].v) + (long long)start * kv->stride_token;
+        lp.scores[l] = const_cast<float *>(layers[l0 + l].scores) + start;
+      }
+      if ((s = score_sequence<T>(h, st, kv, plans[b], nl, lp, gamma, en, 4ll * B, L, wsb, tabs[b])) != FC_OK) return s;
+    }
+  }
+  (void)H;
+  // the caller's stream waits for this call's work right away, unless it asked to have that deferred
+  if (!h->score_overlap || !direct_only) return fc_flush_pending(h, st);
+  return FC_OK;
+}
+
+fc_status score_dispatch(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const fc_layer_buffers *layers,
+                         int num_layers, double gamma, double *energy, void *workspace) {
+  char *wsb = static_cast<char *>(workspace);
+  switch (kv->dtype) {
+    case FC_F32: return score_call<float>(h, st, kv, layers, num_layers, gamma, energy, wsb);
+    case FC_F16: return score_call<__half>(h, st, kv, layers, num_layers, gamma, energy, wsb);
+    default: return score_call<__nv_bfloat16>(h, st, kv, layers, num_layers, gamma, energy, wsb);
+  }
 }
 
 // Column slices of one launch of k_pass2_power that run side by side (the rest are looped over).
@@ -1375,8 +1402,8 @@ fc_status power_sequence(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, in
   const int N = kv->cu_seqlens[b + 1] - start;
   if (N == 0) return FC_OK;
   const int d = kv->head_dim, H = kv->num_heads;
-  const SeqPlan sp = plan_sequence(N, false);
-  const ScoreLayout L = layout_for(h, sp, H, d);
+  const SeqPlan sp = plan_sequence(N);
+  const GenericLayout L = generic_layout(h, sp, H, d);
   float2 *ws = reinterpret_cast<float2 *>(wsb + L.off_ws);
   float2 *spec = reinterpret_cast<float2 *>(wsb + L.off_spec);
   float2 *hhat = reinterpret_cast<float2 *>(wsb + L.off_hhat);
@@ -1388,7 +1415,7 @@ fc_status power_sequence(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, in
   const FftPlan p1 = make_plan(sp.N1);
   fc_status s;
   if (sp.bluestein) {
-    ChirpKernelLoader cl{N, sp.Nfft, -1};
+    ChirpKernelLoader cl{N, sp.Nfft};
     if ((s = launch_pass1(h, st, cl, sp, 8, 8, hcol, nullptr)) != FC_OK) return s;
     if ((s = launch_pass2<MID_SPEC>(h, st, sp, 8, 8, hcol, 0, hhat, 1.f)) != FC_OK) return s;
   }
@@ -1437,15 +1464,98 @@ fc_status power_sequence(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, in
   return FC_OK;
 }
 
+// Operation count of the chirp form: the yardstick fc_describe_plan reports for lengths that are not powers of two.
+// Smallest of 2^k and 160, 192, 224 x 32..512 that is >= need (0 if none up to 131072).
+inline int chirp_length(long long need) {
+  int best = 0;
+  for (int M = 1024; M <= 131072; M <<= 1)
+    if (M >= need) { best = M; break; }
+  for (int n1 = 160; n1 <= 224; n1 += 32)
+    for (int n2 = 32; n2 <= 512; n2 <<= 1) {
+      const int M = n1 * n2;
+      if (M >= need && (best == 0 || M < best)) best = M;
+    }
+  return best;
+}
+
 }  // namespace
 
+extern "C" fc_status fc_describe_plan(const fc_handle *h, int32_t seqlen, double gamma, int32_t out[4]) {
+  if (!h || !out || seqlen < 1 || !(gamma >= 0.0 && gamma <= 1.0)) return FC_ERR_INVALID_ARG;
+  if (seqlen > h->max_seqlen || (seqlen > 65536 && !is_pow2(seqlen))) return FC_ERR_UNSUPPORTED;
+  const SeqPlan sp = plan_sequence(seqlen);
+  out[0] = sp.bluestein ? 1 : 0;
+  out[1] = sp.Nfft;
+  const PassPlan p = plan_passes(seqlen);
+  out[2] = (p.ok && !p.pad) ? p.N1 : sp.N1;
+  out[3] = (p.ok && !p.pad) ? p.N2 : sp.N2;
+  if (sp.bluestein) {
+    const int omega = cutoff_index(gamma, seqlen), Mf = chirp_length(2LL * seqlen - 1);
+    bool shaped = Mf != 0 && Mf <= sp.Nfft;
+    if (shaped) out[1] = Mf;
+    if (h->band_form && 2LL * omega + 1 < seqlen) {
+      const int Mb = chirp_length((long long)seqlen + 2LL * omega + 1);
+      if (Mb != 0 && Mb < out[1]) { out[0] = 2; out[1] = Mb; shaped = true; }
+    }
+    if (shaped) {
+      const PassPlan c = pad_shape(out[1]);
+      out[2] = c.N1;
+      out[3] = c.N2;
+    }
+  }
+  return FC_OK;
+}
+
+extern "C" size_t fc_score_layers_workspace_bytes(const fc_handle *h, const fc_kv_view *shape, int32_t num_layers) {
+  if (validate_view(h, shape, false) != FC_OK || num_layers < 1) return 0;
+  return score_layout(h, shape, num_layers).total;
+}
+
+extern "C" size_t fc_score_workspace_bytes(const fc_handle *h, const fc_kv_view *kv) {
+  if (validate_view(h, kv, true) != FC_OK) return 0;
+  return score_layout(h, kv, 1).total;
+}
+
+extern "C" fc_status fc_score_layers(fc_handle *h, const fc_kv_view *shape, const fc_layer_buffers *layers,
+                                     int32_t num_layers, double gamma, double *energy, void *workspace,
+                                     size_t workspace_bytes, fc_stream stream) {
+  fc_status s = validate_view(h, shape, false);
+  if (s != FC_OK) return s;
+  if (!layers || !energy || num_layers < 1) return FC_ERR_INVALID_ARG;
+  if (!(gamma >= 0.0 && gamma <= 1.0)) return FC_ERR_INVALID_ARG;
+  for (int l = 0; l < num_layers; ++l)
+    if (!layers[l].k || !layers[l].v || !layers[l].scores || ((uintptr_t)layers[l].k & 15) || ((uintptr_t)layers[l].v & 15))
+      return FC_ERR_INVALID_ARG;
+  if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < score_layout(h, shape, num_layers).total)
+    return FC_ERR_WORKSPACE;
+  int dev = -1;
+  FC_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev != h->device) FC_CUDA_TRY(cudaSetDevice(h->device));
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  claim_persisting_l2(h, shape, num_layers, st);
+  return score_dispatch(h, st, shape, layers, num_layers, gamma, energy, workspace);
+}
+
+extern "C" fc_status fc_score_layer(fc_handle *h, const fc_kv_view *kv, double gamma, float *scores,
+                                    double *energy, void *workspace, size_t workspace_bytes,
+                                    fc_stream stream) {
+  const fc_status s = validate_view(h, kv, true);
+  if (s != FC_OK) return s;
+  if (!scores || !energy) return FC_ERR_INVALID_ARG;
+  fc_layer_buffers one = {};
+  one.k = kv->k;
+  one.v = kv->v;
+  one.scores = scores;
+  return fc_score_layers(h, kv, &one, 1, gamma, energy, workspace, workspace_bytes, stream);
+}
+
 extern "C" size_t fc_power_spectrum_workspace_bytes(const fc_handle *h, const fc_kv_view *kv) {
-  if (validate_view(h, kv) != FC_OK) return 0;
+  if (validate_view(h, kv, true) != FC_OK) return 0;
   size_t need = 256;
   for (int b = 0; b < kv->batch; ++b) {
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0) continue;
-    const size_t t = layout_for(h, plan_sequence(N, false), kv->num_heads, kv->head_dim).total + power_partial_bytes(N);
+    const size_t t = generic_layout(h, plan_sequence(N), kv->num_heads, kv->head_dim).total + power_partial_bytes(N);
     if (t > need) need = t;
   }
   return need;
@@ -1453,7 +1563,7 @@ extern "C" size_t fc_power_spectrum_workspace_bytes(const fc_handle *h, const fc
 
 extern "C" fc_status fc_power_spectrum(fc_handle *h, const fc_kv_view *kv, double *spectrum, void *workspace,
                                        size_t workspace_bytes, fc_stream stream) {
-  fc_status s = validate_view(h, kv);
+  fc_status s = validate_view(h, kv, true);
   if (s != FC_OK) return s;
   if (!spectrum) return FC_ERR_INVALID_ARG;
   const size_t need = fc_power_spectrum_workspace_bytes(h, kv);
@@ -1468,63 +1578,6 @@ extern "C" fc_status fc_power_spectrum(fc_handle *h, const fc_kv_view *kv, doubl
       case FC_F32: s = power_sequence<float>(h, st, kv, b, spectrum, (char *)workspace); break;
       case FC_F16: s = power_sequence<__half>(h, st, kv, b, spectrum, (char *)workspace); break;
       default: s = power_sequence<__nv_bfloat16>(h, st, kv, b, spectrum, (char *)workspace); break;
-    }
-  }
-  return s;
-}
-
-extern "C" fc_status fc_describe_plan(const fc_handle *h, int32_t seqlen, double gamma, int32_t out[4]) {
-  if (!h || !out || seqlen < 1 || !(gamma >= 0.0 && gamma <= 1.0)) return FC_ERR_INVALID_ARG;
-  if (seqlen > h->max_seqlen || (seqlen > 65536 && !is_pow2(seqlen))) return FC_ERR_UNSUPPORTED;
-  const SeqPlan sp = plan_sequence(seqlen);
-  out[0] = sp.bluestein ? 1 : 0;
-  out[1] = sp.Nfft;
-  out[2] = sp.N1;
-  out[3] = sp.N2;
-  if (sp.bluestein) {
-    const ChirpChoice c = choose_chirp(h, sp, seqlen, cutoff_index(gamma, seqlen), true);
-    out[0] = c.band >= 0 ? 2 : 1;
-    out[1] = c.M;
-    if (c.fast) {
-      const ChirpShape cs = chirp_shape(c.M);
-      out[2] = cs.n1();
-      out[3] = cs.n2();
-    }
-  }
-  return FC_OK;
-}
-
-extern "C" size_t fc_score_workspace_bytes(const fc_handle *h, const fc_kv_view *kv) {
-  if (validate_view(h, kv) != FC_OK) return 0;
-  size_t need = 256;
-  for (int b = 0; b < kv->batch; ++b) {
-    const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
-    if (N == 0) continue;
-    const ScoreLayout L = layout_for(h, plan_sequence(N, !h->generic_only), kv->num_heads, kv->head_dim);
-    if (L.total > need) need = L.total;
-  }
-  return need;
-}
-
-extern "C" fc_status fc_score_layer(fc_handle *h, const fc_kv_view *kv, double gamma, float *scores,
-                                    double *energy, void *workspace, size_t workspace_bytes,
-                                    fc_stream stream) {
-  fc_status s = validate_view(h, kv);
-  if (s != FC_OK) return s;
-  if (!scores || !energy) return FC_ERR_INVALID_ARG;
-  if (!(gamma >= 0.0 && gamma <= 1.0)) return FC_ERR_INVALID_ARG;
-  const size_t need = fc_score_workspace_bytes(h, kv);
-  if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < need) return FC_ERR_WORKSPACE;
-  int dev = -1;
-  FC_CUDA_TRY(cudaGetDevice(&dev));
-  if (dev != h->device) FC_CUDA_TRY(cudaSetDevice(h->device));
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  claim_persisting_l2(h, kv, st);
-  for (int b = 0; b < kv->batch && s == FC_OK; ++b) {
-    switch (kv->dtype) {
-      case FC_F32: s = score_sequence<float>(h, st, kv, b, gamma, scores, energy, (char *)workspace); break;
-      case FC_F16: s = score_sequence<__half>(h, st, kv, b, gamma, scores, energy, (char *)workspace); break;
-      default: s = score_sequence<__nv_bfloat16>(h, st, kv, b, gamma, scores, energy, (char *)workspace); break;
     }
   }
   return s;
@@ -1709,25 +1762,17 @@ extern "C" fc_status fc_score_layer_static(const fc_kv_view *kv, double gamma, f
   hs.status_word = su.status;
   hs.done_counter = su.counter;
   hs.group_bytes = 1;                 // one head per transform group: the smallest workspace
-  hs.tune_cpw = 32;
-  hs.tune_cp = 8;
   hs.prof_class = FC_K_NONE;
   hs.generic_only = true;
   hs.num_sms = su.num_sms;
-  s = validate_view(&hs, kv);         // lengths above kStaticMaxSeqlen come back as FC_ERR_UNSUPPORTED
+  s = validate_view(&hs, kv, true);         // lengths above kStaticMaxSeqlen come back as FC_ERR_UNSUPPORTED
   if (s != FC_OK) return s;
-  const size_t need = fc_score_workspace_bytes(&hs, kv);
-  if (need == 0) return FC_ERR_INVALID_ARG;
-  if (need > kStaticScratchBytes) return FC_ERR_WORKSPACE;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  for (int b = 0; b < kv->batch && s == FC_OK; ++b) {
-    switch (kv->dtype) {
-      case FC_F32: s = score_sequence<float>(&hs, st, kv, b, gamma, scores, energy, (char *)su.scratch); break;
-      case FC_F16: s = score_sequence<__half>(&hs, st, kv, b, gamma, scores, energy, (char *)su.scratch); break;
-      default: s = score_sequence<__nv_bfloat16>(&hs, st, kv, b, gamma, scores, energy, (char *)su.scratch); break;
-    }
-  }
-  return s;
+  if (score_layout(&hs, kv, 1).total > kStaticScratchBytes) return FC_ERR_WORKSPACE;
+  fc_layer_buffers one = {};
+  one.k = kv->k;
+  one.v = kv->v;
+  one.scores = scores;
+  return score_dispatch(&hs, static_cast<cudaStream_t>(stream), kv, &one, 1, gamma, energy, su.scratch);
 }
 
 extern "C" fc_status fc_static_last_device_status(fc_stream stream) {
