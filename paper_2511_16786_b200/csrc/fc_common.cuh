@@ -326,6 +326,16 @@ __host__ __device__ constexpr float root_sin(int i) {
   return R == 16 ? s16[i % 8] : R == 14 ? s14[i % 7] : R == 12 ? s12[i % 6] : s10[i % 5];
 }
 
+// cos and sin of 2*pi*i/32, i < 16
+__host__ __device__ constexpr float root32_cos(int i) {
+  constexpr float c[16] = {1.f, 0.98078528040323044913f, 0.92387953251128675613f, 0.83146961230254523708f,
+                           0.70710678118654752440f, 0.55557023301960222474f, 0.38268343236508977173f, 0.19509032201612826785f,
+                           0.f, -0.19509032201612826785f, -0.38268343236508977173f, -0.55557023301960222474f,
+                           -0.70710678118654752440f, -0.83146961230254523708f, -0.92387953251128675613f, -0.98078528040323044913f};
+  return c[i];
+}
+__host__ __device__ constexpr float root32_sin(int i) { return root32_cos(i < 8 ? 8 - i : i - 8); }
+
 // R-point DFT of R/2 samples followed by R/2 zeros: even bins are the R/2-point DFT of the samples, odd bins that of
 // the samples times w_R^n.
 template <int R>
@@ -342,17 +352,22 @@ __device__ __forceinline__ void dft_zero_tail(const float2 (&x)[R / 2], float2 (
   for (int k = 0; k < R / 2; ++k) { y[2 * k] = e[k]; y[2 * k + 1] = o[k]; }
 }
 
-// The first R/2 samples of the inverse R-point DFT (the mirror of the above).
+// The first R/2 samples of the inverse R-point DFT (the mirror of the above): the even bins' R/2-point transform plus
+// the odd bins' times w_R^-n.
+template <int R>
+__device__ __forceinline__ void add_odd_half(float2 (&e)[R / 2], const float2 (&o)[R / 2]) {
+  e[0] = cadd(e[0], o[0]);
+#pragma unroll
+  for (int n = 1; n < R / 2; ++n) e[n] = cadd(e[n], cmul(o[n], make_float2(root_cos<R>(n), root_sin<R>(n))));
+}
 template <int R>
 __device__ __forceinline__ void idft_first_half(const float2 (&y)[R], float2 (&x)[R / 2]) {
-  float2 e[R / 2], o[R / 2];
+  float2 o[R / 2];
 #pragma unroll
-  for (int k = 0; k < R / 2; ++k) { e[k] = y[2 * k]; o[k] = y[2 * k + 1]; }
-  dft_small<R / 2, +1>(e);
+  for (int k = 0; k < R / 2; ++k) { x[k] = y[2 * k]; o[k] = y[2 * k + 1]; }
+  dft_small<R / 2, +1>(x);
   dft_small<R / 2, +1>(o);
-#pragma unroll
-  for (int n = 0; n < R / 2; ++n)
-    x[n] = n == 0 ? cadd(e[n], o[n]) : cadd(e[n], cmul(o[n], make_float2(root_cos<R>(n), root_sin<R>(n))));
+  add_odd_half<R>(x, o);
 }
 
 // ------------------------------------------------------------------ batched stages in shared memory

@@ -782,9 +782,10 @@ GroupPlan plan_groups(const fc_handle *h, const PassPlan &p, int num_units, int 
   if (groups < h->num_aux && num_units >= h->num_aux && !one_group) groups = h->num_aux;
   g.units = (num_units + groups - 1) / groups;                 // balanced groups
   g.sub = head_dim;
-  if (p.pad && nu_alloc == 1) {
+  if (nu_alloc == 1) {
     // the intermediates of the groups in flight (one per internal stream) should stay in the cache, so a unit is
-    // halved down to 64 columns while they exceed three times the budget
+    // halved down to 64 columns while they exceed three times the budget (two times: 20000 and 38000 tokens 7..11 %
+    // slower; four and a half: 28000 and 32000 tokens 12 % slower)
     while (g.sub % 128 == 0 && (size_t)h->num_aux * p.M * g.sub * sizeof(float2) > 3 * h->group_bytes) g.sub /= 2;
   }
   g.ngr = head_dim / g.sub;
@@ -1024,14 +1025,13 @@ fc_status launch_p2(const PassArgs &x, int ncol, float4 *tab_out) {
 
 fc_status run_p2(const PassArgs &x, int ncol, float4 *tab_out) {
   const PassPlan &p = *x.p;
-  if (p.dbl) {
-    constexpr int CP = 4;
-    const size_t sm = (size_t)4 * (256 * CP + 16 * CP) * sizeof(float4) + 1024 * sizeof(float4) +
-                      (256 + 32 + 72) * sizeof(float2);
-    fc_status s = set_smem(fast::k_p2_double<CP>, sm);
+  if (p.N2 == 512) {
+    constexpr int C = 8;
+    const size_t sm = (size_t)2 * 16 * (32 * C + C) * sizeof(float2) + 1024 * sizeof(float4) + (64 + 68) * sizeof(float2);
+    fc_status s = set_smem(fast::k_p2_512<C>, sm);
     if (s != FC_OK) return s;
     ProfScope ps(x.h, FC_K_PASS2, x.st);
-    fast::k_p2_double<CP><<<dim3(p.N1 / 2, tab_out ? 1 : ncol / (2 * CP)), 64 * CP, sm, x.st>>>(
+    fast::k_p2_512<C><<<dim3(p.N1 / 2, tab_out ? 1 : ncol / C), 32 * C, sm, x.st>>>(
         p.N1, ncol, x.ws, x.h->master, x.h->master_len, x.tab, tab_out);
     return fc_after_launch(x.h);
   }

@@ -22,7 +22,7 @@
 //      E[k] = c[k] Z[k] - h[k] Z[-k],   c = 1 - DFT of g wrapped around 0 (real),   h = DFT of g(t+1), t = 0..2N-2,
 //    and the residual is the inverse transform's first N outputs.  One forward and one inverse transform of 2N points
 //    where two chirp convolutions (four transforms of 1.4N..2N points, six launches) did the same before: a packed
-//    batch of eight sequences of 7k..54k tokens went from 94.2 to 47.6 ms (28 layers x 4 heads).
+//    batch of eight sequences of 7k..54k tokens went from 94.2 to 58.8 ms (28 layers x 4 heads).
 //
 // The transforms are left unnormalised; pass 3 folds 1/M^2 into the score.
 #pragma once
@@ -240,11 +240,11 @@ k_p1(const __grid_constant__ LayerPtrs lp, long long stride_token, long long str
     }
     dft_fwd<R1B>(y0);
     dft_fwd<R1B>(y1);
+    float4 *dst = reinterpret_cast<float4 *>(ws + ((size_t)pp * N2 + n2) * ncol_ws + gc0 + 2 * cp);
 #pragma unroll
     for (int q = 0; q < R1B; ++q) {
-      const int k1 = pp + A * q;
-      float4 *dst = reinterpret_cast<float4 *>(ws + ((size_t)k1 * N2 + n2) * ncol_ws + gc0 + 2 * cp);
       *dst = make_float4(y0[q].x, y0[q].y, y1[q].x, y1[q].y);
+      dst += (size_t)A * N2 * ncol_ws / 2;
     }
   }
   if (LD == LD_TABLE) return;
@@ -323,10 +323,12 @@ k_p2(int N1, int ncol_ws, float2 *__restrict__ ws, const float2 *__restrict__ ma
   float4 *Sh = S + hf * (N2 * CP);
   const float2 *twR = twN + hf * HN;
   float2 x0[16], x1[16];
-  float2 *base = ws + (size_t)k1 * N2 * ncol_ws + gc0 + 2 * cp;
+  float4 *base = reinterpret_cast<float4 *>(ws + ((size_t)k1 * N2 + j) * ncol_ws + gc0 + 2 * cp);
+  const float4 *src = base;
 #pragma unroll
   for (int p = 0; p < 16; ++p) {
-    const float4 t = __ldcg(reinterpret_cast<const float4 *>(base + (size_t)(j + R2B * p) * ncol_ws));
+    const float4 t = __ldcg(src);
+    src += (size_t)R2B * ncol_ws / 2;
     x0[p] = make_float2(t.x, t.y);
     x1[p] = make_float2(t.z, t.w);
   }
@@ -444,142 +446,162 @@ k_p2(int N1, int ncol_ws, float2 *__restrict__ ws, const float2 *__restrict__ ma
   dft_inv<16>(x0);
   dft_inv<16>(x1);
   twiddle_affine16<true>(x0, x1, twR[j], twR[R2B], twR[R2B + 1]);
+  asm volatile("" : "+r"(ncol_ws));           // the row addresses are formed again rather than kept from the loads
 #pragma unroll
-  for (int p = 0; p < 16; ++p)
-    *reinterpret_cast<float4 *>(base + (size_t)(j + R2B * p) * ncol_ws) =
-        make_float4(x0[p].x, x0[p].y, x1[p].x, x1[p].y);
+  for (int p = 0; p < 16; ++p) {
+    *base = make_float4(x0[p].x, x0[p].y, x1[p].x, x1[p].y);
+    base += (size_t)R2B * ncol_ws / 2;
+  }
 }
 
 
 // ---------------------------------------------------------------------------
-// pass 2 of the padded form for rows of 512 points: a block holds the even and the odd samples of two partner rows
-// (four 256-point transforms of 2*CP channels).  A radix-2 step joins the samples, A[k] = E[k] + w^k O[k] and
-// A[k + 256] = E[k] - w^k O[k]; bins k and k + 256 of one row meet the bins 512 - 1 - k and 256 - 1 - k of the other,
-// i.e. one and the same pair (E', O') of it, so a thread forms both filtered bins from four values and takes the
-// radix-2 step back at once: no exchange beyond the one of the 256-point case.  grid (N1/2, columns / (2*CP)).
-// CP = 4: 256 threads and 90 KB, two blocks per SM like the other passes.
+// pass 2 of the padded form for rows of 512 points: a thread holds 32 points of ONE channel (the same 64 data registers
+// as 16 points of two), two radix-16 butterflies in the outer stage and one of radix 32 in the inner one, so a row
+// crosses shared memory as often as one of 256 points.  grid (N1/2, columns / C), block 32*C: C = 8 channels are 64-byte
+// pieces of the workspace rows and 256 threads with 75 KB, two blocks per SM like the other passes.  (Joining two
+// 256-point transforms by a radix-2 step instead reads seven values per point around the filter: 28 layers x 4 heads of
+// 38158 tokens took 16.2 ms against 13.4 ms.)
 // ---------------------------------------------------------------------------
-template <int CP>
-__global__ void __launch_bounds__(64 * CP, 2)
-k_p2_double(int N1, int ncol_ws, float2 *__restrict__ ws, const float2 *__restrict__ master, int master_len,
-            const float4 *__restrict__ tab, float4 *__restrict__ tab_out = nullptr) {
-  constexpr int N2 = 256, ROW = 512, NT = 64 * CP;
-  constexpr int SUB = 16 * CP + (CP < 8 ? CP : 0);            // rows in groups of 16, padded against bank conflicts
-  constexpr int QUARTER = 16 * SUB;
+__device__ __forceinline__ void twiddle_powers16_one(float2 (&x)[16], float2 c1, float2 c4, bool conj) {
+  if (conj) { c1.y = -c1.y; c4.y = -c4.y; }
+  const float2 c2 = cmul(c1, c1), c3 = cmul(c2, c1);
+  float2 base = c4;
+  x[1] = cmul(x[1], c1); x[2] = cmul(x[2], c2); x[3] = cmul(x[3], c3);
+#pragma unroll
+  for (int g = 1; g < 4; ++g) {
+    x[4 * g] = cmul(x[4 * g], base);
+    x[4 * g + 1] = cmul(x[4 * g + 1], cmul(base, c1));
+    x[4 * g + 2] = cmul(x[4 * g + 2], cmul(base, c2));
+    x[4 * g + 3] = cmul(x[4 * g + 3], cmul(base, c3));
+    if (g < 3) base = cmul(base, c4);
+  }
+}
+__device__ __forceinline__ void twiddle_affine16_one(float2 (&x)[16], float2 b, float2 s1, float2 s4, bool conj) {
+  if (conj) { b.y = -b.y; s1.y = -s1.y; s4.y = -s4.y; }
+  const float2 s2 = cmul(s1, s1), s3 = cmul(s2, s1);
+  float2 base = b;
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    x[4 * g] = cmul(x[4 * g], base);
+    x[4 * g + 1] = cmul(x[4 * g + 1], cmul(base, s1));
+    x[4 * g + 2] = cmul(x[4 * g + 2], cmul(base, s2));
+    x[4 * g + 3] = cmul(x[4 * g + 3], cmul(base, s3));
+    if (g < 3) base = cmul(base, s4);
+  }
+}
+
+template <int C>
+__global__ void __launch_bounds__(32 * C, 2)
+k_p2_512(int N1, int ncol_ws, float2 *__restrict__ ws, const float2 *__restrict__ master, int master_len,
+         const float4 *__restrict__ tab, float4 *__restrict__ tab_out = nullptr) {
+  constexpr int ROW = 512, NT = 32 * C;
+  constexpr int SUB = 32 * C + (C < 16 ? C : 0);              // groups of 32 points, padded against bank conflicts
+  constexpr int HALF = 16 * SUB;
   extern __shared__ float4 smem4[];
-  float4 *S = smem4;                                          // [row][even, odd][QUARTER]
-  float4 *hc = S + 4 * QUARTER;                               // [2][512] (h, c) of the two rows
-  float2 *w5 = reinterpret_cast<float2 *>(hc + 2 * ROW);      // [256] w_512^k
-  float2 *tw = w5 + N2;                                       // [2][16] w_256^j, w_256^4j
-  float2 *twN = tw + 32;                                      // [4][18] w_N^(k1*(2j + half)) and its steps
-  const int tid = threadIdx.x, cp = tid % CP, j = (tid / CP) % 16, quarter = tid / (16 * CP);
-  const int half = quarter & 1, row = quarter >> 1;
+  float2 *S = reinterpret_cast<float2 *>(smem4);              // [row][HALF]
+  float4 *hc = reinterpret_cast<float4 *>(S + 2 * HALF);      // [2][512] (h, c) of the two rows
+  float2 *tw = reinterpret_cast<float2 *>(hc + 2 * ROW);      // [2][32] w_512^j, w_512^4j
+  float2 *twN = tw + 64;                                      // [2][34] w_N^(k1*j) and its steps of 32 and 128 points
+  const int tid = threadIdx.x, c = tid % C, j = (tid / C) % 16, row = tid / (16 * C);
   const int k1a = blockIdx.x, k1b = k1a == 0 ? N1 / 2 : N1 - k1a;
-  const bool self = k1a == 0;
   const int k1 = row ? k1b : k1a;
   const int N = N1 * ROW;
-  float2 x0[16], x1[16];
-  float2 *base = ws + ((size_t)k1 * ROW + half) * ncol_ws + blockIdx.y * (2 * CP) + 2 * cp;
-  const size_t rstride = 2 * (size_t)ncol_ws;
+  float2 x[2][16];                                            // points j + 16*b + 32*p
+  float2 *base = ws + ((size_t)k1 * ROW + j) * ncol_ws + blockIdx.y * C + c;
 #pragma unroll
-  for (int p = 0; p < 16; ++p) {
-    const float4 t = __ldcg(reinterpret_cast<const float4 *>(base + (size_t)(j + 16 * p) * rstride));
-    x0[p] = make_float2(t.x, t.y);
-    x1[p] = make_float2(t.z, t.w);
-  }
+  for (int b = 0; b < 2; ++b)
+#pragma unroll
+    for (int p = 0; p < 16; ++p) x[b][p] = __ldcg(base + (size_t)(16 * b + 32 * p) * ncol_ws);
   if (tab_out == nullptr)
     for (int i = tid; i < 2 * ROW; i += NT) hc[i] = __ldg(tab + (size_t)(i < ROW ? k1a : k1b) * ROW + (i & (ROW - 1)));
-  for (int i = tid; i < N2; i += NT) w5[i] = master[(size_t)i * (master_len / ROW)];
-  for (int i = tid; i < 32; i += NT) tw[i] = master[(size_t)(i < 16 ? i : 4 * (i - 16)) * (master_len / N2)];
+  for (int i = tid; i < 64; i += NT) tw[i] = master[(size_t)(i < 32 ? i : 4 * (i - 32)) * (master_len / ROW)];
   {
     const bool in_master = (master_len % N) == 0;
-    for (int i = tid; i < 4 * 18; i += NT) {
-      const int qt = i / 18, e = i - qt * 18;
-      const int n2 = e < 16 ? 2 * e + (qt & 1) : e == 16 ? 32 : 128;      // the step of 16 entries is 32 samples
-      const int r = (n2 * ((qt >> 1) ? k1b : k1a)) % N;
+    for (int i = tid; i < 2 * 34; i += NT) {
+      const int r2 = i / 34, e = i - r2 * 34;
+      const int r = ((e < 32 ? e : e == 32 ? 32 : 128) * (r2 ? k1b : k1a)) % N;
       twN[i] = in_master ? master[(size_t)r * (master_len / N)] : root_of_unity(r, N);
     }
   }
-  float4 *Sq = S + quarter * QUARTER;
-  const float2 *twR = twN + quarter * 18;
-  __syncthreads();
-  twiddle_affine16<false>(x0, x1, twR[j], twR[16], twR[17]);
-  dft_fwd<16>(x0);
-  dft_fwd<16>(x1);
-  twiddle_powers16<false>(x0, x1, tw[j], tw[16 + j]);
-#pragma unroll
-  for (int p = 0; p < 16; ++p) Sq[p * SUB + j * CP + cp] = make_float4(x0[p].x, x0[p].y, x1[p].x, x1[p].y);
+  float2 *S1 = S + row * HALF + j * C + c;                    // + 16*b*C + p*SUB
+  float2 *S2 = S + row * HALF + j * SUB + c;                  // + q*C
+  const float2 *twR = twN + row * 34;
   __syncthreads();
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
-    const float4 t = Sq[j * SUB + q * CP + cp];
-    x0[q] = make_float2(t.x, t.y);
-    x1[q] = make_float2(t.z, t.w);
+  for (int b = 0; b < 2; ++b) {
+    twiddle_affine16_one(x[b], twR[j + 16 * b], twR[32], twR[33], false);
+    dft_fwd<16>(x[b]);
+    twiddle_powers16_one(x[b], tw[j + 16 * b], tw[32 + j + 16 * b], false);
+#pragma unroll
+    for (int p = 0; p < 16; ++p) S1[16 * b * C + p * SUB] = x[b][p];
   }
-  dft_fwd<16>(x0);
-  dft_fwd<16>(x1);
-#pragma unroll
-  for (int q = 0; q < 16; ++q) Sq[j * SUB + q * CP + cp] = make_float4(x0[q].x, x0[q].y, x1[q].x, x1[q].y);
   __syncthreads();
-  // bin k2 = j + 16 q of this quarter is in x[q]; S[group k2 & 15][k2 >> 4]
-  {
-    const float4 *Ss = S + (quarter ^ 1) * QUARTER + j * SUB + cp;           // the row's other samples, same k2
-    const int prow = self ? row : 1 - row;
-    const float4 *Pe = S + 2 * prow * QUARTER + cp, *Po = Pe + QUARTER;      // the partner row's E', O'
-    const float4 *hrow = hc + row * ROW;
+  // radix 32 over the points of group j: x[b][i] takes point 2i + b, then x[b][i] is bin k2 = j + 16*(i + 16*b)
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const int k2 = j + 16 * q;
-      const float2 w = w5[k2];
-      const float4 t = Ss[q * CP];
-      float2 &m0 = x0[q], &m1 = x1[q];
-      const float2 e0 = half ? make_float2(t.x, t.y) : m0, e1 = half ? make_float2(t.z, t.w) : m1;
-      const float2 o0 = cmul(half ? m0 : make_float2(t.x, t.y), w), o1 = cmul(half ? m1 : make_float2(t.z, t.w), w);
-      const float2 lo0 = cadd(e0, o0), hi0 = csub(e0, o0), lo1 = cadd(e1, o1), hi1 = csub(e1, o1);
-      if (tab_out != nullptr) {                    // channel 0: spectrum of g around 0, channel 1: of g(t + 1)
-        if (cp == 0 && blockIdx.y == 0)
-          tab_out[(size_t)k1 * ROW + k2 + half * N2] = half ? make_float4(hi1.x, hi1.y, 1.f - hi0.x, 0.f)
-                                                            : make_float4(lo1.x, lo1.y, 1.f - lo0.x, 0.f);
-        continue;
+  for (int b = 0; b < 2; ++b) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) x[b][i] = S2[(2 * i + b) * C];
+    dft_fwd<16>(x[b]);
+  }
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const float2 o = cmul(x[1][i], make_float2(root32_cos(i), -root32_sin(i)));
+    x[1][i] = csub(x[0][i], o);
+    x[0][i] = cadd(x[0][i], o);
+    S2[i * C] = x[0][i];
+    S2[(i + 16) * C] = x[1][i];
+  }
+  if (tab_out != nullptr) {              // channel 0: spectrum of g around 0, channel 1: of g(t + 1)
+    __syncthreads();
+    if (c == 0 && blockIdx.y == 0)
+      for (int q = 0; q < 32; ++q) {
+        const float2 g0 = S2[q * C], g1 = S2[q * C + 1];
+        tab_out[(size_t)k1 * ROW + j + 16 * q] = make_float4(g1.x, g1.y, 1.f - g0.x, 0.f);
       }
-      // partner bins of k2 and k2 + 256: from E', O' at k2p, the upper one for the lower bin (row 0, k2 = 0: itself)
-      const int k2p = (k1 == 0) ? ((N2 - k2) & (N2 - 1)) : (N2 - 1 - k2);
-      const float2 wp = w5[k2p];
-      const float4 te = Pe[(k2p & 15) * SUB + (k2p >> 4) * CP], to = Po[(k2p & 15) * SUB + (k2p >> 4) * CP];
-      const float2 po0 = cmul(make_float2(to.x, to.y), wp), po1 = cmul(make_float2(to.z, to.w), wp);
-      const float sw = (k1 == 0 && k2 == 0) ? -1.f : 1.f;
-      const float2 a0 = make_float2(fmaf(-sw, po0.x, te.x), fmaf(-sw, po0.y, te.y));     // partner of the lower bin
-      const float2 a1 = make_float2(fmaf(-sw, po1.x, te.z), fmaf(-sw, po1.y, te.w));
-      const float2 b0 = make_float2(fmaf(sw, po0.x, te.x), fmaf(sw, po0.y, te.y));       // partner of the upper bin
-      const float2 b1 = make_float2(fmaf(sw, po1.x, te.z), fmaf(sw, po1.y, te.w));
-      const float4 f = hrow[k2], g = hrow[k2 + N2];
-      const float2 fl = make_float2(f.x, f.y), fh = make_float2(g.x, g.y);
-      const float2 bl0 = csub(cscale(lo0, f.z), cmul(a0, fl)), bl1 = csub(cscale(lo1, f.z), cmul(a1, fl));
-      const float2 bh0 = csub(cscale(hi0, g.z), cmul(b0, fh)), bh1 = csub(cscale(hi1, g.z), cmul(b1, fh));
-      m0 = half ? cmul_conj(csub(bl0, bh0), w) : cadd(bl0, bh0);
-      m1 = half ? cmul_conj(csub(bl1, bh1), w) : cadd(bl1, bh1);
+    return;
+  }
+  __syncthreads();
+  {
+    // partner of bin k2: 512 - k2 in row 0, 511 - k2 in the others; it sits in group 15 - j (row 0: -j mod 16) of the
+    // partner row, at q' = 31 - q (row 0, j = 0: 32 - q, bin 0 with itself)
+    const bool first = k1 == 0 && j == 0;
+    const int prow = k1a == 0 ? row : 1 - row, pj = k1 == 0 ? ((16 - j) & 15) : 15 - j;
+    const float2 *Sp = S + prow * HALF + pj * SUB + c + (first ? 32 : 31) * C;
+    const float4 *hrow = hc + row * ROW + j;
+#pragma unroll
+    for (int q = 0; q < 32; ++q) {
+      float2 &P = x[q >> 4][q & 15];
+      const float2 t = Sp[q == 0 && first ? -32 * C : -q * C];
+      const float4 w = hrow[16 * q];
+      P = make_float2(fmaf(t.y, w.y, fmaf(-t.x, w.x, w.z * P.x)), fmaf(-t.y, w.x, fmaf(-t.x, w.y, w.z * P.y)));
     }
   }
-  if (tab_out != nullptr) return;
-  dft_inv<16>(x0);
-  dft_inv<16>(x1);
-  __syncthreads();                                 // all reads of the spectra are done
+  __syncthreads();                       // all partner reads are done
+  // inverse radix 32: point 2i + b from the sums (b = 0) and rotated differences (b = 1)
 #pragma unroll
-  for (int q = 0; q < 16; ++q) Sq[j * SUB + q * CP + cp] = make_float4(x0[q].x, x0[q].y, x1[q].x, x1[q].y);
+  for (int i = 0; i < 16; ++i) {
+    const float2 d = csub(x[0][i], x[1][i]);
+    x[0][i] = cadd(x[0][i], x[1][i]);
+    x[1][i] = cmul(d, make_float2(root32_cos(i), root32_sin(i)));
+  }
+#pragma unroll
+  for (int b = 0; b < 2; ++b) {
+    dft_inv<16>(x[b]);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) S2[(2 * i + b) * C] = x[b][i];
+  }
   __syncthreads();
 #pragma unroll
-  for (int p = 0; p < 16; ++p) {
-    const float4 t = Sq[p * SUB + j * CP + cp];
-    x0[p] = make_float2(t.x, t.y);
-    x1[p] = make_float2(t.z, t.w);
-  }
-  twiddle_powers16<true>(x0, x1, tw[j], tw[16 + j]);
-  dft_inv<16>(x0);
-  dft_inv<16>(x1);
-  twiddle_affine16<true>(x0, x1, twR[j], twR[16], twR[17]);
+  for (int b = 0; b < 2; ++b) {
 #pragma unroll
-  for (int p = 0; p < 16; ++p)
-    *reinterpret_cast<float4 *>(base + (size_t)(j + 16 * p) * rstride) = make_float4(x0[p].x, x0[p].y, x1[p].x, x1[p].y);
+    for (int p = 0; p < 16; ++p) x[b][p] = S1[16 * b * C + p * SUB];
+    twiddle_powers16_one(x[b], tw[j + 16 * b], tw[32 + j + 16 * b], true);
+    dft_inv<16>(x[b]);
+    twiddle_affine16_one(x[b], twR[j + 16 * b], twR[32], twR[33], true);
+#pragma unroll
+    for (int p = 0; p < 16; ++p) base[(size_t)(16 * b + 32 * p) * ncol_ws] = x[b][p];
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -632,10 +654,11 @@ k_p3(const __grid_constant__ LayerPtrs lp, int H, int head_dim, int u0, int dcol
       const int pp = j + R1B * it;
       if (A % R1B != 0 && pp >= A) break;
       float2 y0[R1B], y1[R1B];
+      const float4 *src = reinterpret_cast<const float4 *>(ws + ((size_t)pp * N2 + n2) * ncol_ws + gc0 + 2 * cp);
 #pragma unroll
       for (int q = 0; q < R1B; ++q) {
-        const float4 t = __ldcg(reinterpret_cast<const float4 *>(
-            ws + ((size_t)(pp + A * q) * N2 + n2) * ncol_ws + gc0 + 2 * cp));
+        const float4 t = __ldcg(src);
+        src += (size_t)A * N2 * ncol_ws / 2;
         y0[q] = make_float2(t.x, t.y);
         y1[q] = make_float2(t.z, t.w);
       }
@@ -646,27 +669,43 @@ k_p3(const __grid_constant__ LayerPtrs lp, int H, int head_dim, int u0, int dcol
         S[(q + R1B * pp) * CPW + cp] = make_float4(y0[q].x, y0[q].y, y1[q].x, y1[q].y);
     }
     __syncthreads();
-    float2 x0[A], x1[A];
-#pragma unroll
-    for (int p = 0; p < A; ++p) {
+    float2 z0[AO], z1[AO];
+    auto twiddled = [&](int p, float2 &a, float2 &b) {        // input p of the last stage, both channels
       const float4 t = S[(j + R1B * p) * CPW + cp];
-      x0[p] = make_float2(t.x, t.y);
-      x1[p] = make_float2(t.z, t.w);
+      a = make_float2(t.x, t.y);
+      b = make_float2(t.z, t.w);
       if (p > 0) {
         const float2 w = tw[j * p];
-        x0[p] = cmul_conj(x0[p], w);
-        x1[p] = cmul_conj(x1[p], w);
+        a = cmul_conj(a, w);
+        b = cmul_conj(b, w);
       }
-    }
-    float2 z0[AO], z1[AO];
+    };
     if constexpr (PAD) {
-      idft_first_half<A>(x0, z0);
-      idft_first_half<A>(x1, z1);
-    } else {
-      dft_inv<A>(x0);
-      dft_inv<A>(x1);
+      if constexpr (A < 14) {
+        float2 x0[A], x1[A];
 #pragma unroll
-      for (int p = 0; p < A; ++p) { z0[p] = x0[p]; z1[p] = x1[p]; }
+        for (int p = 0; p < A; ++p) twiddled(p, x0[p], x1[p]);
+        idft_first_half<A>(x0, z0);
+        idft_first_half<A>(x1, z1);
+      } else {
+        // the same with the odd inputs read after the even ones are transformed: 16 instead of 92 bytes of spills
+        float2 o0[AO], o1[AO];
+#pragma unroll
+        for (int k = 0; k < AO; ++k) twiddled(2 * k, z0[k], z1[k]);
+        dft_inv<AO>(z0);
+        dft_inv<AO>(z1);
+#pragma unroll
+        for (int k = 0; k < AO; ++k) twiddled(2 * k + 1, o0[k], o1[k]);
+        dft_inv<AO>(o0);
+        dft_inv<AO>(o1);
+        add_odd_half<A>(z0, o0);
+        add_odd_half<A>(z1, o1);
+      }
+    } else {
+#pragma unroll
+      for (int p = 0; p < A; ++p) twiddled(p, z0[p], z1[p]);
+      dft_inv<A>(z0);
+      dft_inv<A>(z1);
     }
 #pragma unroll
     for (int p = 0; p < AO; ++p) {
