@@ -192,8 +192,14 @@ def _check(code: int, where: str):
         raise FlashCacheError(code, where)
 
 
-def _stream() -> c_void_p:
-    return c_void_p(torch.cuda.current_stream().cuda_stream)
+# the raw handle of the current stream, without building a torch.cuda.Stream object on every call
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _stream() -> int:
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _cu_array(cu_seqlens):
@@ -413,8 +419,9 @@ def fc_decode_workspace_bytes(handle, args) -> int:
 
 def fc_decode_attention(handle, args, out, workspace) -> None:
     """out: [B, Hq, d] device tensor of the cache dtype."""
-    _check(_lib.fc_decode_attention(handle, byref(args), c_void_p(out.data_ptr()), c_void_p(workspace.data_ptr()),
-                                    workspace.numel() * workspace.element_size(), _stream()), "fc_decode_attention")
+    rc = _lib.fc_decode_attention(handle, byref(args), out.data_ptr(), workspace.data_ptr(), workspace.nbytes, _stream())
+    if rc != FC_OK:
+        raise FlashCacheError(rc, "fc_decode_attention")
 
 
 def fc_reset_ordering(handle) -> None:

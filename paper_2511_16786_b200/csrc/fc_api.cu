@@ -131,6 +131,7 @@ extern "C" fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen) 
   h->master = nullptr;
   h->status_word = nullptr;
   h->done_counter = nullptr;
+  h->decode_ready = false;
   h->group_bytes = (size_t)32 << 20;
   h->launches = 0;
   h->num_aux = 2;

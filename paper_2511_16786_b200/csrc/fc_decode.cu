@@ -1,13 +1,19 @@
 // Decoding step on the compacted cache (Sec. 3.1, Eq. 3-4): Softmax(q K^T / sqrt(d)) V over the rows the
 // compressor kept plus the uncompressed tail.  The step reads every K and V row once and is bound by
-// that read, so the design is about keeping HBM busy:
+// that read (or, on short caches, by the chain of latencies of one launch), so the design is about keeping HBM busy:
 //
-//  * grid (splits, KV heads, sequences); a block walks its share of the rows in tiles of 64, filled by
-//    tiled TMA loads (128-byte swizzle) into a four-stage shared-memory ring behind mbarriers;
+//  * the tiles (64 rows) of all sequences of all KV heads form one line, and the grid's blocks, one per SM, take equal
+//    shares of it, whatever the lengths of the sequences are: a block's share is one or more runs of consecutive tiles
+//    of one sequence and head each (28 layers of kept rows 1638, 205, 3277, 820: 382 -> 335 us per step, where a grid of
+//    splits sized for the longest sequence left half of the SMs without rows);
+//  * a producer warp fills a four-stage shared-memory ring by tiled TMA loads (128-byte swizzle), one mbarrier pair per
+//    stage; the four other warps wait for nothing but the tile they use;
 //  * all query heads of a KV head (up to 16) are one 16-row operand of m16n8k16 tensor-core products,
 //    so a K/V tile is read from shared memory once for the whole group; each of the 4 warps owns 16
 //    rows of the tile and keeps its own running maximum, sum and 16 x 128 fp32 output;
-//  * the warps' partial results are merged in shared memory, the splits' in a second small kernel.
+//  * the warps' partial results are merged in shared memory; a sequence covered by one block is finished there, else a
+//    second small kernel merges the blocks' shares (28 layers of 65536 rows: 926 -> 808 us per step).
+// Both launches are programmatic dependents: they are set up while the kernel before them in the stream ends.
 #include <cuda.h>
 
 #include "fc_common.cuh"
@@ -16,25 +22,25 @@ namespace {
 
 constexpr int kD = 128;                 // head_dim
 constexpr int kTile = 64;               // rows per tile
-constexpr int kWarps = 4;
-constexpr int kThreadsD = 32 * kWarps;
+constexpr int kWarps = 4;               // consumer warps; one more loads
+constexpr int kConsumers = 32 * kWarps;
+constexpr int kThreadsD = kConsumers + 32;
 constexpr int kBoxBytes = kTile * 128;  // one TMA box: 64 rows x 64 elements of 2 bytes
 constexpr int kStageBytes = 4 * kBoxBytes;   // K low/high halves, V low/high halves
-// tiles in the shared-memory ring: 4 (one resident block per SM, three tiles in flight) measured best;
-// 2 and 3 (three and two blocks per SM) and 5..7 were slower (1.05, 0.98, 0.84..0.91 against 0.82 ms for
-// 28 layers of 65536 rows)
 constexpr int kStages = 4;
 constexpr unsigned kSuspendNs = 2000u;        // a blocking test of an mbarrier sleeps at most about this long
 constexpr unsigned kSpinLimit = 1u << 17;    // such tests before a wait gives up (a quarter of a second)
 
 struct DecodeParams {
   const void *q;
+  void *out;
   const long long *offsets;
   const int *tail_len;
-  float *part_o;        // [batch][q heads][splits][128]
-  float2 *part_ml;      // [batch][q heads][splits]: (running maximum in log2 units, sum)
+  float *part_o;        // [slot][query heads of a KV head][128]
+  float2 *part_ml;      // [slot][query heads of a KV head]: (running maximum in log2 units, sum)
+  int2 *span;           // [H][batch]: first and last block with tiles of the sequence (first > last: none)
   int *status;
-  int H, Hq, G, nsplit, chunk, tail_cap, has_tail;
+  int B, H, Hq, G, nb, tail_cap, has_tail;
   float scale_log2;     // log2(e) / sqrt(d)
 };
 
@@ -48,6 +54,10 @@ __device__ __forceinline__ void mbar_init(unsigned long long *bar, unsigned coun
 __device__ __forceinline__ void mbar_expect_tx(unsigned long long *bar, unsigned bytes) {
   asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n"
                ::"r"((unsigned)__cvta_generic_to_shared(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(unsigned long long *bar) {
+  asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n"
+               ::"r"((unsigned)__cvta_generic_to_shared(bar)) : "memory");
 }
 // One potentially blocking test: the thread sleeps until the phase completes or a hardware time limit passes.
 __device__ __forceinline__ bool mbar_try(unsigned long long *bar, unsigned parity) {
@@ -74,6 +84,10 @@ __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *map, i
   asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];\n"
                ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(reinterpret_cast<unsigned long long>(map)),
                  "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"((unsigned)__cvta_generic_to_shared(bar)) : "memory");
+}
+
+__device__ __forceinline__ void prefetch_map(const CUtensorMap *map) {
+  asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<unsigned long long>(map)) : "memory");
 }
 
 __device__ __forceinline__ void ldmatrix_x4(unsigned addr, unsigned (&r)[4]) {
@@ -121,236 +135,399 @@ __device__ __forceinline__ unsigned tile_offset(int row, int chunk) {
 
 constexpr int kMergeStride = kD + 4;    // floats per row of a warp's output in the merge buffer
 
-// One block: KV head h of sequence b, logical rows [split*chunk, (split+1)*chunk).  Logical rows are the kept
-// rows, padded to a multiple of the tile, followed by the tail rows, so that every tile lies in one segment.
+// One sequence: its rows in the cache and in the tail, as tiles (main rows first; a tile lies in one of the two).
+struct SeqRows {
+  long long off0;
+  int n_main, n_tail, tiles_main, tiles;
+};
+__device__ __forceinline__ SeqRows seq_rows(const DecodeParams &P, int b) {
+  SeqRows s;
+  s.off0 = P.offsets[b];
+  const long long nm = P.offsets[b + 1] - s.off0;
+  s.n_main = nm < 0 ? 0 : (int)nm;
+  int nt = P.has_tail ? P.tail_len[b] : 0;
+  s.n_tail = nt < 0 ? 0 : (nt > P.tail_cap ? P.tail_cap : nt);
+  s.tiles_main = (s.n_main + kTile - 1) / kTile;
+  s.tiles = s.tiles_main + (s.n_tail + kTile - 1) / kTile;
+  return s;
+}
+
+// The line of T tiles, head after head and sequence after sequence: block i takes the tiles [i*T/nb, (i+1)*T/nb).
+// (32-bit division where the product fits: a 64-bit one costs some hundred cycles before the first load.)
+__device__ __forceinline__ long long muldiv(long long a, int m, long long d) {
+  const unsigned long long x = (unsigned long long)a * (unsigned)m;
+  return (x >> 32) == 0 && ((unsigned long long)d >> 32) == 0 ? (long long)((unsigned)x / (unsigned)d) : (long long)(x / (unsigned long long)d);
+}
+__device__ __forceinline__ long long share_start(int i, long long T, int nb) { return muldiv(T, i, nb); }
+__device__ __forceinline__ int share_of(long long t, long long T, int nb) {
+  const unsigned long long x = (unsigned long long)(t + 1) * (unsigned)nb - 1;
+  return (x >> 32) == 0 && ((unsigned long long)T >> 32) == 0 ? (int)((unsigned)x / (unsigned)T) : (int)(x / (unsigned long long)T);
+}
+
+__device__ __forceinline__ void consumers_sync() { asm volatile("bar.sync 1, %0;\n" ::"n"(kConsumers) : "memory"); }
+
+struct DecodeShared {
+  unsigned long long full[kStages], empty[kStages];
+};
+
+__device__ __forceinline__ void fold(float4 &acc, const float4 &v, float f) {      // acc += f * v
+  acc.x = fmaf(v.x, f, acc.x);
+  acc.y = fmaf(v.y, f, acc.y);
+  acc.z = fmaf(v.z, f, acc.z);
+  acc.w = fmaf(v.w, f, acc.w);
+}
+template <typename T>
+__device__ __forceinline__ void store_head(T *out, const float4 &o, float l) {      // four channels of o / l
+  const float inv = l > 0.f ? 1.f / l : 0.f;
+  uint2 pk;
+  pk.x = Mma<T>::pack(o.x * inv, o.y * inv);
+  pk.y = Mma<T>::pack(o.z * inv, o.w * inv);
+  *reinterpret_cast<uint2 *>(out) = pk;
+}
+
+// One block: its share of the line of tiles.
 template <typename T>
 __global__ void __launch_bounds__(kThreadsD)
-k_decode_partial(const DecodeParams P, const __grid_constant__ DecodeMaps M) {
+k_decode(const DecodeParams P, const __grid_constant__ DecodeMaps M) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  unsigned long long *full = reinterpret_cast<unsigned long long *>(smem + kStages * kStageBytes);
-  const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
+  float *mbuf = reinterpret_cast<float *>(smem + kStages * kStageBytes);
+  __shared__ DecodeShared sh;
+  const int blk = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;
 
-  const long long off0 = P.offsets[b];
-  long long nm = P.offsets[b + 1] - off0;
-  const int n_main = nm < 0 ? 0 : (int)nm;
-  const int n_main_pad = (n_main + kTile - 1) / kTile * kTile;
-  int n_tail = P.has_tail ? P.tail_len[b] : 0;
-  n_tail = n_tail < 0 ? 0 : (n_tail > P.tail_cap ? P.tail_cap : n_tail);
-  const int total = n_tail > 0 ? n_main_pad + n_tail : n_main;
-  const int lo = split * P.chunk;
-  const int hi = lo + P.chunk < total ? lo + P.chunk : total;
-  const int ntiles = lo < hi ? (hi - lo + kTile - 1) / kTile : 0;
-
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   if (tid == 0) {
-    for (int i = 0; i < kStages; ++i) mbar_init(&full[i], 1u);
+    for (int i = 0; i < kStages; ++i) { mbar_init(&sh.full[i], 1u); mbar_init(&sh.empty[i], kWarps); }
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
+  if (tid == kConsumers) {
+    prefetch_map(&M.k);
+    prefetch_map(&M.v);
+    if (P.has_tail) { prefetch_map(&M.tk); prefetch_map(&M.tv); }
+  }
   __syncthreads();
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");       // what the kernels before this one wrote is visible from here
 
-  // the query heads of this KV head as the 16 x 128 left operand (rows past the group are zero)
-  unsigned qf[kD / 16][4];
+  // Tiles of all sequences, 32 at a time, in every warp for itself (no barrier before the first load): the sum, then
+  // the sequence that holds the first tile of this block's share.
+  auto tiles_of = [&](int i) { return i < P.B ? seq_rows(P, i).tiles : 0; };
+  const int first32 = tiles_of(lane);
+  long long total = __reduce_add_sync(0xffffffffu, first32);
+  for (int b0 = 32; b0 < P.B; b0 += 32) total += __reduce_add_sync(0xffffffffu, tiles_of(b0 + lane));
+  const long long line_len = total * P.H;                    // every head has the same tiles
+  const int nb = line_len < P.nb ? (int)line_len : P.nb;     // blocks that have tiles
+  const long long lo = blk < nb ? share_start(blk, line_len, nb) : 0, hi = blk < nb ? share_start(blk + 1, line_len, nb) : 0;
+  int h = lo > 0 ? (int)muldiv(lo, 1, total) : 0;
+  const long long lo_head = lo - h * total;                  // within the head
+  int b = 0;
+  long long line = 0;                          // position of the first tile of (h, b)
   {
-    const T *qb = static_cast<const T *>(P.q) + ((long long)b * P.Hq + (long long)h * P.G) * kD;
-    const bool r0 = g < P.G, r1 = g + 8 < P.G;
+    long long at = 0;
+    for (int b0 = 0; b0 < P.B; b0 += 32) {
+      const int mine = b0 == 0 ? first32 : tiles_of(b0 + lane);
+      int incl = mine;
 #pragma unroll
-    for (int kk = 0; kk < kD / 16; ++kk) {
-      const int c = 16 * kk + 2 * t;
-      qf[kk][0] = r0 ? *reinterpret_cast<const unsigned *>(qb + g * kD + c) : 0u;
-      qf[kk][1] = r1 ? *reinterpret_cast<const unsigned *>(qb + (g + 8) * kD + c) : 0u;
-      qf[kk][2] = r0 ? *reinterpret_cast<const unsigned *>(qb + g * kD + c + 8) : 0u;
-      qf[kk][3] = r1 ? *reinterpret_cast<const unsigned *>(qb + (g + 8) * kD + c + 8) : 0u;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      const unsigned past = __ballot_sync(0xffffffffu, at + incl > lo_head);
+      if (past) {
+        const int first = __ffs(past) - 1;
+        b = b0 + first;
+        line = h * total + at + __shfl_sync(0xffffffffu, incl - mine, first);
+        break;
+      }
+      at += __shfl_sync(0xffffffffu, incl, 31);
     }
   }
-
-  auto issue = [&](int ti, int s) {
-    const int row0 = lo + ti * kTile;
-    unsigned char *dst = smem + s * kStageBytes;
-    mbar_expect_tx(&full[s], (unsigned)kStageBytes);
-    if (row0 < n_main_pad) {
-      const int r = (int)(off0 + row0);
-      tma_load_3d(dst, &M.k, 0, h, r, &full[s]);
-      tma_load_3d(dst + kBoxBytes, &M.k, 64, h, r, &full[s]);
-      tma_load_3d(dst + 2 * kBoxBytes, &M.v, 0, h, r, &full[s]);
-      tma_load_3d(dst + 3 * kBoxBytes, &M.v, 64, h, r, &full[s]);
-    } else {
-      const int r = row0 - n_main_pad;
-      tma_load_4d(dst, &M.tk, 0, h, r, b, &full[s]);
-      tma_load_4d(dst + kBoxBytes, &M.tk, 64, h, r, b, &full[s]);
-      tma_load_4d(dst + 2 * kBoxBytes, &M.tv, 0, h, r, b, &full[s]);
-      tma_load_4d(dst + 3 * kBoxBytes, &M.tv, 64, h, r, b, &full[s]);
+  if (blk == 0)                                // sequences without rows
+    for (int i = tid; i < P.B; i += kThreadsD)
+      if (seq_rows(P, i).tiles == 0) {
+        for (int hh = 0; hh < P.H; ++hh) P.span[(size_t)hh * P.B + i] = make_int2(0, -1);
+        for (int c = 0; c < P.Hq * kD / 8; ++c)
+          reinterpret_cast<uint4 *>(static_cast<T *>(P.out) + (size_t)i * P.Hq * kD)[c] = make_uint4(0u, 0u, 0u, 0u);
+      }
+  if (lo >= hi) return;
+  SeqRows s = seq_rows(P, b);
+  auto advance = [&](long long ti) {           // on to the sequence and head that tile ti belongs to
+    while (ti >= line + s.tiles) {
+      line += s.tiles;
+      if (++b == P.B) { b = 0; ++h; }
+      s = seq_rows(P, b);
     }
   };
 
-  float oacc[kD / 8][4];
-#pragma unroll
-  for (int j = 0; j < kD / 8; ++j) oacc[j][0] = oacc[j][1] = oacc[j][2] = oacc[j][3] = 0.f;
-  float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
-  const unsigned sbase = (unsigned)__cvta_generic_to_shared(smem);
-  bool failed = false;
-  int issued = 0, consumed = 0;
-
-  if (tid == 0)
-    for (int ti = 0; ti < kStages - 1 && ti < ntiles; ++ti) { issue(ti, ti); issued = ti + 1; }
-
-  for (int ti = 0; ti < ntiles; ++ti) {
-    const int s = ti % kStages;
-    if (tid == 0 && ti + kStages - 1 < ntiles) {          // into the stage that the barrier below released last time round
-      issue(ti + kStages - 1, (ti + kStages - 1) % kStages);
-      issued = ti + kStages;
+  if (warp == kWarps) {
+    // producer
+    if (lane == 0) {
+      int n = 0;
+      bool ok = true;
+      for (long long ti = lo; ti < hi; ++ti, ++n) {
+        advance(ti);
+        const int st = n % kStages;
+        if (n >= kStages && !mbar_wait(&sh.empty[st], (unsigned)(n / kStages - 1) & 1u)) { ok = false; break; }
+        unsigned char *dst = smem + st * kStageBytes;
+        mbar_expect_tx(&sh.full[st], (unsigned)kStageBytes);
+        const int lt = (int)(ti - line);
+        if (lt < s.tiles_main) {
+          const int r = (int)(s.off0 + (long long)lt * kTile);
+          tma_load_3d(dst, &M.k, 0, h, r, &sh.full[st]);
+          tma_load_3d(dst + kBoxBytes, &M.k, 64, h, r, &sh.full[st]);
+          tma_load_3d(dst + 2 * kBoxBytes, &M.v, 0, h, r, &sh.full[st]);
+          tma_load_3d(dst + 3 * kBoxBytes, &M.v, 64, h, r, &sh.full[st]);
+        } else {
+          const int r = (lt - s.tiles_main) * kTile;
+          tma_load_4d(dst, &M.tk, 0, h, r, b, &sh.full[st]);
+          tma_load_4d(dst + kBoxBytes, &M.tk, 64, h, r, b, &sh.full[st]);
+          tma_load_4d(dst + 2 * kBoxBytes, &M.tv, 0, h, r, b, &sh.full[st]);
+          tma_load_4d(dst + 3 * kBoxBytes, &M.tv, 64, h, r, b, &sh.full[st]);
+        }
+      }
+      // a consumer gave up: the loads still in flight write this block's shared memory, give them a bounded chance
+      if (!ok) {
+        atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
+        for (int i = n > kStages ? n - kStages : 0; i < n; ++i)
+          mbar_wait(&sh.full[i % kStages], (unsigned)(i / kStages) & 1u);
+      }
     }
-    const bool got = mbar_wait(&full[s], (unsigned)(ti / kStages) & 1u);
-    if (__syncthreads_or(got ? 0 : 1)) { failed = true; consumed = ti; break; }
-    const int row0 = lo + ti * kTile;
-    int valid = (row0 < n_main_pad ? n_main : total) - row0;
-    valid = valid > kTile ? kTile : valid;
-    const int wrow = 16 * warp;
-    if (wrow < valid) {
-      const unsigned sb = sbase + (unsigned)(s * kStageBytes);
-      float sacc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-      const int mi = lane >> 3;
+    return;
+  }
+
+  // consumers
+  const unsigned sbase = (unsigned)__cvta_generic_to_shared(smem);
+  float *mo = mbuf;                                                            // [warp][16][kMergeStride]
+  float2 *mml = reinterpret_cast<float2 *>(mo + kWarps * 16 * kMergeStride);   // [warp][16]
+  bool failed = false;
+  int n = 0;
+  for (long long ti = lo; ti < hi;) {
+    advance(ti);
+    const long long seg_end = line + s.tiles < hi ? line + s.tiles : hi;
+    // the query heads of this KV head as the 16 x 128 left operand (rows past the group are zero)
+    unsigned qf[kD / 16][4];
+    {
+      const T *qb = static_cast<const T *>(P.q) + ((long long)b * P.Hq + (long long)h * P.G) * kD;
+      const bool r0 = g < P.G, r1 = g + 8 < P.G;
 #pragma unroll
       for (int kk = 0; kk < kD / 16; ++kk) {
-        unsigned r[4];
-        ldmatrix_x4(sb + tile_offset(wrow + (mi >> 1) * 8 + (lane & 7), 2 * kk + (mi & 1)), r);
-        Mma<T>::run(sacc[0], qf[kk], r[0], r[1]);
-        Mma<T>::run(sacc[1], qf[kk], r[2], r[3]);
-      }
-      float mx[2] = {-INFINITY, -INFINITY};
-#pragma unroll
-      for (int nb = 0; nb < 2; ++nb)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int key = wrow + 8 * nb + 2 * t + (e & 1);
-          const float sv = key < valid ? sacc[nb][e] * P.scale_log2 : -INFINITY;
-          sacc[nb][e] = sv;
-          mx[e >> 1] = fmaxf(mx[e >> 1], sv);
-        }
-      float corr[2], ms[2];
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        mx[i] = fmaxf(mx[i], __shfl_xor_sync(0xffffffffu, mx[i], 1));
-        mx[i] = fmaxf(mx[i], __shfl_xor_sync(0xffffffffu, mx[i], 2));
-        const float mn = fmaxf(m[i], mx[i]);
-        ms[i] = (mn == -INFINITY) ? 0.f : mn;
-        corr[i] = exp2f(m[i] - ms[i]);
-        m[i] = mn;
-      }
-      float ps[2] = {0.f, 0.f};
-#pragma unroll
-      for (int nb = 0; nb < 2; ++nb)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float p = exp2f(sacc[nb][e] - ms[e >> 1]);
-          sacc[nb][e] = p;
-          ps[e >> 1] += p;
-        }
-      l[0] = l[0] * corr[0] + ps[0];
-      l[1] = l[1] * corr[1] + ps[1];
-#pragma unroll
-      for (int j = 0; j < kD / 8; ++j) {
-        oacc[j][0] *= corr[0]; oacc[j][1] *= corr[0];
-        oacc[j][2] *= corr[1]; oacc[j][3] *= corr[1];
-      }
-      // rows at or past `valid` (another sequence's rows, or memory nobody wrote) have probability 0, but
-      // 0 x NaN is NaN: their value rows are cleared before the product.  k0 = first of the two rows a
-      // fragment register holds (low half k0, high half k0 + 1).
-      const int rem = valid - wrow;
-      unsigned vm0 = 0xffffffffu, vm1 = 0xffffffffu;
-      if (rem < 16) {
-        vm0 = (2 * t < rem ? 0x0000ffffu : 0u) | (2 * t + 1 < rem ? 0xffff0000u : 0u);
-        vm1 = (2 * t + 8 < rem ? 0x0000ffffu : 0u) | (2 * t + 9 < rem ? 0xffff0000u : 0u);
-      }
-      unsigned pa[4];
-      pa[0] = Mma<T>::pack(sacc[0][0], sacc[0][1]);
-      pa[1] = Mma<T>::pack(sacc[0][2], sacc[0][3]);
-      pa[2] = Mma<T>::pack(sacc[1][0], sacc[1][1]);
-      pa[3] = Mma<T>::pack(sacc[1][2], sacc[1][3]);
-#pragma unroll
-      for (int jj = 0; jj < kD / 16; ++jj) {
-        unsigned r[4];
-        ldmatrix_x4_trans(sb + 2 * kBoxBytes + tile_offset(wrow + (mi & 1) * 8 + (lane & 7), 2 * jj + (mi >> 1)), r);
-        r[0] &= vm0; r[2] &= vm0;
-        r[1] &= vm1; r[3] &= vm1;
-        Mma<T>::run(oacc[2 * jj], pa, r[0], r[1]);
-        Mma<T>::run(oacc[2 * jj + 1], pa, r[2], r[3]);
+        const int c = 16 * kk + 2 * t;
+        qf[kk][0] = r0 ? *reinterpret_cast<const unsigned *>(qb + g * kD + c) : 0u;
+        qf[kk][1] = r1 ? *reinterpret_cast<const unsigned *>(qb + (g + 8) * kD + c) : 0u;
+        qf[kk][2] = r0 ? *reinterpret_cast<const unsigned *>(qb + g * kD + c + 8) : 0u;
+        qf[kk][3] = r1 ? *reinterpret_cast<const unsigned *>(qb + (g + 8) * kD + c + 8) : 0u;
       }
     }
-    __syncthreads();                       // everyone is through with stage s before it is filled again
-  }
-  if (failed) {
-    // a load did not arrive in time: say so, give the loads still in flight a bounded chance to land
-    // (they write this block's shared memory), and report an empty share
-    if (tid == 0) {
-      atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
-      for (int ti = consumed; ti < issued; ++ti) mbar_wait(&full[ti % kStages], (unsigned)(ti / kStages) & 1u);
-    }
-    m[0] = m[1] = -INFINITY;
-    l[0] = l[1] = 0.f;
+    float oacc[kD / 8][4];
 #pragma unroll
     for (int j = 0; j < kD / 8; ++j) oacc[j][0] = oacc[j][1] = oacc[j][2] = oacc[j][3] = 0.f;
-    __syncthreads();
-  }
+    float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
 
-  // merge the four warps (each saw a quarter of every tile), then write this split's share
-  float *mo = reinterpret_cast<float *>(smem);                          // [warp][16][kMergeStride]
-  float2 *mml = reinterpret_cast<float2 *>(mo + kWarps * 16 * kMergeStride);   // [warp][16]
+    for (; ti < seg_end; ++ti, ++n) {
+      if (failed) continue;
+      const int st = n % kStages;
+      if (!mbar_wait(&sh.full[st], (unsigned)(n / kStages) & 1u)) {
+        // a load did not arrive in time: say so and report an empty share
+        failed = true;
+        if (lane == 0) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
+        continue;
+      }
+      const int lt = (int)(ti - line);
+      int valid = lt < s.tiles_main ? s.n_main - lt * kTile : s.n_tail - (lt - s.tiles_main) * kTile;
+      valid = valid > kTile ? kTile : valid;
+      const int wrow = 16 * warp;
+      if (wrow < valid) {
+        const unsigned sb = sbase + (unsigned)(st * kStageBytes);
+        float sacc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+        const int mi = lane >> 3;
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    l[i] += __shfl_xor_sync(0xffffffffu, l[i], 1);
-    l[i] += __shfl_xor_sync(0xffffffffu, l[i], 2);
-  }
-  {
-    float *w0 = mo + ((size_t)warp * 16 + g) * kMergeStride, *w1 = w0 + 8 * kMergeStride;
+        for (int kk = 0; kk < kD / 16; ++kk) {
+          unsigned r[4];
+          ldmatrix_x4(sb + tile_offset(wrow + (mi >> 1) * 8 + (lane & 7), 2 * kk + (mi & 1)), r);
+          Mma<T>::run(sacc[0], qf[kk], r[0], r[1]);
+          Mma<T>::run(sacc[1], qf[kk], r[2], r[3]);
+        }
+        float mx[2] = {-INFINITY, -INFINITY};
 #pragma unroll
-    for (int j = 0; j < kD / 8; ++j) {
-      *reinterpret_cast<float2 *>(w0 + 8 * j + 2 * t) = make_float2(oacc[j][0], oacc[j][1]);
-      *reinterpret_cast<float2 *>(w1 + 8 * j + 2 * t) = make_float2(oacc[j][2], oacc[j][3]);
+        for (int nb = 0; nb < 2; ++nb)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int key = wrow + 8 * nb + 2 * t + (e & 1);
+            const float sv = key < valid ? sacc[nb][e] * P.scale_log2 : -INFINITY;
+            sacc[nb][e] = sv;
+            mx[e >> 1] = fmaxf(mx[e >> 1], sv);
+          }
+        float corr[2], ms[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          mx[i] = fmaxf(mx[i], __shfl_xor_sync(0xffffffffu, mx[i], 1));
+          mx[i] = fmaxf(mx[i], __shfl_xor_sync(0xffffffffu, mx[i], 2));
+          const float mn = fmaxf(m[i], mx[i]);
+          ms[i] = (mn == -INFINITY) ? 0.f : mn;
+          corr[i] = exp2f(m[i] - ms[i]);
+          m[i] = mn;
+        }
+        float ps[2] = {0.f, 0.f};
+#pragma unroll
+        for (int nb = 0; nb < 2; ++nb)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float p = exp2f(sacc[nb][e] - ms[e >> 1]);
+            sacc[nb][e] = p;
+            ps[e >> 1] += p;
+          }
+        l[0] = l[0] * corr[0] + ps[0];
+        l[1] = l[1] * corr[1] + ps[1];
+#pragma unroll
+        for (int j = 0; j < kD / 8; ++j) {
+          oacc[j][0] *= corr[0]; oacc[j][1] *= corr[0];
+          oacc[j][2] *= corr[1]; oacc[j][3] *= corr[1];
+        }
+        // rows at or past `valid` (another sequence's rows, or memory nobody wrote) have probability 0, but
+        // 0 x NaN is NaN: their value rows are cleared before the product.  k0 = first of the two rows a
+        // fragment register holds (low half k0, high half k0 + 1).
+        const int rem = valid - wrow;
+        unsigned vm0 = 0xffffffffu, vm1 = 0xffffffffu;
+        if (rem < 16) {
+          vm0 = (2 * t < rem ? 0x0000ffffu : 0u) | (2 * t + 1 < rem ? 0xffff0000u : 0u);
+          vm1 = (2 * t + 8 < rem ? 0x0000ffffu : 0u) | (2 * t + 9 < rem ? 0xffff0000u : 0u);
+        }
+        unsigned pa[4];
+        pa[0] = Mma<T>::pack(sacc[0][0], sacc[0][1]);
+        pa[1] = Mma<T>::pack(sacc[0][2], sacc[0][3]);
+        pa[2] = Mma<T>::pack(sacc[1][0], sacc[1][1]);
+        pa[3] = Mma<T>::pack(sacc[1][2], sacc[1][3]);
+#pragma unroll
+        for (int jj = 0; jj < kD / 16; ++jj) {
+          unsigned r[4];
+          ldmatrix_x4_trans(sb + 2 * kBoxBytes + tile_offset(wrow + (mi & 1) * 8 + (lane & 7), 2 * jj + (mi >> 1)), r);
+          r[0] &= vm0; r[2] &= vm0;
+          r[1] &= vm1; r[3] &= vm1;
+          Mma<T>::run(oacc[2 * jj], pa, r[0], r[1]);
+          Mma<T>::run(oacc[2 * jj + 1], pa, r[2], r[3]);
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sh.empty[st]);             // this warp is through with the stage
     }
-    if (t == 0) {
-      mml[warp * 16 + g] = make_float2(m[0], l[0]);
-      mml[warp * 16 + g + 8] = make_float2(m[1], l[1]);
-    }
-  }
-  __syncthreads();
-  for (int r = 0; r < P.G; ++r) {
-    float mm = -INFINITY;
+    if (failed) {
+      m[0] = m[1] = -INFINITY;
+      l[0] = l[1] = 0.f;
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) mm = fmaxf(mm, mml[w * 16 + r].x);
-    const float msafe = (mm == -INFINITY) ? 0.f : mm;
-    float o = 0.f, ll = 0.f;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-      const float2 v = mml[w * 16 + r];
-      const float f = exp2f(v.x - msafe);
-      o += mo[((size_t)w * 16 + r) * kMergeStride + tid] * f;
-      ll += v.y * f;
+      for (int j = 0; j < kD / 8; ++j) oacc[j][0] = oacc[j][1] = oacc[j][2] = oacc[j][3] = 0.f;
     }
-    const size_t slot = ((size_t)b * P.Hq + (size_t)h * P.G + r) * P.nsplit + split;
-    P.part_o[slot * kD + tid] = o;
-    if (tid == 0) P.part_ml[slot] = make_float2(mm, ll);
+
+    // merge the four warps (each saw a quarter of every tile)
+    consumers_sync();                                        // the merge buffer is free again
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      l[i] += __shfl_xor_sync(0xffffffffu, l[i], 1);
+      l[i] += __shfl_xor_sync(0xffffffffu, l[i], 2);
+    }
+    {
+      float *w0 = mo + ((size_t)warp * 16 + g) * kMergeStride, *w1 = w0 + 8 * kMergeStride;
+#pragma unroll
+      for (int j = 0; j < kD / 8; ++j) {
+        *reinterpret_cast<float2 *>(w0 + 8 * j + 2 * t) = make_float2(oacc[j][0], oacc[j][1]);
+        *reinterpret_cast<float2 *>(w1 + 8 * j + 2 * t) = make_float2(oacc[j][2], oacc[j][3]);
+      }
+      if (t == 0) {
+        mml[warp * 16 + g] = make_float2(m[0], l[0]);
+        mml[warp * 16 + g + 8] = make_float2(m[1], l[1]);
+      }
+    }
+    consumers_sync();
+    const int i0 = share_of(line, line_len, nb), i1 = share_of(line + s.tiles - 1, line_len, nb);
+    const size_t slot = ((size_t)blk + (size_t)h * P.B + b) * P.G;
+    for (int r = warp; r < P.G; r += kWarps) {               // a warp per query head, four channels per lane
+      float2 v[kWarps];
+      float mm = -INFINITY, ll = 0.f;
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) { v[w] = mml[w * 16 + r]; mm = fmaxf(mm, v[w].x); }
+      const float msafe = (mm == -INFINITY) ? 0.f : mm;
+      float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) {
+        const float f = exp2f(v[w].x - msafe);
+        fold(o, *reinterpret_cast<const float4 *>(mo + ((size_t)w * 16 + r) * kMergeStride + 4 * lane), f);
+        ll += v[w].y * f;
+      }
+      if (i0 == i1) {
+        store_head(static_cast<T *>(P.out) + ((size_t)b * P.Hq + (size_t)h * P.G + r) * kD + 4 * lane, o, ll);
+      } else {
+        *reinterpret_cast<float4 *>(P.part_o + (slot + r) * kD + 4 * lane) = o;
+        if (lane == 0) P.part_ml[slot + r] = make_float2(mm, ll);
+      }
+    }
+    if (blk == i0 && tid == 0) P.span[(size_t)h * P.B + b] = make_int2(i0, i1);
   }
 }
 
-// out[b][j] = sum over splits of their shares, rescaled to the common maximum, divided by the common sum.
+// out[b][h*G + r] = sum over the blocks i0..i1 of their shares, rescaled to the common maximum, divided by the common
+// sum.  Shares sit in slot i + (h*B + b) (both only ever advance along the line, so slots do not collide).  One block per
+// query head; each warp folds every fourth share, loads ahead of the arithmetic, and the warps' results meet in shared
+// memory: two rounds of latency.  Launched early as a programmatic dependent, it is resident when the shares are complete
+// (merging in the block that finishes last instead costs an atomic and 3..5 us on one SM: 14.0 against 11.9 us per
+// layer of the small case above).
 template <typename T>
-__global__ void __launch_bounds__(kD)
-k_decode_combine(const float *__restrict__ part_o, const float2 *__restrict__ part_ml, int nsplit, T *__restrict__ out) {
-  const size_t bj = blockIdx.x;
-  const int c = threadIdx.x;
-  float mm = -INFINITY;
-  for (int s = 0; s < nsplit; ++s) mm = fmaxf(mm, part_ml[bj * nsplit + s].x);
-  const float msafe = (mm == -INFINITY) ? 0.f : mm;
-  float o = 0.f, ll = 0.f;
-  for (int s = 0; s < nsplit; ++s) {
-    const float2 v = part_ml[bj * nsplit + s];
-    const float f = exp2f(v.x - msafe);
-    o += part_o[(bj * nsplit + s) * kD + c] * f;
-    ll += v.y * f;
+__global__ void __launch_bounds__(32 * kWarps)
+k_decode_combine(const DecodeParams P) {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  __shared__ float4 so[kWarps][32];
+  __shared__ float2 sml[kWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int b = blockIdx.x / P.Hq, hq = blockIdx.x - b * P.Hq, h = hq / P.G, r = hq - h * P.G;
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  const int2 span = __ldcg(P.span + (size_t)h * P.B + b);
+  if (span.y <= span.x) return;                              // no rows, or finished by its only block
+  const size_t slot0 = ((size_t)span.x + (size_t)h * P.B + b) * P.G + r;
+  const int cnt = span.y - span.x + 1;
+  constexpr int kAhead = 10;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  float m = -INFINITY, l = 0.f;
+  for (int s0 = warp; s0 < cnt; s0 += kWarps * kAhead) {
+    float4 v[kAhead];
+    float2 ml[kAhead];
+#pragma unroll
+    for (int a = 0; a < kAhead; ++a) {
+      const int i = s0 + a * kWarps < cnt ? s0 + a * kWarps : s0;
+      ml[a] = __ldcg(P.part_ml + slot0 + (size_t)i * P.G);
+      v[a] = __ldcg(reinterpret_cast<const float4 *>(P.part_o + (slot0 + (size_t)i * P.G) * kD) + lane);
+    }
+    float mn = m;
+#pragma unroll
+    for (int a = 0; a < kAhead; ++a) {
+      if (s0 + a * kWarps >= cnt) ml[a] = make_float2(-INFINITY, 0.f);
+      mn = fmaxf(mn, ml[a].x);
+    }
+    const float ms = mn == -INFINITY ? 0.f : mn, keep = exp2f(m - ms);
+    m = mn;
+    l *= keep;
+    acc.x *= keep; acc.y *= keep; acc.z *= keep; acc.w *= keep;
+#pragma unroll
+    for (int a = 0; a < kAhead; ++a) {
+      const float f = exp2f(ml[a].x - ms);
+      fold(acc, v[a], f);
+      l += ml[a].y * f;
+    }
   }
-  out[bj * kD + c] = Mma<T>::from_float(ll > 0.f ? o / ll : 0.f);
+  so[warp][lane] = acc;
+  if (lane == 0) sml[warp] = make_float2(m, l);
+  __syncthreads();
+  if (warp != 0) return;
+  float mm = -INFINITY, ll = 0.f;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) mm = fmaxf(mm, sml[w].x);
+  const float ms = mm == -INFINITY ? 0.f : mm;
+  float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) {
+    const float f = exp2f(sml[w].x - ms);
+    fold(o, so[w][lane], f);
+    ll += sml[w].y * f;
+  }
+  store_head(static_cast<T *>(P.out) + ((size_t)b * P.Hq + hq) * kD + 4 * lane, o, ll);
 }
 
 // ---------------------------------------------------------------------------
@@ -387,26 +564,12 @@ fc_status encode_rows(CUtensorMap *m, CUtensorMapDataType dt, int rank, const vo
   return r == CUDA_SUCCESS ? FC_OK : FC_ERR_INTERNAL;
 }
 
-constexpr size_t kDecodeSmem = (size_t)kStages * kStageBytes + 64 + 1024;   // ring, barriers, slack to align the ring to 1024 bytes
-
-// Resident blocks of k_decode_partial per SM (the launch is sized to one full wave of them).
-int decode_blocks_per_sm() {
-  static int n = 0;
-  if (n == 0) {
-    int v = 0;
-    if (cudaFuncSetAttribute(k_decode_partial<__half>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmem) == cudaSuccess &&
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_decode_partial<__half>, kThreadsD, kDecodeSmem) == cudaSuccess && v > 0)
-      n = v;
-    else
-      n = 1;
-    cudaGetLastError();
-  }
-  return n;
-}
+// ring, merge buffer (the warps' outputs, padded), slack to align the ring to 1024 bytes
+constexpr size_t kDecodeSmem = (size_t)kStages * kStageBytes + kWarps * 16 * (kMergeStride + 2) * sizeof(float) + 1024;
 
 struct DecodePlan {
-  int nsplit, chunk;
-  size_t off_ml, total;
+  int nb;
+  size_t off_ml, off_span, total;
 };
 
 fc_status check_decode(const fc_handle *h, const fc_decode_args *a) {
@@ -429,19 +592,14 @@ fc_status check_decode(const fc_handle *h, const fc_decode_args *a) {
 
 DecodePlan plan_decode(const fc_handle *h, const fc_decode_args *a) {
   DecodePlan p;
-  const long long logical = a->max_rows + (a->tail_k ? kTile - 1 : 0);      // the kept rows are padded to a tile before the tail
-  long long tiles = (logical + kTile - 1) / kTile;
-  if (tiles < 1) tiles = 1;
-  const long long groups = (long long)a->batch * a->num_heads;
-  long long want = (long long)decode_blocks_per_sm() * h->num_sms / groups;           // one full wave of resident blocks
-  if (want < 1) want = 1;
-  if (want > tiles) want = tiles;
-  const long long per = (tiles + want - 1) / want;
-  p.chunk = (int)(per * kTile);
-  p.nsplit = (int)((tiles + per - 1) / per);
-  const size_t slots = (size_t)a->batch * a->num_q_heads * p.nsplit;
+  // one block per SM (the ring takes most of its shared memory), or as many as there can be tiles
+  const long long tiles = (long long)a->batch * a->num_heads * ((a->max_rows + kTile - 1) / kTile + (a->tail_k ? 1 : 0));
+  p.nb = (int)(tiles < h->num_sms ? (tiles < 1 ? 1 : tiles) : h->num_sms);
+  const size_t units = (size_t)a->batch * a->num_heads;
+  const size_t slots = (p.nb + units) * (size_t)(a->num_q_heads / a->num_heads);
   p.off_ml = (slots * kD * sizeof(float) + 255) & ~(size_t)255;
-  p.total = p.off_ml + ((slots * sizeof(float2) + 255) & ~(size_t)255);
+  p.off_span = p.off_ml + ((slots * sizeof(float2) + 255) & ~(size_t)255);
+  p.total = p.off_span + ((units * sizeof(int2) + 255) & ~(size_t)255);
   return p;
 }
 
@@ -469,25 +627,48 @@ fc_status launch_decode(fc_handle *h, const fc_decode_args *a, const DecodePlan 
   }
   DecodeParams P;
   P.q = a->q;
+  P.out = out;
   P.offsets = reinterpret_cast<const long long *>(a->offsets);
   P.tail_len = a->tail_len;
   P.part_o = reinterpret_cast<float *>(ws);
   P.part_ml = reinterpret_cast<float2 *>(ws + pl.off_ml);
+  P.span = reinterpret_cast<int2 *>(ws + pl.off_span);
   P.status = h->status_word;
+  P.B = a->batch;
   P.H = a->num_heads;
   P.Hq = a->num_q_heads;
   P.G = a->num_q_heads / a->num_heads;
-  P.nsplit = pl.nsplit;
-  P.chunk = pl.chunk;
+  P.nb = pl.nb;
   P.tail_cap = a->tail_k ? a->tail_capacity : 0;
   P.has_tail = a->tail_k ? 1 : 0;
   P.scale_log2 = (float)(1.4426950408889634 / sqrt((double)kD));
-  const size_t sm = kDecodeSmem;
-  FC_CUDA_TRY(cudaFuncSetAttribute(k_decode_partial<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  k_decode_partial<T><<<dim3(pl.nsplit, a->num_heads, a->batch), kThreadsD, sm, st>>>(P, M);
+  if (!h->decode_ready) {              // once per handle
+    FC_CUDA_TRY(cudaFuncSetAttribute(k_decode<__half>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmem));
+    FC_CUDA_TRY(cudaFuncSetAttribute(k_decode<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmem));
+    h->decode_ready = true;
+  }
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(pl.nb);
+  lc.blockDim = dim3(kThreadsD);
+  lc.dynamicSmemBytes = kDecodeSmem;
+  lc.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  if (cudaLaunchKernelEx(&lc, k_decode<T>, P, M) != cudaSuccess) {
+    cudaGetLastError();
+    return FC_ERR_CUDA;
+  }
   if ((s = fc_after_launch(h)) != FC_OK) return s;
-  k_decode_combine<T><<<(unsigned)(a->batch * a->num_q_heads), kD, 0, st>>>(P.part_o, P.part_ml, pl.nsplit,
-                                                                              static_cast<T *>(out));
+  lc.gridDim = dim3((unsigned)(a->batch * a->num_q_heads));
+  lc.blockDim = dim3(32 * kWarps);
+  lc.dynamicSmemBytes = 0;
+  if (cudaLaunchKernelEx(&lc, k_decode_combine<T>, P) != cudaSuccess) {
+    cudaGetLastError();
+    return FC_ERR_CUDA;
+  }
   return fc_after_launch(h);
 }
 
