@@ -131,6 +131,7 @@ extern "C" fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen) 
   h->master = nullptr;
   h->status_word = nullptr;
   h->done_counter = nullptr;
+  h->small_counter = nullptr;
   h->decode_ready = false;
   h->group_bytes = (size_t)32 << 20;
   h->launches = 0;
@@ -164,6 +165,8 @@ extern "C" fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen) 
       cudaMemset(h->status_word, 0, sizeof(int)) != cudaSuccess ||
       cudaMalloc(&h->done_counter, 2 * FC_LAYER_CHUNK * sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(h->done_counter, 0, 2 * FC_LAYER_CHUNK * sizeof(unsigned)) != cudaSuccess ||
+      cudaMalloc(&h->small_counter, FC_LAYER_CHUNK * 32 * sizeof(unsigned)) != cudaSuccess ||
+      cudaMemset(h->small_counter, 0, FC_LAYER_CHUNK * 32 * sizeof(unsigned)) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
       !create_streams(h)) {
     fc_destroy(h);
@@ -265,6 +268,7 @@ extern "C" void fc_destroy(fc_handle *h) {
   if (h->master) cudaFree(h->master);
   if (h->status_word) cudaFree(h->status_word);
   if (h->done_counter) cudaFree(h->done_counter);
+  if (h->small_counter) cudaFree(h->small_counter);
   delete h;
 }
 

@@ -29,6 +29,7 @@ struct fc_handle {
   int *status_word;        // DEVICE
   unsigned *done_counter;  // DEVICE [2][FC_LAYER_CHUNK], zero between calls (the last block of a layer's sequence resets it)
   bool decode_ready;       // the decoding kernel has been allowed its shared memory on this device
+  unsigned *small_counter; // DEVICE [FC_LAYER_CHUNK * 32], zero between launches (fc_score_small.cuh)
   size_t group_bytes;
   int num_sms;
   // L2 residency of the transform intermediates: the per-stream workspace buffers are declared a

@@ -26,6 +26,7 @@
 // through Bluestein's chirp convolution on a power-of-two length M >= 2N-1.
 #include "fc_common.cuh"
 #include "fc_score_fast.cuh"
+#include "fc_score_small.cuh"
 
 #include <math.h>
 #include <mutex>
@@ -681,6 +682,7 @@ GenericLayout generic_layout(const fc_handle *h, const SeqPlan &sp, int num_head
 // ---- the specialised passes (fc_score_fast.cuh) ----
 struct PassPlan {
   bool ok;                   // false: the length is left to the generic kernels
+  bool small;                // one kernel does it all (fc_score_small.cuh); only pad, N and M are set besides
   bool pad;                  // padded form (else direct: M == N)
   int N, M, N1, N2;
   int a, r1b, r2b;           // N1 = a * r1b, N2 = 16 * r2b (32 * r2b with dbl)
@@ -722,9 +724,28 @@ inline PassPlan pad_shape(int M) {
   return p;
 }
 
-// How a sequence of N tokens is transformed.
-PassPlan plan_passes(int N) {
+// Channel pairs per block of the small kernel for M points.
+constexpr int small_cp(int M) { return M <= 128 ? 32 : 4096 / M; }
+
+// How a sequence of N tokens and head_dim channels is transformed (head_dim 0: the three passes wherever they apply).
+PassPlan plan_passes(int N, int head_dim) {
   PassPlan p = {};
+  // one kernel where a cluster of at most 16 blocks holds a head
+  if (N <= 1024 && head_dim > 0) {
+    int M = 64;
+    const bool pad = !(is_pow2(N) && N >= 64);
+    while (M < (pad ? 2 * N - 1 : N)) M <<= 1;
+    if (M <= 1024) {
+      const int width = 2 * small_cp(M), blocks = head_dim / width;
+      if (head_dim % width == 0 && is_pow2(blocks) && blocks <= 16) {
+        p.ok = p.small = true;
+        p.pad = pad;
+        p.N = N;
+        p.M = M;
+        return p;
+      }
+    }
+  }
   if (is_pow2(N) && N >= 1024) {
     if (N > 65536) return p;
     const int bits = ilog2(N);
@@ -796,7 +817,7 @@ GroupPlan plan_groups(const fc_handle *h, const PassPlan &p, int num_units, int 
 // Workspace carve-up of one scoring call: the regions hold the largest sequence of the view.
 struct ScoreLayout {
   size_t buf_bytes;          // intermediates, one buffer per internal stream
-  size_t off_buf, off_tab, off_tot, off_hi, total;
+  size_t off_buf, off_tab, off_tot, off_hi, off_small, total;
   size_t tot_bytes, hi_bytes;   // per-block partial sums of one step; two copies, used in turn
 };
 
@@ -810,23 +831,24 @@ inline bool first_of_its_length(const fc_kv_view *kv, int b) {
 ScoreLayout score_layout(const fc_handle *h, const fc_kv_view *kv, int num_layers) {
   ScoreLayout L = {};
   const int H = kv->num_heads, d = kv->head_dim, nl = num_layers < FC_LAYER_CHUNK ? num_layers : FC_LAYER_CHUNK;
-  size_t tab = 0, generic = 0;
+  size_t tab = 0, generic = 0, nsmall = 0;
   for (int b = 0; b < kv->batch; ++b) {
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0) continue;
-    const PassPlan p = plan_passes(N);
+    const PassPlan p = plan_passes(N, kv->head_dim);
     if (!p.ok || h->generic_only) {
       const size_t t = generic_layout(h, plan_sequence(N), H, d).total;
       if (t > generic) generic = t;
       continue;
     }
+    if (p.pad && first_of_its_length(kv, b)) tab += (size_t)p.M * sizeof(float4);
+    if (p.small) { ++nsmall; continue; }
     const GroupPlan g = plan_groups(h, p, nl * H, H, d);
     const size_t tot = (size_t)nl * H * (d / (2 * p.cpw)) * p.N2 * 2 * sizeof(double);
     const size_t hi = (size_t)nl * H * g.ngr * p.N2 * 2 * sizeof(double);
     if (g.buf_bytes > L.buf_bytes) L.buf_bytes = g.buf_bytes;
     if (tot > L.tot_bytes) L.tot_bytes = tot;
     if (hi > L.hi_bytes) L.hi_bytes = hi;
-    if (p.pad && first_of_its_length(kv, b)) tab += (size_t)p.M * sizeof(float4);
   }
   L.tot_bytes = align_up(L.tot_bytes, 256);
   L.hi_bytes = align_up(L.hi_bytes, 256);
@@ -835,6 +857,7 @@ ScoreLayout score_layout(const fc_handle *h, const fc_kv_view *kv, int num_layer
   L.off_tab = off; off += align_up(tab, 256);
   L.off_tot = off; off += 2 * L.tot_bytes;
   L.off_hi = off;  off += 2 * L.hi_bytes;
+  L.off_small = off; off += align_up(nl * nsmall * H * 4 * sizeof(double), 256);
   L.total = off > generic ? off : generic;
   if (L.total < 256) L.total = 256;
   return L;
@@ -859,8 +882,8 @@ void claim_persisting_l2(fc_handle *h, const fc_kv_view *kv, int num_layers, cud
   for (int b = 0; b < kv->batch && !claim; ++b) {
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0) continue;
-    const PassPlan p = plan_passes(N);
-    if (!p.ok || p.pad) continue;
+    const PassPlan p = plan_passes(N, kv->head_dim);
+    if (!p.ok || p.pad || p.small) continue;
     claim = window_fits(h, p, plan_groups(h, p, nl * kv->num_heads, kv->num_heads, kv->head_dim));
   }
   if (claim == (h->persist_on != 0)) return;
@@ -913,6 +936,22 @@ fc_status set_smem(Kern kern, size_t bytes) {
   if (it == done.end())
     FC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
   done[key] = bytes;
+  return FC_OK;
+}
+
+// Clusters of more than 8 blocks, once per kernel and device.
+template <class Kern>
+fc_status allow_wide_clusters(Kern kern) {
+  static std::mutex mu;
+  static std::unordered_map<unsigned long long, bool> done;
+  int dev = 0;
+  FC_CUDA_TRY(cudaGetDevice(&dev));
+  const unsigned long long key = (unsigned long long)reinterpret_cast<uintptr_t>(reinterpret_cast<const void *>(kern)) ^
+                                 ((unsigned long long)dev << 56);
+  std::lock_guard<std::mutex> lock(mu);
+  if (done[key]) return FC_OK;
+  FC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  done[key] = true;
   return FC_OK;
 }
 
@@ -1096,7 +1135,7 @@ fc_status prepare_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, do
     tabs[b] = nullptr;
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0) continue;
-    const PassPlan p = plan_passes(N);
+    const PassPlan p = plan_passes(N, kv->head_dim);
     if (!p.ok || !p.pad) continue;
     if (!any) {
       any = true;
@@ -1113,7 +1152,7 @@ fc_status prepare_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, do
   for (int b = 0; b < kv->batch; ++b) {
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0 || tabs[b]) continue;
-    const PassPlan p = plan_passes(N);
+    const PassPlan p = plan_passes(N, kv->head_dim);
     if (!p.ok || !p.pad) continue;
     if (!first_of_its_length(kv, b)) {
       for (int i = 0; i < b && !tabs[b]; ++i)
@@ -1138,6 +1177,14 @@ fc_status prepare_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, do
     } else {
       dst = spare;
       spare += p.M;
+    }
+    if (p.small) {
+      small::k_small_table<<<(p.M + 63) / 64, 64, (N + 1) * sizeof(float), st>>>(dst, N, cutoff_index(gamma, N), p.M, h->master,
+                                                                                h->master_len);
+      if ((s = fc_after_launch(h)) != FC_OK) return s;
+      if (slot >= 0) h->tab_key[slot] = key_of(b);
+      tabs[b] = dst;
+      continue;
     }
     static const fast::LayerPtrs none = {};
     const PassArgs x{h, st, &p, &none, kv, 0, 1, 0, 2 * p.cpw, cutoff_index(gamma, N), reinterpret_cast<float2 *>(wsb + L.off_buf), nullptr};
@@ -1212,6 +1259,78 @@ fc_status score_sequence(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, co
   for (int i = 0; i < h->num_aux; ++i) FC_CUDA_TRY(cudaEventRecord(h->ev_done[par][i], h->aux[i]));
   h->step++;
   h->pending_join = true;
+  return FC_OK;
+}
+
+// The short sequences of a chunk of layers, one launch per transform length and form (and 32 sequences), on the caller's
+// stream.
+template <typename T, class S, bool PADDED>
+fc_status launch_small(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const fast::LayerPtrs &lp, int nl,
+                       const small::SeqTable &tab, int nseq, double *part, double *energy) {
+  const size_t sm = S::smem(PADDED);
+  fc_status s = set_smem(small::k_small<T, S, PADDED>, sm);
+  if (s != FC_OK) return s;
+  const unsigned blocks = (unsigned)(kv->head_dim / (2 * S::CP));
+  if (blocks > 8 && (s = allow_wide_clusters(small::k_small<T, S, PADDED>)) != FC_OK) return s;
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(blocks, kv->num_heads, nl * nseq);
+  lc.blockDim = dim3(S::NT);
+  lc.dynamicSmemBytes = sm;
+  lc.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = blocks;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  ProfScope ps(h, FC_K_PASS2, st);
+  if (cudaLaunchKernelEx(&lc, small::k_small<T, S, PADDED>, lp, tab, nseq, (long long)kv->stride_token,
+                         (long long)kv->stride_head, (int)kv->num_heads, (int)kv->head_dim, (const float2 *)h->master,
+                         h->master_len, (long long)kv->cu_seqlens[kv->batch], part, h->small_counter, energy,
+                         4ll * kv->batch) != cudaSuccess) {
+    cudaGetLastError();
+    return FC_ERR_CUDA;
+  }
+  return fc_after_launch(h);
+}
+
+template <typename T>
+fc_status score_small(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const fc_layer_buffers *layers, int nl,
+                      const std::vector<PassPlan> &plans, const std::vector<const float4 *> &tabs, double gamma,
+                      double *energy, double *part) {
+  fast::LayerPtrs lp = {};
+  for (int l = 0; l < nl; ++l) {
+    lp.k[l] = layers[l].k;
+    lp.v[l] = layers[l].v;
+    lp.scores[l] = const_cast<float *>(layers[l].scores);
+  }
+  for (int M = 64; M <= 1024; M <<= 1)
+    for (int pad = 0; pad < 2; ++pad) {
+      small::SeqTable tab = {};
+      int n = 0;
+      for (int b = 0; b <= kv->batch; ++b) {
+        if (n > 0 && (n == small::kSeqs || b == kv->batch)) {
+          fc_status s = FC_ERR_INTERNAL;
+#define FC_SMALL(M_, A_, B_, C_)                                                                                        \
+  if (M == M_)                                                                                                          \
+    s = pad ? launch_small<T, small::Shape<A_, B_, C_, small_cp(M_)>, true>(h, st, kv, lp, nl, tab, n, part, energy)    \
+            : launch_small<T, small::Shape<A_, B_, C_, small_cp(M_)>, false>(h, st, kv, lp, nl, tab, n, part, energy);
+          FC_SMALL(64, 8, 1, 8) FC_SMALL(128, 16, 1, 8) FC_SMALL(256, 16, 1, 16) FC_SMALL(512, 8, 8, 8)
+          FC_SMALL(1024, 16, 8, 8)
+#undef FC_SMALL
+          if (s != FC_OK) return s;
+          part += (size_t)nl * n * kv->num_heads * 4;
+          n = 0;
+        }
+        if (b == kv->batch || !plans[b].small || plans[b].M != M || plans[b].pad != (pad != 0)) continue;
+        tab.start[n] = kv->cu_seqlens[b];
+        tab.N[n] = plans[b].N;
+        tab.omega[n] = cutoff_index(gamma, plans[b].N);
+        tab.index[n] = b;
+        tab.tab[n] = tabs[b];
+        ++n;
+      }
+    }
   return FC_OK;
 }
 
@@ -1312,26 +1431,36 @@ fc_status score_generic(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, int
   return fc_after_launch(h);
 }
 
+// The internal streams wait for everything `st` has been given so far.
+fc_status fork_streams(fc_handle *h, cudaStream_t st) {
+  FC_CUDA_TRY(cudaEventRecord(h->ev_fork, st));
+  for (int i = 0; i < h->num_aux; ++i) FC_CUDA_TRY(cudaStreamWaitEvent(h->aux[i], h->ev_fork, 0));
+  return FC_OK;
+}
+
 // All sequences of `num_layers` layers that share the view's layout; energy[l][B][4].
 template <typename T>
 fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const fc_layer_buffers *layers, int num_layers,
                      double gamma, double *energy, char *wsb) {
-  const int B = kv->batch, H = kv->num_heads;
+  const int B = kv->batch;
   const ScoreLayout L = score_layout(h, kv, num_layers);
   fc_status s;
-  bool fork = true, direct_only = true, any_fast = false;
+  bool fork = true, direct_only = true, any_fast = false, any_small = false, any_passes = false;
   std::vector<PassPlan> plans(B);
   std::vector<const float4 *> tabs(B, nullptr);
   for (int b = 0; b < B; ++b) {
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0) continue;
-    if (!h->generic_only) plans[b] = plan_passes(N);
+    if (!h->generic_only) plans[b] = plan_passes(N, kv->head_dim);
     any_fast = any_fast || plans[b].ok;
-    if (!plans[b].ok || plans[b].pad) direct_only = false;
+    any_small = any_small || plans[b].small;
+    any_passes = any_passes || (plans[b].ok && !plans[b].small);
+    if (!plans[b].ok || (plans[b].pad && !plans[b].small)) direct_only = false;
   }
   if (any_fast && (s = prepare_tables(h, st, kv, gamma, L, wsb, tabs.data())) != FC_OK) return s;
   // a call that carves the workspace differently: nothing of the previous call may be in flight on the other streams
   const size_t sig = reinterpret_cast<size_t>(wsb) ^ (L.buf_bytes << 20) ^ (L.tot_bytes << 8) ^ L.hi_bytes ^ (L.off_tot << 12);
+  if (any_small && sig != h->last_sig && (s = fc_flush_pending(h, st)) != FC_OK) return s;
   if (any_fast && h->step >= 1 && sig != h->last_sig) {
     for (int i = 0; i < h->num_aux; ++i)
       for (int o = 0; o < h->num_aux; ++o)
@@ -1340,6 +1469,13 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
   if (any_fast) h->last_sig = sig;
   for (int l0 = 0; l0 < num_layers; l0 += FC_LAYER_CHUNK) {
     const int nl = num_layers - l0 < FC_LAYER_CHUNK ? num_layers - l0 : FC_LAYER_CHUNK;
+    if (any_small && any_passes && fork) {          // the internal streams need not wait for the short sequences
+      if ((s = fork_streams(h, st)) != FC_OK) return s;
+      fork = false;
+    }
+    if (any_small && (s = score_small<T>(h, st, kv, layers + l0, nl, plans, tabs, gamma, energy + 4 * (size_t)l0 * B,
+                                         reinterpret_cast<double *>(wsb + L.off_small))) != FC_OK)
+      return s;
     for (int b = 0; b < B; ++b) {
       const int start = kv->cu_seqlens[b];
       double *en = energy + 4 * ((size_t)l0 * B + b);
@@ -1360,9 +1496,9 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
         }
         continue;
       }
+      if (plans[b].small) continue;
       if (fork) {
-        FC_CUDA_TRY(cudaEventRecord(h->ev_fork, st));
-        for (int i = 0; i < h->num_aux; ++i) FC_CUDA_TRY(cudaStreamWaitEvent(h->aux[i], h->ev_fork, 0));
+        if ((s = fork_streams(h, st)) != FC_OK) return s;
         fork = false;
       }
       fast::LayerPtrs lp = {};
@@ -1374,7 +1510,6 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
       if ((s = score_sequence<T>(h, st, kv, plans[b], nl, lp, gamma, en, 4ll * B, L, wsb, tabs[b])) != FC_OK) return s;
     }
   }
-  (void)H;
   // the caller's stream waits for this call's work right away, unless it asked to have that deferred
   if (!h->score_overlap || !direct_only) return fc_flush_pending(h, st);
   return FC_OK;
@@ -1486,7 +1621,7 @@ extern "C" fc_status fc_describe_plan(const fc_handle *h, int32_t seqlen, double
   const SeqPlan sp = plan_sequence(seqlen);
   out[0] = sp.bluestein ? 1 : 0;
   out[1] = sp.Nfft;
-  const PassPlan p = plan_passes(seqlen);
+  const PassPlan p = plan_passes(seqlen, 0);
   out[2] = (p.ok && !p.pad) ? p.N1 : sp.N1;
   out[3] = (p.ok && !p.pad) ? p.N2 : sp.N2;
   if (sp.bluestein) {
