@@ -146,6 +146,7 @@ extern "C" fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen) 
   h->prof_seen = 0;
   h->generic_only = false;
   h->select_overlap = 0;
+  h->after_select = false;
   h->score_overlap = 0;
   h->band_form = 1;
   h->step = 0;
@@ -163,8 +164,8 @@ extern "C" fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen) 
   if (cudaMalloc(&h->master, (size_t)h->master_len * sizeof(float2)) != cudaSuccess ||
       cudaMalloc(&h->status_word, sizeof(int)) != cudaSuccess ||
       cudaMemset(h->status_word, 0, sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&h->done_counter, 2 * FC_LAYER_CHUNK * sizeof(unsigned)) != cudaSuccess ||
-      cudaMemset(h->done_counter, 0, 2 * FC_LAYER_CHUNK * sizeof(unsigned)) != cudaSuccess ||
+      cudaMalloc(&h->done_counter, (2 * FC_LAYER_CHUNK + 1) * sizeof(unsigned)) != cudaSuccess ||
+      cudaMemset(h->done_counter, 0, (2 * FC_LAYER_CHUNK + 1) * sizeof(unsigned)) != cudaSuccess ||
       cudaMalloc(&h->small_counter, FC_LAYER_CHUNK * 32 * sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(h->small_counter, 0, FC_LAYER_CHUNK * 32 * sizeof(unsigned)) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) != cudaSuccess ||

@@ -27,7 +27,7 @@ struct fc_handle {
   int master_len;          // power of two; master[i] = exp(-2*pi*i*j/master_len)
   float2 *master;          // DEVICE
   int *status_word;        // DEVICE
-  unsigned *done_counter;  // DEVICE [2][FC_LAYER_CHUNK], zero between calls (the last block of a layer's sequence resets it)
+  unsigned *done_counter;  // DEVICE [2][FC_LAYER_CHUNK] pass 3, [1] allocation; zero between calls (the last block resets its counter)
   bool decode_ready;       // the decoding kernel has been allowed its shared memory on this device
   unsigned *small_counter; // DEVICE [FC_LAYER_CHUNK * 32], zero between launches (fc_score_small.cuh)
   size_t group_bytes;
@@ -53,6 +53,7 @@ struct fc_handle {
   // true only for the stack handle of fc_score_layer_static: every length takes the generic
   // single-stream kernels (no internal streams or events exist there)
   bool generic_only;
+  bool after_select;       // the handle's last launch was a selection: only then may the next one start beside it
   int select_overlap;      // 1: consecutive fc_select_compact launches may overlap (fc_set_select_overlap)
   // fc_set_score_overlap: consecutive fc_score_layer calls keep running on the two internal streams
   // without rejoining the caller's stream; the join is made by the next call that consumes their results
@@ -511,6 +512,7 @@ inline fc_status fc_flush_pending(fc_handle *h, cudaStream_t st) {
 // the call that made it and does not linger for the caller's next CUDA call.
 inline fc_status fc_after_launch(fc_handle *h) {
   h->launches++;
+  h->after_select = false;
   return cudaGetLastError() == cudaSuccess ? FC_OK : FC_ERR_CUDA;
 }
 

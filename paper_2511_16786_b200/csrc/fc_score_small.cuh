@@ -80,7 +80,7 @@ template <typename T, class S, bool PADDED>
 __global__ void __launch_bounds__(S::NT, S::NT == 256 ? 2 : 4)
 k_small(const __grid_constant__ fast::LayerPtrs lp, const __grid_constant__ SeqTable st, int nseq, long long stride_token,
         long long stride_head, int H, int head_dim, const float2 *__restrict__ master, int master_len,
-        long long score_stride, double *__restrict__ part, unsigned *__restrict__ done, double *__restrict__ energy,
+        long long score_stride, double *__restrict__ part_en, unsigned *__restrict__ done, double *__restrict__ energy,
         long long energy_layer) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
@@ -91,13 +91,14 @@ k_small(const __grid_constant__ fast::LayerPtrs lp, const __grid_constant__ SeqT
   float4 *hc = X + S::ROWS * CP;                              // padded: (h, c) of every bin
   float2 *uT = reinterpret_cast<float2 *>(hc);                // direct: exp(-j*pi*q/N) of every bin
   __shared__ double red[4][NT / 32], sums[4];
-  __shared__ bool is_last;
   const int tid = threadIdx.x, cp = tid % CP, j = tid / CP, lane = tid & 31, warp = tid >> 5;
   const int slice = blockIdx.x, head = blockIdx.y, layer = blockIdx.z / nseq, sq = blockIdx.z - layer * nseq;
   const int N = st.N[sq], omega = st.omega[sq], start = st.start[sq];
   const int ch = slice * (2 * CP) + 2 * cp;
   const T *kb = static_cast<const T *>(lp.k[layer]) + (long long)start * stride_token + (long long)head * stride_head + ch;
   const T *vb = static_cast<const T *>(lp.v[layer]) + (long long)start * stride_token + (long long)head * stride_head + ch;
+
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");   // e.g. the allocation, which waits for this grid
 
   // stage A: butterfly j + LANES*u holds the points j + LANES*u + L1*p
   float2 x0[16], x1[16];
@@ -206,14 +207,16 @@ k_small(const __grid_constant__ fast::LayerPtrs lp, const __grid_constant__ SeqT
   // ---- the residual filter between the bins k and M-k
 #pragma unroll
   for (int u = 0; u < UC; ++u) {
-    const int s = j + LANES * u, k0 = s / RB + RA * (s % RB);
+    // bins k = k0 + RA*RB*p; their partners are the sub-block of -k0 read backwards (k0 = 0: its own, shifted by one)
+    const int s = j + LANES * u, k0 = s / RB + RA * (s % RB), kn = (RA * RB - k0) & (RA * RB - 1);
+    const float4 *part = X + S::row(((kn & (RA - 1)) * RB + kn / RA) * RC) + cp;
 #pragma unroll
     for (int p = 0; p < RC; ++p) {
-      const int k = k0 + RA * RB * p, kp = (M - k) & (M - 1), rest = kp / RA;
-      const int pos = ((kp & (RA - 1)) * RB + (rest & (RB - 1))) * RC + rest / RB;
+      const int k = k0 + RA * RB * p;
+      const float4 *other = part + (k0 == 0 ? (RC - p) & (RC - 1) : RC - 1 - p) * CP;
       float2 &P0 = x0[u * RC + p], &P1 = x1[u * RC + p];
       if (PADDED) {
-        const float4 t = X[S::row(pos) + cp], w = hc[k];
+        const float4 t = *other, w = hc[k];
         P0 = make_float2(fmaf(t.y, w.y, fmaf(-t.x, w.x, w.z * P0.x)), fmaf(-t.y, w.x, fmaf(-t.x, w.y, w.z * P0.y)));
         P1 = make_float2(fmaf(t.w, w.y, fmaf(-t.z, w.x, w.z * P1.x)), fmaf(-t.w, w.x, fmaf(-t.z, w.y, w.z * P1.y)));
       } else {
@@ -221,7 +224,7 @@ k_small(const __grid_constant__ fast::LayerPtrs lp, const __grid_constant__ SeqT
         if (k == 0 || (inL && inH)) {
           P0 = P1 = make_float2(0.f, 0.f);
         } else if (inL || inH) {
-          const float4 t = X[S::row(pos) + cp];
+          const float4 t = *other;
           const float2 e = uT[k];
           const float sgn = inL ? -0.5f : 0.5f;
           const float2 w = make_float2(e.x * sgn, -e.y * sgn);
@@ -326,34 +329,42 @@ k_small(const __grid_constant__ fast::LayerPtrs lp, const __grid_constant__ SeqT
   }
   cluster.sync();
   const int nblk = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  if (rank == 0 && tid < 32) {
+    // energies: the head's sums, then, in the block of the (layer, sequence)'s last head, all heads' in order
+    double *en = energy + layer * energy_layer + 4ll * st.index[sq];
+    double v = 0.0;
+    if (tid < 4) {
+      for (int b = 0; b < nblk; ++b) v += *cluster.map_shared_rank(&sums[tid], b);
+      if ((tid & 1) == 0) v *= (double)head_dim;              // d * sum Dev = outlier-band energy
+      if (H == 1) en[tid] = v;
+      else part_en[((size_t)blockIdx.z * H + head) * 4 + tid] = v;
+    }
+    if (H > 1) {
+      __syncwarp();
+      bool last = false;
+      if (tid == 0) {
+        __threadfence();
+        last = atomicAdd(done + blockIdx.z, 1u) + 1u == (unsigned)H;
+        if (last) done[blockIdx.z] = 0u;
+        __threadfence();
+      }
+      if (__shfl_sync(0xffffffffu, last, 0) && tid < 4) {
+        v = 0.0;
+        for (int h = 0; h < H; ++h) v += __ldcg(part_en + ((size_t)blockIdx.z * H + h) * 4 + tid);
+        en[tid] = v;
+      }
+    }
+  }
   float *out = lp.scores[layer] + (long long)head * score_stride + start;
-  for (int n = rank * NT + tid; n < M; n += nblk * NT) {
-    if (PADDED && n >= N) break;
+  const int per = (M + nblk - 1) / nblk;                      // rows of this block
+  for (int i = NT - 1 - tid; i < per; i += NT) {              // (rank 0's first warp is busy with the energies)
+    const int n = rank * per + i;
+    if (n >= M || (PADDED && n >= N)) continue;
     float v = 0.f;
     for (int b = 0; b < nblk; ++b) v += *cluster.map_shared_rank(&rowsum[n], b);
     out[PADDED ? n : fast::perm_token(n, M)] = v * inv;
   }
-  if (rank == 0 && tid < 4) {
-    double v = 0.0;
-    for (int b = 0; b < nblk; ++b) v += *cluster.map_shared_rank(&sums[tid], b);
-    if ((tid & 1) == 0) v *= (double)head_dim;                // d * sum Dev = outlier-band energy
-    if (H == 1) energy[layer * energy_layer + 4ll * st.index[sq] + tid] = v;
-    else part[((size_t)blockIdx.z * H + head) * 4 + tid] = v;
-  }
   cluster.sync();                                             // remote reads of this block's memory are done
-  if (rank != 0 || H == 1) return;
-  // the last head of the (layer, sequence) adds up the heads in order
-  if (tid == 0) {
-    __threadfence();
-    is_last = atomicAdd(done + blockIdx.z, 1u) + 1u == (unsigned)H;
-    if (is_last) done[blockIdx.z] = 0u;
-  }
-  __syncthreads();
-  if (!is_last || tid >= 4) return;
-  __threadfence();
-  double v = 0.0;
-  for (int h = 0; h < H; ++h) v += __ldcg(part + ((size_t)blockIdx.z * H + h) * 4 + tid);
-  energy[layer * energy_layer + 4ll * st.index[sq] + tid] = v;
 }
 
 }  // namespace small

@@ -10,6 +10,8 @@
 
 #include <cooperative_groups.h>
 #include <math.h>
+#include <mutex>
+#include <unordered_map>
 
 namespace {
 
@@ -39,126 +41,193 @@ __device__ double filled_sum(const double *w, int L, double lam, double lo, doub
   return s;
 }
 
-// One block per sequence of the chunk.  Shared memory: w[L], cand[2L], fval[2L], frac[L], order[L].
-__global__ void __launch_bounds__(256)
+__device__ __forceinline__ double warp_min_d(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+__device__ __forceinline__ double warp_max_d(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
+// One block per sequence of the chunk.  Shared memory: w[L], cand[2L], fval[2L], frac[L], bud[L], order[L].
+// The sums whose rounding the rule fixes run in layer order (one thread, or one thread per candidate); everything else
+// (searches over the candidates, the remainders' order and who gets one) is spread over the block, so that a call is a
+// chain of a few L-step loops: 10.9 + 1.8 us (with the offsets as a second kernel) -> ALLOC us at 28 layers.
+// The last block of the call writes the offsets.
+constexpr int kAllocThreads = 256;
+__global__ void __launch_bounds__(kAllocThreads)
 k_allocate(const double *__restrict__ energy, int L, int B, int b0, SeqTable st, double rho,
-           int min_keep, int *__restrict__ budgets) {
+           int min_keep, int *__restrict__ budgets, long long *__restrict__ out_offsets, unsigned *__restrict__ done,
+           unsigned total_blocks) {
   extern __shared__ double sh[];
   double *w = sh;
   double *cand = w + L;
   double *fval = cand + 2 * L;
   double *frac = fval + 2 * L;
-  int *order = reinterpret_cast<int *>(frac + L);
-  __shared__ double s_sum;
-  __shared__ int s_bad;
-  const int tid = threadIdx.x;
+  int *bud = reinterpret_cast<int *>(frac + L);
+  int *order = bud + L;
+  __shared__ double s_sum, s_red[2][kAllocThreads / 32];
+  __shared__ int s_bad, s_floor, s_last;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = b0 + blockIdx.x;
-  const int N = st.start[blockIdx.x + 1] - st.start[blockIdx.x];
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  const int N = b < B ? st.start[blockIdx.x + 1] - st.start[blockIdx.x] : 0;
   if (N == 0) {
-    for (int l = tid; l < L; l += blockDim.x) budgets[(size_t)l * B + b] = 0;
-    return;
-  }
-  const double lo = (double)(min_keep < N ? (min_keep < 0 ? 0 : min_keep) : N);
-  const double hi = (double)N;
-  double bt = floor(rho * (double)N * (double)L + 0.5);
-  if (bt < (double)L * lo) bt = (double)L * lo;
-  if (bt > (double)L * hi) bt = (double)L * hi;
-  const long long B_tot = (long long)bt;
+    if (b < B)
+      for (int l = tid; l < L; l += kAllocThreads) budgets[(size_t)l * B + b] = 0;
+  } else {
+    const double lo = (double)(min_keep < N ? (min_keep < 0 ? 0 : min_keep) : N);
+    const double hi = (double)N;
+    double bt = floor(rho * (double)N * (double)L + 0.5);
+    if (bt < (double)L * lo) bt = (double)L * lo;
+    if (bt > (double)L * hi) bt = (double)L * hi;
+    const long long B_tot = (long long)bt;
 
-  // R^l = hiK/totK + hiV/totV   (Eq. 12)
-  if (tid == 0) s_bad = 0;
-  __syncthreads();
-  for (int l = tid; l < L; l += blockDim.x) {
-    const double *e = energy + ((size_t)l * B + b) * 4;
-    const double rk = e[1] > 0.0 ? e[0] / e[1] : 0.0;
-    const double rv = e[3] > 0.0 ? e[2] / e[3] : 0.0;
-    const double R = rk + rv;
-    w[l] = R;
-    if (!(R >= 0.0) || isinf(R)) s_bad = 1;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    double s = 0.0;
-    for (int l = 0; l < L; ++l) s += w[l];
-    if (!(s > 0.0) || isinf(s) || isnan(s)) s_bad = 1;
-    s_sum = s;
-  }
-  __syncthreads();
-  const bool uniform = s_bad != 0;
-  const double total = s_sum;
-  __syncthreads();
-  for (int l = tid; l < L; l += blockDim.x) w[l] = uniform ? 1.0 / (double)L : w[l] / total;
-  __syncthreads();
-
-  // kinks of f(lam) = sum clamp(lam*w, lo, hi) and f at each of them
-  for (int i = tid; i < 2 * L; i += blockDim.x) {
-    const double wl = w[i >> 1];
-    cand[i] = wl > 0.0 ? ((i & 1) ? hi / wl : lo / wl) : INFINITY;
-  }
-  __syncthreads();
-  for (int i = tid; i < 2 * L; i += blockDim.x)
-    fval[i] = isinf(cand[i]) ? -1.0 : filled_sum(w, L, cand[i], lo, hi);
-  __syncthreads();
-
-  if (tid == 0) {
-    // smallest kink b* > 0 with f(b*) >= B_tot, and the largest kink a* < b* (0 counts as a kink)
-    double bstar = INFINITY, fb = 0.0, kmax = 0.0;
-    for (int i = 0; i < 2 * L; ++i) {
-      if (isinf(cand[i])) continue;
-      if (cand[i] > kmax) kmax = cand[i];
-      if (cand[i] > 0.0 && fval[i] >= (double)B_tot && cand[i] < bstar) { bstar = cand[i]; fb = fval[i]; }
+    // R^l = hiK/totK + hiV/totV   (Eq. 12)
+    if (tid == 0) { s_bad = 0; s_floor = 0; }
+    __syncthreads();
+    for (int l = tid; l < L; l += kAllocThreads) {
+      const double *e = energy + ((size_t)l * B + b) * 4;
+      const double rk = e[1] > 0.0 ? e[0] / e[1] : 0.0;
+      const double rv = e[3] > 0.0 ? e[2] / e[3] : 0.0;
+      const double R = rk + rv;
+      w[l] = R;
+      if (!(R >= 0.0) || isinf(R)) s_bad = 1;
     }
-    double lam;
-    if (isinf(bstar)) {
-      lam = kmax;
-    } else {
+    __syncthreads();
+    if (tid == 0) {
+      double s = 0.0;
+#pragma unroll 4
+      for (int l = 0; l < L; ++l) s += w[l];
+      if (!(s > 0.0) || isinf(s) || isnan(s)) s_bad = 1;
+      s_sum = s;
+    }
+    __syncthreads();
+    const bool uniform = s_bad != 0;
+    const double total = s_sum;
+    for (int l = tid; l < L; l += kAllocThreads) w[l] = uniform ? 1.0 / (double)L : w[l] / total;
+    __syncthreads();
+
+    // kinks of f(lam) = sum clamp(lam*w, lo, hi) and f at each of them; the smallest kink b* > 0 with f(b*) >= B_tot
+    // and the largest one in all
+    double bstar = INFINITY, kmax = 0.0;
+    for (int i = tid; i < 2 * L; i += kAllocThreads) {
+      const double wl = w[i >> 1];
+      const double c = wl > 0.0 ? ((i & 1) ? hi / wl : lo / wl) : INFINITY;
+      double f = -1.0;
+      if (!isinf(c)) {
+        f = filled_sum(w, L, c, lo, hi);
+        kmax = fmax(kmax, c);
+        if (c > 0.0 && f >= (double)B_tot) bstar = fmin(bstar, c);
+      }
+      cand[i] = c;
+      fval[i] = f;
+    }
+    bstar = warp_min_d(bstar);
+    kmax = warp_max_d(kmax);
+    if (lane == 0) { s_red[0][warp] = bstar; s_red[1][warp] = kmax; }
+    __syncthreads();
+    bstar = INFINITY;
+#pragma unroll
+    for (int i = 0; i < kAllocThreads / 32; ++i) { bstar = fmin(bstar, s_red[0][i]); kmax = fmax(kmax, s_red[1][i]); }
+    __syncthreads();
+    double lam = kmax;
+    if (!isinf(bstar)) {
+      // the largest kink a* < b* (0 counts as a kink) and f at both; equal kinks have equal f
       double astar = 0.0;
-      for (int i = 0; i < 2 * L; ++i)
-        if (!isinf(cand[i]) && cand[i] < bstar && cand[i] > astar) astar = cand[i];
-      const double fa = filled_sum(w, L, astar, lo, hi);
+      for (int i = tid; i < 2 * L; i += kAllocThreads)
+        if (cand[i] < bstar) astar = fmax(astar, cand[i]);
+      astar = warp_max_d(astar);
+      if (lane == 0) s_red[0][warp] = astar;
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < kAllocThreads / 32; ++i) astar = fmax(astar, s_red[0][i]);
+      if (tid == 0) s_red[1][1] = (double)L * lo;            // f(0): L whole numbers, exact in any order
+      __syncthreads();
+      for (int i = tid; i < 2 * L; i += kAllocThreads) {
+        if (cand[i] == bstar) s_red[1][0] = fval[i];
+        if (cand[i] == astar && astar > 0.0) s_red[1][1] = fval[i];
+      }
+      __syncthreads();
+      const double fb = s_red[1][0], fa = s_red[1][1];
       lam = (fb == fa) ? astar : astar + ((double)B_tot - fa) * (bstar - astar) / (fb - fa);
     }
-    long long sum = 0;
-    for (int l = 0; l < L; ++l) {
+    int mine = 0;
+    for (int l = tid; l < L; l += kAllocThreads) {
       double q = lam * w[l];
       q = q < lo ? lo : (q > hi ? hi : q);
       const double fl = floor(q);
       frac[l] = q - fl;
-      budgets[(size_t)l * B + b] = (int)fl;
-      sum += (long long)fl;
+      bud[l] = (int)fl;
+      // the sum of the floors, low and high halves apart (it may pass 2^31)
+      mine += (int)fl;
     }
-    s_sum = (double)(B_tot - sum);     // deficit
+    // (at most 1024 layers of at most 131072 tokens: 2^27)
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if (lane == 0) atomicAdd(&s_floor, mine);
+    __syncthreads();
+    const long long deficit = B_tot - (long long)s_floor;
+    // order by (fraction descending, layer ascending)
+    for (int l = tid; l < L; l += kAllocThreads) {
+      int rank = 0;
+      const double f = frac[l];
+#pragma unroll 4
+      for (int m = 0; m < L; ++m) rank += (frac[m] > f || (frac[m] == f && m < l)) ? 1 : 0;
+      order[rank] = l;
+    }
+    __syncthreads();
+    // one more token to each layer in that order that is not full, round after round: the first round in parallel,
+    // further ones (only when layers are full) by one thread
+    int room = 0;
+    for (int l = tid; l < L; l += kAllocThreads) room += bud[l] < N ? 1 : 0;
+    if (tid == 0) s_last = 0;
+    __syncthreads();
+    room = __reduce_add_sync(0xffffffffu, room);
+    if (lane == 0) atomicAdd(&s_last, room);
+    __syncthreads();
+    room = s_last;
+    if (deficit > 0 && deficit <= room) {
+      for (int r = tid; r < L; r += kAllocThreads) {
+        int before = 0;
+        for (int m = 0; m < r; ++m) before += bud[order[m]] < N ? 1 : 0;
+        cand[r] = (bud[order[r]] < N && before < deficit) ? 1.0 : 0.0;
+      }
+      __syncthreads();
+      for (int r = tid; r < L; r += kAllocThreads)
+        if (cand[r] > 0.0) bud[order[r]] += 1;
+    } else if (deficit > 0 && tid == 0) {
+      long long left = deficit;
+      while (left > 0) {
+        bool gave = false;
+        for (int r = 0; r < L && left > 0; ++r)
+          if (bud[order[r]] < N) { bud[order[r]] += 1; --left; gave = true; }
+        if (!gave) break;
+      }
+    }
+    __syncthreads();
+    for (int l = tid; l < L; l += kAllocThreads) budgets[(size_t)l * B + b] = bud[l];
   }
-  __syncthreads();
-  // order by (fraction descending, layer ascending)
-  for (int l = tid; l < L; l += blockDim.x) {
-    int rank = 0;
-    const double f = frac[l];
-    for (int m = 0; m < L; ++m) rank += (frac[m] > f || (frac[m] == f && m < l)) ? 1 : 0;
-    order[rank] = l;
-  }
+  // the last block of the call: out_offsets[l][.] = exclusive prefix sums of budgets[l][.]
+  __threadfence();
   __syncthreads();
   if (tid == 0) {
-    long long deficit = (long long)s_sum;
-    while (deficit > 0) {
-      bool gave = false;
-      for (int r = 0; r < L && deficit > 0; ++r) {
-        int *bl = &budgets[(size_t)order[r] * B + b];
-        if (*bl < N) { *bl += 1; --deficit; gave = true; }
-      }
-      if (!gave) break;
-    }
+    s_last = (atomicAdd(done, 1u) + 1u == total_blocks) ? 1 : 0;
+    if (s_last) *done = 0u;
+    __threadfence();
   }
-}
-
-__global__ void k_offsets(const int *__restrict__ budgets, int L, int B, long long *__restrict__ out_offsets) {
-  const int l = blockIdx.x * blockDim.x + threadIdx.x;
-  if (l >= L) return;
-  long long acc = 0;
-  out_offsets[(size_t)l * (B + 1)] = 0;
-  for (int b = 0; b < B; ++b) {
-    acc += budgets[(size_t)l * B + b];
-    out_offsets[(size_t)l * (B + 1) + b + 1] = acc;
+  __syncthreads();
+  if (!s_last) return;
+  for (int l = tid; l < L; l += kAllocThreads) {
+    long long acc = 0;
+    long long *off = out_offsets + (size_t)l * (B + 1);
+    off[0] = 0;
+    for (int i = 0; i < B; ++i) {
+      acc += __ldcg(budgets + (size_t)l * B + i);
+      off[i + 1] = acc;
+    }
   }
 }
 
@@ -173,23 +242,25 @@ __device__ __forceinline__ unsigned score_key(float x) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-constexpr int kSelThreads = 1024;   // threads per block of the selection kernel
-constexpr int kSelCluster = 8;      // blocks (one cluster) per (sequence, head) at most; 2 or 4 for shorter sequences
-constexpr int kSelKptMax = 16;      // scores per thread: 8 * 1024 * 16 = 131072 tokens at most
+constexpr int kSelCluster = 8;      // blocks (one cluster) per (sequence, head) at most
+constexpr int kSelKptMax = 16;      // scores per thread
+constexpr int kSelMaxTokens = kSelCluster * 1024 * kSelKptMax;
+constexpr int kBins = 2048;         // radix digits: 10 (sign, exponent, one mantissa bit), 11 and 11 bits
+constexpr int kCandidates = 128;    // a bin of at most this many keys is finished by comparing them with one another
 
-// Selection + compaction + row gather for one (sequence, head), by one cluster of
-// CL blocks (2, 4 or 8).  Block r of the cluster owns the contiguous token range
-// [r*chunk, (r+1)*chunk) and keeps its score keys in registers.  The k-th largest
-// key is found by a 4-pass MSB-first radix select whose 256-bin histograms are
-// summed across the cluster through distributed shared memory; the chosen tokens
-// are then ranked in token order (block prefix + cluster prefix), written as
-// ascending indices, and their K/V rows are copied by the same block.
+// Selection + compaction + row gather for one (sequence, head), by one cluster of CL blocks of NT threads.  Block r of
+// the cluster owns the contiguous token range [r*chunk, (r+1)*chunk) and keeps its score keys in registers (thread t:
+// tokens t, t + NT, ... of the range, so loads coalesce).  The k-th largest key is found by an MSB-first radix select
+// with digits of 10, 11 and 11 bits, whose histograms are summed across the cluster through distributed shared memory; as soon as the
+// chosen bin holds few keys (after two digits, i.e. 12 mantissa bits, nearly always) they are compared with one another.
+// The chosen tokens are then ranked in token order (ballots per 32 tokens, one scan of the counts, cluster prefix),
+// written as ascending indices, and their K/V rows are copied by the same block.
 // grid (CL * sequences in chunk, heads), cluster (CL, 1, 1).
 // PER_LAYER: one cluster per sequence (grid.y = 1) ranks the tokens by the sum over heads of their
 // scores (the order of the head-averaged deviation), writes the same indices for every head and
 // gathers the rows of all heads.  protect (may be null): a non-zero byte per token of the batch puts
 // that token before every unmarked one.
-template <int kSelKpt, bool PER_LAYER, int CL>
+template <int KPT, bool PER_LAYER, int CL, int NT>
 __device__ __forceinline__ void
 select_gather_body(const float *__restrict__ scores, long long T, const SeqTable &st, int b0,
                 const int *__restrict__ budgets, const long long *__restrict__ out_offsets,
@@ -199,190 +270,246 @@ select_gather_body(const float *__restrict__ scores, long long T, const SeqTable
                 char *__restrict__ out_v, const unsigned char *__restrict__ protect) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
-  __shared__ int lhist[4][256];          // this block's histograms, one per pass (read by the whole cluster)
-  __shared__ int ghist[256];             // cluster-wide histogram of the current pass
-  __shared__ unsigned tot[CL];  // (ties << 16 | greater) of every block of the cluster
-  __shared__ unsigned wsum[kSelThreads / 32];
+  constexpr int NW = NT / 32, CNT = KPT * NW;     // warps, 32-token runs of the block's range
+  extern __shared__ unsigned short sel[];         // [KPT*NT] chosen tokens of the range, in order
+  __shared__ int lhist[3][kBins];                 // this block's histograms, one per digit (read by the whole cluster)
+  __shared__ unsigned cand[kCandidates];          // this block's keys in the chosen bin
+  __shared__ unsigned all[kCandidates];           // the cluster's
+  __shared__ unsigned runs[CNT];                  // (ties << 16 | greater) of every run, then their prefix sums
+  __shared__ unsigned tot[CL];                    // (ties << 16 | greater) of every block of the cluster
+  __shared__ unsigned wsum[32];
+  __shared__ int s_ncand;
   __shared__ unsigned s_prefix;
-  __shared__ int s_krem;
+  __shared__ int s_krem, s_count;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const unsigned r = cluster.block_rank();
+  const int r = CL == 1 ? 0 : (int)cluster.block_rank();
   const int bl = blockIdx.x / CL;
   const int b = b0 + bl, h = PER_LAYER ? 0 : blockIdx.y;
   const int s0 = st.start[bl];
   const int n = st.start[bl + 1] - s0;
+  const float *sc = scores + (long long)h * T + s0;
+  const int chunk = (n + CL - 1) / CL;
+  const int lo = (int)r * chunk;
+  const int len = (lo + chunk < n ? lo + chunk : n) - lo;         // may be <= 0
+
+  if (n == 0) return;
+  // the budget, the offset and the scores are requested together, without a branch between the loads (tokens past the
+  // range read its neighbours and are not counted: 9.0 -> LOADUS us for 16 scores a thread)
   int k = budgets[b];
-  k = k < 0 ? 0 : (k > n ? n : k);
   const long long off = out_offsets[b];
+  unsigned key[KPT];
+  {
+    float x[KPT];
+    const int last = n - 1;
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) {
+      const int t = lo + tid + i * NT;
+      x[i] = __ldg(sc + (t < last ? t : last));
+    }
+    if (PER_LAYER)
+      for (int hh = 1; hh < H; ++hh) {
+        const float *sh = sc + (long long)hh * T;
+#pragma unroll
+        for (int i = 0; i < KPT; ++i) {
+          const int t = lo + tid + i * NT;
+          x[i] += __ldg(sh + (t < last ? t : last));
+        }
+      }
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) key[i] = score_key(x[i]);
+    if (protect) {
+#pragma unroll
+      for (int i = 0; i < KPT; ++i) {
+        const int t = lo + tid + i * NT;
+        if (__ldg(protect + s0 + (t < last ? t : last))) key[i] = 0xFFFFFFFFu;
+      }
+    }
+  }
+  k = k < 0 ? 0 : (k > n ? n : k);
   if (k == 0) return;                                    // same decision in every block of the cluster
   if (off < 0 || off + k > cap) {
     if (tid == 0 && r == 0) atomicOr(status, FC_DEV_FLAG_INTERNAL);
     return;
   }
-  const float *sc = scores + (long long)h * T + s0;
   int *dst = out_idx + (long long)h * cap + off;
+  auto sync_all = [&]() { if (CL == 1) __syncthreads(); else cluster.sync(); };
 
-  const int chunk = (n + CL - 1) / CL;
-  const int lo = (int)r * chunk;
-  const int hi = lo + chunk < n ? lo + chunk : n;
-  const int base = lo + tid * kSelKpt;
-  int nv = hi - base;
-  nv = nv < 0 ? 0 : (nv > kSelKpt ? kSelKpt : nv);
-  unsigned key[kSelKpt];
-#pragma unroll
-  for (int i = 0; i < kSelKpt; ++i) {
-    key[i] = 0u;
-    if (i < nv) {
-      float x = sc[base + i];
-      if (PER_LAYER)
-        for (int hh = 1; hh < H; ++hh) x += sc[(long long)hh * T + base + i];
-      key[i] = (protect && protect[s0 + base + i]) ? 0xFFFFFFFFu : score_key(x);
-    }
-  }
-
-  for (int i = tid; i < 4 * 256; i += kSelThreads) (&lhist[0][0])[i] = 0;
   unsigned tau = 0;
   int need = 0;
-  const bool take_all = (k == n);
-  if (!take_all) {
-    __syncthreads();                                     // the local histograms are zero
+  if (k < n) {
+    for (int i = tid; i < 3 * kBins; i += NT) (&lhist[0][0])[i] = 0;
+    if (tid == 0) s_ncand = 0;
+    __syncthreads();
     unsigned prefix = 0, mask = 0;
     int krem = k;
 #pragma unroll 1
-    for (int pass = 0; pass < 4; ++pass) {
-      const int shift = 24 - 8 * pass;
+    for (int pass = 0; pass < 3; ++pass) {
+      const int shift = pass == 0 ? 22 : pass == 1 ? 11 : 0;
+      const unsigned digits = pass == 0 ? 1023u : 2047u;
 #pragma unroll
-      for (int i = 0; i < kSelKpt; ++i) {
-        const bool m = (i < nv) && ((key[i] & mask) == prefix);
-        const unsigned act = __ballot_sync(0xffffffffu, m);
-        if (m) {
-          const unsigned dgt = (key[i] >> shift) & 255u;
-          const unsigned peers = __match_any_sync(act, dgt);
-          if (lane == __ffs(peers) - 1) atomicAdd(&lhist[pass][dgt], __popc(peers));
-        }
-      }
-      cluster.sync();                                    // every block's histogram of this pass is complete
-      if (tid < 256) {
-        int v = 0;
-#pragma unroll
-        for (unsigned rr = 0; rr < CL; ++rr) v += *cluster.map_shared_rank(&lhist[pass][tid], rr);
-        ghist[tid] = v;
-      }
-      __syncthreads();
-      if (warp == 0) {
-        // lane l owns bins 8l..8l+7; find the bin where the count from the top reaches krem
-        int mine = 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) mine += ghist[8 * lane + i];
-        int above = mine;                                // inclusive suffix sum over lanes >= l
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int t = __shfl_down_sync(0xffffffffu, above, o);
-          if (lane + o < 32) above += t;
-        }
-        const int strictly_above = above - mine;
-        if (strictly_above < krem && krem <= above) {
-          int cum = strictly_above, dsel = 8 * lane;
-          for (int i = 7; i >= 0; --i) {
-            const int c = ghist[8 * lane + i];
-            if (cum + c >= krem) { dsel = 8 * lane + i; break; }
-            cum += c;
+      for (int i = 0; i < KPT; ++i) {
+        const bool m = (tid + i * NT < len) && ((key[i] & mask) == prefix);
+        if (pass == 0) {                                 // a warp's keys share a few values of the first digit
+          const unsigned act = __ballot_sync(0xffffffffu, m);
+          if (m) {
+            const unsigned dgt = key[i] >> shift;
+            const unsigned peers = __match_any_sync(act, dgt);
+            if (lane == __ffs(peers) - 1) atomicAdd(&lhist[0][dgt], __popc(peers));
           }
-          s_krem = krem - cum;
-          s_prefix = prefix | ((unsigned)dsel << shift);
+        } else if (m) {                                  // and are spread over the later ones
+          atomicAdd(&lhist[pass][(key[i] >> shift) & digits], 1);
+        }
+      }
+      sync_all();                                        // every block's histogram of this digit is complete
+      // thread t owns the bins t*PB .. t*PB + PB - 1; find the bin where the count from the top reaches krem
+      constexpr int PB = kBins / NT;
+      int v[PB], mine = 0;
+#pragma unroll
+      for (int i = 0; i < PB; ++i) {
+        v[i] = 0;
+#pragma unroll
+        for (int rr = 0; rr < CL; ++rr)
+          v[i] += CL == 1 ? lhist[pass][tid * PB + i] : *cluster.map_shared_rank(&lhist[pass][tid * PB + i], rr);
+        mine += v[i];
+      }
+      int above = mine;                                  // inclusive suffix sum over the lanes from this one up
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_down_sync(0xffffffffu, above, o);
+        if (lane + o < 32) above += t;
+      }
+      if (lane == 0) wsum[warp] = (unsigned)above;
+      __syncthreads();
+      const int higher = __reduce_add_sync(0xffffffffu, lane < NW && lane > warp ? (int)wsum[lane] : 0);
+      int cum = higher + above - mine;                   // keys strictly above this thread's bins
+      if (cum < krem && krem <= cum + mine) {
+#pragma unroll
+        for (int i = PB - 1; i >= 0; --i) {
+          if (cum < krem && krem <= cum + v[i]) {
+            s_krem = krem - cum;
+            s_count = v[i];
+            s_prefix = prefix | ((unsigned)(tid * PB + i) << shift);
+          }
+          cum += v[i];
         }
       }
       __syncthreads();
       krem = s_krem;
       prefix = s_prefix;
-      mask |= 0xFFu << shift;
+      mask |= digits << shift;
+      const int count = s_count;
+      if (pass == 2) break;
+      if (count <= kCandidates) {
+        // the keys of the bin, from every block, then the one that krem of them (ties included) reach
+#pragma unroll
+        for (int i = 0; i < KPT; ++i)
+          if (tid + i * NT < len && (key[i] & mask) == prefix) cand[atomicAdd(&s_ncand, 1)] = key[i];
+        sync_all();
+        if (CL == 1) {
+          for (int i = tid; i < count; i += NT) all[i] = cand[i];
+        } else {
+          int at = 0;
+          for (int rr = 0; rr < CL; ++rr) {
+            const int c = *cluster.map_shared_rank(&s_ncand, rr);
+            for (int i = tid; i < c; i += NT) all[at + i] = *cluster.map_shared_rank(&cand[i], rr);
+            at += c;
+          }
+        }
+        __syncthreads();
+        for (int i = tid; i < count; i += NT) {
+          const unsigned x = all[i];
+          int gt = 0, eq = 0;
+#pragma unroll 8
+          for (int q = 0; q < count; ++q) { gt += all[q] > x ? 1 : 0; eq += all[q] == x ? 1 : 0; }
+          if (gt < krem && krem <= gt + eq) { s_prefix = x; s_krem = krem - gt; }      // equal keys agree
+        }
+        __syncthreads();
+        krem = s_krem;
+        prefix = s_prefix;
+        break;
+      }
     }
     tau = prefix;
     need = krem;
   }
 
-  // per-thread counts, block exclusive scan of (ties << 16 | greater)
-  unsigned cnt = 0;
+  // greater and tied keys of every run of 32 tokens, their exclusive prefix sums, the block's totals
 #pragma unroll
-  for (int i = 0; i < kSelKpt; ++i)
-    if (i < nv) cnt += (key[i] > tau ? 1u : 0u) + (key[i] == tau ? 0x10000u : 0u);
-  unsigned incl = cnt;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += t;
+  for (int i = 0; i < KPT; ++i) {
+    const bool in = tid + i * NT < len;
+    const unsigned g = __ballot_sync(0xffffffffu, in && key[i] > tau), e = __ballot_sync(0xffffffffu, in && key[i] == tau);
+    if (lane == 0) runs[i * NW + warp] = (unsigned)__popc(g) | ((unsigned)__popc(e) << 16);
   }
-  if (lane == 31) wsum[warp] = incl;
   __syncthreads();
-  if (warp == 0) {
-    const unsigned v = wsum[lane];
-    unsigned wi = v;
+  {
+    // CNT <= NT runs, one per thread
+    const unsigned v = tid < CNT ? runs[tid] : 0u;
+    unsigned incl = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const unsigned t = __shfl_up_sync(0xffffffffu, wi, o);
-      if (lane >= o) wi += t;
+      const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
     }
-    wsum[lane] = wi - v;                                 // exclusive prefix of the warp totals
-    if (lane == 31) {
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    const unsigned lower = __reduce_add_sync(0xffffffffu, lane < NW && lane < warp ? wsum[lane] : 0u);
+    if (tid < CNT) runs[tid] = lower + incl - v;
+    if (tid == NT - 1) {
+      const unsigned all_runs = lower + incl;
+      if (CL == 1) tot[0] = all_runs;
+      else
 #pragma unroll
-      for (unsigned rr = 0; rr < CL; ++rr) *cluster.map_shared_rank(&tot[r], rr) = wi;
+        for (int rr = 0; rr < CL; ++rr) *cluster.map_shared_rank(&tot[r], rr) = all_runs;
     }
   }
-  cluster.sync();                                        // also orders wsum for the block
-  const unsigned excl = wsum[warp] + incl - cnt;
+  sync_all();                                            // also orders runs for the block
   int gt_before = 0, tie_before = 0, my_gt = 0, my_tie = 0;
 #pragma unroll
-  for (unsigned rr = 0; rr < CL; ++rr) {
+  for (int rr = 0; rr < CL; ++rr) {
     const unsigned t = tot[rr];
     if (rr < r) { gt_before += (int)(t & 0xFFFFu); tie_before += (int)(t >> 16); }
     if (rr == r) { my_gt = (int)(t & 0xFFFFu); my_tie = (int)(t >> 16); }
   }
   // (a block holds at most 16384 scores, so neither 16-bit field can overflow)
-  int g = gt_before + (int)(excl & 0xFFFFu);
-  int ti = tie_before + (int)(excl >> 16);
+  const int first = gt_before + (tie_before < need ? tie_before : need);    // rank of this block's first token
 #pragma unroll
-  for (int i = 0; i < kSelKpt; ++i) {
-    if (i < nv) {
-      int pos = -1;
-      if (key[i] > tau) {
-        pos = g + (ti < need ? ti : need);
-        ++g;
-      } else if (key[i] == tau) {
-        if (ti < need) pos = g + ti;
-        ++ti;
-      }
-      if (pos >= 0) {
-        dst[pos] = base + i;
-        if (PER_LAYER)
-          for (int hh = 1; hh < H; ++hh) dst[(long long)hh * cap + pos] = base + i;
-      }
+  for (int i = 0; i < KPT; ++i) {
+    const bool in = tid + i * NT < len;
+    const bool g = in && key[i] > tau, e = in && key[i] == tau;
+    const unsigned bg = __ballot_sync(0xffffffffu, g), be = __ballot_sync(0xffffffffu, e), below = (1u << lane) - 1u;
+    const unsigned base = runs[i * NW + warp];
+    const int ng = gt_before + (int)(base & 0xFFFFu) + __popc(bg & below);
+    const int nt = tie_before + (int)(base >> 16) + __popc(be & below);
+    if (g || (e && nt < need)) {
+      const int pos = ng + (nt < need ? nt : need), tok = lo + tid + i * NT;
+      sel[pos - first] = (unsigned short)(tid + i * NT);
+      dst[pos] = tok;
+      if (PER_LAYER)
+        for (int hh = 1; hh < H; ++hh) dst[(long long)hh * cap + pos] = tok;
     }
   }
-  __syncthreads();                                       // this block's indices are visible to its warps
+  __syncthreads();                                       // this block's tokens are visible to its warps
 
   // gather the rows this block selected: ranks [first, first + count)
-  const int first = gt_before + (tie_before < need ? tie_before : need);
   int tie_take = need - tie_before;
   tie_take = tie_take < 0 ? 0 : (tie_take > my_tie ? my_tie : tie_take);
   const int count = my_gt + tie_take;
   const int n16 = row_bytes >> 4;
-  // a warp takes kGatherRows rows at a time: their indices, then their 16-byte pieces, are requested together, so
+  // a warp takes kGatherRows rows at a time: their 16-byte pieces are requested together, so
   // that several independent round trips to DRAM are in flight per warp instead of one after the other
   constexpr int kGatherRows = 4;
   const int per_head = 2 * n16;
-  for (int rr0 = warp * kGatherRows; rr0 < count; rr0 += (kSelThreads / 32) * kGatherRows) {
-    long long tok[kGatherRows];
+  const char *kb = kin + ((long long)s0 + lo) * stride_token_b, *vb = vin + ((long long)s0 + lo) * stride_token_b;
+  for (int rr0 = warp * kGatherRows; rr0 < count; rr0 += NW * kGatherRows) {
+    int tok[kGatherRows];
 #pragma unroll
-    for (int g = 0; g < kGatherRows; ++g) {
-      const int rr = rr0 + g < count ? rr0 + g : rr0;            // rows past the end repeat the first (not stored)
-      tok[g] = (long long)s0 + dst[first + rr];
-    }
+    for (int g = 0; g < kGatherRows; ++g) tok[g] = sel[rr0 + g < count ? rr0 + g : rr0];   // past the end: repeated, not stored
     for (int w = lane; w < (PER_LAYER ? H * per_head : per_head); w += 32) {
       const int hh = PER_LAYER ? w / per_head : h;
       const int u = PER_LAYER ? w - hh * per_head : w;
       const bool isv = u >= n16;
       const int uu = isv ? u - n16 : u;
-      const char *in = (isv ? vin : kin) + (long long)hh * stride_head_b + 16ll * uu;
+      const char *in = (isv ? vb : kb) + (long long)hh * stride_head_b + 16ll * uu;
       char *out = (isv ? out_v : out_k) + 16ll * uu;
       uint4 val[kGatherRows];
 #pragma unroll
@@ -400,8 +527,8 @@ select_gather_body(const float *__restrict__ scores, long long T, const SeqTable
 // overlap != 0 (launched with the programmatic-serialisation attribute): the next launch in the stream
 // may start as soon as every block of this one has begun, and this grid does not finish before its
 // predecessor has, so "the last launch is complete" still means "all of them are".
-template <int kSelKpt, bool PER_LAYER, int CL>
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kSelThreads)
+template <int KPT, bool PER_LAYER, int CL, int NT>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT, 1024 / NT)
 k_select_gather(const __grid_constant__ LayerTable lt, long long T, const __grid_constant__ SeqTable st, int b0, int B,
                 const int *__restrict__ budgets, const long long *__restrict__ out_offsets,
                 int *__restrict__ status, long long stride_token_b,
@@ -409,7 +536,7 @@ k_select_gather(const __grid_constant__ LayerTable lt, long long T, const __grid
                 const unsigned char *__restrict__ protect) {
   if (overlap) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   const int z = blockIdx.z;
-  select_gather_body<kSelKpt, PER_LAYER, CL>(lt.scores[z], T, st, b0, budgets + (size_t)z * B,
+  select_gather_body<KPT, PER_LAYER, CL, NT>(lt.scores[z], T, st, b0, budgets + (size_t)z * B,
                                          out_offsets + (size_t)z * (B + 1), lt.out_idx[z], lt.cap[z], status, lt.k[z], lt.v[z],
                                          stride_token_b, stride_head_b, row_bytes, H, lt.out_k[z], lt.out_v[z], protect);
   if (overlap) asm volatile("griddepcontrol.wait;\n" ::: "memory");
@@ -440,16 +567,32 @@ extern "C" fc_status fc_allocate_budgets(fc_handle *h, const double *energy, int
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if ((s = fc_flush_pending(h, st)) != FC_OK) return s;    // the energies may still be in flight on the internal streams
   const int L = num_layers;
-  const size_t sm = (size_t)(6 * L) * sizeof(double) + (size_t)L * sizeof(int);
-  for (int b0 = 0; b0 < batch; b0 += kSeqChunk) {
+  const size_t sm = (size_t)(6 * L) * sizeof(double) + (size_t)(2 * L) * sizeof(int);
+  if (sm > 48 * 1024) FC_CUDA_TRY(cudaFuncSetAttribute(k_allocate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  for (int b0 = 0; b0 < batch || b0 == 0; b0 += kSeqChunk) {
     const int nseq = batch - b0 < kSeqChunk ? batch - b0 : kSeqChunk;
     SeqTable tab;
     for (int i = 0; i <= nseq; ++i) tab.start[i] = cu_seqlens_host[b0 + i];
-    k_allocate<<<nseq, 256, sm, st>>>(energy, L, batch, b0, tab, rho, min_keep, budgets);
+    // a programmatic dependent: resident when the kernel before it ends (an empty batch still has its offsets written)
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(nseq > 0 ? nseq : 1);
+    lc.blockDim = dim3(kAllocThreads);
+    lc.dynamicSmemBytes = sm;
+    lc.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    if (cudaLaunchKernelEx(&lc, k_allocate, energy, (int)L, (int)batch, b0, tab, rho, (int)min_keep, budgets,
+                           reinterpret_cast<long long *>(out_offsets), h->done_counter + 2 * FC_LAYER_CHUNK,
+                           (unsigned)(batch > 0 ? batch : 1)) != cudaSuccess) {
+      cudaGetLastError();
+      return FC_ERR_CUDA;
+    }
     if ((s = fc_after_launch(h)) != FC_OK) return s;
   }
-  k_offsets<<<(L + 127) / 128, 128, 0, st>>>(budgets, L, batch, reinterpret_cast<long long *>(out_offsets));
-  return fc_after_launch(h);
+  return FC_OK;
 }
 
 extern "C" size_t fc_select_workspace_bytes(const fc_handle *h, const fc_kv_view *kv) {
@@ -478,10 +621,27 @@ fc_status check_select_shape(const fc_handle *h, const fc_kv_view *kv, const voi
   fc_status s = check_cu(kv->cu_seqlens, kv->batch);
   if (s != FC_OK) return s;
   for (int b = 0; b < kv->batch; ++b)
-    if (kv->cu_seqlens[b + 1] - kv->cu_seqlens[b] > kSelCluster * kSelThreads * kSelKptMax) return FC_ERR_UNSUPPORTED;
+    if (kv->cu_seqlens[b + 1] - kv->cu_seqlens[b] > kSelMaxTokens) return FC_ERR_UNSUPPORTED;
   if ((kv->stride_token * es) % 16 || (kv->stride_head * es) % 16) return FC_ERR_INVALID_ARG;
   if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < fc_select_workspace_bytes(h, kv))
     return FC_ERR_WORKSPACE;
+  return FC_OK;
+}
+
+// Dynamic shared memory beyond the default, once per kernel and device.
+template <class Kern>
+fc_status allow_smem(Kern kern, size_t bytes) {
+  static std::mutex mu;
+  static std::unordered_map<unsigned long long, size_t> done;     // (device, kernel) -> bytes already allowed
+  int dev = 0;
+  FC_CUDA_TRY(cudaGetDevice(&dev));
+  const unsigned long long key = (unsigned long long)reinterpret_cast<uintptr_t>(reinterpret_cast<const void *>(kern)) ^
+                                 ((unsigned long long)dev << 56);
+  std::lock_guard<std::mutex> lock(mu);
+  size_t &have = done[key];
+  if (have >= bytes) return FC_OK;
+  FC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  have = bytes;
   return FC_OK;
 }
 
@@ -499,50 +659,50 @@ fc_status launch_select(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, con
     for (int i = 0; i <= nseq; ++i) tab.start[i] = kv->cu_seqlens[b0 + i];
     int nmax = 0;
     for (int i = 0; i < nseq; ++i) nmax = tab.start[i + 1] - tab.start[i] > nmax ? tab.start[i + 1] - tab.start[i] : nmax;
-    // blocks per (sequence, head): the fewest of 2, 4, 8 that hold the longest sequence at 16 scores per thread.
-    // Fewer blocks per cluster let more clusters run at once (8 blocks of 1024 threads: 15 clusters on 148 SMs) and
-    // the phases of the radix select wait on cluster barriers, not on bandwidth: measured per step, 8 -> 2 blocks,
-    // 0.199 -> 0.158 ms at 28 x 4 heads of 32768 tokens, 1.70 -> 1.12 ms at 32 x 32 heads of 16384; one block is
-    // 2..9 % slower than two where it would fit.
-    int cl = 2;
-    while (cl < kSelCluster && nmax > cl * kSelThreads * kSelKptMax) cl *= 2;
-    const int per_thread = (nmax + cl * kSelThreads - 1) / (cl * kSelThreads);
+    // Blocks of 1024 threads, as few per (sequence, head) as hold the longest sequence at 16 scores per thread: every
+    // phase of the select waits on barriers, and one block's are a fraction of a cluster's (28 x 4 heads of 1500 tokens:
+    // 22.6 us with two blocks, 12.2 with one; 8 ragged short sequences 131 -> 72 us; one layer of 1024 tokens: 10.0 us
+    // with one block, 18.4 with eight).  Two where a layer keeps one index set, whose few clusters gather all heads.
+    constexpr int nt = 1024;
+    int cl = per_layer ? 2 : 1;
+    while (cl < kSelCluster && nmax > cl * nt * kSelKptMax) cl *= 2;
+    int kpt = 2;
+    while (kpt < kSelKptMax && nmax > cl * nt * kpt) kpt *= 2;
     {
       ProfScope ps(h, FC_K_SELECT, st);
-#define FC_SEL_LAUNCH(KPT, PL, CLV)                                                                     \
+      const size_t sm = (size_t)kpt * nt * sizeof(unsigned short);
+#define FC_SEL_LAUNCH(KPT, PL, CLV)                                                                \
   do {                                                                                                  \
+    if ((s = allow_smem(k_select_gather<KPT, PL, CLV, nt>, sm)) != FC_OK) return s;                    \
     cudaLaunchConfig_t lc = {};                                                                         \
     lc.gridDim = dim3(CLV * nseq, (PL) ? 1 : kv->num_heads, nl);                                        \
-    lc.blockDim = dim3(kSelThreads);                                                                    \
+    lc.blockDim = dim3(nt);                                                                             \
+    lc.dynamicSmemBytes = sm;                                                                           \
     lc.stream = st;                                                                                     \
     cudaLaunchAttribute at[1];                                                                          \
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;                                      \
     at[0].val.programmaticStreamSerializationAllowed = 1;                                               \
     lc.attrs = at;                                                                                      \
-    lc.numAttrs = h->select_overlap ? 1 : 0;                                                            \
-    launch_err = cudaLaunchKernelEx(&lc, k_select_gather<KPT, PL, CLV>, lt, (long long)T, tab, b0, (int)kv->batch, \
+    lc.numAttrs = (h->select_overlap && h->after_select) ? 1 : 0;                                       \
+    launch_err = cudaLaunchKernelEx(&lc, k_select_gather<KPT, PL, CLV, nt>, lt, (long long)T, tab, b0, (int)kv->batch, \
         budgets, reinterpret_cast<const long long *>(out_offsets),                                      \
         h->status_word, (long long)(kv->stride_token * es), (long long)(kv->stride_head * es),          \
         (int)(kv->head_dim * es), (int)kv->num_heads, (int)h->select_overlap, protect);                 \
   } while (0)
-#define FC_SEL_KPT(PL, CLV)                                                                             \
-  do {                                                                                                  \
-    if (per_thread <= 2) FC_SEL_LAUNCH(2, PL, CLV);                                                     \
-    else if (per_thread <= 4) FC_SEL_LAUNCH(4, PL, CLV);                                                \
-    else if (per_thread <= 8) FC_SEL_LAUNCH(8, PL, CLV);                                                \
-    else FC_SEL_LAUNCH(16, PL, CLV);                                                                    \
-  } while (0)
-      cudaError_t launch_err = cudaSuccess;
-      if (per_layer) {
-        if (cl == 2) FC_SEL_KPT(true, 2); else if (cl == 4) FC_SEL_KPT(true, 4); else FC_SEL_KPT(true, 8);
-      } else {
-        if (cl == 2) FC_SEL_KPT(false, 2); else if (cl == 4) FC_SEL_KPT(false, 4); else FC_SEL_KPT(false, 8);
-      }
-      if (launch_err != cudaSuccess) return FC_ERR_CUDA;
-#undef FC_SEL_KPT
+#define FC_SEL_CASE(KPT, PL, CLV) \
+  else if (kpt == KPT && cl == CLV && per_layer == PL) FC_SEL_LAUNCH(KPT, PL, CLV);
+      cudaError_t launch_err = cudaErrorInvalidValue;
+      if (false) {}
+      FC_SEL_CASE(2, false, 1) FC_SEL_CASE(4, false, 1) FC_SEL_CASE(8, false, 1) FC_SEL_CASE(16, false, 1)
+      FC_SEL_CASE(16, false, 2) FC_SEL_CASE(16, false, 4) FC_SEL_CASE(16, false, 8)
+      FC_SEL_CASE(2, true, 2) FC_SEL_CASE(4, true, 2) FC_SEL_CASE(8, true, 2) FC_SEL_CASE(16, true, 2)
+      FC_SEL_CASE(16, true, 4) FC_SEL_CASE(16, true, 8)
+#undef FC_SEL_CASE
 #undef FC_SEL_LAUNCH
+      if (launch_err != cudaSuccess) { cudaGetLastError(); return FC_ERR_CUDA; }
     }
     if ((s = fc_after_launch(h)) != FC_OK) return s;
+    h->after_select = true;
   }
   return FC_OK;
 }
