@@ -21,9 +21,10 @@
 //           twiddle, DFT over n2, the filter above, inverse DFT over k2, twiddle -> B[k1][n2]
 //   pass 3  for every n2: inverse DFT over k1, |.|^2 summed over the channels -> scores
 // Every other length up to 65536 takes the same three passes on a longer transform with the residual written as one
-// padded convolution (fc_score_fast.cuh).  The generic kernels of this file serve the power of two 131072, the spectrum
-// diagnostics and the entry point without allocation; there, lengths that are not a power of two (or are below 16) go
-// through Bluestein's chirp convolution on a power-of-two length M >= 2N-1.
+// padded convolution (fc_score_fast.cuh); the spectrum diagnostics run on the same passes.  The generic kernels of this
+// file serve the power of two 131072, spectra of short powers of two and the entry point without allocation; there,
+// lengths that are not a power of two (or are below 16) go through Bluestein's chirp convolution on a power-of-two
+// length M >= 2N-1.
 #include "fc_common.cuh"
 #include "fc_score_fast.cuh"
 #include "fc_score_small.cuh"
@@ -47,13 +48,7 @@ __device__ __forceinline__ int perm_token(int p, int N) {
   return p < half ? 2 * p : 2 * (N - 1 - p) + 1;
 }
 
-// exp(j*pi*n^2/N), the Bluestein chirp; the phase is reduced exactly in integers.
-__device__ __forceinline__ float2 chirp(int n, int N) {
-  const unsigned long long r = ((unsigned long long)n * (unsigned long long)n) % (2ull * (unsigned long long)N);
-  float s, c;
-  sincospif(__fdiv_rn((float)(unsigned)r, (float)N), &s, &c);
-  return make_float2(c, s);
-}
+using fast::chirp;
 
 template <typename T> struct Elem;
 template <> struct Elem<float> {
@@ -553,7 +548,7 @@ k_pass2_power(FftPlan plan, int N1, int ncol_ws, int cs2_log2, const float2 *__r
   }
 }
 
-// Other N (chirp path): from the N-point spectrum spec[q][col].  grid (N/2 + 1): block q sums the pair
+// Chirp convolutions: from the N-point spectrum spec[q][col].  grid (N/2 + 1): block q sums the pair
 // {q, N-q} over all columns of the group and writes partial[q], partial[N-q].
 __global__ void __launch_bounds__(kThreads)
 k_spec_power(const float2 *__restrict__ spec, int ncol, int N, float2 *__restrict__ partial) {
@@ -585,14 +580,17 @@ k_spec_power(const float2 *__restrict__ spec, int ncol, int N, float2 *__restric
   }
 }
 
-// spectrum[m] (+)= sum over y of partial[y][m], in fp64 and in a fixed order.
-__global__ void k_power_accumulate(const float2 *__restrict__ partial, int ny, int N, double *__restrict__ spectrum,
+// spectrum[m] (+)= sum over y of partial[y][m], in fp64 and in a fixed order.  The partial sums of the direct form are in
+// the order [k1][k2] of pass 2, bin k1 + N1*k2; N1 == 1: in the order of the bins.
+__global__ void k_power_accumulate(const float2 *__restrict__ partial, int ny, int N, int N1, double *__restrict__ spectrum,
                                    int first) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= N) return;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= N) return;
+  const int N2 = N / N1, m = N1 == 1 ? i : i / N2 + N1 * (i % N2);
   double a = first ? 0.0 : spectrum[2 * m], b = first ? 0.0 : spectrum[2 * m + 1];
+#pragma unroll 4
   for (int y = 0; y < ny; ++y) {
-    const float2 p = partial[(size_t)y * N + m];
+    const float2 p = __ldcs(partial + (size_t)y * N + i);
     a += (double)p.x;
     b += (double)p.y;
   }
@@ -612,7 +610,7 @@ inline int ilog2(int x) { int b = 0; while ((1 << b) < x) ++b; return b; }
 inline bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// ---- generic kernels: the power of two 131072, the spectrum diagnostics and the no-allocation entry point ----
+// ---- generic kernels: the power of two 131072, spectra of powers of two below 1024, the no-allocation entry point ----
 struct SeqPlan {
   bool bluestein;
   int N, Nfft, N1, N2;
@@ -724,6 +722,20 @@ inline PassPlan pad_shape(int M) {
   return p;
 }
 
+// The smallest padded length >= 2N - 1, N <= 65536.
+PassPlan plan_padded(int N) {
+  int best = 0;
+  const int need = 2 * N - 1;
+  for (int k = 10; k <= 17; ++k)
+    for (int f = 4; f <= 7; ++f) {
+      const int M = (1 << k) / 4 * f;
+      if (M >= need && (best == 0 || M < best) && pad_shape(M).ok) best = M;
+    }
+  PassPlan p = pad_shape(best);
+  p.N = N;
+  return p;
+}
+
 // Channel pairs per block of the small kernel for M points.
 constexpr int small_cp(int M) { return M <= 128 ? 32 : 4096 / M; }
 
@@ -763,19 +775,7 @@ PassPlan plan_passes(int N, int head_dim) {
     p.ok = true;
     return p;
   }
-  if (N > 65536) return p;
-  // smallest padded length >= 2N - 1
-  int best = 0;
-  const int need = 2 * N - 1;
-  for (int k = 10; k <= 17; ++k)
-    for (int f = 4; f <= 7; ++f) {
-      const int M = (1 << k) / 4 * f;
-      if (M >= need && (best == 0 || M < best) && pad_shape(M).ok) best = M;
-    }
-  if (best == 0) return p;
-  p = pad_shape(best);
-  p.N = N;
-  return p;
+  return N > 65536 ? p : plan_padded(N);
 }
 
 // How one sequence's units (layer, head) are grouped into launches.
@@ -854,12 +854,12 @@ ScoreLayout score_layout(const fc_handle *h, const fc_kv_view *kv, int num_layer
   L.hi_bytes = align_up(L.hi_bytes, 256);
   size_t off = 0;
   L.off_buf = off; off += L.buf_bytes * h->num_aux;
+  if (off < generic) off = generic;            // tables outlive a sequence on the generic kernels
   L.off_tab = off; off += align_up(tab, 256);
   L.off_tot = off; off += 2 * L.tot_bytes;
   L.off_hi = off;  off += 2 * L.hi_bytes;
   L.off_small = off; off += align_up(nl * nsmall * H * 4 * sizeof(double), 256);
-  L.total = off > generic ? off : generic;
-  if (L.total < 256) L.total = 256;
+  L.total = off < 256 ? 256 : off;
   return L;
 }
 
@@ -1013,7 +1013,7 @@ fc_status launch_p1(const PassArgs &x, double *part_tot, int layer_slots) {
   ProfScope ps(x.h, FC_K_PASS1, x.st);
   fast::k_p1<T, R1B, CPW, LD, A><<<dim3(p.N2, ncol / (2 * CPW)), CPW * R1B, sm, x.st>>>(
       *x.lp, x.kv->stride_token, x.kv->stride_head, x.kv->num_heads, x.kv->head_dim, x.u0, x.c0, x.cols, p.N, p.N2, ncol,
-      x.ws, x.h->master, x.h->master_len, part_tot, layer_slots, x.omega);
+      x.ws, x.h->master, x.h->master_len, part_tot, layer_slots, x.omega, x.tab);
   return fc_after_launch(x.h);
 }
 
@@ -1039,6 +1039,17 @@ fc_status run_p1(const PassArgs &x, double *part_tot, int layer_slots) {
   return FC_ERR_INTERNAL;
 }
 
+// The rows of a chirp convolution (spectrum diagnostics).
+template <typename T>
+fc_status run_p1_chirp(const PassArgs &x) {
+  const PassPlan &p = *x.p;
+#define FC_P1(A_, R_, C_) \
+  if (p.a == A_ && p.r1b == R_ && p.cpw == C_) return launch_p1<T, A_, R_, C_, fast::LD_CHIRP>(x, nullptr, 0);
+  FC_OUTER_PAD_SHAPES(FC_P1)
+#undef FC_P1
+  return FC_ERR_INTERNAL;
+}
+
 fc_status run_p1_table(const PassArgs &x) {
   const PassPlan &p = *x.p;
 #define FC_P1(A_, R_, C_) \
@@ -1049,50 +1060,59 @@ fc_status run_p1_table(const PassArgs &x) {
 }
 
 // tab_out != nullptr: the forward half on the two kernel columns, `ncol` columns wide (run_p1_table)
-template <int R2B, int CP, bool PAD>
-fc_status launch_p2(const PassArgs &x, int ncol, float4 *tab_out) {
+template <int R2B, int CP, int MODE>
+fc_status launch_p2(const PassArgs &x, int ncol, float4 *tab_out, float2 *power) {
   const PassPlan &p = *x.p;
+  constexpr bool TAB = MODE == fast::MODE_PAD || MODE == fast::MODE_MUL;
   const size_t sm = (size_t)2 * (16 * R2B) * CP * sizeof(float4) + (4 * R2B + 4) * sizeof(float2) +
-                    (PAD ? 2 * (16 * R2B) * sizeof(float4) : (2 * (16 * R2B) + 4) * sizeof(float2));
-  fc_status s = set_smem(fast::k_p2<R2B, CP, PAD>, sm);
+                    (TAB ? 2 * (16 * R2B) * sizeof(float4) : (2 * (16 * R2B) + 4) * sizeof(float2));
+  fc_status s = set_smem(fast::k_p2<R2B, CP, MODE>, sm);
   if (s != FC_OK) return s;
   ProfScope ps(x.h, FC_K_PASS2, x.st);
-  fast::k_p2<R2B, CP, PAD><<<dim3(p.N1 / 2, tab_out ? 1 : ncol / (2 * CP)), 2 * CP * R2B, sm, x.st>>>(
-      p.N1, ncol, x.ws, x.h->master, x.h->master_len, x.omega, x.tab, tab_out);
+  fast::k_p2<R2B, CP, MODE><<<dim3(p.N1 / 2, tab_out ? 1 : ncol / (2 * CP)), 2 * CP * R2B, sm, x.st>>>(
+      p.N1, ncol, x.ws, x.h->master, x.h->master_len, x.omega, x.tab, tab_out, power, p.N);
   return fc_after_launch(x.h);
 }
 
-fc_status run_p2(const PassArgs &x, int ncol, float4 *tab_out) {
+template <int MODE>
+fc_status launch_p2_512(const PassArgs &x, int ncol, float4 *tab_out) {
   const PassPlan &p = *x.p;
-  if (p.N2 == 512) {
-    constexpr int C = 8;
-    const size_t sm = (size_t)2 * 16 * (32 * C + C) * sizeof(float2) + 1024 * sizeof(float4) + (64 + 68) * sizeof(float2);
-    fc_status s = set_smem(fast::k_p2_512<C>, sm);
-    if (s != FC_OK) return s;
-    ProfScope ps(x.h, FC_K_PASS2, x.st);
-    fast::k_p2_512<C><<<dim3(p.N1 / 2, tab_out ? 1 : ncol / C), 32 * C, sm, x.st>>>(
-        p.N1, ncol, x.ws, x.h->master, x.h->master_len, x.tab, tab_out);
-    return fc_after_launch(x.h);
-  }
-#define FC_P2(R_, C_, P_) \
-  if (p.pad == P_ && p.r2b == R_ && p.cp == C_) return launch_p2<R_, C_, P_>(x, ncol, tab_out);
-  FC_P2(2, 32, true) FC_P2(4, 32, true) FC_P2(8, 16, true) FC_P2(16, 8, true)
-  FC_P2(2, 8, false) FC_P2(4, 8, false) FC_P2(4, 32, false) FC_P2(8, 16, false) FC_P2(16, 8, false)
+  constexpr int C = 8;
+  const size_t sm = (size_t)2 * 16 * (32 * C + C) * sizeof(float2) + 1024 * sizeof(float4) + (64 + 68) * sizeof(float2);
+  fc_status s = set_smem(fast::k_p2_512<C, MODE>, sm);
+  if (s != FC_OK) return s;
+  ProfScope ps(x.h, FC_K_PASS2, x.st);
+  fast::k_p2_512<C, MODE><<<dim3(p.N1 / 2, tab_out ? 1 : ncol / C), 32 * C, sm, x.st>>>(
+      p.N1, ncol, x.ws, x.h->master, x.h->master_len, x.tab, tab_out, p.N);
+  return fc_after_launch(x.h);
+}
+
+fc_status run_p2(const PassArgs &x, int ncol, int mode, float4 *tab_out = nullptr, float2 *power = nullptr) {
+  const PassPlan &p = *x.p;
+  using namespace fast;
+  if (p.N2 == 512) return mode == MODE_PAD ? launch_p2_512<MODE_PAD>(x, ncol, tab_out) : launch_p2_512<MODE_MUL>(x, ncol, tab_out);
+#define FC_P2(R_, C_, M_) \
+  if (mode == M_ && p.r2b == R_ && p.cp == C_) return launch_p2<R_, C_, M_>(x, ncol, tab_out, power);
+  FC_P2(2, 32, MODE_PAD) FC_P2(4, 32, MODE_PAD) FC_P2(8, 16, MODE_PAD) FC_P2(16, 8, MODE_PAD)
+  FC_P2(2, 32, MODE_MUL) FC_P2(4, 32, MODE_MUL) FC_P2(8, 16, MODE_MUL) FC_P2(16, 8, MODE_MUL)
+  FC_P2(2, 8, MODE_FILTER) FC_P2(4, 8, MODE_FILTER) FC_P2(4, 32, MODE_FILTER) FC_P2(8, 16, MODE_FILTER) FC_P2(16, 8, MODE_FILTER)
+  FC_P2(2, 8, MODE_POWER) FC_P2(4, 8, MODE_POWER) FC_P2(4, 32, MODE_POWER) FC_P2(8, 16, MODE_POWER) FC_P2(16, 8, MODE_POWER)
 #undef FC_P2
   return FC_ERR_INTERNAL;
 }
 
-template <int A, int R1B, int CPW, bool PAD>
-fc_status launch_p3(const PassArgs &x, long long score_stride, int accumulate, int hi_base, const fast::EnergyOut &eo) {
+template <int A, int R1B, int CPW, int OUT>
+fc_status launch_p3(const PassArgs &x, long long score_stride, int accumulate, int hi_base, const fast::EnergyOut &eo,
+                    float2 *spec = nullptr) {
   const PassPlan &p = *x.p;
   const size_t sm = smem_outer(p);
-  fc_status s = set_smem(fast::k_p3<R1B, CPW, PAD, A>, sm);
+  fc_status s = set_smem(fast::k_p3<R1B, CPW, OUT, A>, sm);
   if (s != FC_OK) return s;
-  const float inv = (float)(1.0 / ((double)p.M * (double)p.M * (double)x.kv->head_dim));
+  const float inv = OUT == fast::OUT_SPEC ? 1.f / (float)p.M : (float)(1.0 / ((double)p.M * (double)p.M * (double)x.kv->head_dim));
   ProfScope ps(x.h, FC_K_PASS3, x.st);
-  fast::k_p3<R1B, CPW, PAD, A><<<dim3(p.N2, x.nu), CPW * R1B, sm, x.st>>>(
+  fast::k_p3<R1B, CPW, OUT, A><<<dim3(p.N2, x.nu), CPW * R1B, sm, x.st>>>(
       *x.lp, x.kv->num_heads, x.kv->head_dim, x.u0, x.cols, p.N, p.N2, x.nu * x.cols, x.ws, x.h->master, x.h->master_len,
-      score_stride, inv, accumulate, hi_base, eo);
+      score_stride, inv, accumulate, hi_base, eo, spec, x.tab);
   return fc_after_launch(x.h);
 }
 
@@ -1100,13 +1120,24 @@ fc_status run_p3(const PassArgs &x, long long score_stride, int accumulate, int 
   const PassPlan &p = *x.p;
 #define FC_P3(A_, R_, C_)                               \
   if (p.pad && p.a == A_ && p.r1b == R_ && p.cpw == C_) \
-    return launch_p3<A_, R_, C_, true>(x, score_stride, accumulate, hi_base, eo);
+    return launch_p3<A_, R_, C_, fast::OUT_PAD>(x, score_stride, accumulate, hi_base, eo);
   FC_OUTER_PAD_SHAPES(FC_P3)
 #undef FC_P3
 #define FC_P3(A_, R_, C_)                                \
   if (!p.pad && p.a == A_ && p.r1b == R_ && p.cpw == C_) \
-    return launch_p3<A_, R_, C_, false>(x, score_stride, accumulate, hi_base, eo);
+    return launch_p3<A_, R_, C_, fast::OUT_SCORE>(x, score_stride, accumulate, hi_base, eo);
   FC_OUTER_DIRECT_SHAPES(FC_P3)
+#undef FC_P3
+  return FC_ERR_INTERNAL;
+}
+
+// The N-point spectrum at the end of a chirp convolution (spectrum diagnostics).
+fc_status run_p3_spec(const PassArgs &x, float2 *spec) {
+  const PassPlan &p = *x.p;
+  static const fast::EnergyOut none = {};
+#define FC_P3(A_, R_, C_) \
+  if (p.a == A_ && p.r1b == R_ && p.cpw == C_) return launch_p3<A_, R_, C_, fast::OUT_SPEC>(x, 0, 0, 0, none, spec);
+  FC_OUTER_PAD_SHAPES(FC_P3)
 #undef FC_P3
   return FC_ERR_INTERNAL;
 }
@@ -1119,23 +1150,32 @@ inline int cutoff_index(double gamma, int N) {
   return (int)om;
 }
 
-// Filter tables of the padded form for every such sequence of the view, tabs[b].  A table depends on the length and the
-// cutoff only, so the handle keeps the last FC_TAB_SLOTS (the layers of a prefill share theirs).  While the stream is
-// being captured, and for lengths beyond the slots, tables go to the workspace, every call: a graph must not depend on
-// what the handle holds when it is replayed.
-fc_status prepare_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, double gamma, const ScoreLayout &L, char *wsb,
-                         const float4 **tabs) {
+// How the spectrum diagnostics transform a sequence: a power of two from 1024 to 65536 directly, a length that is not a
+// power of two by a chirp convolution of >= 2N - 1 points (plan.pad); 131072 points and powers of two below 1024, where
+// launches count and a chirp would add two of them, are left to the generic kernels.
+PassPlan plan_spectrum(int N) {
+  static const PassPlan none = {};
+  if (is_pow2(N) && N >= 16) return N >= 1024 && N <= 65536 ? plan_passes(N, 0) : none;
+  return plan_padded(N);
+}
+
+// Tables of the padded form (filter) or of the chirp (spectrum = true: its spectrum and per-row factors) for every such
+// sequence of the view, tabs[b].  A table depends on the length and the cutoff only, so the handle keeps the last
+// FC_TAB_SLOTS (the layers of a prefill share theirs).  While the stream is being captured, and for lengths beyond the
+// slots, tables go to the workspace (`spare`), every call: a graph must not depend on what the handle holds when it is
+// replayed.  `buf`: an intermediate buffer to build them in.
+fc_status prepare_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, double gamma, bool spectrum, float4 *spare,
+                         float2 *buf, const float4 **tabs) {
   bool cached = true, any = false, flushed = false;
   bool used[FC_TAB_SLOTS] = {};
-  auto key_of = [&](int b) {
-    const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
-    return (long long)N + ((long long)(cutoff_index(gamma, N) + 1) << 32);
-  };
+  auto plan_of = [&](int N) { return spectrum ? plan_spectrum(N) : plan_passes(N, kv->head_dim); };
+  auto omega_of = [&](int N) { return spectrum ? -1 : cutoff_index(gamma, N); };
+  auto key_of = [&](int N) { return (long long)N + ((long long)(omega_of(N) + 2) << 32); };
   for (int b = 0; b < kv->batch; ++b) {
     tabs[b] = nullptr;
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0) continue;
-    const PassPlan p = plan_passes(N, kv->head_dim);
+    const PassPlan p = plan_of(N);
     if (!p.ok || !p.pad) continue;
     if (!any) {
       any = true;
@@ -1145,14 +1185,13 @@ fc_status prepare_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, do
     }
     if (cached)
       for (int i = 0; i < FC_TAB_SLOTS; ++i)
-        if (h->tab_key[i] == key_of(b)) { tabs[b] = h->tab_cache + (size_t)i * h->tab_slot_len; used[i] = true; }
+        if (h->tab_key[i] == key_of(N)) { tabs[b] = h->tab_cache + (size_t)i * h->tab_slot_len; used[i] = true; }
   }
   if (!any) return FC_OK;
-  float4 *spare = reinterpret_cast<float4 *>(wsb + L.off_tab);
   for (int b = 0; b < kv->batch; ++b) {
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0 || tabs[b]) continue;
-    const PassPlan p = plan_passes(N, kv->head_dim);
+    const PassPlan p = plan_of(N);
     if (!p.ok || !p.pad) continue;
     if (!first_of_its_length(kv, b)) {
       for (int i = 0; i < b && !tabs[b]; ++i)
@@ -1171,7 +1210,7 @@ fc_status prepare_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, do
     }
     if (slot >= 0) {
       h->tab_next = (slot + 1) % FC_TAB_SLOTS;
-      h->tab_key[slot] = 0;                                  // not valid until both launches are in the stream
+      h->tab_key[slot] = 0;                                  // not valid until its launches are in the stream
       used[slot] = true;
       dst = h->tab_cache + (size_t)slot * h->tab_slot_len;
     } else {
@@ -1179,18 +1218,16 @@ fc_status prepare_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, do
       spare += p.M;
     }
     if (p.small) {
-      small::k_small_table<<<(p.M + 63) / 64, 64, (N + 1) * sizeof(float), st>>>(dst, N, cutoff_index(gamma, N), p.M, h->master,
+      small::k_small_table<<<(p.M + 63) / 64, 64, (N + 1) * sizeof(float), st>>>(dst, N, omega_of(N), p.M, h->master,
                                                                                 h->master_len);
       if ((s = fc_after_launch(h)) != FC_OK) return s;
-      if (slot >= 0) h->tab_key[slot] = key_of(b);
-      tabs[b] = dst;
-      continue;
+    } else {
+      static const fast::LayerPtrs none = {};
+      const PassArgs x{h, st, &p, &none, kv, 0, 1, 0, 2 * p.cpw, omega_of(N), buf, nullptr};
+      if ((s = run_p1_table(x)) != FC_OK) return s;
+      if ((s = run_p2(x, 2 * p.cpw, spectrum ? fast::MODE_MUL : fast::MODE_PAD, dst)) != FC_OK) return s;
     }
-    static const fast::LayerPtrs none = {};
-    const PassArgs x{h, st, &p, &none, kv, 0, 1, 0, 2 * p.cpw, cutoff_index(gamma, N), reinterpret_cast<float2 *>(wsb + L.off_buf), nullptr};
-    if ((s = run_p1_table(x)) != FC_OK) return s;
-    if ((s = run_p2(x, 2 * p.cpw, dst)) != FC_OK) return s;
-    if (slot >= 0) h->tab_key[slot] = key_of(b);
+    if (slot >= 0) h->tab_key[slot] = key_of(N);
     tabs[b] = dst;
   }
   return FC_OK;
@@ -1252,7 +1289,7 @@ fc_status score_sequence(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, co
     for (int cg = 0; cg < g.ngr; ++cg) {                      // column groups of one unit, in stream order
       x.c0 = cg * g.sub;
       if ((s = run_p1<T>(x, part_tot, eo.tot_slots)) != FC_OK) return s;
-      if ((s = run_p2(x, nu * g.sub, nullptr)) != FC_OK) return s;
+      if ((s = run_p2(x, nu * g.sub, p.pad ? fast::MODE_PAD : fast::MODE_FILTER)) != FC_OK) return s;
       if ((s = run_p3(x, total_tokens, cg > 0 ? 1 : 0, cg * H * p.N2, eo)) != FC_OK) return s;
     }
   }
@@ -1457,7 +1494,8 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
     any_passes = any_passes || (plans[b].ok && !plans[b].small);
     if (!plans[b].ok || (plans[b].pad && !plans[b].small)) direct_only = false;
   }
-  if (any_fast && (s = prepare_tables(h, st, kv, gamma, L, wsb, tabs.data())) != FC_OK) return s;
+  if (any_fast && (s = prepare_tables(h, st, kv, gamma, false, reinterpret_cast<float4 *>(wsb + L.off_tab),
+                                      reinterpret_cast<float2 *>(wsb + L.off_buf), tabs.data())) != FC_OK) return s;
   // a call that carves the workspace differently: nothing of the previous call may be in flight on the other streams
   const size_t sig = reinterpret_cast<size_t>(wsb) ^ (L.buf_bytes << 20) ^ (L.tot_bytes << 8) ^ L.hi_bytes ^ (L.off_tot << 12);
   if (any_small && sig != h->last_sig && (s = fc_flush_pending(h, st)) != FC_OK) return s;
@@ -1530,71 +1568,147 @@ constexpr int kPowerNY = 16;
 
 size_t power_partial_bytes(int N) { return align_up((size_t)kPowerNY * N * sizeof(float2), 256); }
 
-// Power spectrum of one sequence (Eq. 11) into spectrum[2*m .. 2*m+1], m < N.  Generic kernels, caller's stream.
+// Power spectrum of one sequence (Eq. 11) into spectrum[2*m .. 2*m+1], m < N, on the generic kernels (the power of two
+// 131072) and the caller's stream.
 template <typename T>
-fc_status power_sequence(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, int b, double *spectrum, char *wsb) {
+fc_status power_generic(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, int b, double *spectrum, char *wsb) {
   const int start = kv->cu_seqlens[b];
   const int N = kv->cu_seqlens[b + 1] - start;
-  if (N == 0) return FC_OK;
   const int d = kv->head_dim, H = kv->num_heads;
   const SeqPlan sp = plan_sequence(N);
   const GenericLayout L = generic_layout(h, sp, H, d);
   float2 *ws = reinterpret_cast<float2 *>(wsb + L.off_ws);
-  float2 *spec = reinterpret_cast<float2 *>(wsb + L.off_spec);
-  float2 *hhat = reinterpret_cast<float2 *>(wsb + L.off_hhat);
-  float2 *hcol = reinterpret_cast<float2 *>(wsb + L.off_hcol);
   float2 *partial = reinterpret_cast<float2 *>(wsb + L.total);
   double *out = spectrum + 2 * (size_t)start;
   const T *kp = static_cast<const T *>(kv->k) + (long long)start * kv->stride_token;
   const T *vp = static_cast<const T *>(kv->v) + (long long)start * kv->stride_token;
-  const FftPlan p1 = make_plan(sp.N1);
   fc_status s;
-  if (sp.bluestein) {
-    ChirpKernelLoader cl{N, sp.Nfft};
-    if ((s = launch_pass1(h, st, cl, sp, 8, 8, hcol, nullptr)) != FC_OK) return s;
-    if ((s = launch_pass2<MID_SPEC>(h, st, sp, 8, 8, hcol, 0, hhat, 1.f)) != FC_OK) return s;
-  }
-  bool first = true;
   for (int h0 = 0; h0 < H; h0 += L.heads_per_group) {
     const int hg = (H - h0 < L.heads_per_group) ? H - h0 : L.heads_per_group;
     const int ncol_ws = hg * d;
-    if (!sp.bluestein) {
-      KvLoader<T, false> ld{kp, vp, kv->stride_token, kv->stride_head, h0, d, N, 0.f, 0.f};
-      if ((s = launch_pass1(h, st, ld, sp, ncol_ws, sp.cs, ws, nullptr)) != FC_OK) return s;
-      const FftPlan p2 = make_plan(sp.N2);
-      const size_t sm = smem_pass2(sp, sp.cs2) + (size_t)sp.N2 * 2 * sizeof(float2);
-      if ((s = set_smem(k_pass2_power, sm)) != FC_OK) return s;
-      const int slices = ncol_ws / sp.cs2, ny = slices < kPowerNY ? slices : kPowerNY;
-      k_pass2_power<<<dim3(sp.N1 / 2 + 1, ny), kThreads, sm, st>>>(p2, sp.N1, ncol_ws, ilog2(sp.cs2), ws, h->master,
-                                                                   h->master_len, partial);
-      if ((s = fc_after_launch(h)) != FC_OK) return s;
-      k_power_accumulate<<<(N + 255) / 256, 256, 0, st>>>(partial, ny, N, out, first ? 1 : 0);
-      if ((s = fc_after_launch(h)) != FC_OK) return s;
-      first = false;
+    KvLoader<T, false> ld{kp, vp, kv->stride_token, kv->stride_head, h0, d, N, 0.f, 0.f};
+    if ((s = launch_pass1(h, st, ld, sp, ncol_ws, sp.cs, ws, nullptr)) != FC_OK) return s;
+    const FftPlan p2 = make_plan(sp.N2);
+    const size_t sm = smem_pass2(sp, sp.cs2) + (size_t)sp.N2 * 2 * sizeof(float2);
+    if ((s = set_smem(k_pass2_power, sm)) != FC_OK) return s;
+    const int slices = ncol_ws / sp.cs2, ny = slices < kPowerNY ? slices : kPowerNY;
+    k_pass2_power<<<dim3(sp.N1 / 2 + 1, ny), kThreads, sm, st>>>(p2, sp.N1, ncol_ws, ilog2(sp.cs2), ws, h->master,
+                                                                 h->master_len, partial);
+    if ((s = fc_after_launch(h)) != FC_OK) return s;
+    k_power_accumulate<<<(N + 255) / 256, 256, 0, st>>>(partial, ny, N, 1, out, h0 == 0 ? 1 : 0);
+    if ((s = fc_after_launch(h)) != FC_OK) return s;
+  }
+  return FC_OK;
+}
+
+// Workspace of one fc_power_spectrum call: per internal stream an intermediate buffer and (chirp convolutions) an N-point
+// spectrum, tables, and every sequence's partial sums.
+struct PowerLayout {
+  size_t buf_bytes, spec_bytes, off_spec, off_tab, off_part, total;
+};
+
+// Rows of partial sums of one sequence, at most: a 2*cp-channel slice each (direct), or a launch each (chirp).
+inline int power_rows(const PassPlan &p, const GroupPlan &g, int H, int d) { return p.pad ? H * g.ngr : H * d / (2 * p.cp); }
+
+PowerLayout power_layout(const fc_handle *h, const fc_kv_view *kv) {
+  PowerLayout L = {};
+  const int H = kv->num_heads, d = kv->head_dim;
+  size_t tab = 0, part = 0, generic = 256;
+  for (int b = 0; b < kv->batch; ++b) {
+    const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
+    if (N == 0) continue;
+    const PassPlan p = plan_spectrum(N);
+    if (!p.ok) {
+      const size_t t = generic_layout(h, plan_sequence(N), H, d).total + power_partial_bytes(N);
+      if (t > generic) generic = t;
       continue;
     }
-    const float invM = 1.f / (float)sp.Nfft;
-    const int sub = L.sub_cols, cs = (sub % 64 == 0) ? sp.cs : 32;
-    const int ngroups = (hg == 1) ? d / sub : 1;
-    const int ncol = (hg == 1) ? sub : ncol_ws;
-    int cs2 = 2 * sp.cs2 > 64 ? 64 : 2 * sp.cs2;
-    while (ncol % cs2) cs2 >>= 1;
-    const size_t sm3c = smem_pass13(sp, cs);
-    for (int cg = 0; cg < ngroups; ++cg) {
-      const int dd = (hg == 1) ? sub : d;
-      KvLoader<T, true> ld{kp + cg * sub, vp + cg * sub, kv->stride_token, kv->stride_head, h0, dd, N, 0.f, 0.f};
-      if ((s = launch_pass1(h, st, ld, sp, ncol, cs, ws, nullptr)) != FC_OK) return s;
-      if ((s = launch_pass2<MID_MULH>(h, st, sp, ncol, cs2, ws, 0, hhat, invM)) != FC_OK) return s;
-      if ((s = set_smem(k_pass3<EPI_SPEC, true>, sm3c)) != FC_OK) return s;
-      k_pass3<EPI_SPEC, true><<<dim3(sp.N2, ncol / cs), kThreads, sm3c, st>>>(
-          p1, sp.N2, N, ncol, ilog2(cs), ws, h->master, h->master_len, spec, nullptr, 0, dd, 0, 0.f, nullptr, 0.f, 0);
-      if ((s = fc_after_launch(h)) != FC_OK) return s;
-      k_spec_power<<<N / 2 + 1, kThreads, 0, st>>>(spec, ncol, N, partial);
-      if ((s = fc_after_launch(h)) != FC_OK) return s;
-      k_power_accumulate<<<(N + 255) / 256, 256, 0, st>>>(partial, 1, N, out, first ? 1 : 0);
-      if ((s = fc_after_launch(h)) != FC_OK) return s;
-      first = false;
+    const GroupPlan g = plan_groups(h, p, H, H, d);
+    if (g.buf_bytes > L.buf_bytes) L.buf_bytes = g.buf_bytes;
+    if (p.pad) {
+      const size_t sb = align_up(g.buf_bytes / p.M * N, 256);
+      if (sb > L.spec_bytes) L.spec_bytes = sb;
+      if (first_of_its_length(kv, b)) tab += (size_t)p.M * sizeof(float4);
     }
+    part += align_up((size_t)power_rows(p, g, H, d) * N * sizeof(float2), 256);
+  }
+  L.off_spec = L.buf_bytes * h->num_aux;
+  L.off_tab = L.off_spec + L.spec_bytes * h->num_aux;
+  L.off_part = L.off_tab + align_up(tab, 256);
+  L.total = L.off_part + part;
+  if (generic > L.total) L.total = generic;
+  return L;
+}
+
+// Power spectra of all sequences of a layer.  Launches alternate over the internal streams; each writes partial sums of
+// its own, which are added in a fixed order once all streams have joined (4 layers of 32768 + 10000 tokens, 4 heads,
+// cutoffs included: 3.59 ms on the generic kernels and one stream, 1.06 ms now).
+template <typename T>
+fc_status power_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, double *spectrum, char *wsb) {
+  const int B = kv->batch, H = kv->num_heads, d = kv->head_dim;
+  const PowerLayout L = power_layout(h, kv);
+  std::vector<const float4 *> tabs(B, nullptr);
+  std::vector<int> ny(B, 0);
+  fc_status s = FC_OK;
+  bool passes = false;
+  for (int b = 0; b < B; ++b) {
+    const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
+    if (N == 0) continue;
+    if (plan_spectrum(N).ok) passes = true;
+    else if ((s = power_generic<T>(h, st, kv, b, spectrum, wsb)) != FC_OK) return s;
+  }
+  if (!passes) return FC_OK;
+  if ((s = prepare_tables(h, st, kv, 0.0, true, reinterpret_cast<float4 *>(wsb + L.off_tab), reinterpret_cast<float2 *>(wsb),
+                          tabs.data())) != FC_OK)
+    return s;
+  if ((s = fork_streams(h, st)) != FC_OK) return s;
+  size_t part = L.off_part;
+  unsigned turn = 0;
+  for (int b = 0; b < B; ++b) {
+    const int start = kv->cu_seqlens[b], N = kv->cu_seqlens[b + 1] - start;
+    if (N == 0) continue;
+    const PassPlan p = plan_spectrum(N);
+    if (!p.ok) continue;
+    const GroupPlan g = plan_groups(h, p, H, H, d);
+    fast::LayerPtrs lp = {};
+    lp.k[0] = static_cast<const T *>(kv->k) + (long long)start * kv->stride_token;
+    lp.v[0] = static_cast<const T *>(kv->v) + (long long)start * kv->stride_token;
+    float2 *rows = reinterpret_cast<float2 *>(wsb + part);
+    for (int u0 = 0; u0 < H; u0 += g.units)
+      for (int cg = 0; cg < g.ngr; ++cg, ++turn) {
+        const int nu = H - u0 < g.units ? H - u0 : g.units, si = (int)(turn % (unsigned)h->num_aux), ncol = nu * g.sub;
+        PassArgs x{h, h->aux[si], &p, &lp, kv, u0, nu, cg * g.sub, g.sub, 0,
+                   reinterpret_cast<float2 *>(wsb + (size_t)si * L.buf_bytes), tabs[b]};
+        if (p.pad) {
+          float2 *spec = reinterpret_cast<float2 *>(wsb + L.off_spec + (size_t)si * L.spec_bytes);
+          if ((s = run_p1_chirp<T>(x)) != FC_OK) return s;
+          if ((s = run_p2(x, ncol, fast::MODE_MUL)) != FC_OK) return s;
+          if ((s = run_p3_spec(x, spec)) != FC_OK) return s;
+          k_spec_power<<<N / 2 + 1, kThreads, 0, x.st>>>(spec, ncol, N, rows);
+          if ((s = fc_after_launch(h)) != FC_OK) return s;
+          rows += N;
+          ++ny[b];
+        } else {
+          if ((s = run_p1<T>(x, nullptr, 0)) != FC_OK) return s;
+          if ((s = run_p2(x, ncol, fast::MODE_POWER, nullptr, rows)) != FC_OK) return s;
+          rows += (size_t)(ncol / (2 * p.cp)) * N;
+          ny[b] += ncol / (2 * p.cp);
+        }
+      }
+    part += align_up((size_t)power_rows(p, g, H, d) * N * sizeof(float2), 256);
+  }
+  h->pending_join = true;
+  if ((s = fc_flush_pending(h, st)) != FC_OK) return s;
+  part = L.off_part;
+  for (int b = 0; b < B; ++b) {
+    const int start = kv->cu_seqlens[b], N = kv->cu_seqlens[b + 1] - start;
+    if (N == 0) continue;
+    const PassPlan p = plan_spectrum(N);
+    if (!p.ok) continue;
+    k_power_accumulate<<<(N + 255) / 256, 256, 0, st>>>(reinterpret_cast<float2 *>(wsb + part), ny[b], N, p.pad ? 1 : p.N1,
+                                                        spectrum + 2 * (size_t)start, 1);
+    if ((s = fc_after_launch(h)) != FC_OK) return s;
+    part += align_up((size_t)power_rows(p, plan_groups(h, p, H, H, d), H, d) * N * sizeof(float2), 256);
   }
   return FC_OK;
 }
@@ -1686,14 +1800,7 @@ extern "C" fc_status fc_score_layer(fc_handle *h, const fc_kv_view *kv, double g
 
 extern "C" size_t fc_power_spectrum_workspace_bytes(const fc_handle *h, const fc_kv_view *kv) {
   if (validate_view(h, kv, true) != FC_OK) return 0;
-  size_t need = 256;
-  for (int b = 0; b < kv->batch; ++b) {
-    const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
-    if (N == 0) continue;
-    const size_t t = generic_layout(h, plan_sequence(N), kv->num_heads, kv->head_dim).total + power_partial_bytes(N);
-    if (t > need) need = t;
-  }
-  return need;
+  return power_layout(h, kv).total;
 }
 
 extern "C" fc_status fc_power_spectrum(fc_handle *h, const fc_kv_view *kv, double *spectrum, void *workspace,
@@ -1708,79 +1815,109 @@ extern "C" fc_status fc_power_spectrum(fc_handle *h, const fc_kv_view *kv, doubl
   if (dev != h->device) FC_CUDA_TRY(cudaSetDevice(h->device));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if ((s = fc_flush_pending(h, st)) != FC_OK) return s;     // the workspace may still be in use on the internal streams
-  for (int b = 0; b < kv->batch && s == FC_OK; ++b) {
-    switch (kv->dtype) {
-      case FC_F32: s = power_sequence<float>(h, st, kv, b, spectrum, (char *)workspace); break;
-      case FC_F16: s = power_sequence<__half>(h, st, kv, b, spectrum, (char *)workspace); break;
-      default: s = power_sequence<__nv_bfloat16>(h, st, kv, b, spectrum, (char *)workspace); break;
-    }
+  switch (kv->dtype) {
+    case FC_F32: return power_call<float>(h, st, kv, spectrum, (char *)workspace);
+    case FC_F16: return power_call<__half>(h, st, kv, spectrum, (char *)workspace);
+    default: return power_call<__nv_bfloat16>(h, st, kv, spectrum, (char *)workspace);
   }
-  return s;
 }
 
 // ---------------------------------------------------------------------------
 // fc_cutoff_from_spectrum: the smallest omega whose kept band holds a given share of the energy.
-// One block per sequence; thread t adds up a contiguous run of bins, a block scan of the run totals in
-// fp64 finds the run in which the running sum first reaches share * total, and the thread that owns the
-// run walks it.  Sums are taken in a fixed order (deterministic).
+// Bound by reading the spectrum once, so a cluster of 8 blocks shares a sequence: each of its 128 warps sums a contiguous
+// segment of bins with coalesced loads, the segment totals meet in the first block's shared memory, and its first warp
+// finds the segment in which the running sum first reaches share * total and walks that one (32768 + 10000 bins: 37.7 us
+// with one block per sequence and a run of bins per thread, 4.2 us now).  Sums are fp64 in a fixed order (deterministic).
 // ---------------------------------------------------------------------------
 namespace {
 
-constexpr int kCutThreads = 1024;
+constexpr int kCutThreads = 512, kCutCluster = 8, kCutSegs = kCutCluster * kCutThreads / 32;
 struct CutTable { int start[65]; };
 
-__global__ void __launch_bounds__(kCutThreads)
+__device__ __forceinline__ double warp_inclusive(double v, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double t = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += t;
+  }
+  return v;
+}
+
+__global__ void __cluster_dims__(kCutCluster, 1, 1) __launch_bounds__(kCutThreads)
 k_cutoff_from_spectrum(const double *__restrict__ spectrum, const __grid_constant__ CutTable st, int b0, double share,
                        int *__restrict__ omega, double *__restrict__ gamma) {
-  __shared__ double run[kCutThreads];
-  __shared__ double s_total;
-  const int tid = threadIdx.x;
-  const int s0 = st.start[blockIdx.x], N = st.start[blockIdx.x + 1] - s0;
-  const int b = b0 + blockIdx.x;
-  if (N == 0) {
-    if (tid == 0) { omega[b] = 0; gamma[b] = 0.0; }
+  __shared__ double seg_sum[kCutSegs];
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int lane = threadIdx.x & 31, rank = (int)cluster.block_rank();
+  const int seq = blockIdx.x / kCutCluster;
+  const int s0 = st.start[seq], N = st.start[seq + 1] - s0;
+  const int b = b0 + seq;
+  if (N == 0) {                                       // the same for the whole cluster
+    if (rank == 0 && threadIdx.x == 0) { omega[b] = 0; gamma[b] = 0.0; }
     return;
   }
-  const int per = (N + kCutThreads - 1) / kCutThreads;
-  const int lo = tid * per, hi = lo + per < N ? lo + per : N;
   const double *P = spectrum + 2 * (size_t)s0;
-  double mine = 0.0;
-  for (int m = lo; m < hi; ++m) mine += P[2 * m] + P[2 * m + 1];
-  run[tid] = mine;
-  __syncthreads();
-  // inclusive scan of the run totals (Hillis-Steele, fp64)
-  for (int o = 1; o < kCutThreads; o <<= 1) {
-    const double add = tid >= o ? run[tid - o] : 0.0;
-    __syncthreads();
-    run[tid] += add;
-    __syncthreads();
+  const int len = ((N + kCutSegs - 1) / kCutSegs + 31) & ~31;       // bins per segment
+  {
+    const int sg = rank * (kCutThreads / 32) + (threadIdx.x >> 5);
+    const int lo = sg * len, hi = lo + len < N ? lo + len : N;
+    double a = 0.0;
+#pragma unroll 8
+    for (int m = lo + lane; m < hi; m += 32) a += P[2 * m] + P[2 * m + 1];
+    a = warp_sum_d(a);
+    if (lane == 0) *cluster.map_shared_rank(&seg_sum[sg], 0) = a;
   }
-  if (tid == kCutThreads - 1) s_total = run[tid];
-  __syncthreads();
-  const double total = s_total, want = share * total;
+  cluster.sync();
+  if (rank != 0 || threadIdx.x >= 32) return;
+  constexpr int PER = kCutSegs / 32;
+  double run[PER], acc = 0.0;
+#pragma unroll
+  for (int i = 0; i < PER; ++i) { acc += seg_sum[lane * PER + i]; run[i] = acc; }
+  const double incl = warp_inclusive(acc, lane);
+  double before = __shfl_up_sync(0xffffffffu, incl, 1);
+  if (lane == 0) before = 0.0;
+  const double total = __shfl_sync(0xffffffffu, incl, 31), want = share * total;
   if (!(total > 0.0)) {
-    if (tid == 0) { omega[b] = 0; gamma[b] = 0.5 / (double)N; }
+    if (lane == 0) { omega[b] = 0; gamma[b] = 0.5 / (double)N; }
     return;
   }
-  // the run that holds the crossing: the first non-empty one whose running sum has reached `want` (the
-  // scan's sums of one and the same set can differ in the last bit, so "the last run reaches the total"
-  // is not relied on: without a qualifying run the last non-empty one is taken)
-  __shared__ int s_owner;
-  if (tid == 0) s_owner = kCutThreads;
-  __syncthreads();
-  if (lo < hi && run[tid] >= want) atomicMin(&s_owner, tid);
-  __syncthreads();
-  const int owner = s_owner < kCutThreads ? s_owner : (N - 1) / per;
-  if (tid == owner) {
-    double acc = run[tid] - mine;
-    int m = lo;
-    for (; m < hi; ++m) {
-      acc += P[2 * m] + P[2 * m + 1];
-      if (acc >= want) break;
+  // the segment that holds the crossing: the first non-empty one whose running sum has reached `want` (sums of one and
+  // the same set can differ in the last bit, so "the last one reaches the total" is not relied on: without a qualifying
+  // one the last non-empty one is taken)
+  const int last = (N - 1) / len;
+  int mine = kCutSegs;
+#pragma unroll
+  for (int i = PER - 1; i >= 0; --i)
+    if (before + run[i] >= want) mine = lane * PER + i;
+  const int first = __reduce_min_sync(0xffffffffu, mine);
+  const int owner = first < last ? first : last;
+  double base = before;
+#pragma unroll
+  for (int i = 1; i < PER; ++i)
+    if (owner % PER == i) base = before + run[i - 1];
+  base = __shfl_sync(0xffffffffu, base, owner / PER);
+  const int lo = owner * len, hi = lo + len < N ? lo + len : N;
+  int found = hi - 1;
+  for (int m0 = lo; m0 < hi && found == hi - 1; m0 += 8 * 32) {
+    double v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int m = m0 + 32 * i + lane;
+      const int at = 2 * (m < hi ? m : lo);
+      v[i] = m < hi ? P[at] + P[at + 1] : 0.0;
     }
-    if (m >= hi) m = hi - 1;
-    omega[b] = m;
-    gamma[b] = ((double)m + 0.5) / (double)N;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const double sum = base + warp_inclusive(v[i], lane);
+      const int m = m0 + 32 * i + lane;
+      const unsigned hit = __ballot_sync(0xffffffffu, m < hi && sum >= want);
+      if (hit && found == hi - 1) found = m0 + 32 * i + __ffs(hit) - 1;
+      base = __shfl_sync(0xffffffffu, sum, 31);
+    }
+  }
+  if (lane == 0) {
+    omega[b] = found;
+    gamma[b] = ((double)found + 0.5) / (double)N;
   }
 }
 
@@ -1802,7 +1939,7 @@ extern "C" fc_status fc_cutoff_from_spectrum(fc_handle *h, const double *spectru
     const int nseq = batch - b0 < 64 ? batch - b0 : 64;
     CutTable tab;
     for (int i = 0; i <= nseq; ++i) tab.start[i] = cu_seqlens[b0 + i];
-    k_cutoff_from_spectrum<<<nseq, kCutThreads, 0, st>>>(spectrum, tab, b0, share, omega, gamma);
+    k_cutoff_from_spectrum<<<nseq * kCutCluster, kCutThreads, 0, st>>>(spectrum, tab, b0, share, omega, gamma);
     if ((s = fc_after_launch(h)) != FC_OK) return s;
   }
   return FC_OK;

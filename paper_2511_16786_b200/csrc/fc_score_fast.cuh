@@ -76,10 +76,34 @@ __device__ __forceinline__ float base_kernel(int t, int N, int omega) {
   return (float)(sinpi((double)r / (2.0 * (double)N)) / (2.0 * (double)N * sinpi((double)t / (2.0 * (double)N))));
 }
 
+// exp(+j*pi*n*n/N); n*n is reduced modulo 2N (one period) in integers first.
+__device__ __forceinline__ float2 chirp(int n, int N) {
+  const unsigned long long r = ((unsigned long long)n * (unsigned long long)n) % (2ull * (unsigned long long)N);
+  float s, c;
+  sincospif(__fdiv_rn((float)(unsigned)r, (float)N), &s, &c);
+  return make_float2(c, s);
+}
+
+// (|C_k[q]|^2, |C_v[q]|^2) of Eq. 11 from P = Z[q], Q = Z[N-q] of the packed sequence K + jV in the DCT's order and
+// t = exp(-j*pi*q/(2N)): C[q] = alpha[q] Re(t Y[q]) with Y_k = (P + conj Q)/2, Y_v = (P - conj Q)/(2j) (alpha of Eq. 7).
+__device__ __forceinline__ float2 power_of_bin(float2 P, float2 Q, float2 t, float alpha2) {
+  const float ck = 0.5f * ((P.x + Q.x) * t.x - (P.y - Q.y) * t.y);
+  const float cv = 0.5f * ((P.y + Q.y) * t.x - (Q.x - P.x) * t.y);
+  return make_float2(alpha2 * ck * ck, alpha2 * cv * cv);
+}
+
 // What pass 1 transforms: the rows of a sequence whose length is the transform's (LD_KV), the rows of a shorter one
 // with zeros behind (LD_PAD: at most half of the transform, so half of every first-stage butterfly), or the two
 // convolution kernels of the padded form in the columns 0 and 1 (LD_TABLE).
-enum { LD_KV = 0, LD_PAD = 1, LD_TABLE = 2 };
+// The spectrum diagnostics need the N-point spectrum itself: for lengths that are not a power of two LD_CHIRP and the
+// modes MODE_MUL and OUT_SPEC compute it by one chirp convolution (rows in the DCT's even/odd order times the conjugate
+// chirp, product with the chirp's spectrum, outputs times the conjugate chirp).
+enum { LD_KV = 0, LD_PAD = 1, LD_TABLE = 2, LD_CHIRP = 3 };
+// What pass 2 does between its halves: the residual filter of the direct form, of the padded form, a product with a
+// spectrum (rows are independent), or nothing but the sums of the power spectrum (direct form, no way back).
+enum { MODE_FILTER = 0, MODE_PAD = 1, MODE_MUL = 2, MODE_POWER = 3 };
+// What pass 3 does with its rows: scores of the direct and of the padded form, or the N-point spectrum.
+enum { OUT_SCORE = 0, OUT_PAD = 1, OUT_SPEC = 2 };
 
 // x[p] *= w^p (CONJ: conj(w)^p), p = 1..15, for both channels, from w and w^4 alone: the other powers are products of
 // at most three table values (w^p = w^(4g) * w^r), which replaces 13 of 15 shared-memory reads per use by arithmetic.
@@ -136,7 +160,7 @@ template <typename T, int R1B, int CPW, int LD = LD_KV, int A = 16>
 __global__ void __launch_bounds__(CPW * R1B, (768 / (CPW * R1B)) > 0 ? 768 / (CPW * R1B) : 1)
 k_p1(const __grid_constant__ LayerPtrs lp, long long stride_token, long long stride_head, int H, int head_dim, int u0,
      int c0, int dcols, int N, int N2, int ncol_ws, float2 *__restrict__ ws, const float2 *__restrict__ master,
-     int master_len, double *__restrict__ partial, int layer_slots, int omega = 0) {
+     int master_len, double *__restrict__ partial, int layer_slots, int omega = 0, const float4 *__restrict__ tab = nullptr) {
   constexpr int N1 = A * R1B, NT = CPW * R1B, IT = (A + R1B - 1) / R1B, NW = (NT + 31) / 32;
   extern __shared__ float4 smem4[];
   float4 *S = smem4;                                        // [N1][CPW]
@@ -152,13 +176,16 @@ k_p1(const __grid_constant__ LayerPtrs lp, long long stride_token, long long str
     for (int p = 0; p < A; ++p) {
       // columns 0 and 1; this thread's values come back from shared memory, where the loop can stay rolled
       const int n = (j + R1B * p) * N2 + n2, M = N1 * N2;
-      float g0 = 0.f, g1 = 0.f;
-      if (cp == 0 && gc0 == 0) {
+      float g0 = 0.f, g1 = 0.f, gi = 0.f;
+      if (cp == 0 && gc0 == 0 && omega < 0) {             // the chirp, wrapped, in column 0
+        const int a = n < N ? n : n > M - N ? M - n : -1;
+        if (a >= 0) { const float2 c = chirp(a, N); g0 = c.x; gi = c.y; }
+      } else if (cp == 0 && gc0 == 0) {
         if (n < N) g0 = base_kernel(n, N, omega);
         else if (n > M - N) g0 = base_kernel(M - n, N, omega);
         if (n <= 2 * N - 2) g1 = base_kernel(n + 1, N, omega);
       }
-      S[(j + R1B * p) * CPW + cp] = make_float4(g0, 0.f, g1, 0.f);
+      S[(j + R1B * p) * CPW + cp] = make_float4(g0, gi, g1, 0.f);
     }
 #pragma unroll
     for (int p = 0; p < A; ++p) {
@@ -172,13 +199,13 @@ k_p1(const __grid_constant__ LayerPtrs lp, long long stride_token, long long str
     slot = layer * layer_slots + (head * (head_dim / (2 * CPW)) + ch / (2 * CPW)) * gridDim.x + n2;
     const T *kb = static_cast<const T *>(lp.k[layer]) + (long long)head * stride_head + ch + 2 * cp;
     const T *vb = static_cast<const T *>(lp.v[layer]) + (long long)head * stride_head + ch + 2 * cp;
-    if (LD == LD_PAD) {
+    if (LD == LD_PAD || LD == LD_CHIRP) {
       // rows past the sequence read row 0 and are zeroed
       float2 z0[A / 2], z1[A / 2];
 #pragma unroll
       for (int p = 0; p < A / 2; ++p) {
         const int n = (j + R1B * p) * N2 + n2;
-        const long long off = (long long)(n < N ? n : 0) * stride_token;
+        const long long off = (long long)(n < N ? (LD == LD_CHIRP ? perm_token(n, N) : n) : 0) * stride_token;
         const float2 kk = Load2<T>::ld(kb + off), vv = Load2<T>::ld(vb + off);
         z0[p] = n < N ? make_float2(kk.x, vv.x) : make_float2(0.f, 0.f);
         z1[p] = n < N ? make_float2(kk.y, vv.y) : make_float2(0.f, 0.f);
@@ -189,6 +216,15 @@ k_p1(const __grid_constant__ LayerPtrs lp, long long stride_token, long long str
       for (int p = 0; p < A / 2; ++p) {
         accK = fmaf(z0[p].x, z0[p].x, fmaf(z1[p].x, z1[p].x, accK));
         accV = fmaf(z0[p].y, z0[p].y, fmaf(z1[p].y, z1[p].y, accV));
+      }
+      if (LD == LD_CHIRP) {
+#pragma unroll
+        for (int p = 0; p < A / 2; ++p) {
+          const int n = (j + R1B * p) * N2 + n2;
+          const float4 t = __ldg(tab + (n < N ? n : 0));
+          z0[p] = cmul_conj(z0[p], make_float2(t.z, t.w));
+          z1[p] = cmul_conj(z1[p], make_float2(t.z, t.w));
+        }
       }
       dft_zero_tail<A>(z0, x0);
       dft_zero_tail<A>(z1, x1);
@@ -203,7 +239,7 @@ k_p1(const __grid_constant__ LayerPtrs lp, long long stride_token, long long str
       }
     }
   }
-  if (LD != LD_PAD) {
+  if (LD != LD_PAD && LD != LD_CHIRP) {
     for (int i = tid; i < N1; i += NT) tw[i] = (A == 16) ? master[(size_t)i * (master_len / N1)] : root_of_unity(i, N1);
     __syncthreads();
     if (LD == LD_KV) {
@@ -247,7 +283,7 @@ k_p1(const __grid_constant__ LayerPtrs lp, long long stride_token, long long str
       dst += (size_t)A * N2 * ncol_ws / 2;
     }
   }
-  if (LD == LD_TABLE) return;
+  if (LD == LD_TABLE || LD == LD_CHIRP || partial == nullptr) return;
   // per-block sums of squares (total energy of Eq. 12, by Parseval)
   const double a = warp_sum_d((double)accK), b = warp_sum_d((double)accV);
   if ((tid & 31) == 0) { red[0][tid >> 5] = a; red[1][tid >> 5] = b; }
@@ -271,10 +307,11 @@ k_p1(const __grid_constant__ LayerPtrs lp, long long stride_token, long long str
 // tab_out (padded form): forward half only, of the convolution kernels in the columns 0 and 1; the table entries of
 // this block's bins are written instead.  Tables are laid out [k1][k2].
 // ---------------------------------------------------------------------------
-template <int R2B, int CP, bool PAD = false>
+template <int R2B, int CP, int MODE = MODE_FILTER>
 __global__ void __launch_bounds__(2 * CP * R2B, 512 / (2 * CP * R2B > 32 ? 2 * CP * R2B : 32))
 k_p2(int N1, int ncol_ws, float2 *__restrict__ ws, const float2 *__restrict__ master, int master_len, int omega,
-     const float4 *__restrict__ tab = nullptr, float4 *__restrict__ tab_out = nullptr) {
+     const float4 *__restrict__ tab, float4 *__restrict__ tab_out, float2 *__restrict__ power, int Nseq) {
+  constexpr bool TAB = MODE == MODE_PAD || MODE == MODE_MUL;
   constexpr int N2 = 16 * R2B, NT = 2 * CP * R2B, IT = 16 / R2B;
   extern __shared__ float4 smem4[];
   float4 *S = smem4;                                         // [2][N2][CP]
@@ -300,14 +337,15 @@ k_p2(int N1, int ncol_ws, float2 *__restrict__ ws, const float2 *__restrict__ ma
   {
     const int ustep = master_len / (2 * N);
     for (int i = tid; i < N2; i += NT) {
-      if (PAD) {
+      if (TAB) {
         if (tab_out == nullptr) {
           hc[i] = __ldg(tab + (size_t)k1a * N2 + i);
           hc[N2 + i] = __ldg(tab + (size_t)k1b * N2 + i);
         }
       } else {
-        uT[i] = master[(size_t)(k1a + N1 * i) * ustep];
-        uT[H2 + i] = master[(size_t)(k1b + N1 * i) * ustep];
+        // exp(-j*pi*q/N) of the filter, exp(-j*pi*q/(2N)) of the power spectrum
+        uT[i] = master[(size_t)(k1a + N1 * i) * (MODE == MODE_POWER ? ustep / 2 : ustep)];
+        uT[H2 + i] = master[(size_t)(k1b + N1 * i) * (MODE == MODE_POWER ? ustep / 2 : ustep)];
       }
     }
     for (int i = tid; i < 2 * R2B; i += NT)
@@ -361,26 +399,33 @@ k_p2(int N1, int ncol_ws, float2 *__restrict__ ws, const float2 *__restrict__ ma
       x1[it * R2B + q] = y1[q];
       // direct form: only bins inside the two bands are read by their partners (the partner of an in-band bin is
       // in the other band), so the rest, 1 - 2*gamma of them, is not written back
-      bool wanted = true;
-      if (!PAD) {
+      bool wanted = MODE != MODE_MUL;
+      if (MODE == MODE_FILTER) {
         const int bin = k1 + N1 * (pp + 16 * q);
         wanted = bin <= omega || N - bin <= omega;
       }
       if (wanted) Sh[(q + R2B * pp) * CP + cp] = make_float4(y0[q].x, y0[q].y, y1[q].x, y1[q].y);
     }
   }
-  if (PAD && tab_out != nullptr) {            // x0: spectrum of g around 0, x1: spectrum of g(t + 1)
+  if (TAB && tab_out != nullptr) {            // x0: spectrum of g around 0 or of the chirp, x1: spectrum of g(t + 1)
     if (cp == 0 && blockIdx.y == 0) {
 #pragma unroll
       for (int it = 0; it < IT; ++it)
 #pragma unroll
-        for (int q = 0; q < R2B; ++q)
-          tab_out[(size_t)k1 * N2 + j + R2B * it + 16 * q] =
-              make_float4(x1[it * R2B + q].x, x1[it * R2B + q].y, 1.f - x0[it * R2B + q].x, 0.f);
+        for (int q = 0; q < R2B; ++q) {
+          const int at = k1 * N2 + j + R2B * it + 16 * q;
+          const float2 a = x0[it * R2B + q], b = x1[it * R2B + q];
+          if (MODE == MODE_MUL) {             // the chirp of row `at` beside it
+            const float2 c = at < Nseq ? chirp(at, Nseq) : make_float2(0.f, 0.f);
+            tab_out[at] = make_float4(a.x, a.y, c.x, c.y);
+          } else {
+            tab_out[at] = make_float4(b.x, b.y, 1.f - a.x, 0.f);
+          }
+        }
     }
     return;
   }
-  __syncthreads();                            // spectra of both rows are in shared memory
+  if (MODE != MODE_MUL) __syncthreads();      // spectra of both rows are in shared memory
   const float4 *Sp = S + (self ? hf : 1 - hf) * (N2 * CP);
 #pragma unroll
   for (int it = 0; it < IT; ++it) {
@@ -390,7 +435,22 @@ k_p2(int N1, int ncol_ws, float2 *__restrict__ ws, const float2 *__restrict__ ma
       const int k2 = pp + 16 * q;
       const int bin = k1 + N1 * k2;
       const int k2p = (k1 == 0) ? ((N2 - k2) & (N2 - 1)) : (N2 - 1 - k2);
-      if (PAD) {
+      if (MODE == MODE_MUL) {
+        const float4 w = hc[hf * N2 + k2];
+        x0[it * R2B + q] = cmul(x0[it * R2B + q], make_float2(w.x, w.y));
+        x1[it * R2B + q] = cmul(x1[it * R2B + q], make_float2(w.x, w.y));
+        continue;
+      }
+      if (MODE == MODE_POWER) {               // both channels' powers replace the bins
+        const float4 t = Sp[((k2p >> 4) + R2B * (k2p & 15)) * CP + cp];
+        const float2 u = uT[hf * H2 + k2];
+        const float alpha2 = (bin == 0 ? 1.f : 2.f) / (float)N;
+        const float2 a = power_of_bin(x0[it * R2B + q], make_float2(t.x, t.y), u, alpha2);
+        const float2 b = power_of_bin(x1[it * R2B + q], make_float2(t.z, t.w), u, alpha2);
+        x0[it * R2B + q] = make_float2(a.x + b.x, a.y + b.y);
+        continue;
+      }
+      if (MODE == MODE_PAD) {
         const float4 t = Sp[((k2p >> 4) + R2B * (k2p & 15)) * CP + cp], w = hc[hf * N2 + k2];
         float2 &P0 = x0[it * R2B + q], &P1 = x1[it * R2B + q];
         P0 = make_float2(fmaf(t.y, w.y, fmaf(-t.x, w.x, w.z * P0.x)), fmaf(-t.y, w.x, fmaf(-t.x, w.y, w.z * P0.y)));
@@ -415,6 +475,37 @@ k_p2(int N1, int ncol_ws, float2 *__restrict__ ws, const float2 *__restrict__ ma
       }
     }
   }
+  if (MODE == MODE_POWER) {
+    // sums over the slice's channels: transposed reduction over the CP lanes that share (row, j), the 16 bins halved at
+    // every step; bin index = it*R2B + q
+    int count = 16, first = 0;
+#pragma unroll
+    for (int st = CP / 2; st >= 1; st >>= 1) {
+      if (count > 1) {
+        const int half = count / 2;
+        const bool up = (cp & st) != 0;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+          const float2 send = up ? x0[i] : x0[i + half], keep = up ? x0[i + half] : x0[i];
+          x0[i] = make_float2(keep.x + __shfl_xor_sync(0xffffffffu, send.x, st), keep.y + __shfl_xor_sync(0xffffffffu, send.y, st));
+        }
+        if (up) first += half;
+        count = half;
+      } else {
+        x0[0] = make_float2(x0[0].x + __shfl_xor_sync(0xffffffffu, x0[0].x, st), x0[0].y + __shfl_xor_sync(0xffffffffu, x0[0].y, st));
+      }
+    }
+    constexpr int KEEP = CP >= 16 ? 1 : 16 / CP;
+    if (CP <= 16 || (cp & (CP / 16 - 1)) == 0) {
+      float2 *dst = power + (size_t)blockIdx.y * N + (size_t)k1 * N2;
+#pragma unroll
+      for (int i = 0; i < KEEP; ++i) {
+        const int e = first + i;
+        dst[j + R2B * (e / R2B) + 16 * (e % R2B)] = x0[i];
+      }
+    }
+    return;
+  }
   // first inverse stage (mirror of the second forward stage)
 #pragma unroll
   for (int it = 0; it < IT; ++it) {
@@ -426,7 +517,7 @@ k_p2(int N1, int ncol_ws, float2 *__restrict__ ws, const float2 *__restrict__ ma
 #pragma unroll
     for (int q = 0; q < R2B; ++q) { x0[it * R2B + q] = y0[q]; x1[it * R2B + q] = y1[q]; }
   }
-  __syncthreads();                            // all partner reads are done
+  if (MODE != MODE_MUL) __syncthreads();      // all partner reads are done
 #pragma unroll
   for (int it = 0; it < IT; ++it) {
     const int pp = j + R2B * it;
@@ -491,10 +582,10 @@ __device__ __forceinline__ void twiddle_affine16_one(float2 (&x)[16], float2 b, 
   }
 }
 
-template <int C>
+template <int C, int MODE>
 __global__ void __launch_bounds__(32 * C, 2)
 k_p2_512(int N1, int ncol_ws, float2 *__restrict__ ws, const float2 *__restrict__ master, int master_len,
-         const float4 *__restrict__ tab, float4 *__restrict__ tab_out = nullptr) {
+         const float4 *__restrict__ tab, float4 *__restrict__ tab_out, int Nseq) {
   constexpr int ROW = 512, NT = 32 * C;
   constexpr int SUB = 32 * C + (C < 16 ? C : 0);              // groups of 32 points, padded against bank conflicts
   constexpr int HALF = 16 * SUB;
@@ -557,7 +648,13 @@ k_p2_512(int N1, int ncol_ws, float2 *__restrict__ ws, const float2 *__restrict_
     if (c == 0 && blockIdx.y == 0)
       for (int q = 0; q < 32; ++q) {
         const float2 g0 = S2[q * C], g1 = S2[q * C + 1];
-        tab_out[(size_t)k1 * ROW + j + 16 * q] = make_float4(g1.x, g1.y, 1.f - g0.x, 0.f);
+        const int at = k1 * ROW + j + 16 * q;
+        if (MODE == MODE_MUL) {
+          const float2 cf = at < Nseq ? chirp(at, Nseq) : make_float2(0.f, 0.f);
+          tab_out[at] = make_float4(g0.x, g0.y, cf.x, cf.y);
+        } else {
+          tab_out[at] = make_float4(g1.x, g1.y, 1.f - g0.x, 0.f);
+        }
       }
     return;
   }
@@ -572,6 +669,11 @@ k_p2_512(int N1, int ncol_ws, float2 *__restrict__ ws, const float2 *__restrict_
 #pragma unroll
     for (int q = 0; q < 32; ++q) {
       float2 &P = x[q >> 4][q & 15];
+      if (MODE == MODE_MUL) {
+        const float4 m = hrow[16 * q];
+        P = cmul(P, make_float2(m.x, m.y));
+        continue;
+      }
       const float2 t = Sp[q == 0 && first ? -32 * C : -q * C];
       const float4 w = hrow[16 * q];
       P = make_float2(fmaf(t.y, w.y, fmaf(-t.x, w.x, w.z * P.x)), fmaf(-t.y, w.x, fmaf(-t.x, w.y, w.z * P.y)));
@@ -624,11 +726,14 @@ struct EnergyOut {
   long long energy_stride;
 };
 
-template <int R1B, int CPW, bool PAD = false, int A = 16>
+template <int R1B, int CPW, int OUT = OUT_SCORE, int A = 16>
 __global__ void __launch_bounds__(CPW * R1B, 512 / (CPW * R1B))
 k_p3(const __grid_constant__ LayerPtrs lp, int H, int head_dim, int u0, int dcols, int N, int N2, int ncol_ws,
      const float2 *__restrict__ ws, const float2 *__restrict__ master, int master_len, long long score_stride,
-     float inv_scale, int accumulate, int hi_base, const __grid_constant__ EnergyOut eo) {
+     float inv_scale, int accumulate, int hi_base, const __grid_constant__ EnergyOut eo,
+     float2 *__restrict__ spec = nullptr, const float4 *__restrict__ tab = nullptr) {
+  // OUT_SPEC: row n < N times conj(chirp(n)) and inv_scale to spec[n][column]; nothing else
+  constexpr bool PAD = OUT != OUT_SCORE;
   constexpr int N1 = A * R1B, NT = CPW * R1B, IT = (A + R1B - 1) / R1B, NW = (NT + 31) / 32;
   constexpr int AO = PAD ? A / 2 : A;                       // rows a thread ends with
   constexpr int PR = PAD ? 8 : 16;                          // the same, rounded up to a power of two
@@ -710,6 +815,13 @@ k_p3(const __grid_constant__ LayerPtrs lp, int H, int head_dim, int u0, int dcol
 #pragma unroll
     for (int p = 0; p < AO; ++p) {
       if (PAD && (j + R1B * p) * N2 + n2 >= N) continue;
+      if (OUT == OUT_SPEC) {
+        const int n = (j + R1B * p) * N2 + n2;
+        const float4 t = __ldg(tab + n);
+        const float2 c = make_float2(t.z * inv_scale, t.w * inv_scale), a = cmul_conj(z0[p], c), b = cmul_conj(z1[p], c);
+        *reinterpret_cast<float4 *>(spec + (size_t)n * ncol_ws + gc0 + 2 * cp) = make_float4(a.x, a.y, b.x, b.y);
+        continue;
+      }
       const float ek = fmaf(z0[p].x, z0[p].x, z1[p].x * z1[p].x);
       const float ev = fmaf(z0[p].y, z0[p].y, z1[p].y * z1[p].y);
       totK += ek;
@@ -718,6 +830,7 @@ k_p3(const __grid_constant__ LayerPtrs lp, int H, int head_dim, int u0, int dcol
     }
     __syncthreads();
   }
+  if (OUT == OUT_SPEC) return;
   // transposed reduction over the CPW lanes that share j: the PR row sums are halved at every
   // step until one is left, further steps are plain adds; row p = cp >> log2(CPW/PR)
   {

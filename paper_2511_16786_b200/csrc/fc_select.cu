@@ -55,7 +55,7 @@ __device__ __forceinline__ double warp_max_d(double v) {
 // One block per sequence of the chunk.  Shared memory: w[L], cand[2L], fval[2L], frac[L], bud[L], order[L].
 // The sums whose rounding the rule fixes run in layer order (one thread, or one thread per candidate); everything else
 // (searches over the candidates, the remainders' order and who gets one) is spread over the block, so that a call is a
-// chain of a few L-step loops: 10.9 + 1.8 us (with the offsets as a second kernel) -> ALLOC us at 28 layers.
+// chain of a few L-step loops: 10.9 + 1.8 us (with the offsets as a second kernel) -> 9.0 us at 28 layers.
 // The last block of the call writes the offsets.
 constexpr int kAllocThreads = 256;
 __global__ void __launch_bounds__(kAllocThreads)
@@ -294,7 +294,7 @@ select_gather_body(const float *__restrict__ scores, long long T, const SeqTable
 
   if (n == 0) return;
   // the budget, the offset and the scores are requested together, without a branch between the loads (tokens past the
-  // range read its neighbours and are not counted: 9.0 -> LOADUS us for 16 scores a thread)
+  // range read its neighbours and are not counted: with a branch 16 scores took 9.0 us)
   int k = budgets[b];
   const long long off = out_offsets[b];
   unsigned key[KPT];

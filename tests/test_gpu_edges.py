@@ -1,0 +1,122 @@
+"""Spectrum, selection and short-sequence scoring at the edges of their dispatch rules and tiles, against the fp64 oracle
+(selection: exactly)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import flashcache_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fc():
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    from paper_2511_16786_b200 import binding
+    return binding
+
+
+def _kv(T, H, d, dtype, seed):
+    g = torch.Generator().manual_seed(seed)
+    t = torch.arange(T, dtype=torch.float32)[:, None, None] / T
+    k = 0.3 * torch.randn((T, H, d), generator=g) + torch.cos(2.5 * t + torch.randn((1, H, d), generator=g))
+    v = 0.3 * torch.randn((T, H, d), generator=g) + t
+    return k.to(dtype), v.to(dtype)
+
+
+# the generic kernels (512), every direct shape, and chirp lengths just inside a transform length of every first factor,
+# with rows of 32 to 512 points; heads in one launch and in several, a head in column groups
+@pytest.mark.parametrize("lens,H,d,dtype", [((512, 1024, 2048, 640, 641), 2, 64, torch.float32),
+                                            ((4096, 8192, 897, 1793), 3, 128, torch.float16),
+                                            ((16384, 10000), 4, 128, torch.bfloat16),
+                                            ((65536, 24577, 36865), 1, 64, torch.float32),
+                                            ((65535, 57345), 1, 128, torch.bfloat16)])
+def test_power_spectrum_at_its_edges(fc, lens, H, d, dtype):
+    cu = [0] + [int(x) for x in np.cumsum(lens)]
+    k, v = _kv(cu[-1], H, d, dtype, cu[-1])
+    h = fc.fc_create(0, max(lens))
+    try:
+        kd, vd = k.cuda(), v.cuda()
+        ws = torch.empty(fc.fc_power_spectrum_workspace_bytes(h, kd, vd, cu), dtype=torch.uint8, device="cuda")
+        got = []
+        for _ in range(2):                                    # the second call finds its tables kept
+            spec = torch.full((cu[-1], 2), -1.0, dtype=torch.float64, device="cuda")
+            fc.fc_power_spectrum(h, kd, vd, cu, spec, ws)
+            assert fc.fc_last_device_status(h) == 0
+            got.append(spec.cpu())
+            ws.fill_(255)
+    finally:
+        fc.fc_destroy(h)
+    assert torch.equal(got[0], got[1])
+    want = O.power_spectrum(k.double().numpy(), v.double().numpy(), cu, "fft")
+    for b in range(len(lens)):
+        w, g = want[cu[b]:cu[b + 1]], got[0][cu[b]:cu[b + 1]].numpy()
+        for j in range(2):
+            err = np.abs(g[:, j] - w[:, j]) / np.maximum(w[:, j], 1e-6 * w[:, j].max())
+            assert err.max() <= 2e-3, "%d tokens: %.3e" % (lens[b], err.max())
+
+
+# powers of two the small kernel runs directly, padded lengths around each of its transforms, and head dims whose
+# blocks make a cluster (or do not: 192)
+@pytest.mark.parametrize("d", [64, 128, 192, 256])
+def test_short_sequences_at_their_edges(fc, d):
+    lens = (1, 2, 32, 33, 63, 64, 65, 128, 129, 256, 257, 512, 513, 1024)
+    cu = [0] + [int(x) for x in np.cumsum(lens)]
+    k, v = _kv(cu[-1], 2, d, torch.float32, d)
+    h = fc.fc_create(0, max(lens))
+    try:
+        kd, vd = k.cuda(), v.cuda()
+        scores = torch.full((2, cu[-1]), -1.0, device="cuda")
+        energy = torch.empty((len(lens), 4), dtype=torch.float64, device="cuda")
+        ws = torch.empty(fc.fc_score_workspace_bytes(h, kd, vd, cu), dtype=torch.uint8, device="cuda")
+        fc.fc_score_layer(h, kd, vd, cu, 0.2, scores, energy, ws)
+        assert fc.fc_last_device_status(h) == 0
+        scores, energy = scores.cpu().numpy(), energy.cpu().numpy()
+    finally:
+        fc.fc_destroy(h)
+    for b, n in enumerate(lens):
+        ks, vs = k[cu[b]:cu[b + 1]].double().numpy(), v[cu[b]:cu[b + 1]].double().numpy()
+        tot = 0.0
+        for hd in range(2):
+            want, en = O.score_head(ks[:, hd], vs[:, hd], 0.2, "fft")
+            ebar = ((ks[:, hd] ** 2).sum(1) + (vs[:, hd] ** 2).sum(1)).mean() / d
+            err = np.abs(scores[hd, cu[b]:cu[b + 1]] - want) / np.maximum(want, 1e-6 * ebar)
+            assert err.max() <= 1e-3, "%d tokens: %.3e" % (n, err.max())
+            tot += np.asarray(en)[1]
+        np.testing.assert_allclose(energy[b, 1], tot, rtol=1e-5)
+
+
+# lengths around what one block, and a cluster of two, four and eight, hold; budgets at both ends; scores that leave the
+# threshold's bin with few keys (finished directly), with many distinct ones (every digit), and with one value for all
+@pytest.mark.parametrize("per_layer", [False, True])
+@pytest.mark.parametrize("n", [2047, 4097, 16384, 16385, 32769, 65537, 131072])
+def test_selection_at_its_edges(fc, n, per_layer):
+    rng = np.random.default_rng(n)
+    H, d = 3, 64
+    g = torch.Generator().manual_seed(n)
+    k, v = torch.randn((n, H, d), generator=g).half(), torch.randn((n, H, d), generator=g).half()
+    spread = (rng.integers(0, 1 << 17, (H, n)) * 2.0 ** -17).astype(np.float32)          # sums over heads are exact
+    near = (1.0 + rng.integers(0, 4096, (H, n)) * 2.0 ** -20).astype(np.float32)
+    same = np.full((H, n), 0.25, np.float32)
+    h = fc.fc_create(0, 131072)
+    try:
+        kd, vd, cu = k.cuda(), v.cuda(), [0, n]
+        ws = torch.empty(fc.fc_select_workspace_bytes(h, kd, vd, cu), dtype=torch.uint8, device="cuda")
+        for scores in (spread, near, same):
+            for budget in (1, n // 5, n - 1, n):
+                out_k = torch.zeros((budget, H, d), dtype=k.dtype, device="cuda")
+                out_v, idx = torch.zeros_like(out_k), torch.full((H, budget), -1, dtype=torch.int32, device="cuda")
+                bd = torch.tensor([budget], dtype=torch.int32, device="cuda")
+                of = torch.tensor([0, budget], dtype=torch.int64, device="cuda")
+                fc.fc_select_compact_ex(h, kd, vd, cu, torch.from_numpy(scores).cuda(), bd, of, out_k, out_v, idx, ws,
+                                        per_layer=per_layer)
+                assert fc.fc_last_device_status(h) == 0
+                for hd in range(H):
+                    got = idx[hd].cpu().numpy()
+                    dev = scores.astype(np.float64)
+                    np.testing.assert_array_equal(got, O.select_topk(O.layer_score(dev) if per_layer else dev[hd], budget))
+                    at = torch.from_numpy(got.astype(np.int64)).cuda()
+                    assert torch.equal(out_k[:, hd], kd[at, hd]) and torch.equal(out_v[:, hd], vd[at, hd])
+    finally:
+        fc.fc_destroy(h)
