@@ -28,6 +28,7 @@ constexpr int kThreadsD = kConsumers + 32;
 constexpr int kBoxBytes = kTile * 128;  // one TMA box: 64 rows x 64 elements of 2 bytes
 constexpr int kStageBytes = 4 * kBoxBytes;   // K low/high halves, V low/high halves
 constexpr int kStages = 4;
+constexpr int kEarlyTiles = 2;                // tiles brought into L2 ahead
 constexpr unsigned kSuspendNs = 2000u;        // a blocking test of an mbarrier sleeps at most about this long
 constexpr unsigned kSpinLimit = 1u << 17;    // such tests before a wait gives up (a quarter of a second)
 
@@ -42,6 +43,8 @@ struct DecodeParams {
   int *status;
   int B, H, Hq, G, nb, tail_cap, has_tail;
   float scale_log2;     // log2(e) / sqrt(d)
+  int cache_rows;
+  const void *cache_k, *cache_v;
 };
 
 struct DecodeMaps {
@@ -133,6 +136,7 @@ __device__ __forceinline__ unsigned tile_offset(int row, int chunk) {
   return (unsigned)((chunk >> 3) * kBoxBytes + row * 128 + (((chunk & 7) ^ (row & 7)) << 4));
 }
 
+constexpr int kFoldWarps = 4;           // warps of the second kernel
 constexpr int kMergeStride = kD + 4;    // floats per row of a warp's output in the merge buffer
 
 // One sequence: its rows in the cache and in the tail, as tiles (main rows first; a tile lies in one of the two).
@@ -140,12 +144,13 @@ struct SeqRows {
   long long off0;
   int n_main, n_tail, tiles_main, tiles;
 };
+template <bool EARLY = false>            // before the kernels in front are done: nothing of it may stay in L1
 __device__ __forceinline__ SeqRows seq_rows(const DecodeParams &P, int b) {
   SeqRows s;
-  s.off0 = P.offsets[b];
-  const long long nm = P.offsets[b + 1] - s.off0;
+  s.off0 = EARLY ? __ldcg(P.offsets + b) : P.offsets[b];
+  const long long nm = (EARLY ? __ldcg(P.offsets + b + 1) : P.offsets[b + 1]) - s.off0;
   s.n_main = nm < 0 ? 0 : (int)nm;
-  int nt = P.has_tail ? P.tail_len[b] : 0;
+  int nt = P.has_tail ? (EARLY ? __ldcg(P.tail_len + b) : P.tail_len[b]) : 0;
   s.n_tail = nt < 0 ? 0 : (nt > P.tail_cap ? P.tail_cap : nt);
   s.tiles_main = (s.n_main + kTile - 1) / kTile;
   s.tiles = s.tiles_main + (s.n_tail + kTile - 1) / kTile;
@@ -162,6 +167,49 @@ __device__ __forceinline__ long long share_start(int i, long long T, int nb) { r
 __device__ __forceinline__ int share_of(long long t, long long T, int nb) {
   const unsigned long long x = (unsigned long long)(t + 1) * (unsigned)nb - 1;
   return (x >> 32) == 0 && ((unsigned long long)T >> 32) == 0 ? (int)((unsigned)x / (unsigned)T) : (int)(x / (unsigned long long)T);
+}
+
+// A block's share of the line: tiles [lo, hi), the first of them in sequence b of head h, whose tiles start at `line`.
+struct Share {
+  long long lo, hi, line, line_len;
+  int h, b, nb;                                // nb: blocks that have tiles
+};
+// Tiles of all sequences, 32 at a time, in every warp for itself (no barrier before the first load): the sum, then
+// the sequence that holds the first tile of this block's share.
+template <bool EARLY>
+__device__ __forceinline__ Share find_share(const DecodeParams &P, int blk, int lane) {
+  Share r;
+  auto tiles_of = [&](int i) { return i < P.B ? seq_rows<EARLY>(P, i).tiles : 0; };
+  const int first32 = tiles_of(lane);
+  long long total = __reduce_add_sync(0xffffffffu, first32);
+  for (int b0 = 32; b0 < P.B; b0 += 32) total += __reduce_add_sync(0xffffffffu, tiles_of(b0 + lane));
+  r.line_len = total * P.H;                    // every head has the same tiles
+  r.nb = r.line_len < P.nb ? (int)r.line_len : P.nb;
+  r.lo = blk < r.nb ? share_start(blk, r.line_len, r.nb) : 0;
+  r.hi = blk < r.nb ? share_start(blk + 1, r.line_len, r.nb) : 0;
+  r.h = r.lo > 0 ? (int)muldiv(r.lo, 1, total) : 0;
+  const long long lo_head = r.lo - r.h * total;              // within the head
+  r.b = 0;
+  r.line = 0;
+  long long at = 0;
+  for (int b0 = 0; b0 < P.B; b0 += 32) {
+    const int mine = b0 == 0 ? first32 : tiles_of(b0 + lane);
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    const unsigned past = __ballot_sync(0xffffffffu, at + incl > lo_head);
+    if (past) {
+      const int first = __ffs(past) - 1;
+      r.b = b0 + first;
+      r.line = r.h * total + at + __shfl_sync(0xffffffffu, incl - mine, first);
+      break;
+    }
+    at += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  return r;
 }
 
 __device__ __forceinline__ void consumers_sync() { asm volatile("bar.sync 1, %0;\n" ::"n"(kConsumers) : "memory"); }
@@ -208,41 +256,32 @@ k_decode(const DecodeParams P, const __grid_constant__ DecodeMaps M) {
     if (P.has_tail) { prefetch_map(&M.tk); prefetch_map(&M.tv); }
   }
   __syncthreads();
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");       // what the kernels before this one wrote is visible from here
-
-  // Tiles of all sequences, 32 at a time, in every warp for itself (no barrier before the first load): the sum, then
-  // the sequence that holds the first tile of this block's share.
-  auto tiles_of = [&](int i) { return i < P.B ? seq_rows(P, i).tiles : 0; };
-  const int first32 = tiles_of(lane);
-  long long total = __reduce_add_sync(0xffffffffu, first32);
-  for (int b0 = 32; b0 < P.B; b0 += 32) total += __reduce_add_sync(0xffffffffu, tiles_of(b0 + lane));
-  const long long line_len = total * P.H;                    // every head has the same tiles
-  const int nb = line_len < P.nb ? (int)line_len : P.nb;     // blocks that have tiles
-  const long long lo = blk < nb ? share_start(blk, line_len, nb) : 0, hi = blk < nb ? share_start(blk + 1, line_len, nb) : 0;
-  int h = lo > 0 ? (int)muldiv(lo, 1, total) : 0;
-  const long long lo_head = lo - h * total;                  // within the head
-  int b = 0;
-  long long line = 0;                          // position of the first tile of (h, b)
-  {
-    long long at = 0;
-    for (int b0 = 0; b0 < P.B; b0 += 32) {
-      const int mine = b0 == 0 ? first32 : tiles_of(b0 + lane);
-      int incl = mine;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
+  if (warp < kWarps) {
+    // While the kernels in front still run, the first rows of the share are brought into L2.  Nothing is read from them
+    // here, so it does not matter if those kernels are still writing them, or the offsets: a wrong guess only wastes it.
+    // By plain prefetches, since the tensor engine takes as long over a prefetch as over the load; two tiles are what
+    // fits into the wait (four and eight lose again what two gain), and with a share of one tile the load itself is as
+    // early.  28 layers of 65536 rows 799 -> 778 us, of kept rows 1638, 205, 3277, 820 326 -> 309 us.
+    const Share sr = find_share<true>(P, blk, lane);
+    if (sr.hi - sr.lo > 1) {
+      const SeqRows s = seq_rows<true>(P, sr.b);
+      const long long first = sr.lo - sr.line, left = s.tiles_main - first;
+      const int n = (int)(left < kEarlyTiles ? left : kEarlyTiles) * kTile * 4;       // four lines of 128 bytes per row
+      for (int i = tid; i < n; i += kConsumers) {
+        const long long row = s.off0 + first * kTile + (i >> 2);
+        const char *base = static_cast<const char *>(i & 2 ? P.cache_v : P.cache_k);
+        if (row >= 0 && row < P.cache_rows)
+          asm volatile("prefetch.global.L2 [%0];\n" ::"l"(base + ((size_t)row * P.H + sr.h) * (kD * 2) + (i & 1) * 128) : "memory");
       }
-      const unsigned past = __ballot_sync(0xffffffffu, at + incl > lo_head);
-      if (past) {
-        const int first = __ffs(past) - 1;
-        b = b0 + first;
-        line = h * total + at + __shfl_sync(0xffffffffu, incl - mine, first);
-        break;
-      }
-      at += __shfl_sync(0xffffffffu, incl, 31);
     }
   }
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");       // what the kernels before this one wrote is visible from here
+
+  const Share sr = find_share<false>(P, blk, lane);
+  const long long lo = sr.lo, hi = sr.hi, line_len = sr.line_len;
+  const int nb = sr.nb;
+  int h = sr.h, b = sr.b;
+  long long line = sr.line;
   if (blk == 0)                                // sequences without rows
     for (int i = tid; i < P.B; i += kThreadsD)
       if (seq_rows(P, i).tiles == 0) {
@@ -427,10 +466,13 @@ k_decode(const DecodeParams P, const __grid_constant__ DecodeMaps M) {
     }
     {
       float *w0 = mo + ((size_t)warp * 16 + g) * kMergeStride, *w1 = w0 + 8 * kMergeStride;
+      if (g < P.G) {
 #pragma unroll
-      for (int j = 0; j < kD / 8; ++j) {
-        *reinterpret_cast<float2 *>(w0 + 8 * j + 2 * t) = make_float2(oacc[j][0], oacc[j][1]);
-        *reinterpret_cast<float2 *>(w1 + 8 * j + 2 * t) = make_float2(oacc[j][2], oacc[j][3]);
+        for (int j = 0; j < kD / 8; ++j) *reinterpret_cast<float2 *>(w0 + 8 * j + 2 * t) = make_float2(oacc[j][0], oacc[j][1]);
+      }
+      if (g + 8 < P.G) {
+#pragma unroll
+        for (int j = 0; j < kD / 8; ++j) *reinterpret_cast<float2 *>(w1 + 8 * j + 2 * t) = make_float2(oacc[j][2], oacc[j][3]);
       }
       if (t == 0) {
         mml[warp * 16 + g] = make_float2(m[0], l[0]);
@@ -471,11 +513,11 @@ k_decode(const DecodeParams P, const __grid_constant__ DecodeMaps M) {
 // (merging in the block that finishes last instead costs an atomic and 3..5 us on one SM: 14.0 against 11.9 us per
 // layer of the small case above).
 template <typename T>
-__global__ void __launch_bounds__(32 * kWarps)
+__global__ void __launch_bounds__(32 * kFoldWarps)
 k_decode_combine(const DecodeParams P) {
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-  __shared__ float4 so[kWarps][32];
-  __shared__ float2 sml[kWarps];
+  __shared__ float4 so[kFoldWarps][32];
+  __shared__ float2 sml[kFoldWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b = blockIdx.x / P.Hq, hq = blockIdx.x - b * P.Hq, h = hq / P.G, r = hq - h * P.G;
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
@@ -486,19 +528,19 @@ k_decode_combine(const DecodeParams P) {
   constexpr int kAhead = 10;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   float m = -INFINITY, l = 0.f;
-  for (int s0 = warp; s0 < cnt; s0 += kWarps * kAhead) {
+  for (int s0 = warp; s0 < cnt; s0 += kFoldWarps * kAhead) {
     float4 v[kAhead];
     float2 ml[kAhead];
 #pragma unroll
     for (int a = 0; a < kAhead; ++a) {
-      const int i = s0 + a * kWarps < cnt ? s0 + a * kWarps : s0;
+      const int i = s0 + a * kFoldWarps < cnt ? s0 + a * kFoldWarps : s0;
       ml[a] = __ldcg(P.part_ml + slot0 + (size_t)i * P.G);
       v[a] = __ldcg(reinterpret_cast<const float4 *>(P.part_o + (slot0 + (size_t)i * P.G) * kD) + lane);
     }
     float mn = m;
 #pragma unroll
     for (int a = 0; a < kAhead; ++a) {
-      if (s0 + a * kWarps >= cnt) ml[a] = make_float2(-INFINITY, 0.f);
+      if (s0 + a * kFoldWarps >= cnt) ml[a] = make_float2(-INFINITY, 0.f);
       mn = fmaxf(mn, ml[a].x);
     }
     const float ms = mn == -INFINITY ? 0.f : mn, keep = exp2f(m - ms);
@@ -518,11 +560,11 @@ k_decode_combine(const DecodeParams P) {
   if (warp != 0) return;
   float mm = -INFINITY, ll = 0.f;
 #pragma unroll
-  for (int w = 0; w < kWarps; ++w) mm = fmaxf(mm, sml[w].x);
+  for (int w = 0; w < kFoldWarps; ++w) mm = fmaxf(mm, sml[w].x);
   const float ms = mm == -INFINITY ? 0.f : mm;
   float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-  for (int w = 0; w < kWarps; ++w) {
+  for (int w = 0; w < kFoldWarps; ++w) {
     const float f = exp2f(sml[w].x - ms);
     fold(o, so[w][lane], f);
     ll += sml[w].y * f;
@@ -639,6 +681,9 @@ fc_status launch_decode(fc_handle *h, const fc_decode_args *a, const DecodePlan 
   P.Hq = a->num_q_heads;
   P.G = a->num_q_heads / a->num_heads;
   P.nb = pl.nb;
+  P.cache_rows = (int)a->cache_rows;
+  P.cache_k = a->cache_k;
+  P.cache_v = a->cache_v;
   P.tail_cap = a->tail_k ? a->tail_capacity : 0;
   P.has_tail = a->tail_k ? 1 : 0;
   P.scale_log2 = (float)(1.4426950408889634 / sqrt((double)kD));
@@ -663,7 +708,7 @@ fc_status launch_decode(fc_handle *h, const fc_decode_args *a, const DecodePlan 
   }
   if ((s = fc_after_launch(h)) != FC_OK) return s;
   lc.gridDim = dim3((unsigned)(a->batch * a->num_q_heads));
-  lc.blockDim = dim3(32 * kWarps);
+  lc.blockDim = dim3(32 * kFoldWarps);
   lc.dynamicSmemBytes = 0;
   if (cudaLaunchKernelEx(&lc, k_decode_combine<T>, P) != cudaSuccess) {
     cudaGetLastError();
