@@ -159,23 +159,30 @@ __device__ __forceinline__ void dft4(float2 &a0, float2 &a1, float2 &a2, float2 
   a3 = csub(d0, d1);
 }
 
+// a, b = e + w*o, e - w*o for w = exp(DIR*j*phi): with w = c*(1 + j*t) the factor c goes into the two sums, six fused
+// operations instead of eight (a 16-point transform 148 instead of 168; scoring 0.2..1.3 % faster); of cos and sin the
+// larger is taken for c, so |t| <= 1.
+template <int DIR>
+__device__ __forceinline__ void rotated_sums(float2 e, float2 o, float cs, float sn, float2 &a, float2 &b) {
+  const bool by_cos = cs * cs >= sn * sn;                     // constants: folded
+  const float f = by_cos ? cs : (DIR < 0 ? -sn : sn), t = by_cos ? (DIR < 0 ? -sn : sn) / cs : cs / (DIR < 0 ? -sn : sn);
+  const float2 r = by_cos ? make_float2(fmaf(-t, o.y, o.x), fmaf(t, o.x, o.y))
+                          : make_float2(fmaf(t, o.x, -o.y), fmaf(t, o.y, o.x));
+  a = make_float2(fmaf(f, r.x, e.x), fmaf(f, r.y, e.y));
+  b = make_float2(fmaf(-f, r.x, e.x), fmaf(-f, r.y, e.y));
+}
+
 template <int DIR>
 __device__ __forceinline__ void dft8(float2 (&x)[8]) {
   const float h = 0.70710678118654752440f;
   dft4<DIR>(x[0], x[2], x[4], x[6]);   // even samples -> x[0],x[2],x[4],x[6] = E0..E3
   dft4<DIR>(x[1], x[3], x[5], x[7]);   // odd samples  -> x[1],x[3],x[5],x[7] = O0..O3
-  float2 e0 = x[0], e1 = x[2], e2 = x[4], e3 = x[6];
-  float2 o0 = x[1], o1 = x[3], o2 = x[5], o3 = x[7];
-  // w8^1 = (1 + DIR*j)/sqrt2, w8^2 = DIR*j, w8^3 = (-1 + DIR*j)/sqrt2
-  float2 t1 = DIR < 0 ? make_float2((o1.x + o1.y) * h, (o1.y - o1.x) * h)
-                      : make_float2((o1.x - o1.y) * h, (o1.x + o1.y) * h);
-  float2 t2 = mul_j<DIR>(o2);
-  float2 t3 = DIR < 0 ? make_float2((o3.y - o3.x) * h, -(o3.x + o3.y) * h)
-                      : make_float2(-(o3.x + o3.y) * h, (o3.x - o3.y) * h);
+  const float2 e0 = x[0], e1 = x[2], e2 = x[4], e3 = x[6];
+  const float2 o0 = x[1], o1 = x[3], o2 = mul_j<DIR>(x[5]), o3 = x[7];
   x[0] = cadd(e0, o0); x[4] = csub(e0, o0);
-  x[1] = cadd(e1, t1); x[5] = csub(e1, t1);
-  x[2] = cadd(e2, t2); x[6] = csub(e2, t2);
-  x[3] = cadd(e3, t3); x[7] = csub(e3, t3);
+  rotated_sums<DIR>(e1, o1, h, h, x[1], x[5]);
+  x[2] = cadd(e2, o2); x[6] = csub(e2, o2);
+  rotated_sums<DIR>(e3, o3, -h, h, x[3], x[7]);
 }
 
 template <int DIR>
@@ -187,19 +194,15 @@ __device__ __forceinline__ void dft16(float2 (&x)[16]) {
   for (int i = 0; i < 8; ++i) { e[i] = x[2 * i]; o[i] = x[2 * i + 1]; }
   dft8<DIR>(e);
   dft8<DIR>(o);
-  const float sg = DIR < 0 ? -1.f : 1.f;
-  // w16^k = (cos(k*pi/8), DIR*sin(k*pi/8))
-  float2 t[8];
-  t[0] = o[0];
-  t[1] = cmul(o[1], make_float2(c1, sg * s1));
-  t[2] = cmul(o[2], make_float2(h, sg * h));
-  t[3] = cmul(o[3], make_float2(s1, sg * c1));
-  t[4] = mul_j<DIR>(o[4]);
-  t[5] = cmul(o[5], make_float2(-s1, sg * c1));
-  t[6] = cmul(o[6], make_float2(-h, sg * h));
-  t[7] = cmul(o[7], make_float2(-c1, sg * s1));
-#pragma unroll
-  for (int k = 0; k < 8; ++k) { x[k] = cadd(e[k], t[k]); x[k + 8] = csub(e[k], t[k]); }
+  o[4] = mul_j<DIR>(o[4]);
+  x[0] = cadd(e[0], o[0]); x[8] = csub(e[0], o[0]);
+  rotated_sums<DIR>(e[1], o[1], c1, s1, x[1], x[9]);
+  rotated_sums<DIR>(e[2], o[2], h, h, x[2], x[10]);
+  rotated_sums<DIR>(e[3], o[3], s1, c1, x[3], x[11]);
+  x[4] = cadd(e[4], o[4]); x[12] = csub(e[4], o[4]);
+  rotated_sums<DIR>(e[5], o[5], -s1, c1, x[5], x[13]);
+  rotated_sums<DIR>(e[6], o[6], -h, h, x[6], x[14]);
+  rotated_sums<DIR>(e[7], o[7], -c1, s1, x[7], x[15]);
 }
 
 // Odd lengths by the symmetric form: with a_m = x[m] + x[P-m], b_m = x[m] - x[P-m],
@@ -361,7 +364,10 @@ template <int R>
 __device__ __forceinline__ void add_odd_half(float2 (&e)[R / 2], const float2 (&o)[R / 2]) {
   e[0] = cadd(e[0], o[0]);
 #pragma unroll
-  for (int n = 1; n < R / 2; ++n) e[n] = cadd(e[n], cmul(o[n], make_float2(root_cos<R>(n), root_sin<R>(n))));
+  for (int n = 1; n < R / 2; ++n) {
+    const float c = root_cos<R>(n), s = root_sin<R>(n);
+    e[n] = make_float2(fmaf(c, o[n].x, fmaf(-s, o[n].y, e[n].x)), fmaf(c, o[n].y, fmaf(s, o[n].x, e[n].y)));
+  }
 }
 template <int R>
 __device__ __forceinline__ void idft_first_half(const float2 (&y)[R], float2 (&x)[R / 2]) {
