@@ -663,20 +663,28 @@ fc_status launch_select(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, con
     // phase of the select waits on barriers, and one block's are a fraction of a cluster's (28 x 4 heads of 1500 tokens:
     // 22.6 us with two blocks, 12.2 with one; 8 ragged short sequences 131 -> 72 us; one layer of 1024 tokens: 10.0 us
     // with one block, 18.4 with eight).  Two where a layer keeps one index set, whose few clusters gather all heads.
-    constexpr int nt = 1024;
     int cl = per_layer ? 2 : 1;
-    while (cl < kSelCluster && nmax > cl * nt * kSelKptMax) cl *= 2;
+    while (cl < kSelCluster && nmax > cl * 1024 * kSelKptMax) cl *= 2;
     int kpt = 2;
-    while (kpt < kSelKptMax && nmax > cl * nt * kpt) kpt *= 2;
+    while (kpt < kSelKptMax && nmax > cl * 1024 * kpt) kpt *= 2;
+    // Short sequences in more blocks than SMs: fewer threads with more scores each, so that several blocks share an SM
+    // and some gather rows (bound by memory) while others select (bound by barriers): 28 x 32 heads of 1000 tokens
+    // 62 -> 43 us, of 300 34 -> 15, 28 x 4 heads of 8 ragged sequences up to 2311 69 -> 60.  Not beyond 4096 tokens,
+    // where the gather fills the time (8192: 128 -> 137, 16384: 1.12 -> 1.20 ms).
+    int nt = 1024;
+    if (!per_layer && kpt <= 4 && (long long)nseq * kv->num_heads * nl > h->num_sms) {
+      nt = nmax <= 1024 ? 256 : 512;
+      kpt = nmax <= 2048 ? 4 : 8;
+    }
     {
       ProfScope ps(h, FC_K_SELECT, st);
       const size_t sm = (size_t)kpt * nt * sizeof(unsigned short);
-#define FC_SEL_LAUNCH(KPT, PL, CLV)                                                                \
+#define FC_SEL_LAUNCH(KPT, PL, CLV, NTV)                                                                \
   do {                                                                                                  \
-    if ((s = allow_smem(k_select_gather<KPT, PL, CLV, nt>, sm)) != FC_OK) return s;                    \
+    if ((s = allow_smem(k_select_gather<KPT, PL, CLV, NTV>, sm)) != FC_OK) return s;                    \
     cudaLaunchConfig_t lc = {};                                                                         \
     lc.gridDim = dim3(CLV * nseq, (PL) ? 1 : kv->num_heads, nl);                                        \
-    lc.blockDim = dim3(nt);                                                                             \
+    lc.blockDim = dim3(NTV);                                                                             \
     lc.dynamicSmemBytes = sm;                                                                           \
     lc.stream = st;                                                                                     \
     cudaLaunchAttribute at[1];                                                                          \
@@ -684,19 +692,22 @@ fc_status launch_select(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, con
     at[0].val.programmaticStreamSerializationAllowed = 1;                                               \
     lc.attrs = at;                                                                                      \
     lc.numAttrs = (h->select_overlap && h->after_select) ? 1 : 0;                                       \
-    launch_err = cudaLaunchKernelEx(&lc, k_select_gather<KPT, PL, CLV, nt>, lt, (long long)T, tab, b0, (int)kv->batch, \
+    launch_err = cudaLaunchKernelEx(&lc, k_select_gather<KPT, PL, CLV, NTV>, lt, (long long)T, tab, b0, (int)kv->batch, \
         budgets, reinterpret_cast<const long long *>(out_offsets),                                      \
         h->status_word, (long long)(kv->stride_token * es), (long long)(kv->stride_head * es),          \
         (int)(kv->head_dim * es), (int)kv->num_heads, (int)h->select_overlap, protect);                 \
   } while (0)
 #define FC_SEL_CASE(KPT, PL, CLV) \
-  else if (kpt == KPT && cl == CLV && per_layer == PL) FC_SEL_LAUNCH(KPT, PL, CLV);
+  else if (nt == 1024 && kpt == KPT && cl == CLV && per_layer == PL) FC_SEL_LAUNCH(KPT, PL, CLV, 1024);
+#define FC_SEL_MANY(KPT, NTV) else if (nt == NTV && kpt == KPT && cl == 1) FC_SEL_LAUNCH(KPT, false, 1, NTV);
       cudaError_t launch_err = cudaErrorInvalidValue;
       if (false) {}
       FC_SEL_CASE(2, false, 1) FC_SEL_CASE(4, false, 1) FC_SEL_CASE(8, false, 1) FC_SEL_CASE(16, false, 1)
       FC_SEL_CASE(16, false, 2) FC_SEL_CASE(16, false, 4) FC_SEL_CASE(16, false, 8)
       FC_SEL_CASE(2, true, 2) FC_SEL_CASE(4, true, 2) FC_SEL_CASE(8, true, 2) FC_SEL_CASE(16, true, 2)
       FC_SEL_CASE(16, true, 4) FC_SEL_CASE(16, true, 8)
+      FC_SEL_MANY(4, 256) FC_SEL_MANY(4, 512) FC_SEL_MANY(8, 512)
+#undef FC_SEL_MANY
 #undef FC_SEL_CASE
 #undef FC_SEL_LAUNCH
       if (launch_err != cudaSuccess) { cudaGetLastError(); return FC_ERR_CUDA; }

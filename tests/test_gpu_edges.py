@@ -120,3 +120,32 @@ def test_selection_at_its_edges(fc, n, per_layer):
                     assert torch.equal(out_k[:, hd], kd[at, hd]) and torch.equal(out_v[:, hd], vd[at, hd])
     finally:
         fc.fc_destroy(h)
+
+
+# short sequences in more blocks than SMs (smaller blocks that share an SM), around the lengths they hold
+@pytest.mark.parametrize("lens", [(1024, 1, 0, 300), (1025, 2048, 7), (2049, 64, 4096), (4097, 100, 1000)])
+def test_selection_of_many_short_sequences(fc, lens):
+    rng = np.random.default_rng(sum(lens))
+    H, d, cu = 256, 64, [0] + [int(x) for x in np.cumsum(lens)]
+    budgets = [(n + 3) // 4 for n in lens]
+    offs = [0] + [int(x) for x in np.cumsum(budgets)]
+    g = torch.Generator().manual_seed(sum(lens))
+    k = torch.randn((cu[-1], H, d), generator=g).half().cuda()
+    scores = (rng.integers(0, 1 << 12, (H, cu[-1])) * 2.0 ** -9).astype(np.float32)
+    h = fc.fc_create(0, 8192)
+    try:
+        ws = torch.empty(fc.fc_select_workspace_bytes(h, k, k, cu), dtype=torch.uint8, device="cuda")
+        out_k = torch.zeros((offs[-1], H, d), dtype=k.dtype, device="cuda")
+        out_v, idx = torch.zeros_like(out_k), torch.full((H, offs[-1]), -1, dtype=torch.int32, device="cuda")
+        fc.fc_select_compact_ex(h, k, k, cu, torch.from_numpy(scores).cuda(),
+                                torch.tensor(budgets, dtype=torch.int32, device="cuda"),
+                                torch.tensor(offs, dtype=torch.int64, device="cuda"), out_k, out_v, idx, ws)
+        assert fc.fc_last_device_status(h) == 0
+        for hd in range(H):
+            for b in range(len(lens)):
+                got = idx[hd, offs[b]:offs[b + 1]].cpu().numpy()
+                np.testing.assert_array_equal(got, O.select_topk(scores[hd, cu[b]:cu[b + 1]].astype(np.float64), budgets[b]))
+            at = torch.cat([idx[hd, offs[b]:offs[b + 1]].long() + cu[b] for b in range(len(lens))])
+            assert torch.equal(out_k[:, hd], k[at, hd]) and torch.equal(out_v[:, hd], k[at, hd])
+    finally:
+        fc.fc_destroy(h)
