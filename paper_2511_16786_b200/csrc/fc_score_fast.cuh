@@ -172,21 +172,25 @@ k_p1(const __grid_constant__ LayerPtrs lp, long long stride_token, long long str
   float2 x0[A], x1[A];
   float accK = 0.f, accV = 0.f;
   if (LD == LD_TABLE) {
-#pragma unroll 1
-    for (int p = 0; p < A; ++p) {
-      // columns 0 and 1; this thread's values come back from shared memory, where the loop can stay rolled
-      const int n = (j + R1B * p) * N2 + n2, M = N1 * N2;
-      float g0 = 0.f, g1 = 0.f, gi = 0.f;
-      if (cp == 0 && gc0 == 0 && omega < 0) {             // the chirp, wrapped, in column 0
-        const int a = n < N ? n : n > M - N ? M - n : -1;
-        if (a >= 0) { const float2 c = chirp(a, N); g0 = c.x; gi = c.y; }
-      } else if (cp == 0 && gc0 == 0) {
-        if (n < N) g0 = base_kernel(n, N, omega);
-        else if (n > M - N) g0 = base_kernel(M - n, N, omega);
-        if (n <= 2 * N - 2) g1 = base_kernel(n + 1, N, omega);
+    // columns 0 and 1, the N1 rows of this n2 shared out over the block (fp64 sines: 17 us at 96 rows with a column's own
+    // threads, 5.3 us now)
+    const int M = N1 * N2;
+    for (int i = tid; i < N1 * CPW; i += NT) S[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+    if (gc0 == 0)
+      for (int i = tid; i < 2 * N1; i += NT) {
+        const int n = (i >> 1) * N2 + n2;
+        float2 *at = reinterpret_cast<float2 *>(S + (i >> 1) * CPW) + (i & 1);
+        if (omega < 0) {                                  // the chirp, wrapped, in column 0
+          const int m = n < N ? n : n > M - N ? M - n : -1;
+          if ((i & 1) == 0 && m >= 0) *at = chirp(m, N);
+        } else if (i & 1) {
+          if (n <= 2 * N - 2) at->x = base_kernel(n + 1, N, omega);
+        } else if (n < N || n > M - N) {
+          at->x = base_kernel(n < N ? n : M - n, N, omega);
+        }
       }
-      S[(j + R1B * p) * CPW + cp] = make_float4(g0, gi, g1, 0.f);
-    }
+    __syncthreads();
 #pragma unroll
     for (int p = 0; p < A; ++p) {
       const float4 t = S[(j + R1B * p) * CPW + cp];
