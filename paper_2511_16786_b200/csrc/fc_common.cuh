@@ -14,7 +14,7 @@
 
 #define FC_MAX_STAGES 4
 #define FC_MAX_AUX 4     // internal streams a handle may use
-#define FC_TAB_SLOTS 8   // filter tables a handle keeps (one per sequence length and cutoff)
+#define FC_TAB_SLOTS 8   // filter tables a handle keeps (one per sequence length, cutoff and form)
 #define FC_LAYER_CHUNK 32  // layers one launch of the scoring kernels can span (kernel-argument table)
 
 // Bits of the device status word.
@@ -63,7 +63,7 @@ struct fc_handle {
   size_t last_sig;               // how the previous call carved its workspace
   bool pending_join;             // internal streams hold work the caller's stream has not waited for
   cudaEvent_t ev_done[2][FC_MAX_AUX];   // [step parity][internal stream]: that stream finished that step
-  // filter tables of the last FC_TAB_SLOTS (length, cutoff) pairs that took the padded path (DEVICE, allocated by
+  // filter tables of the last FC_TAB_SLOTS (length, cutoff, form) triples that took the padded path (DEVICE, allocated by
   // fc_create: FC_TAB_SLOTS x tab_slot_len entries; tab_key[i] = what slot i holds, 0 = nothing; round robin)
   float4 *tab_cache;
   int tab_slot_len, tab_next;

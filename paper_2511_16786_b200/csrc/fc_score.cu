@@ -1160,8 +1160,8 @@ PassPlan plan_spectrum(int N) {
 }
 
 // Tables of the padded form (filter) or of the chirp (spectrum = true: its spectrum and per-row factors) for every such
-// sequence of the view, tabs[b].  A table depends on the length and the cutoff only, so the handle keeps the last
-// FC_TAB_SLOTS (the layers of a prefill share theirs).  While the stream is being captured, and for lengths beyond the
+// sequence of the view, tabs[b].  A table depends on the length, the cutoff and the form (small kernel or passes) only, so
+// the handle keeps the last FC_TAB_SLOTS (the layers of a prefill share theirs).  While the stream is being captured, and for lengths beyond the
 // slots, tables go to the workspace (`spare`), every call: a graph must not depend on what the handle holds when it is
 // replayed.  `buf`: an intermediate buffer to build them in.
 fc_status prepare_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, double gamma, bool spectrum, float4 *spare,
@@ -1170,7 +1170,11 @@ fc_status prepare_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, do
   bool used[FC_TAB_SLOTS] = {};
   auto plan_of = [&](int N) { return spectrum ? plan_spectrum(N) : plan_passes(N, kv->head_dim); };
   auto omega_of = [&](int N) { return spectrum ? -1 : cutoff_index(gamma, N); };
-  auto key_of = [&](int N) { return (long long)N + ((long long)(omega_of(N) + 2) << 32); };
+  // head_dim decides between the small kernel and the passes, whose tables differ in length and order, so the form is
+  // part of the key (with it N fixes the transform length)
+  auto key_of = [&](int N) {
+    return (long long)N + (plan_of(N).small ? 1ll << 24 : 0ll) + ((long long)(omega_of(N) + 2) << 32);
+  };
   for (int b = 0; b < kv->batch; ++b) {
     tabs[b] = nullptr;
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];

@@ -78,3 +78,23 @@ def test_padded_lengths_at_their_edges(fc, N, gamma):
     _check_head(k[:, 0], v[:, 0], s[0, 0], gamma, torch.float32)
     _, eo = O.score_head(k[:, 0].double().numpy(), v[:, 0].double().numpy(), gamma, "fft")
     np.testing.assert_allclose(e[0, 0, [1, 3]].numpy(), np.asarray(eo)[[1, 3]], rtol=1e-5)
+
+
+# one handle, one length, head dimensions that fill a cluster of the small kernel (128) and that do not (192, 256 at more
+# than 256 tokens, 384): each finds a filter table of its own form
+@pytest.mark.parametrize("N", [100, 300, 333, 500, 1000])
+def test_head_dims_that_take_different_kernels_share_a_handle(fc, N):
+    h = fc.fc_create(0, N)
+    try:
+        for d in (128, 192, 256, 384, 128, 192):
+            k, v = _kv(N, 2, d, torch.float32, N + d)
+            kd, vd = k.cuda(), v.cuda()
+            scores = torch.full((2, N), -1.0, dtype=torch.float32, device="cuda")
+            energy = torch.full((1, 4), -1.0, dtype=torch.float64, device="cuda")
+            ws = torch.empty(fc.fc_score_workspace_bytes(h, kd, vd, [0, N]), dtype=torch.uint8, device="cuda")
+            fc.fc_score_layer(h, kd, vd, [0, N], 0.2, scores, energy, ws)
+            assert fc.fc_last_device_status(h) == 0
+            for head in range(2):
+                _check_head(k[:, head], v[:, head], scores[head].cpu(), 0.2, torch.float32)
+    finally:
+        fc.fc_destroy(h)
