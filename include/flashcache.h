@@ -119,9 +119,10 @@ fc_status fc_proto_dft16_stage(fc_handle *h, const void *x, void *y, int32_t nco
                                int32_t repeat, fc_stream stream);
 
 /* Self test of the failure path of the bounded device-side waits (diagnostic; the paper has no
- * counterpart): enqueues one small kernel that waits, at most 1000 tries, on a barrier nothing will ever
- * complete, gives up, and records it.  The next fc_last_device_status returns FC_ERR_TIMEOUT; the
- * context stays usable (nothing traps, nothing spins without a limit). */
+ * counterpart): enqueues one small kernel in which half of a warp waits, at most 1000 tries, on a barrier
+ * nothing will ever complete, gives up, and the warp as a whole records it.  The next fc_last_device_status
+ * returns FC_ERR_TIMEOUT (FC_ERR_INTERNAL if the warp's lanes disagreed); the context stays usable (nothing
+ * traps, nothing spins without a limit). */
 fc_status fc_selftest_bounded_wait(fc_handle *h, fc_stream stream);
 
 /* Number of kernels this handle has launched since fc_create (diagnostic). */

@@ -1,5 +1,6 @@
 // Handle life cycle, status reporting and the twiddle table of the FlashCache library.
 #include "fc_common.cuh"
+#include "fc_mbar.cuh"
 
 #include <mutex>
 #include <new>
@@ -35,25 +36,21 @@ __global__ void __launch_bounds__(256) k_fma_probe(float *out, int iters, float 
   out[blockIdx.x * blockDim.x + threadIdx.x] = s;
 }
 
-// Self test of the failure path every bounded device-side wait takes: one block waits on a shared-memory
-// barrier that nothing ever arrives on, gives up after `limit` tries, records the timeout in the status
-// word and returns normally.
+// Self test of the failure path of the bounded device-side waits.  One warp waits, half of its lanes on a barrier that is
+// complete and half on one that nothing ever arrives on: the latter give up after `limit` tries, every lane must get that
+// verdict, and the timeout is recorded in the status word.  A verdict that differs from lane to lane is an internal error.
 __global__ void k_selftest_bounded_wait(int *status, unsigned limit) {
-  __shared__ unsigned long long bar;
-  const unsigned addr = (unsigned)__cvta_generic_to_shared(&bar);
+  __shared__ unsigned long long complete, never;
   if (threadIdx.x == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(addr) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    mbar::init(&complete, 1u);
+    mbar::init(&never, 1u);
+    mbar::init_done();
+    mbar::arrive(&complete);
   }
   __syncthreads();
-  bool done = false;
-  for (unsigned it = 0; it < limit && !done; ++it) {
-    unsigned ok;
-    asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}\n"
-                 : "=r"(ok) : "r"(addr) : "memory");
-    done = ok != 0;
-  }
-  if (!done && threadIdx.x == 0) atomicOr(status, FC_DEV_FLAG_TIMEOUT);
+  const bool ok = mbar::wait_warp(threadIdx.x & 1 ? &never : &complete, 0u, limit);
+  const unsigned through = __ballot_sync(0xffffffffu, ok);
+  if (threadIdx.x == 0) atomicOr(status, through == 0u ? FC_DEV_FLAG_TIMEOUT : FC_DEV_FLAG_INTERNAL);
 }
 
 }  // namespace

@@ -17,6 +17,7 @@
 #include <cuda.h>
 
 #include "fc_common.cuh"
+#include "fc_mbar.cuh"
 
 namespace {
 
@@ -29,8 +30,6 @@ constexpr int kBoxBytes = kTile * 128;  // one TMA box: 64 rows x 64 elements of
 constexpr int kStageBytes = 4 * kBoxBytes;   // K low/high halves, V low/high halves
 constexpr int kStages = 4;
 constexpr int kEarlyTiles = 2;                // tiles brought into L2 ahead
-constexpr unsigned kSuspendNs = 2000u;        // a blocking test of an mbarrier sleeps at most about this long
-constexpr unsigned kSpinLimit = 1u << 17;    // such tests before a wait gives up (a quarter of a second)
 
 struct DecodeParams {
   const void *q;
@@ -51,30 +50,6 @@ struct DecodeMaps {
   CUtensorMap k, v, tk, tv;
 };
 
-__device__ __forceinline__ void mbar_init(unsigned long long *bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"((unsigned)__cvta_generic_to_shared(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long *bar, unsigned bytes) {
-  asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n"
-               ::"r"((unsigned)__cvta_generic_to_shared(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(unsigned long long *bar) {
-  asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n"
-               ::"r"((unsigned)__cvta_generic_to_shared(bar)) : "memory");
-}
-// One potentially blocking test: the thread sleeps until the phase completes or a hardware time limit passes.
-__device__ __forceinline__ bool mbar_try(unsigned long long *bar, unsigned parity) {
-  unsigned ok;
-  asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
-               : "=r"(ok) : "r"((unsigned)__cvta_generic_to_shared(bar)), "r"(parity), "r"(kSuspendNs) : "memory");
-  return ok != 0u;
-}
-// Bounded wait; false = gave up.
-__device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned parity) {
-  for (unsigned it = 0; it < kSpinLimit; ++it)
-    if (mbar_try(bar, parity)) return true;
-  return false;
-}
 // Tiled loads into this block's shared memory; completion is counted in bytes on `bar`.  One destination block only.
 __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, int c0, int c1, int c2,
                                             unsigned long long *bar) {
@@ -247,8 +222,8 @@ k_decode(const DecodeParams P, const __grid_constant__ DecodeMaps M) {
 
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   if (tid == 0) {
-    for (int i = 0; i < kStages; ++i) { mbar_init(&sh.full[i], 1u); mbar_init(&sh.empty[i], kWarps); }
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    for (int i = 0; i < kStages; ++i) { mbar::init(&sh.full[i], 1u); mbar::init(&sh.empty[i], kWarps); }
+    mbar::init_done();
   }
   if (tid == kConsumers) {
     prefetch_map(&M.k);
@@ -307,9 +282,9 @@ k_decode(const DecodeParams P, const __grid_constant__ DecodeMaps M) {
       for (long long ti = lo; ti < hi; ++ti, ++n) {
         advance(ti);
         const int st = n % kStages;
-        if (n >= kStages && !mbar_wait(&sh.empty[st], (unsigned)(n / kStages - 1) & 1u)) { ok = false; break; }
+        if (n >= kStages && !mbar::wait(&sh.empty[st], (unsigned)(n / kStages - 1) & 1u)) { ok = false; break; }
         unsigned char *dst = smem + st * kStageBytes;
-        mbar_expect_tx(&sh.full[st], (unsigned)kStageBytes);
+        mbar::expect_tx(&sh.full[st], (unsigned)kStageBytes);
         const int lt = (int)(ti - line);
         if (lt < s.tiles_main) {
           const int r = (int)(s.off0 + (long long)lt * kTile);
@@ -329,7 +304,7 @@ k_decode(const DecodeParams P, const __grid_constant__ DecodeMaps M) {
       if (!ok) {
         atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
         for (int i = n > kStages ? n - kStages : 0; i < n; ++i)
-          mbar_wait(&sh.full[i % kStages], (unsigned)(i / kStages) & 1u);
+          mbar::wait(&sh.full[i % kStages], (unsigned)(i / kStages) & 1u);
       }
     }
     return;
@@ -366,8 +341,8 @@ k_decode(const DecodeParams P, const __grid_constant__ DecodeMaps M) {
     for (; ti < seg_end; ++ti, ++n) {
       if (failed) continue;
       const int st = n % kStages;
-      if (!mbar_wait(&sh.full[st], (unsigned)(n / kStages) & 1u)) {
-        // a load did not arrive in time: say so and report an empty share
+      if (!mbar::wait_warp(&sh.full[st], (unsigned)(n / kStages) & 1u)) {
+        // a load did not arrive in time (for any lane): say so and report an empty share
         failed = true;
         if (lane == 0) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
         continue;
@@ -448,7 +423,7 @@ k_decode(const DecodeParams P, const __grid_constant__ DecodeMaps M) {
         }
       }
       __syncwarp();
-      if (lane == 0) mbar_arrive(&sh.empty[st]);             // this warp is through with the stage
+      if (lane == 0) mbar::arrive(&sh.empty[st]);             // this warp is through with the stage
     }
     if (failed) {
       m[0] = m[1] = -INFINITY;

@@ -156,3 +156,15 @@ def test_decode_rejects_bad_arguments(fc):
         assert e.value.code == 3
     finally:
         fc.fc_destroy(h)
+
+
+def test_a_warp_that_waits_in_vain_gives_up_as_one(fc):
+    # half of the lanes' barrier is complete, the other half's never will be: the warp's collective instructions may only
+    # follow if every lane gets the same verdict (lanes that disagree would be reported as FC_ERR_INTERNAL, 6)
+    h = fc.fc_create(0, 64)
+    try:
+        for _ in range(3):
+            fc.fc_selftest_bounded_wait(h)
+            assert fc.fc_last_device_status(h) == 5                 # FC_ERR_TIMEOUT
+    finally:
+        fc.fc_destroy(h)
