@@ -120,9 +120,10 @@ fc_status fc_proto_dft16_stage(fc_handle *h, const void *x, void *y, int32_t nco
 
 /* Self test of the failure path of the bounded device-side waits (diagnostic; the paper has no
  * counterpart): enqueues one small kernel in which half of a warp waits, at most 1000 tries, on a barrier
- * nothing will ever complete, gives up, and the warp as a whole records it.  The next fc_last_device_status
- * returns FC_ERR_TIMEOUT (FC_ERR_INTERNAL if the warp's lanes disagreed); the context stays usable (nothing
- * traps, nothing spins without a limit). */
+ * nothing will ever complete, gives up, and the warp as a whole records it, while another thread issues loads
+ * nobody consumes and waits for them before the block ends.  The next fc_last_device_status returns
+ * FC_ERR_TIMEOUT (FC_ERR_INTERNAL if the warp's lanes disagreed or a load was missing); the context stays
+ * usable (nothing traps, nothing spins without a limit). */
 fc_status fc_selftest_bounded_wait(fc_handle *h, fc_stream stream);
 
 /* Number of kernels this handle has launched since fc_create (diagnostic). */

@@ -36,21 +36,44 @@ __global__ void __launch_bounds__(256) k_fma_probe(float *out, int iters, float 
   out[blockIdx.x * blockDim.x + threadIdx.x] = s;
 }
 
-// Self test of the failure path of the bounded device-side waits.  One warp waits, half of its lanes on a barrier that is
-// complete and half on one that nothing ever arrives on: the latter give up after `limit` tries, every lane must get that
+// Self test of the failure path of the bounded device-side waits.  The first warp waits, half of its lanes on a barrier that
+// is complete and half on one that nothing ever arrives on: the latter give up after `limit` tries, every lane must get that
 // verdict, and the timeout is recorded in the status word.  A verdict that differs from lane to lane is an internal error.
-__global__ void k_selftest_bounded_wait(int *status, unsigned limit) {
-  __shared__ unsigned long long complete, never;
+// Meanwhile a thread of the second warp loads five pieces of `src` into a ring of three stages, none of which anyone
+// consumes, and drains it: what was loaded last into each stage must be there afterwards.
+__global__ void k_selftest_bounded_wait(int *status, unsigned limit, const float2 *src) {
+  constexpr int S = 3, ITEMS = 5, PIECE = 16;                 // PIECE float2 values: 128 bytes
+  __shared__ __align__(128) float2 ring[S][PIECE];
+  __shared__ unsigned long long complete, never, full[S];
   if (threadIdx.x == 0) {
     mbar::init(&complete, 1u);
     mbar::init(&never, 1u);
+    for (int i = 0; i < S; ++i) mbar::init(&full[i], 1u);
     mbar::init_done();
     mbar::arrive(&complete);
   }
   __syncthreads();
-  const bool ok = mbar::wait_warp(threadIdx.x & 1 ? &never : &complete, 0u, limit);
-  const unsigned through = __ballot_sync(0xffffffffu, ok);
-  if (threadIdx.x == 0) atomicOr(status, through == 0u ? FC_DEV_FLAG_TIMEOUT : FC_DEV_FLAG_INTERNAL);
+  if (threadIdx.x < 32) {
+    const bool ok = mbar::wait_warp(threadIdx.x & 1 ? &never : &complete, 0u, limit);
+    const unsigned through = __ballot_sync(0xffffffffu, ok);
+    if (threadIdx.x == 0) atomicOr(status, through == 0u ? FC_DEV_FLAG_TIMEOUT : FC_DEV_FLAG_INTERNAL);
+  } else if (threadIdx.x == 32) {
+    bool good = true;
+    for (int i = 0; i < ITEMS; ++i) {
+      if (i >= S) good &= mbar::wait(&full[i % S], (unsigned)(i / S - 1) & 1u);
+      mbar::expect_tx(&full[i % S], (unsigned)sizeof(ring[0]));
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+                   ::"r"(mbar::address(ring[i % S])), "l"(__cvta_generic_to_global(src + i * PIECE)),
+                     "r"((unsigned)sizeof(ring[0])), "r"(mbar::address(&full[i % S])) : "memory");
+    }
+    good &= mbar::drain(full, ITEMS);
+    for (int i = ITEMS - S; i < ITEMS; ++i)
+      for (int e = 0; e < PIECE; ++e) {
+        const float2 a = ring[i % S][e], b = src[i * PIECE + e];
+        good &= a.x == b.x && a.y == b.y;
+      }
+    if (!good) atomicOr(status, FC_DEV_FLAG_INTERNAL);
+  }
 }
 
 }  // namespace
@@ -331,7 +354,7 @@ done:
 
 extern "C" fc_status fc_selftest_bounded_wait(fc_handle *h, fc_stream stream) {
   if (!h) return FC_ERR_INVALID_ARG;
-  k_selftest_bounded_wait<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(h->status_word, 1000u);
+  k_selftest_bounded_wait<<<1, 64, 0, static_cast<cudaStream_t>(stream)>>>(h->status_word, 1000u, h->master);
   return fc_after_launch(h);
 }
 

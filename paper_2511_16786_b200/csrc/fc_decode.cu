@@ -300,12 +300,10 @@ k_decode(const DecodeParams P, const __grid_constant__ DecodeMaps M) {
           tma_load_4d(dst + 3 * kBoxBytes, &M.tv, 64, h, r, b, &sh.full[st]);
         }
       }
-      // a consumer gave up: the loads still in flight write this block's shared memory, give them a bounded chance
-      if (!ok) {
-        atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
-        for (int i = n > kStages ? n - kStages : 0; i < n; ++i)
-          mbar::wait(&sh.full[i % kStages], (unsigned)(i / kStages) & 1u);
-      }
+      // not before its loads have landed may the block end, also where consumers gave up (they no longer wait for them);
+      // where none did, this waits for what the consumers wait for
+      if (!mbar::drain(sh.full, n)) ok = false;
+      if (!ok) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
     }
     return;
   }

@@ -40,4 +40,14 @@ __device__ __forceinline__ bool wait_warp(unsigned long long *bar, unsigned pari
   return __all_sync(0xffffffffu, wait(bar, parity, limit)) != 0;
 }
 
+// A ring of S stages, item i in stage i % S: waits (bounded, S limits at most) for the loads of the last items of `issued`,
+// each of which is the last one its stage was given.  Whoever issued loads into a block's shared memory calls this before
+// it ends, whatever the consumers did: a block that has gone may have its memory given to another one.
+template <int S>
+__device__ __forceinline__ bool drain(unsigned long long (&full)[S], int issued, unsigned limit = kSpinLimit) {
+  bool landed = true;
+  for (int i = issued > S ? issued - S : 0; i < issued; ++i) landed &= wait(&full[i % S], (unsigned)(i / S) & 1u, limit);
+  return landed;
+}
+
 }  // namespace mbar

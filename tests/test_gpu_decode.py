@@ -168,3 +168,20 @@ def test_a_warp_that_waits_in_vain_gives_up_as_one(fc):
             assert fc.fc_last_device_status(h) == 5                 # FC_ERR_TIMEOUT
     finally:
         fc.fc_destroy(h)
+
+
+def test_loads_nobody_consumes_have_landed_before_the_block_ends(fc):
+    # the self test's second half: five loads into a ring of three stages that no one empties, then the wait that the
+    # decoding kernel's producer ends with; a piece that is not there afterwards would be reported as FC_ERR_INTERNAL.
+    # Then the shapes in which the producer has issued everything before the first tile is used: one to five tiles a block
+    h = fc.fc_create(0, 64)
+    try:
+        for _ in range(20):
+            fc.fc_selftest_bounded_wait(h)
+        assert fc.fc_last_device_status(h) == 5                     # FC_ERR_TIMEOUT of the other half
+    finally:
+        fc.fc_destroy(h)
+    for rows in (64, 64 * 148 * 3, 64 * 148 * 4, 64 * 148 * 4 + 1, 64 * 148 * 5):
+        q, ck, cv = _inputs(rows, 1, 1, 4, torch.bfloat16, rows)
+        got = _run(fc, q, ck, cv, [0, rows])
+        _check(got, O.decode_attention(q.double().numpy(), ck.double().numpy(), cv.double().numpy(), [0, rows]))
