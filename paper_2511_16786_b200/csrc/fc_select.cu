@@ -431,6 +431,8 @@ select_gather_body(const float *__restrict__ scores, long long T, const SeqTable
     }
     tau = prefix;
     need = krem;
+  } else if (CL > 1) {
+    cluster.sync();      // every block has started (elsewhere the digits' barriers see to it): the totals below go to all
   }
 
   // greater and tied keys of every run of 32 tokens, their exclusive prefix sums, the block's totals

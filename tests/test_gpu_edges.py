@@ -149,3 +149,26 @@ def test_selection_of_many_short_sequences(fc, lens):
             assert torch.equal(out_k[:, hd], k[at, hd]) and torch.equal(out_v[:, hd], k[at, hd])
     finally:
         fc.fc_destroy(h)
+
+
+# every token kept by clusters of two, four and eight blocks, more of them than run at a time: no digit is counted, so
+# nothing but its own barrier lets a block write into its neighbours' memory
+@pytest.mark.parametrize("n,batch,per_layer", [(300, 200, True), (16385, 60, False), (32769, 24, True), (65537, 10, False)])
+def test_selection_that_keeps_every_token_in_clusters(fc, n, batch, per_layer):
+    H, d, cu = 2, 64, [i * n for i in range(batch + 1)]
+    g = torch.Generator(device="cuda").manual_seed(n)
+    k = torch.randn((cu[-1], H, d), generator=g, device="cuda").half()
+    scores = torch.rand((H, cu[-1]), generator=g, device="cuda")
+    h = fc.fc_create(0, 131072)
+    try:
+        ws = torch.empty(fc.fc_select_workspace_bytes(h, k, k, cu), dtype=torch.uint8, device="cuda")
+        out_k = torch.zeros_like(k)
+        out_v, idx = torch.zeros_like(k), torch.full((H, cu[-1]), -1, dtype=torch.int32, device="cuda")
+        fc.fc_select_compact_ex(h, k, k, cu, scores, torch.full((batch,), n, dtype=torch.int32, device="cuda"),
+                                torch.tensor(cu, dtype=torch.int64, device="cuda"), out_k, out_v, idx, ws,
+                                per_layer=per_layer)
+        assert fc.fc_last_device_status(h) == 0
+        assert torch.equal(idx, torch.arange(n, dtype=torch.int32, device="cuda").repeat(H, batch))
+        assert torch.equal(out_k, k) and torch.equal(out_v, k)
+    finally:
+        fc.fc_destroy(h)
