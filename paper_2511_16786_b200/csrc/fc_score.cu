@@ -1860,6 +1860,7 @@ k_cutoff_from_spectrum(const double *__restrict__ spectrum, const __grid_constan
     if (rank == 0 && threadIdx.x == 0) { omega[b] = 0; gamma[b] = 0.0; }
     return;
   }
+  cluster.barrier_arrive();
   const double *P = spectrum + 2 * (size_t)s0;
   const int len = ((N + kCutSegs - 1) / kCutSegs + 31) & ~31;       // bins per segment
   {
@@ -1869,6 +1870,7 @@ k_cutoff_from_spectrum(const double *__restrict__ spectrum, const __grid_constan
 #pragma unroll 8
     for (int m = lo + lane; m < hi; m += 32) a += P[2 * m] + P[2 * m + 1];
     a = warp_sum_d(a);
+    cluster.barrier_wait();                           // the first block has started: its memory may be written
     if (lane == 0) *cluster.map_shared_rank(&seg_sum[sg], 0) = a;
   }
   cluster.sync();

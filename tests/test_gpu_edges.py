@@ -172,3 +172,33 @@ def test_selection_that_keeps_every_token_in_clusters(fc, n, batch, per_layer):
         assert torch.equal(out_k, k) and torch.equal(out_v, k)
     finally:
         fc.fc_destroy(h)
+
+
+# more sequences than clusters run at a time (and than one launch describes), short and long in turn, so that clusters start
+# while others end: every block may write to its cluster's first one only once that has started
+def test_cutoff_of_many_sequences(fc):
+    rng = np.random.default_rng(3)
+    lens = [int(n) for n in rng.integers(1, 9000, 150)]
+    lens[7] = lens[80] = 0
+    cu = [0] + [int(x) for x in np.cumsum(lens)]
+    P = rng.random((cu[-1], 2)) * np.exp(-rng.random((cu[-1], 1)) * 6.0)
+    h = fc.fc_create(0, 9000)
+    try:
+        om = torch.full((150,), -7, dtype=torch.int32, device="cuda")
+        ga = torch.full((150,), -7.0, dtype=torch.float64, device="cuda")
+        fc.fc_cutoff_from_spectrum(h, torch.from_numpy(P).cuda(), cu, 0.7, om, ga)
+        assert fc.fc_last_device_status(h) == 0
+        om, ga = om.cpu().numpy(), ga.cpu().numpy()
+    finally:
+        fc.fc_destroy(h)
+    for b, n in enumerate(lens):
+        if n == 0:
+            assert om[b] == 0 and ga[b] == 0.0
+            continue
+        seg = P[cu[b]:cu[b + 1]]
+        wo, wg = O.cutoff_for_energy_share(seg, 0.7)
+        if om[b] != wo:                                      # only where rounding of the running sum decides
+            c, tot = np.cumsum(seg.sum(1)), seg.sum()
+            assert abs(c[min(om[b], wo)] - 0.7 * tot) <= 1e-12 * tot
+        else:
+            assert ga[b] == wg
