@@ -667,6 +667,12 @@ fc_status launch_select(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, con
     // with one block, 18.4 with eight).  Two where a layer keeps one index set, whose few clusters gather all heads.
     int cl = per_layer ? 2 : 1;
     while (cl < kSelCluster && nmax > cl * 1024 * kSelKptMax) cl *= 2;
+    // But a block also gathers the rows it chose, so where the clusters would leave most of the SMs idle, sequences of
+    // more than 2048 tokens get two blocks and of more than 4096 four (one layer of 4 heads of 4096, 8192, 16384 tokens:
+    // 23.5 -> 19.5, 35.8 -> 23.4, 62.5 -> 29.6 us; 64 heads of 16384 with two: 68.6 -> 56.3).  Not with eight, whose
+    // clusters run 15 at a time, and not to the last SM: 36 clusters of four do not fit at once (32768 tokens: 53 -> 68).
+    const long long units = (long long)nseq * kv->num_heads * nl;
+    while (!per_layer && cl < 4 && nmax > 2048 * cl && units * 2 * cl <= h->num_sms - h->num_sms / 8) cl *= 2;
     int kpt = 2;
     while (kpt < kSelKptMax && nmax > cl * 1024 * kpt) kpt *= 2;
     // Short sequences in more blocks than SMs: fewer threads with more scores each, so that several blocks share an SM
@@ -674,7 +680,7 @@ fc_status launch_select(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, con
     // 62 -> 43 us, of 300 34 -> 15, 28 x 4 heads of 8 ragged sequences up to 2311 69 -> 60.  Not beyond 4096 tokens,
     // where the gather fills the time (8192: 128 -> 137, 16384: 1.12 -> 1.20 ms).
     int nt = 1024;
-    if (!per_layer && kpt <= 4 && (long long)nseq * kv->num_heads * nl > h->num_sms) {
+    if (!per_layer && kpt <= 4 && units > h->num_sms) {
       nt = nmax <= 1024 ? 256 : 512;
       kpt = nmax <= 2048 ? 4 : 8;
     }
@@ -705,7 +711,9 @@ fc_status launch_select(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, con
       cudaError_t launch_err = cudaErrorInvalidValue;
       if (false) {}
       FC_SEL_CASE(2, false, 1) FC_SEL_CASE(4, false, 1) FC_SEL_CASE(8, false, 1) FC_SEL_CASE(16, false, 1)
-      FC_SEL_CASE(16, false, 2) FC_SEL_CASE(16, false, 4) FC_SEL_CASE(16, false, 8)
+      FC_SEL_CASE(2, false, 2) FC_SEL_CASE(4, false, 2) FC_SEL_CASE(8, false, 2) FC_SEL_CASE(16, false, 2)
+      FC_SEL_CASE(2, false, 4) FC_SEL_CASE(4, false, 4) FC_SEL_CASE(8, false, 4) FC_SEL_CASE(16, false, 4)
+      FC_SEL_CASE(16, false, 8)
       FC_SEL_CASE(2, true, 2) FC_SEL_CASE(4, true, 2) FC_SEL_CASE(8, true, 2) FC_SEL_CASE(16, true, 2)
       FC_SEL_CASE(16, true, 4) FC_SEL_CASE(16, true, 8)
       FC_SEL_MANY(4, 256) FC_SEL_MANY(4, 512) FC_SEL_MANY(8, 512)

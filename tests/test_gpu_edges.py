@@ -202,3 +202,31 @@ def test_cutoff_of_many_sequences(fc):
             assert abs(c[min(om[b], wo)] - 0.7 * tot) <= 1e-12 * tot
         else:
             assert ga[b] == wg
+
+
+# few (sequence, head) pairs: one, two and four blocks each by length, around the numbers of pairs whose clusters fit
+# at once (33 pairs of 4, 65 of 2 on 148 SMs do not)
+@pytest.mark.parametrize("n", [2048, 2049, 4096, 4097, 8193, 16384, 16385])
+@pytest.mark.parametrize("H", [1, 32, 33, 64, 65])
+def test_selection_of_few_heads_takes_clusters(fc, n, H):
+    rng = np.random.default_rng(n + H)
+    d = 64
+    scores = (rng.integers(0, 1 << 11, (H, n)) * 2.0 ** -9).astype(np.float32)          # many ties
+    g = torch.Generator(device="cuda").manual_seed(n)
+    k = torch.randn((n, H, d), generator=g, device="cuda").half()
+    budget, cu = n // 3, [0, n]
+    h = fc.fc_create(0, 16385)
+    try:
+        ws = torch.empty(fc.fc_select_workspace_bytes(h, k, k, cu), dtype=torch.uint8, device="cuda")
+        out_k = torch.zeros((budget, H, d), dtype=k.dtype, device="cuda")
+        out_v, idx = torch.zeros_like(out_k), torch.full((H, budget), -1, dtype=torch.int32, device="cuda")
+        fc.fc_select_compact_ex(h, k, k, cu, torch.from_numpy(scores).cuda(),
+                                torch.tensor([budget], dtype=torch.int32, device="cuda"),
+                                torch.tensor([0, budget], dtype=torch.int64, device="cuda"), out_k, out_v, idx, ws)
+        assert fc.fc_last_device_status(h) == 0
+        for hd in {0, H // 2, H - 1}:
+            np.testing.assert_array_equal(idx[hd].cpu().numpy(), O.select_topk(scores[hd].astype(np.float64), budget))
+            at = idx[hd].long()
+            assert torch.equal(out_k[:, hd], k[at, hd]) and torch.equal(out_v[:, hd], k[at, hd])
+    finally:
+        fc.fc_destroy(h)
