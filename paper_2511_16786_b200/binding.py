@@ -9,6 +9,7 @@ raises on import.
 from __future__ import annotations
 
 import ctypes
+import operator
 import os
 from ctypes import POINTER, byref, c_char_p, c_double, c_int, c_int32, c_int64, c_size_t, c_uint64, c_void_p
 
@@ -506,6 +507,10 @@ def fc_select_compact_layers(handle, K_layers, V_layers, cu_seqlens, scores, bud
 # ----------------------------------------------------------------------------
 # convenience: buffers for a whole model and the three-phase pass
 # ----------------------------------------------------------------------------
+_data_ptr, _strides = torch.Tensor.data_ptr, torch.Tensor.stride
+_shape_and_dtype = operator.attrgetter("shape", "dtype")
+
+
 class Compressor:
     """Owns a handle and the device buffers of one workload shape; `compress`
     issues fc_score_layer x L, fc_allocate_budgets, fc_select_compact x L on the
@@ -546,6 +551,7 @@ class Compressor:
         self.out_v = None
         self.out_idx = None
         self._ws = None
+        self._m = self._mkey = self._mbuffers = None
 
     def close(self):
         if self.handle is not None:
@@ -568,21 +574,42 @@ class Compressor:
         return self._ws
 
     def _outputs(self, per_layer_capacity: int):
-        if self.out_k is None or self.out_k.shape[1] < per_layer_capacity:
+        if self.out_k is None or min(self.out_k.shape[1], self.out_v.shape[1], self.out_idx.shape[2]) < per_layer_capacity:
             dev = self.device
             self.out_k = torch.empty((self.L, per_layer_capacity, self.H, self.d), dtype=self.dtype, device=dev)
             self.out_v = torch.empty_like(self.out_k)
             self.out_idx = torch.empty((self.L, self.H, per_layer_capacity), dtype=torch.int32, device=dev)
 
-    # The per-layer calls below go straight to the C entry points with arguments that are marshalled
-    # once per set of tensors (views, pointers, the cu_seqlens array): the per-call Python work would
-    # otherwise cost more than the selection kernels it launches.
+    # The C entry points get arguments that are marshalled once per set of tensors (views, pointers, the cu_seqlens
+    # array): the Python work would otherwise cost more than the kernels of short calls.  A set is known by everything
+    # that goes into the arguments: address, strides, shape and dtype of every input, address of every buffer.
+    def _arguments_key(self, K_layers, V_layers):
+        key = []
+        for tensors in (K_layers, V_layers):
+            key += map(_data_ptr, tensors)
+            key += map(_strides, tensors)
+            key += map(_shape_and_dtype, tensors)
+        return key
+
+    def _buffers_key(self):
+        return [0 if t is None else t.data_ptr() for t in (self.scores, self.energy, self.budgets, self.offsets,
+                                                           self.out_k, self.out_v, self.out_idx, self._ws)]
+
     def _marshal(self, K_layers, V_layers):
-        key = tuple(k.data_ptr() for k in K_layers) + tuple(v.data_ptr() for v in V_layers)
-        if getattr(self, "_mkey", None) == key and self._m_out == (id(self.out_k), id(self._ws)):
+        key = self._arguments_key(K_layers, V_layers)
+        if self._mkey == key and self._mbuffers == self._buffers_key():
             return self._m
+        if len(K_layers) != self.L or len(V_layers) != self.L:
+            raise ValueError("one K and one V tensor per layer")
+        size = self.dtype.itemsize
+        for k in K_layers:
+            if k.dim() != 3 or k.shape[0] < self.T or tuple(k.shape[1:]) != (self.H, self.d) or k.element_size() != size:
+                raise ValueError("expected [T, H, d] tensors with elements of the compressor's size")
         ws = self._workspace(K_layers[0], V_layers[0])
         self._outputs(self.capacity)
+        cap = int(self.out_idx.shape[2])
+        if min(self.out_k.shape[1], self.out_v.shape[1]) < cap:
+            raise ValueError("out_k and out_v need as many rows as out_idx has entries")
         cu = _cu_array(self.cu)
         views = [make_view(K_layers[l], V_layers[l], cu) for l in range(self.L)]
         P = c_void_p
@@ -596,7 +623,8 @@ class Compressor:
             out_k=[P(self.out_k[l].data_ptr()) for l in range(self.L)],
             out_v=[P(self.out_v[l].data_ptr()) for l in range(self.L)],
             out_idx=[P(self.out_idx[l].data_ptr()) for l in range(self.L)],
-            cap=int(self.out_k.shape[1]))
+            cap=cap, all_energy=P(self.energy.data_ptr()), all_budgets=P(self.budgets.data_ptr()),
+            all_offsets=P(self.offsets.data_ptr()), cu_ptr=ctypes.cast(cu, POINTER(c_int32)))
         tab = (fc_layer_buffers * self.L)()
         for l in range(self.L):
             tab[l] = fc_layer_buffers(K_layers[l].data_ptr(), V_layers[l].data_ptr(), self.scores[l].data_ptr(),
@@ -606,15 +634,16 @@ class Compressor:
         # layers laid out alike are scored in one call
         m["alike"] = all((k.stride(), v.stride(), k.dtype) == (K_layers[0].stride(), V_layers[0].stride(), K_layers[0].dtype)
                          for k, v in zip(K_layers, V_layers))
-        self._m, self._mkey, self._m_out = m, key, (id(self.out_k), id(self._ws))
+        self._m, self._mkey, self._mbuffers = m, key, self._buffers_key()
         return m
 
     def score(self, K_layers, V_layers):
-        m = self._marshal(K_layers, V_layers)
-        st, h, gamma = _stream(), self.handle, c_double(self.gamma)
+        self._score(self._marshal(K_layers, V_layers), _stream())
+
+    def _score(self, m, st):
+        h, gamma = self.handle, self.gamma
         if m["alike"]:
-            rc = _lib.fc_score_layers(h, m["refs"][0], m["layers"], self.L, gamma, c_void_p(self.energy.data_ptr()),
-                                      m["ws"], m["ws_bytes"], st)
+            rc = _lib.fc_score_layers(h, m["refs"][0], m["layers"], self.L, gamma, m["all_energy"], m["ws"], m["ws_bytes"], st)
             if rc != FC_OK:
                 raise FlashCacheError(rc, "fc_score_layers")
             return
@@ -629,12 +658,14 @@ class Compressor:
                             self.budgets, self.offsets)
 
     def select_compact(self, K_layers, V_layers, one_launch: bool = True):
-        m = self._marshal(K_layers, V_layers)
-        st, h = _stream(), self.handle
+        self._select_compact(self._marshal(K_layers, V_layers), _stream(), one_launch)
+
+    def _select_compact(self, m, st, one_launch: bool = True):
+        h = self.handle
         opt = byref(self._opt)
         if one_launch:         # every layer side by side (fc_select_compact_layers)
-            rc = _lib.fc_select_compact_layers(h, m["refs"][0], m["layers"], self.L, c_void_p(self.budgets.data_ptr()),
-                                               c_void_p(self.offsets.data_ptr()), opt, m["ws"], m["ws_bytes"], st)
+            rc = _lib.fc_select_compact_layers(h, m["refs"][0], m["layers"], self.L, m["all_budgets"], m["all_offsets"], opt,
+                                               m["ws"], m["ws_bytes"], st)
             if rc != FC_OK:
                 raise FlashCacheError(rc, "fc_select_compact_layers")
             return
@@ -646,9 +677,13 @@ class Compressor:
                 raise FlashCacheError(rc, "fc_select_compact_ex")
 
     def compress(self, K_layers, V_layers):
-        self.score(K_layers, V_layers)
-        self.allocate()
-        self.select_compact(K_layers, V_layers)
+        m, st = self._marshal(K_layers, V_layers), _stream()
+        self._score(m, st)
+        rc = _lib.fc_allocate_budgets(self.handle, m["all_energy"], self.L, self.B, m["cu_ptr"], self.rho, self.min_keep,
+                                      m["all_budgets"], m["all_offsets"], st)
+        if rc != FC_OK:
+            raise FlashCacheError(rc, "fc_allocate_budgets")
+        self._select_compact(m, st)
 
     def capture(self, K_layers, V_layers):
         """The whole `compress` sequence on these tensors as a CUDA graph (torch.cuda.CUDAGraph): one
