@@ -337,6 +337,12 @@ def fc_score_layer(handle, k, v, cu_seqlens, gamma: float, scores, energy, works
                                workspace.numel() * workspace.element_size(), _stream()), "fc_score_layer")
 
 
+def _alike(K_layers, V_layers) -> bool:
+    """Whether one layer's view describes all of them."""
+    first = (K_layers[0].stride(), K_layers[0].shape[1:], K_layers[0].dtype)
+    return all((t.stride(), t.shape[1:], t.dtype) == first for ts in (K_layers, V_layers) for t in ts)
+
+
 def fc_score_layers_workspace_bytes(handle, k, v, cu_seqlens, num_layers: int) -> int:
     cu = _cu_array(cu_seqlens)
     view = make_view(k, v, cu)
@@ -346,6 +352,8 @@ def fc_score_layers_workspace_bytes(handle, k, v, cu_seqlens, num_layers: int) -
 def fc_score_layers(handle, K_layers, V_layers, cu_seqlens, gamma: float, scores, energy, workspace) -> None:
     """fc_score_layer for all layers (one layout) in one call.  scores: float32 [L, H, T]; energy: float64 [L, B, 4]."""
     L = len(K_layers)
+    if len(V_layers) != L or not _alike(K_layers, V_layers):
+        raise ValueError("layers of one layout: the same strides, heads, channels and dtype")
     cu = _cu_array(cu_seqlens)
     view = make_view(K_layers[0], V_layers[0], cu)
     tab = (fc_layer_buffers * L)()
@@ -489,6 +497,8 @@ def fc_select_compact_layers(handle, K_layers, V_layers, cu_seqlens, scores, bud
     """All layers in one launch.  scores [L, H, T]; budgets [L, B]; out_offsets [L, B+1];
     out_k / out_v [L, capacity, H, d]; out_idx [L, H, capacity]."""
     L = len(K_layers)
+    if len(V_layers) != L or not _alike(K_layers, V_layers):
+        raise ValueError("layers of one layout: the same strides, heads, channels and dtype")
     cu = _cu_array(cu_seqlens)
     view = make_view(K_layers[0], V_layers[0], cu)
     cap = int(out_k.shape[1])
@@ -631,9 +641,8 @@ class Compressor:
                                       self.out_k[l].data_ptr(), self.out_v[l].data_ptr(),
                                       self.out_idx[l].data_ptr(), m["cap"])
         m["layers"] = tab
-        # layers laid out alike are scored in one call
-        m["alike"] = all((k.stride(), v.stride(), k.dtype) == (K_layers[0].stride(), V_layers[0].stride(), K_layers[0].dtype)
-                         for k, v in zip(K_layers, V_layers))
+        # layers laid out alike are scored in one call and selected in one launch
+        m["alike"] = _alike(K_layers, V_layers)
         self._m, self._mkey, self._mbuffers = m, key, self._buffers_key()
         return m
 
@@ -663,7 +672,7 @@ class Compressor:
     def _select_compact(self, m, st, one_launch: bool = True):
         h = self.handle
         opt = byref(self._opt)
-        if one_launch:         # every layer side by side (fc_select_compact_layers)
+        if one_launch and m["alike"]:         # every layer side by side (fc_select_compact_layers)
             rc = _lib.fc_select_compact_layers(h, m["refs"][0], m["layers"], self.L, m["all_budgets"], m["all_offsets"], opt,
                                                m["ws"], m["ws_bytes"], st)
             if rc != FC_OK:

@@ -86,3 +86,20 @@ def test_tensors_that_do_not_fit_are_refused(fc):
     c.compress(K, V)
     assert _same(_results(c), _fresh(fc, K, V))
     c.close()
+
+
+def test_layers_of_unlike_layouts(fc):
+    # one layer token-major, one head-major: each is read by its own strides, in the selection too
+    mem = _tensors(4)
+    K = [mem[0], mem[1].view(H, T, D).transpose(0, 1)]
+    V = [mem[2], mem[3].view(H, T, D).transpose(0, 1)]
+    c = _compressor(fc)
+    c.compress(K, V)
+    assert _same(_results(c), _fresh(fc, K, V))
+    # the entry points that describe all layers by one view refuse them
+    cu = [0, T]
+    with pytest.raises(ValueError):
+        fc.fc_score_layers(c.handle, K, V, cu, 0.2, c.scores, c.energy, c._ws)
+    with pytest.raises(ValueError):
+        fc.fc_select_compact_layers(c.handle, K, V, cu, c.scores, c.budgets, c.offsets, c.out_k, c.out_v, c.out_idx, c._ws)
+    c.close()
