@@ -704,9 +704,9 @@ extern "C" fc_status fc_decode_attention(fc_handle *h, const fc_decode_args *a, 
   if (!out || ((uintptr_t)out & 15)) return FC_ERR_INVALID_ARG;
   const DecodePlan pl = plan_decode(h, a);
   if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < pl.total) return FC_ERR_WORKSPACE;
-  int dev = -1;
-  FC_CUDA_TRY(cudaGetDevice(&dev));
-  if (dev != h->device) FC_CUDA_TRY(cudaSetDevice(h->device));
+  // always set, not only where it differs: in a thread that has made no CUDA call yet device 0 is current but no context is,
+  // and the tensor maps are encoded by the driver, which wants one
+  FC_CUDA_TRY(cudaSetDevice(h->device));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if ((s = fc_flush_pending(h, st)) != FC_OK) return s;
   if (a->dtype == FC_F16) return launch_decode<__half>(h, a, pl, out, static_cast<char *>(workspace), st);

@@ -185,3 +185,32 @@ def test_loads_nobody_consumes_have_landed_before_the_block_ends(fc):
         q, ck, cv = _inputs(rows, 1, 1, 4, torch.bfloat16, rows)
         got = _run(fc, q, ck, cv, [0, rows])
         _check(got, O.decode_attention(q.double().numpy(), ck.double().numpy(), cv.double().numpy(), [0, rows]))
+
+
+def test_a_thread_whose_first_cuda_call_is_a_decoding_step(fc):
+    import threading
+    q, ck, cv = _inputs(200, 1, 2, 2, torch.float16, 9)
+    h = fc.fc_create(0, 64)
+    try:
+        qd, kd, vd, off = q.cuda(), ck.cuda(), cv.cuda(), torch.tensor([0, 200], device="cuda")
+        args = fc.make_decode_args(qd, kd, vd, off, 200)
+        ws = torch.empty(fc.fc_decode_workspace_bytes(h, args), dtype=torch.uint8, device="cuda")
+        out = torch.full_like(qd, float("nan"))
+        torch.cuda.synchronize()
+        raised = []
+
+        def step():
+            try:
+                fc.fc_decode_attention(h, args, out, ws)
+            except Exception as e:
+                raised.append(e)
+
+        t = threading.Thread(target=step)
+        t.start()
+        t.join()
+        assert not raised, raised
+        assert fc.fc_last_device_status(h) == 0
+        torch.cuda.synchronize()
+        _check(out.double().cpu().numpy(), O.decode_attention(q.double().numpy(), ck.double().numpy(), cv.double().numpy(), [0, 200]))
+    finally:
+        fc.fc_destroy(h)
