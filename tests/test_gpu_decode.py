@@ -214,3 +214,44 @@ def test_a_thread_whose_first_cuda_call_is_a_decoding_step(fc):
         _check(out.double().cpu().numpy(), O.decode_attention(q.double().numpy(), ck.double().numpy(), cv.double().numpy(), [0, 200]))
     finally:
         fc.fc_destroy(h)
+
+
+_THREADS = r"""
+import sys, threading
+sys.path.insert(0, sys.argv[1])
+import torch
+from paper_2511_16786_b200 import binding as fc
+n = 8
+jobs = []
+for i in range(n):
+    h = fc.fc_create(0, 64)
+    q, k, v = (torch.randn(s, device="cuda").half() for s in ((1, 4, 128), (200, 2, 128), (200, 2, 128)))
+    off = torch.tensor([0, 200], device="cuda")
+    a = fc.make_decode_args(q, k, v, off, 200)
+    ws = torch.empty(fc.fc_decode_workspace_bytes(h, a), dtype=torch.uint8, device="cuda")
+    jobs.append((h, a, torch.empty_like(q), ws, torch.cuda.Stream(), (q, k, v, off)))
+torch.cuda.synchronize()
+gate, bad = threading.Barrier(n), []
+def go(job):
+    h, a, out, ws, st, _ = job
+    gate.wait()
+    try:
+        with torch.cuda.stream(st):
+            fc.fc_decode_attention(h, a, out, ws)
+    except Exception as e:
+        bad.append(str(e))
+ts = [threading.Thread(target=go, args=(j,)) for j in jobs]
+[t.start() for t in ts]
+[t.join() for t in ts]
+torch.cuda.synchronize()
+assert not bad, bad
+assert all(fc.fc_last_device_status(j[0]) == 0 and bool(j[2].isfinite().all()) for j in jobs)
+"""
+
+
+def test_first_calls_from_several_threads(fc, repo_root):
+    # a handle each; what the library looks up on its first decoding call is there for all of them
+    import subprocess
+    import sys
+    r = subprocess.run([sys.executable, "-c", _THREADS, repo_root], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
