@@ -170,7 +170,7 @@ extern "C" fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen) 
   h->score_overlap = 0;
   h->band_form = 1;
   h->step = 0;
-  h->last_sig = 0;
+  h->last_carve = FcCarve{};
   h->pending_join = false;
   for (int a = 0; a < 2; ++a) for (int b = 0; b < FC_MAX_AUX; ++b) h->ev_done[a][b] = nullptr;
   cudaDeviceProp prop;
@@ -396,7 +396,7 @@ extern "C" fc_status fc_set_l2_persist(fc_handle *h, int32_t enabled) {
 extern "C" fc_status fc_reset_ordering(fc_handle *h) {
   if (!h) return FC_ERR_INVALID_ARG;
   h->step = 0;
-  h->last_sig = 0;
+  h->last_carve = FcCarve{};
   h->pending_join = false;
   h->host_last_arena = nullptr;
   for (int i = 0; i < FC_TAB_SLOTS; ++i) h->tab_key[i] = 0;

@@ -21,6 +21,15 @@
 #define FC_DEV_FLAG_INTERNAL 1
 #define FC_DEV_FLAG_TIMEOUT 2
 
+// Where one scoring call keeps its intermediates and partial sums.
+struct FcCarve {
+  const char *base;
+  size_t buf_bytes, tot_bytes, hi_bytes, off_tot;
+  bool operator==(const FcCarve &o) const {
+    return base == o.base && buf_bytes == o.buf_bytes && tot_bytes == o.tot_bytes && hi_bytes == o.hi_bytes && off_tot == o.off_tot;
+  }
+};
+
 struct fc_handle {
   int device;
   int max_seqlen;
@@ -60,7 +69,7 @@ struct fc_handle {
   int score_overlap;
   int band_form;           // fc_set_chirp_band: which chirp form fc_describe_plan counts
   unsigned step;                 // specialised-path sequences scored so far (parity picks partial-sum buffers)
-  size_t last_sig;               // how the previous call carved its workspace
+  FcCarve last_carve;            // how the previous call carved its workspace
   bool pending_join;             // internal streams hold work the caller's stream has not waited for
   cudaEvent_t ev_done[2][FC_MAX_AUX];   // [step parity][internal stream]: that stream finished that step
   // filter tables of the last FC_TAB_SLOTS (length, cutoff, form) triples that took the padded path (DEVICE, allocated by

@@ -1501,14 +1501,15 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
   if (any_fast && (s = prepare_tables(h, st, kv, gamma, false, reinterpret_cast<float4 *>(wsb + L.off_tab),
                                       reinterpret_cast<float2 *>(wsb + L.off_buf), tabs.data())) != FC_OK) return s;
   // a call that carves the workspace differently: nothing of the previous call may be in flight on the other streams
-  const size_t sig = reinterpret_cast<size_t>(wsb) ^ (L.buf_bytes << 20) ^ (L.tot_bytes << 8) ^ L.hi_bytes ^ (L.off_tot << 12);
-  if (any_small && sig != h->last_sig && (s = fc_flush_pending(h, st)) != FC_OK) return s;
-  if (any_fast && h->step >= 1 && sig != h->last_sig) {
+  const FcCarve carve = {wsb, L.buf_bytes, L.tot_bytes, L.hi_bytes, L.off_tot};
+  const bool recarved = !(carve == h->last_carve);
+  if (any_small && recarved && (s = fc_flush_pending(h, st)) != FC_OK) return s;
+  if (any_fast && h->step >= 1 && recarved) {
     for (int i = 0; i < h->num_aux; ++i)
       for (int o = 0; o < h->num_aux; ++o)
         if (o != i) FC_CUDA_TRY(cudaStreamWaitEvent(h->aux[i], h->ev_done[(h->step - 1) & 1u][o], 0));
   }
-  if (any_fast) h->last_sig = sig;
+  if (any_fast) h->last_carve = carve;
   for (int l0 = 0; l0 < num_layers; l0 += FC_LAYER_CHUNK) {
     const int nl = num_layers - l0 < FC_LAYER_CHUNK ? num_layers - l0 : FC_LAYER_CHUNK;
     if (any_small && any_passes && fork) {          // the internal streams need not wait for the short sequences

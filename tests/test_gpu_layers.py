@@ -98,3 +98,36 @@ def test_head_dims_that_take_different_kernels_share_a_handle(fc, N):
                 _check_head(k[:, head], v[:, head], scores[head].cpu(), 0.2, torch.float32)
     finally:
         fc.fc_destroy(h)
+
+
+# calls left on the internal streams, one after the other, that put their buffers at different places of one workspace: the
+# second waits for the first (the two pairs' sizes are such that a sum or exclusive-or of them does not tell them apart)
+@pytest.mark.parametrize("N,first,second", [(2048, (31, 11, 64), (17, 5, 256)), (4096, (31, 11, 64), (17, 5, 256)),
+                                            (8192, (2, 4, 128), (3, 2, 64))])
+def test_deferred_calls_share_a_workspace(fc, N, first, second):
+    cu = [0, N]
+    h = fc.fc_create(0, N)
+    try:
+        calls = []
+        for L, H, d in (first, second):
+            layers = [_kv(N, H, d, torch.bfloat16, 100 * l + H) for l in range(L)]
+            K, V = [k.cuda() for k, _ in layers], [v.cuda() for _, v in layers]
+            need = fc.fc_score_layers_workspace_bytes(h, K[0], V[0], cu, L)
+            calls.append((K, V, need, torch.empty((L, H, N), device="cuda"), torch.empty((L, 1, 4), dtype=torch.float64, device="cuda")))
+        ws = torch.empty(max(c[2] for c in calls), dtype=torch.uint8, device="cuda")
+        want = []
+        for K, V, _, scores, energy in calls:
+            fc.fc_score_layers(h, K, V, cu, 0.2, scores, energy, ws)
+            want.append((scores.clone(), energy.clone()))
+        fc.fc_set_score_overlap(h, True)
+        for _ in range(3):
+            for K, V, _, scores, energy in calls:
+                scores.zero_()
+                energy.zero_()
+            for K, V, _, scores, energy in calls:
+                fc.fc_score_layers(h, K, V, cu, 0.2, scores, energy, ws)
+            assert fc.fc_last_device_status(h) == 0
+            for (_, _, _, scores, energy), (ws_, we) in zip(calls, want):
+                assert torch.equal(scores, ws_) and torch.equal(energy, we)
+    finally:
+        fc.fc_destroy(h)
