@@ -113,8 +113,9 @@ def physical_gpu_index(local_rank: int) -> int:
 
 # --------------------------------------------------------------------------- accounting
 def step_accounting(binding, handle, cfg):
-    """Algorithmic flops and HBM bytes of one step, per kernel class (what the shipped
-    algorithm has to compute and move, not what the hardware happened to do)."""
+    """Algorithmic flops and HBM bytes of one step, per kernel class: what the path cannot do without (one transform of
+    N points each way per complex column, whatever N is), not what the hardware or the padding of lengths that are not a
+    power of two happened to add."""
     d, H, L = cfg.head_dim, cfg.num_heads, cfg.num_layers
     s = 4 if cfg.dtype == "f32" else 2
     acc = {k: dict(flops=0.0, bytes=0.0) for k in ("pass1", "pass2", "pass3", "select", "gather")}
@@ -123,12 +124,12 @@ def step_accounting(binding, handle, cfg):
         if N == 0:
             continue
         plan = binding.fc_describe_plan(handle, N, cfg.gamma)
-        M, n1, n2 = plan["nfft"], plan["n1"], plan["n2"]
+        n1 = plan["n1"] if not plan["bluestein"] else math.sqrt(N)      # share of the outer passes
+        n2 = N / n1
         cols = H * d * L                       # complex columns (K + jV) of this sequence
-        reps = 2 if plan["bluestein"] else 1   # chirp path: two convolutions, each a forward+inverse transform
-        acc["pass1"]["flops"] += reps * cols * M * 5.0 * math.log2(n1)
-        acc["pass2"]["flops"] += reps * cols * M * (10.0 * math.log2(n2) + 8.0)
-        acc["pass3"]["flops"] += reps * cols * M * 5.0 * math.log2(n1) + cols * N * 4.0
+        acc["pass1"]["flops"] += cols * N * 5.0 * math.log2(n1)
+        acc["pass2"]["flops"] += cols * N * (10.0 * math.log2(n2) + 8.0)
+        acc["pass3"]["flops"] += cols * N * 5.0 * math.log2(n1) + cols * N * 4.0
         acc["pass1"]["bytes"] += N * H * L * 2.0 * d * s               # K and V rows, read once
         acc["pass3"]["bytes"] += N * H * L * 4.0                       # score write
         acc["select"]["bytes"] += N * H * L * 4.0                      # score read
