@@ -17,10 +17,11 @@
  *     and never frees or writes caller inputs.
  *   - Streams.  `stream` is a cudaStream_t passed as void*.  Results are ordered
  *     on it: work enqueued on `stream` after a call sees that call's outputs.
- *     fc_score_layer runs sequences of up to 65536 tokens on the handle's
- *     internal streams (two by default), which wait for everything enqueued on `stream` before the call
- *     and which `stream` waits for before the call returns, through events; no
- *     host synchronisation is involved (see fc_set_score_overlap for the
+ *     Short sequences (powers of two up to 1024 tokens, others up to 512, where head_dim
+ *     allows it) are scored by one kernel on `stream`, longer ones of up to 65536 tokens on
+ *     the handle's internal streams (two by default), which wait for everything enqueued on
+ *     `stream` before the call and which `stream` waits for before the call returns, through
+ *     events; no host synchronisation is involved (see fc_set_score_overlap for the
  *     variant that defers the second wait).  Nothing uses the default stream.
  *   - Calls that block the host: fc_create and fc_destroy (device
  *     synchronisation), fc_last_device_status and fc_static_last_device_status
@@ -89,8 +90,9 @@ typedef struct {
 /* Create a handle on `device`.  max_seqlen bounds every N_b later passed in
  * (1 <= max_seqlen <= 131072; lengths that are not a power of two, or below 16,
  * are limited to 65536).  Allocates the twiddle table (8 bytes * 4 * next power of two of
- * max_seqlen), room for eight filter tables (16 bytes * the power of two from 2*max_seqlen-1 up each, at most
- * 2 MiB; lengths that are not a power of two reuse theirs from layer to layer) and a status word.  Returns FC_ERR_CUDA if the device cannot be
+ * max_seqlen, at least 64), room for eight filter tables (16 bytes * the power of two from 2*max_seqlen-1 up each, at
+ * least 16 KiB and at most 2 MiB; lengths that are not a power of two reuse theirs from layer to layer and call to call,
+ * a batch of more than eight unlike ones builds the rest in the workspace on every call) and a status word.  Returns FC_ERR_CUDA if the device cannot be
  * used, FC_ERR_UNSUPPORTED if max_seqlen is out of range. */
 fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen);
 void fc_destroy(fc_handle *h);
@@ -142,8 +144,8 @@ fc_status fc_profile_begin(fc_handle *h, int32_t kernel_class, int32_t max_launc
 fc_status fc_profile_stride(fc_handle *h, int32_t stride);
 fc_status fc_profile_end(fc_handle *h, double *total_ms, uint64_t *launches);
 
-/* enabled = 1: fc_score_layer calls for power-of-two lengths of 1024..65536 tokens leave their
- * work on the library's two internal streams instead of making `stream` wait for it, so that the
+/* enabled = 1: fc_score_layer calls all of whose sequences are short or have power-of-two lengths of up
+ * to 65536 tokens leave their work on the library's internal streams instead of making `stream` wait for it, so that the
  * next layer starts while the last kernels of this one drain.  Inputs are still taken in stream
  * order (the internal streams wait for everything enqueued on `stream` before the call).  The
  * scores and energies of such calls are ordered on a stream only by the next
@@ -161,9 +163,10 @@ fc_status fc_set_score_overlap(fc_handle *h, int32_t enabled);
  * call waits for the one before it. */
 fc_status fc_set_select_overlap(fc_handle *h, int32_t enabled);
 
-/* Which chirp form fc_describe_plan counts for lengths that are not a power of two: enabled = 1 (default) the
+/* Which chirp form fc_describe_plan reports for lengths that are not a power of two: enabled = 1 (default) the
  * band form (only the bins -omega .. omega of the spectrum, padded length >= N + 2*omega + 1) where it is shorter than
- * the full-length form (>= 2N - 1), enabled = 0 always the latter.  No effect on how such lengths are computed. */
+ * the full-length form (>= 2N - 1), enabled = 0 always the latter.  No effect on how anything is computed: the library
+ * scores such lengths by one padded convolution, whatever this says. */
 fc_status fc_set_chirp_band(fc_handle *h, int32_t enabled);
 
 /* Number of internal streams fc_score_layer spreads the head groups of a sequence over (1..4,
@@ -188,11 +191,11 @@ fc_status fc_reset_ordering(fc_handle *h);
  * Default 32 MiB.  Affects speed only. */
 fc_status fc_set_group_bytes(fc_handle *h, size_t bytes);
 
-/* The transform of a sequence of length seqlen at cutoff ratio gamma that roofline figures are counted on
- * (diagnostic; head_dim a multiple of 64 assumed): out = { power of two: the transform itself (0); other lengths: the
- * shortest chirp convolutions in the full-length (1) or band form (2, see fc_set_chirp_band) -- a yardstick: the
- * library computes such lengths as one padded convolution of at least 2N - 1 points --,
- * transform length, first factor N1, second factor N2 }. */
+/* How a sequence of length seqlen could be transformed at cutoff ratio gamma (diagnostic): out = { form, transform
+ * length, first factor N1, second factor N2 }.  Form 0, powers of two: the transform itself, as the three passes run it.
+ * Forms 1 and 2, other lengths: the shortest chirp convolutions in the full-length or band form (see fc_set_chirp_band),
+ * kept for callers that compare with them; the library scores such lengths by one padded convolution of at least
+ * 2N - 1 points instead. */
 fc_status fc_describe_plan(const fc_handle *h, int32_t seqlen, double gamma, int32_t out[4]);
 
 /* Workspace sizes (bytes) the next two calls need for this view.  0 on bad input. */
@@ -275,8 +278,9 @@ fc_status fc_select_compact(fc_handle *h, const fc_kv_view *kv, const float *sco
  * the power spectrum of one layer, P_k[m] = |C_k[m]|^2 and P_v[m] = |C_v[m]|^2, where C[m] is the row of
  * DCT coefficients (Eq. 6-7) of frequency m over all channels of all KV heads.  Its band sums are the
  * numerators and denominators of Eq. 12 (what fc_score_layer returns as `energy`), its running sum is
- * the cumulative-energy curve from which a cutoff gamma can be read.  Not on the compression path:
- * it runs the generic transform kernels on the caller's stream.
+ * the cumulative-energy curve from which a cutoff gamma can be read.  Not on the compression path.
+ * It runs on the internal streams like fc_score_layer and is complete in stream order when it returns
+ * (131072 points and powers of two below 1024: on the caller's stream).
  *
  *   spectrum   DEVICE double[T][2]: row cu_seqlens[b] + m = (P_k[m], P_v[m]) of sequence b.
  *   workspace  DEVICE, 256-byte aligned, >= fc_power_spectrum_workspace_bytes().
@@ -370,7 +374,7 @@ fc_status fc_select_compact_ex(fc_handle *h, const fc_kv_view *kv, const float *
 /*
  * fc_select_compact_ex for several layers in ONE launch (Sec. 3.2.1, last sentence; same selection, same
  * results bit for bit).  After fc_allocate_budgets every layer's scores, budgets and offsets are known, and
- * one layer's selection fills only a fraction of the GPU (8 blocks per sequence and head), so the layers
+ * one layer's selection fills only a fraction of the GPU (one to eight blocks per sequence and head), so the layers
  * are best selected side by side.
  *
  *   shape        the layout all layers share: strides, dtype, num_heads, head_dim, batch, cu_seqlens

@@ -4,16 +4,18 @@
 //
 //  * the tiles (64 rows) of all sequences of all KV heads form one line, and the grid's blocks, one per SM, take equal
 //    shares of it, whatever the lengths of the sequences are: a block's share is one or more runs of consecutive tiles
-//    of one sequence and head each (28 layers of kept rows 1638, 205, 3277, 820: 382 -> 335 us per step, where a grid of
-//    splits sized for the longest sequence left half of the SMs without rows);
+//    of one sequence and head each (a seventh of a step over kept rows of 1638, 205, 3277 and 820 tokens, where a grid
+//    of splits sized for the longest sequence left half of the SMs without rows);
 //  * a producer warp fills a four-stage shared-memory ring by tiled TMA loads (128-byte swizzle), one mbarrier pair per
 //    stage; the four other warps wait for nothing but the tile they use;
 //  * all query heads of a KV head (up to 16) are one 16-row operand of m16n8k16 tensor-core products,
 //    so a K/V tile is read from shared memory once for the whole group; each of the 4 warps owns 16
 //    rows of the tile and keeps its own running maximum, sum and 16 x 128 fp32 output;
 //  * the warps' partial results are merged in shared memory; a sequence covered by one block is finished there, else a
-//    second small kernel merges the blocks' shares (28 layers of 65536 rows: 926 -> 808 us per step).
+//    second small kernel merges the blocks' shares.
 // Both launches are programmatic dependents: they are set up while the kernel before them in the stream ends.
+// Together: 28 layers of 65536 rows 965 -> 784 us per step, of those kept rows with tails 397 -> 310 us (from a graph 754
+// and 294; the host enqueues the 28 calls in 230..370 us, behind the device).
 #include <cuda.h>
 
 #include "fc_common.cuh"
@@ -236,7 +238,7 @@ k_decode(const DecodeParams P, const __grid_constant__ DecodeMaps M) {
     // here, so it does not matter if those kernels are still writing them, or the offsets: a wrong guess only wastes it.
     // By plain prefetches, since the tensor engine takes as long over a prefetch as over the load; two tiles are what
     // fits into the wait (four and eight lose again what two gain), and with a share of one tile the load itself is as
-    // early.  28 layers of 65536 rows 799 -> 778 us, of kept rows 1638, 205, 3277, 820 326 -> 309 us.
+    // early.  3 % of a step over 65536 rows, 5 % over the short caches named above.
     const Share sr = find_share<true>(P, blk, lane);
     if (sr.hi - sr.lo > 1) {
       const SeqRows s = seq_rows<true>(P, sr.b);
@@ -483,8 +485,8 @@ k_decode(const DecodeParams P, const __grid_constant__ DecodeMaps M) {
 // sum.  Shares sit in slot i + (h*B + b) (both only ever advance along the line, so slots do not collide).  One block per
 // query head; each warp folds every fourth share, loads ahead of the arithmetic, and the warps' results meet in shared
 // memory: two rounds of latency.  Launched early as a programmatic dependent, it is resident when the shares are complete
-// (merging in the block that finishes last instead costs an atomic and 3..5 us on one SM: 14.0 against 11.9 us per
-// layer of the small case above).
+// (merging in the block that finishes last instead costs an atomic and 3..5 us on one SM: a sixth more per layer of the
+// short caches named above).
 template <typename T>
 __global__ void __launch_bounds__(32 * kFoldWarps)
 k_decode_combine(const DecodeParams P) {

@@ -22,7 +22,7 @@
 //      E[k] = c[k] Z[k] - h[k] Z[-k],   c = 1 - DFT of g wrapped around 0 (real),   h = DFT of g(t+1), t = 0..2N-2,
 //    and the residual is the inverse transform's first N outputs.  One forward and one inverse transform of 2N points
 //    where two chirp convolutions (four transforms of 1.4N..2N points, six launches) did the same before: a packed
-//    batch of eight sequences of 7k..54k tokens went from 94.2 to 58.8 ms (28 layers x 4 heads).
+//    batch of eight sequences of 7k..54k tokens went from 94.5 to 58.4 ms (28 layers x 4 heads).
 //
 // The transforms are left unnormalised; pass 3 folds 1/M^2 into the score.
 #pragma once

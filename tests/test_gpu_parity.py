@@ -1,7 +1,7 @@
 """GPU parity: the CUDA library (through its C ABI) against the fp64 CPU oracle on
 the same seeded inputs, element by element.
 
-Tolerances (the build's stated bar): score error |g-o| / max(o, 1e-6*e_bar) <= 1e-3
+Tolerances: score error |g-o| / max(o, 1e-6*e_bar) <= 1e-3
 for fp32 inputs and <= 2e-2 for fp16/bf16 inputs, where e_bar is the head's mean
 of (|k_x|^2+|v_x|^2)/d (so the gamma=1 case, whose true scores are 0, is still
 testable); index sets identical except for tokens whose oracle score is within that
@@ -177,9 +177,9 @@ def test_scores_long_arbitrary_length(fc):
 
 
 def test_scores_mixed_paths_in_one_call(fc):
-    # power-of-two and other lengths alternate in one batch: the specialised transform path (two internal
-    # streams, work left pending), the chirp path on the same streams (joined per sequence), a 131072-point chirp
-    # transform and a tiny generic one; results match the oracle and do not change from run to run
+    # power-of-two and other lengths alternate in one batch: the direct and the padded form of the three passes (two
+    # internal streams, up to 81920 points) and a tiny sequence on the caller's stream; results match the oracle and do
+    # not change from run to run
     lens = [5000, 4096, 3000, 8192, 33000, 7, 2048]
     cu = [0] + [int(x) for x in np.cumsum(lens)]
     k, v = _rand_kv(cu[-1], 4, 128, torch.bfloat16, 12)
@@ -190,7 +190,7 @@ def test_scores_mixed_paths_in_one_call(fc):
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.float16])
 def test_scores_131072_point_chirp_transform(fc, dtype):
-    # full-length form (all N bins): 2N - 1 pads to 131072
+    # 2N - 1 = 66001, just past a power of two (131072 points where only powers of two are padded to, 81920 here)
     N = 33001
     k, v = _rand_kv(N, 2, 128, dtype, 13)
     _check_layer(fc, k, v, [0, N], 0.2, band=False)
@@ -206,8 +206,10 @@ def test_scores_131072_point_chirp_transform(fc, dtype):
     (46800, 0.2, 64, None),      # 65521 -> 65536: the longest sequence the band form shortens at this cutoff
 ])
 def test_scores_chirp_band_form(fc, N, gamma, d, group_bytes):
-    # The band form of the chirp path (bins -omega .. omega, Base KV transformed back, score against the input
-    # rows) and the full-length form both match the oracle, and each other.
+    # The lengths at which a chirp transform of the band -omega .. omega would be shorter than one of all bins.  Every one
+    # of them is scored by one padded convolution, whatever fc_set_chirp_band says: both settings match the oracle and
+    # give the same values.  (The chirp form itself, which the entry point without allocation runs, is compared with this
+    # one in test_zz_no_alloc.py.)
     k, v = _rand_kv(N, 2, d, torch.float32, 500 + N)
     g1, e1 = _check_layer(fc, k, v, [0, N], gamma, band=True, group_bytes=group_bytes)
     g2, e2 = _check_layer(fc, k, v, [0, N], gamma, band=False, group_bytes=group_bytes)
@@ -218,9 +220,8 @@ def test_scores_chirp_band_form(fc, N, gamma, d, group_bytes):
 @pytest.mark.parametrize("M", [5120, 6144, 7168, 10240, 12288, 14336, 20480, 24576, 28672, 40960, 49152, 57344,
                                81920, 98304, 114688])
 def test_scores_chirp_lengths_with_an_odd_factor(fc, M):
-    # Full form of the chirp path at N = M/2 - 1: 2N - 1 = M - 3 pads to M = 2^k * {5, 3, 7}, every shape the
-    # specialised kernels have for such lengths (first-stage radix 10, 12, 14; rows of 32..512 points).  The band form
-    # of the same sequence picks another length; both match the oracle.
+    # N = M/2 - 1: 2N - 1 = M - 3 pads to M = 2^k * {5, 3, 7}, every shape the specialised kernels have for such lengths
+    # (first-stage radix 10, 12, 14; rows of 32..512 points), against the oracle; fc_set_chirp_band changes nothing
     N = M // 2 - 1
     k, v = _rand_kv(N, 1, 64, torch.float32, 900 + M % 1000)
     g1, e1 = _check_layer(fc, k, v, [0, N], 0.2, band=False)
@@ -230,12 +231,13 @@ def test_scores_chirp_lengths_with_an_odd_factor(fc, M):
 
 @pytest.mark.parametrize("N", [5118, 20478, 29255, 35107, 40958, 58513])
 def test_scores_chirp_band_form_on_lengths_with_an_odd_factor(fc, N):
-    # N + 2*floor(0.2 N) + 1 lands just under 7168, 28672, 40960, 49152, 57344 and 81920
+    # lengths whose band would fill a chirp transform with an odd factor; padded to 10240 ... 131072 points
     k, v = _rand_kv(N, 2, 128, torch.bfloat16, 30 + N % 100)
     _check_layer(fc, k, v, [0, N], 0.2)
 
 
 def test_describe_plan_reports_the_convolution_length_in_use(fc):
+    # powers of two: the transform in use; other lengths: the chirp lengths (form and size) it documents
     h = fc.fc_create(0, 65536)
     try:
         p = fc.fc_describe_plan(h, 32768, 0.2)
@@ -249,7 +251,7 @@ def test_describe_plan_reports_the_convolution_length_in_use(fc):
         fc.fc_set_chirp_band(h, False)
         p = fc.fc_describe_plan(h, 2500, 0.2)                    # 4999 -> 5120 = 160 x 32
         assert (p["band_form"], p["nfft"], p["n1"], p["n2"]) == (False, 5120, 160, 32)
-        p = fc.fc_describe_plan(h, 300, 0.2)                     # short: generic kernels, power of two
+        p = fc.fc_describe_plan(h, 300, 0.2)                     # short: a power of two
         assert (p["bluestein"], p["nfft"]) == (True, 1024)
     finally:
         fc.fc_destroy(h)
@@ -264,10 +266,10 @@ def test_scores_chirp_band_form_16bit_ragged(fc):
     assert np.array_equal(g1, g2) and np.array_equal(e1, e2)
 
 
-@pytest.mark.parametrize("d,group_bytes", [(128, 1), (128, 1 << 20), (192, 1), (64, 1)])
+@pytest.mark.parametrize("d,group_bytes", [(128, 1), (128, 1 << 20), (192, 1), (64, 1), (256, 1)])
 def test_scores_arbitrary_length_in_column_groups(fc, d, group_bytes):
-    # a small cache budget makes the chirp path transform each head in groups of 32..96 columns
-    # and add the groups' contributions to the score one after the other
+    # a small cache budget makes a head of 128 or 256 channels go in two or four groups of 64 columns, whose contributions
+    # are added to the score one after the other (64 channels, and 192, which does not halve to whole groups, go whole)
     N = 3000
     k, v = _rand_kv(N, 2, d, torch.float32, 40 + d)
     g1, _ = _check_layer(fc, k, v, [0, N], 0.2, group_bytes=group_bytes)
