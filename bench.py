@@ -33,10 +33,10 @@ DEFAULT_CONFIG = "cfg3"          # the 32k-token workload the target fraction is
 
 # DRAM bytes read + written per launch of the dominant kernel as an ncu capture counted them (a constant from
 # that capture, not a measurement of this run; None where no capture of the kernel and workload exists):
-# pass 2 of cfg3, 0.73 MB read + 0.84 MB written on average over 8 launches with the intermediate in the
-# persisting part of L2 (ncu --cache-control none, one pass per launch).
+# pass 2 of cfg3, 0.46 MB read + 1.94 MB written on average over 24 launches with the intermediate in the
+# persisting part of L2 (ncu --cache-control none, one pass per launch; profiles/transform_passes_ncu.md).
 NCU_TRAFFIC_BYTES = {
-    ("cfg3", "pass2"): 1.57e6,
+    ("cfg3", "pass2"): 2.40e6,
 }
 
 
