@@ -1,0 +1,38 @@
+// Scoring in the kept band (fc_band.cuh): what the scoring calls use of it.
+#pragma once
+#include "fc_common.cuh"
+
+struct FcBandSizes {
+  size_t tables, unit;     // bytes: one sequence's tables, one unit's (layer, head) intermediates
+  int steps;               // 128-token steps of a sequence
+};
+// Upper bounds over all cutoffs for a sequence of N tokens; false: no cutoff takes this form.
+bool fc_band_bounds(const fc_kv_view *kv, int N, FcBandSizes *s);
+// Intermediates of one launch group, one copy per internal stream, of a call with so many units.
+size_t fc_band_buffer_bytes(const fc_handle *h, const FcBandSizes *s, int units);
+
+// Whether a cutoff takes this form.
+bool fc_band_takes(const fc_kv_view *kv, int N, int omega);
+
+// One sequence of a chunk of layers.
+struct FcBandJob;
+// nullptr where the other forms are used.  Freed with fc_band_release.
+FcBandJob *fc_band_plan(const fc_handle *h, const fc_kv_view *kv, int N, int omega);
+void fc_band_release(FcBandJob *j);
+int fc_band_units(const fc_handle *h, const FcBandJob *j, int units, size_t buf_bytes);   // units per launch
+int fc_band_ranges(const FcBandJob *j, int units);      // blocks a unit's rows are spread over where a launch has so many units
+// The sequence's tables, built on `st`.
+fc_status fc_band_tables(fc_handle *h, cudaStream_t st, const FcBandJob *j, char *tables);
+struct FcBandLaunch {
+  const void *const *k, *const *v;     // first token of the sequence, layer by layer
+  float *const *scores;
+  int layers;
+  const char *tables;
+  double *part, *energy;
+  unsigned *done;
+  long long score_stride, energy_stride;
+};
+// Tensor maps of the layers' rows; the launches of fc_band_group use them until the next call.
+fc_status fc_band_bind(fc_handle *h, FcBandJob *j, const fc_kv_view *kv, const FcBandLaunch &l);
+// Units [u0, u0 + nu) on `st`, intermediates at `buf`.
+fc_status fc_band_group(fc_handle *h, cudaStream_t st, const FcBandJob *j, const FcBandLaunch &l, int u0, int nu, int ranges, char *buf);

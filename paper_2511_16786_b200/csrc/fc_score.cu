@@ -27,6 +27,7 @@
 // length M >= 2N-1.
 #include "fc_common.cuh"
 #include "fc_score_fast.cuh"
+#include "fc_band.h"
 #include "fc_score_small.cuh"
 
 #include <math.h>
@@ -817,9 +818,17 @@ GroupPlan plan_groups(const fc_handle *h, const PassPlan &p, int num_units, int 
 // Workspace carve-up of one scoring call: the regions hold the largest sequence of the view.
 struct ScoreLayout {
   size_t buf_bytes;          // intermediates, one buffer per internal stream
-  size_t off_buf, off_tab, off_tot, off_hi, off_small, total;
+  size_t off_buf, off_tab, off_band, off_tot, off_hi, off_small, total;
   size_t tot_bytes, hi_bytes;   // per-block partial sums of one step; two copies, used in turn
 };
+
+// Cutoff index omega of Eq. 8 for a sequence of N tokens.
+inline int cutoff_index(double gamma, int N) {
+  long long om = (long long)floor(gamma * (double)N);
+  if (om > N - 1) om = N - 1;
+  if (om < 0) om = 0;
+  return (int)om;
+}
 
 inline bool first_of_its_length(const fc_kv_view *kv, int b) {
   const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
@@ -831,11 +840,19 @@ inline bool first_of_its_length(const fc_kv_view *kv, int b) {
 ScoreLayout score_layout(const fc_handle *h, const fc_kv_view *kv, int num_layers) {
   ScoreLayout L = {};
   const int H = kv->num_heads, d = kv->head_dim, nl = num_layers < FC_LAYER_CHUNK ? num_layers : FC_LAYER_CHUNK;
-  size_t tab = 0, generic = 0, nsmall = 0;
+  size_t tab = 0, generic = 0, nsmall = 0, band = 0;
   for (int b = 0; b < kv->batch; ++b) {
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0) continue;
     const PassPlan p = plan_passes(N, kv->head_dim);
+    FcBandSizes bs;
+    if (!h->generic_only && fc_band_bounds(kv, N, &bs)) {      // whether it is taken depends on the cutoff: room for both
+      if (first_of_its_length(kv, b)) band += bs.tables;
+      const size_t buf = fc_band_buffer_bytes(h, &bs, nl * H);
+      const size_t part = (size_t)nl * H * bs.steps * 4 * sizeof(double);
+      if (align_up(buf, 256) > L.buf_bytes) L.buf_bytes = align_up(buf, 256);
+      if (part > L.tot_bytes) L.tot_bytes = part;
+    }
     if (!p.ok || h->generic_only) {
       const size_t t = generic_layout(h, plan_sequence(N), H, d).total;
       if (t > generic) generic = t;
@@ -856,6 +873,7 @@ ScoreLayout score_layout(const fc_handle *h, const fc_kv_view *kv, int num_layer
   L.off_buf = off; off += L.buf_bytes * h->num_aux;
   if (off < generic) off = generic;            // tables outlive a sequence on the generic kernels
   L.off_tab = off; off += align_up(tab, 256);
+  L.off_band = off; off += band;
   L.off_tot = off; off += 2 * L.tot_bytes;
   L.off_hi = off;  off += 2 * L.hi_bytes;
   L.off_small = off; off += align_up(nl * nsmall * H * 4 * sizeof(double), 256);
@@ -875,7 +893,7 @@ bool window_fits(const fc_handle *h, const PassPlan &p, const GroupPlan &g) {
 // The persisting part of L2 is a limit of the whole context, shared by the handles of a device (fc_persist_acquire):
 // held while calls contain a sequence that wants it, let go when a call has none.  Decided once per call; left as it is
 // while `st` is being captured into a graph, where device-wide settings cannot change.
-void claim_persisting_l2(fc_handle *h, const fc_kv_view *kv, int num_layers, cudaStream_t st) {
+void claim_persisting_l2(fc_handle *h, const fc_kv_view *kv, int num_layers, double gamma, cudaStream_t st) {
   if (!h->l2_persist) return;
   const int nl = num_layers < FC_LAYER_CHUNK ? num_layers : FC_LAYER_CHUNK;
   bool claim = false;
@@ -883,7 +901,7 @@ void claim_persisting_l2(fc_handle *h, const fc_kv_view *kv, int num_layers, cud
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0) continue;
     const PassPlan p = plan_passes(N, kv->head_dim);
-    if (!p.ok || p.pad || p.small) continue;
+    if (!p.ok || p.pad || p.small || fc_band_takes(kv, N, cutoff_index(gamma, N))) continue;
     claim = window_fits(h, p, plan_groups(h, p, nl * kv->num_heads, kv->num_heads, kv->head_dim));
   }
   if (claim == (h->persist_on != 0)) return;
@@ -1142,14 +1160,6 @@ fc_status run_p3_spec(const PassArgs &x, float2 *spec) {
   return FC_ERR_INTERNAL;
 }
 
-// Cutoff index omega of Eq. 8 for a sequence of N tokens.
-inline int cutoff_index(double gamma, int N) {
-  long long om = (long long)floor(gamma * (double)N);
-  if (om > N - 1) om = N - 1;
-  if (om < 0) om = 0;
-  return (int)om;
-}
-
 // How the spectrum diagnostics transform a sequence: a power of two from 1024 to 65536 directly, a length that is not a
 // power of two by a chirp convolution of >= 2N - 1 points (plan.pad); 131072 points and powers of two below 1024, where
 // launches count and a chirp would add two of them, are left to the generic kernels.
@@ -1165,7 +1175,7 @@ PassPlan plan_spectrum(int N) {
 // slots, tables go to the workspace (`spare`), every call: a graph must not depend on what the handle holds when it is
 // replayed.  `buf`: an intermediate buffer to build them in.
 fc_status prepare_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, double gamma, bool spectrum, float4 *spare,
-                         float2 *buf, const float4 **tabs) {
+                         float2 *buf, const float4 **tabs, const FcBandJob *const *band = nullptr) {
   bool cached = true, any = false, flushed = false;
   bool used[FC_TAB_SLOTS] = {};
   auto plan_of = [&](int N) { return spectrum ? plan_spectrum(N) : plan_passes(N, kv->head_dim); };
@@ -1180,7 +1190,7 @@ fc_status prepare_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, do
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0) continue;
     const PassPlan p = plan_of(N);
-    if (!p.ok || !p.pad) continue;
+    if (!p.ok || !p.pad || (band && band[b])) continue;
     if (!any) {
       any = true;
       cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -1196,7 +1206,7 @@ fc_status prepare_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, do
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0 || tabs[b]) continue;
     const PassPlan p = plan_of(N);
-    if (!p.ok || !p.pad) continue;
+    if (!p.ok || !p.pad || (band && band[b])) continue;
     if (!first_of_its_length(kv, b)) {
       for (int i = 0; i < b && !tabs[b]; ++i)
         if (kv->cu_seqlens[i + 1] - kv->cu_seqlens[i] == N) tabs[b] = tabs[i];
@@ -1296,6 +1306,33 @@ fc_status score_sequence(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, co
       if ((s = run_p2(x, nu * g.sub, p.pad ? fast::MODE_PAD : fast::MODE_FILTER)) != FC_OK) return s;
       if ((s = run_p3(x, total_tokens, cg > 0 ? 1 : 0, cg * H * p.N2, eo)) != FC_OK) return s;
     }
+  }
+  for (int i = 0; i < h->num_aux; ++i) FC_CUDA_TRY(cudaEventRecord(h->ev_done[par][i], h->aux[i]));
+  h->step++;
+  h->pending_join = true;
+  return FC_OK;
+}
+
+// One sequence in the kept band, for a chunk of layers.  `lp` points at the sequence's first token.
+fc_status score_band(fc_handle *h, const fc_kv_view *kv, FcBandJob *job, int nl, const fast::LayerPtrs &lp, double *energy,
+                     long long energy_stride, const ScoreLayout &L, char *wsb, const char *tables) {
+  const int U = nl * kv->num_heads;
+  const int nu = fc_band_units(h, job, U, L.buf_bytes);
+  const int ranges = fc_band_ranges(job, nu);
+  const unsigned par = h->step & 1u;               // as in score_sequence
+  if (h->step >= 2)
+    for (int i = 0; i < h->num_aux; ++i)
+      for (int o = 0; o < h->num_aux; ++o)
+        if (o != i) FC_CUDA_TRY(cudaStreamWaitEvent(h->aux[i], h->ev_done[par][o], 0));
+  FcBandLaunch l = {lp.k, lp.v, lp.scores, nl, tables, reinterpret_cast<double *>(wsb + L.off_tot + par * L.tot_bytes), energy,
+                    h->done_counter + par * FC_LAYER_CHUNK, (long long)kv->cu_seqlens[kv->batch], energy_stride};
+  fc_status s = fc_band_bind(h, job, kv, l);
+  if (s != FC_OK) return s;
+  int group = 0;
+  for (int u0 = 0; u0 < U; u0 += nu, ++group) {
+    const int si = (int)((group + h->step) % (unsigned)h->num_aux);
+    s = fc_band_group(h, h->aux[si], job, l, u0, U - u0 < nu ? U - u0 : nu, ranges, wsb + L.off_buf + (size_t)si * L.buf_bytes);
+    if (s != FC_OK) return s;
   }
   for (int i = 0; i < h->num_aux; ++i) FC_CUDA_TRY(cudaEventRecord(h->ev_done[par][i], h->aux[i]));
   h->step++;
@@ -1489,17 +1526,41 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
   bool fork = true, direct_only = true, any_fast = false, any_small = false, any_passes = false;
   std::vector<PassPlan> plans(B);
   std::vector<const float4 *> tabs(B, nullptr);
+  struct Jobs : std::vector<FcBandJob *> {
+    using std::vector<FcBandJob *>::vector;
+    ~Jobs() { for (FcBandJob *j : *this) fc_band_release(j); }
+  } band(B, nullptr);
+  std::vector<const char *> band_tabs(B, nullptr);
   for (int b = 0; b < B; ++b) {
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0) continue;
     if (!h->generic_only) plans[b] = plan_passes(N, kv->head_dim);
+    band[b] = fc_band_plan(h, kv, N, cutoff_index(gamma, N));
+    if (band[b]) {
+      plans[b].ok = true;
+      plans[b].small = plans[b].pad = false;
+    }
     any_fast = any_fast || plans[b].ok;
     any_small = any_small || plans[b].small;
     any_passes = any_passes || (plans[b].ok && !plans[b].small);
     if (!plans[b].ok || (plans[b].pad && !plans[b].small)) direct_only = false;
   }
   if (any_fast && (s = prepare_tables(h, st, kv, gamma, false, reinterpret_cast<float4 *>(wsb + L.off_tab),
-                                      reinterpret_cast<float2 *>(wsb + L.off_buf), tabs.data())) != FC_OK) return s;
+                                      reinterpret_cast<float2 *>(wsb + L.off_buf), tabs.data(), band.data())) != FC_OK) return s;
+  char *band_at = wsb + L.off_band;
+  for (int b = 0; b < B; ++b) {
+    if (!band[b]) continue;
+    const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
+    for (int i = 0; i < b && !band_tabs[b]; ++i)
+      if (kv->cu_seqlens[i + 1] - kv->cu_seqlens[i] == N) band_tabs[b] = band_tabs[i];
+    if (band_tabs[b]) continue;
+    // the tables' place may still be in use on the internal streams
+    if ((s = fc_flush_pending(h, st)) != FC_OK || (s = fc_band_tables(h, st, band[b], band_at)) != FC_OK) return s;
+    band_tabs[b] = band_at;
+    FcBandSizes bs;
+    fc_band_bounds(kv, N, &bs);
+    band_at += bs.tables;
+  }
   // a call that carves the workspace differently: nothing of the previous call may be in flight on the other streams
   const FcCarve carve = {wsb, L.buf_bytes, L.tot_bytes, L.hi_bytes, L.off_tot};
   const bool recarved = !(carve == h->last_carve);
@@ -1550,7 +1611,9 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
         lp.v[l] = static_cast<const T *>(layers[l0 + l].v) + (long long)start * kv->stride_token;
         lp.scores[l] = const_cast<float *>(layers[l0 + l].scores) + start;
       }
-      if ((s = score_sequence<T>(h, st, kv, plans[b], nl, lp, gamma, en, 4ll * B, L, wsb, tabs[b])) != FC_OK) return s;
+      s = band[b] ? score_band(h, kv, band[b], nl, lp, en, 4ll * B, L, wsb, band_tabs[b])
+                  : score_sequence<T>(h, st, kv, plans[b], nl, lp, gamma, en, 4ll * B, L, wsb, tabs[b]);
+      if (s != FC_OK) return s;
     }
   }
   // the caller's stream waits for this call's work right away, unless it asked to have that deferred
@@ -1786,7 +1849,7 @@ extern "C" fc_status fc_score_layers(fc_handle *h, const fc_kv_view *shape, cons
   FC_CUDA_TRY(cudaGetDevice(&dev));
   if (dev != h->device) FC_CUDA_TRY(cudaSetDevice(h->device));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  claim_persisting_l2(h, shape, num_layers, st);
+  claim_persisting_l2(h, shape, num_layers, gamma, st);
   return score_dispatch(h, st, shape, layers, num_layers, gamma, energy, workspace);
 }
 

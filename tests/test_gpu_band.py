@@ -1,0 +1,119 @@
+"""Scoring in the kept band (16-bit inputs, cutoffs of up to about two fifths of the bins) at the edges of its windows, grids
+and dispatch rule, against the fp64 oracle."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import flashcache_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fc():
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    from paper_2511_16786_b200 import binding
+    return binding
+
+
+def _kv(T, H, d, dtype, seed):
+    g = torch.Generator().manual_seed(seed)
+    t = torch.arange(T, dtype=torch.float32)[:, None, None] / T
+    far = torch.rand((T, H, 1), generator=g) < 0.1
+    out = []
+    for a in (2.5, 7.0):
+        n = torch.randn((T, H, d), generator=g)
+        trend = 3.0 * torch.cos(a * t + torch.randn((1, H, d), generator=g))
+        out.append(torch.where(far, 5.0 * n, trend + 0.1 * n).to(dtype))
+    return out
+
+
+def _score(fc, k, v, cu, gamma, repeat=1):
+    """scores [H, T] and energies [B, 4] of one layer, the same in every repetition"""
+    H, d, T = k.shape[1], k.shape[2], cu[-1]
+    h = fc.fc_create(0, max(cu[b + 1] - cu[b] for b in range(len(cu) - 1)))
+    try:
+        ws = torch.empty(fc.fc_score_workspace_bytes(h, k, v, cu), dtype=torch.uint8, device="cuda")
+        got = []
+        for i in range(repeat):
+            ws.fill_(255 if i % 2 else 0)
+            s = torch.full((H, T), -1.0, dtype=torch.float32, device="cuda")
+            e = torch.full((len(cu) - 1, 4), -1.0, dtype=torch.float64, device="cuda")
+            fc.fc_score_layer(h, k, v, cu, gamma, s, e, ws)
+            assert fc.fc_last_device_status(h) == 0
+            got.append((s.cpu(), e.cpu()))
+    finally:
+        fc.fc_destroy(h)
+    for s, e in got[1:]:
+        assert torch.equal(s, got[0][0]) and torch.equal(e, got[0][1])
+    return got[0]
+
+
+def _check(k, v, cu, gamma, scores, energy):
+    d = k.shape[2]
+    for b in range(len(cu) - 1):
+        sums = np.zeros(4)
+        for h in range(k.shape[1]):
+            kk, vv = (x[cu[b]:cu[b + 1], h].double().numpy() for x in (k, v))
+            o, _ = O.score_head(kk, vv, gamma, "fft")
+            g = scores[h, cu[b]:cu[b + 1]].double().numpy()
+            # A residual is z - base, the base a sum of fp32 products: its error per element is bounded by a small
+            # multiple (here 24) of 2^-24 times the head's values, and a score, the mean of the squares of 2d residuals,
+            # moves by at most twice its own root times that (plus the error's square).
+            eps = 24 * 2.0 ** -24 * math.sqrt(((kk ** 2).sum(1) + (vv ** 2).sum(1)).max() / d)
+            bound = 2 * np.sqrt(o) * eps + eps * eps + 1e-6 * o
+            assert (np.abs(g - o) <= bound).all(), "%d tokens, head %d: %.2f of the bound" % (
+                cu[b + 1] - cu[b], h, (np.abs(g - o) / bound).max())
+            rk, rv = kk - O.base_kv(kk, gamma, "fft")[0], vv - O.base_kv(vv, gamma, "fft")[0]
+            sums += [(rk ** 2).sum(), (kk ** 2).sum(), (rv ** 2).sum(), (vv ** 2).sum()]
+        assert np.allclose(energy[b].numpy(), sums, rtol=2e-6, atol=1e-12)
+
+
+# the smallest and largest sequences, every transform length, whole and broken ratios of tokens to grid points, lengths
+# around the 128-token and 16-point steps, cutoffs from none to beyond what the form takes, head widths of one to four tiles
+@pytest.mark.parametrize("N,H,d,gamma,dtype", [
+    (1024, 3, 128, 0.2, torch.bfloat16), (1025, 2, 64, 0.2, torch.float16), (1151, 1, 192, 0.15, torch.bfloat16),
+    (1281, 2, 128, 0.0, torch.bfloat16), (2047, 2, 128, 0.2, torch.float16), (2048, 1, 256, 0.3, torch.bfloat16),
+    (2500, 2, 128, 0.39, torch.bfloat16), (3072, 2, 64, 0.25, torch.float16), (4096, 2, 128, 0.2, torch.bfloat16),
+    (4097, 2, 128, 0.2, torch.bfloat16), (5119, 3, 128, 0.1, torch.float16), (8192, 2, 64, 0.2, torch.bfloat16),
+    (10164, 2, 128, 0.2, torch.bfloat16), (16384, 1, 128, 0.3, torch.float16), (32768, 1, 128, 0.3, torch.bfloat16),
+    (53602, 1, 128, 0.2, torch.float16), (65535, 1, 64, 0.2, torch.bfloat16), (65536, 1, 128, 0.2, torch.bfloat16),
+    (65536, 1, 64, 0.45, torch.bfloat16)])
+def test_band_scores(fc, N, H, d, gamma, dtype):
+    k, v = _kv(N, H, d, dtype, N)
+    s, e = _score(fc, k.cuda(), v.cuda(), [0, N], gamma, repeat=3)
+    _check(k, v, [0, N], gamma, s, e)
+
+
+def test_band_ragged_batch_strided_views_and_neighbours(fc):
+    # sequences of every form side by side, rows and heads strided, and non-finite rows of one sequence next to another's
+    lens = [1100, 300, 1100, 4096, 2311]
+    cu = [0] + [int(x) for x in np.cumsum(lens)]
+    k, v = _kv(cu[-1], 3, 64, torch.bfloat16, 5)
+    wide = [torch.full((cu[-1], 5, 80), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    kd, vd = (w[:, 1:4, :64] for w in wide)
+    kd.copy_(k)
+    vd.copy_(v)
+    s, e = _score(fc, kd, vd, cu, 0.2, repeat=2)
+    _check(k, v, cu, 0.2, s, e)
+    bad = k.clone()
+    bad[cu[2]:cu[2] + 40, 1, 3] = float("nan")
+    bad[cu[3] - 1, 1, 60] = float("inf")
+    kd.copy_(bad)
+    s2, _ = _score(fc, kd, vd, cu, 0.2)
+    assert torch.isnan(s2[1, cu[2]:cu[3]]).all()
+    s2[1, cu[2]:cu[3]] = s[1, cu[2]:cu[3]]
+    assert torch.equal(s, s2)
+
+
+def test_band_scales(fc):
+    # rows whose channels differ by many powers of two: a channel's values are scaled by themselves
+    k, v = _kv(2048, 1, 128, torch.bfloat16, 11)
+    f = torch.exp2(torch.arange(128) % 61 - 30.0)
+    k, v = (k.float() * f).to(torch.bfloat16), (v.float() * f.flip(0)).to(torch.bfloat16)
+    k[:, 0, 5] = 0.0
+    s, e = _score(fc, k.cuda(), v.cuda(), [0, 2048], 0.2)
+    _check(k, v, [0, 2048], 0.2, s, e)
