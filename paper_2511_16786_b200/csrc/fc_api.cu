@@ -202,7 +202,10 @@ extern "C" fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen) 
     h->tab_slot_len = m;
     for (int i = 0; i < FC_TAB_SLOTS; ++i) h->tab_key[i] = 0;
     h->tab_next = 0;
-    if (cudaMalloc(&h->tab_cache, (size_t)FC_TAB_SLOTS * h->tab_slot_len * sizeof(float4)) != cudaSuccess) {
+    for (int i = 0; i < FC_BAND_SLOTS; ++i) h->band_key[i] = 0;
+    h->band_next = 0;
+    if (cudaMalloc(&h->band_cache, FC_BAND_SLOTS * FC_BAND_SLOT_BYTES) != cudaSuccess ||
+        cudaMalloc(&h->tab_cache, (size_t)FC_TAB_SLOTS * h->tab_slot_len * sizeof(float4)) != cudaSuccess) {
       fc_destroy(h);
       return FC_ERR_CUDA;
     }
@@ -286,6 +289,7 @@ extern "C" void fc_destroy(fc_handle *h) {
   if (h->ev_inputs_free) cudaEventDestroy(h->ev_inputs_free);
   if (h->ev_outputs_done) cudaEventDestroy(h->ev_outputs_done);
   if (h->tab_cache) cudaFree(h->tab_cache);
+  if (h->band_cache) cudaFree(h->band_cache);
   if (h->master) cudaFree(h->master);
   if (h->status_word) cudaFree(h->status_word);
   if (h->done_counter) cudaFree(h->done_counter);

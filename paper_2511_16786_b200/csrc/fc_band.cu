@@ -52,10 +52,10 @@ const double (*responses())[band::kCheb] {
   return cheb;
 }
 
-constexpr int kMinGrid = 256, kMaxGrid = 16384;
+constexpr int kMinGrid = 128, kMaxGrid = 16384;
 
 bool eligible(const fc_kv_view *kv, int N) {
-  return kv->dtype != FC_F32 && N >= 1024 && N <= 65536 && kv->head_dim <= 512;
+  return kv->dtype != FC_F32 && N > 512 && N != 1024 && N <= 65536 && kv->head_dim <= 512;
 }
 
 // The coarsest grid on which the band fits: N/4 <= M <= N/2 and omega <= 0.8 M.
@@ -76,27 +76,53 @@ bool make_geometry(int N, int omega, Geometry *g) {
   g->fmax = kKernels[k].fmax;
   for (int i = 0; i < band::kCheb; ++i) g->cheb[i] = responses()[k][i];
   g->same = N == 2 * M || N == 4 * M;                      // 128 tokens are whole quads of the grid
-  g->ks = 0;
-  for (int b = 0; b < g->down_steps(); ++b) {
-    const int s = (band::down_end(*g, b) - band::down_start(*g, b) + 15) / 16;
-    if (s > g->ks) g->ks = s;
+  // The longest windows, over all steps or, where most are alike, over the first and last few and one between.
+  auto over = [&](int n, auto f) {
+    for (int b = 0; b < n; ++b) {
+      if (g->same && b == 4 && n > 8) b = n - 4;
+      f(b);
+    }
+  };
+  // floors of (a + i*d) / m for i = 0, 1, ..: one division, not one per step
+  struct Line {
+    long long q, r, dq, dr, m;
+    Line(long long a, long long d, long long m_) : q(band::floor_div(a, m_)), r(a - q * m_), dq(d / m_), dr(d % m_), m(m_) {}
+    void step() { q += dq; r += dr; if (r >= m) { r -= m; ++q; } }
+  };
+  int ks = 4, need = 8;
+  const auto down = [&](long long lo, long long hi) {            // window [lo, hi] before it is cut to the sequence
+    const int s = lo <= 0 ? 0 : (int)lo & ~15, e = hi + 1 > N ? N : (int)hi + 1, k = (e - s + 15) / 16;
+    if (k > ks) ks = k;
+  };
+  const auto up = [&](long long lo, long long hi) {
+    const int q = lo <= 0 ? 0 : (int)(lo >> 2) & ~3, e = (int)((hi > M - 1 ? M - 1 : hi) >> 2) + 1;
+    if (e - q > need) need = e - q;
+  };
+  if (g->same) {
+    over(g->down_steps(), [&](int b) {
+      down(band::ceil_div((2ll * band::kJ * b + 1 - g->W) * N - M, 2ll * M),
+           band::floor_div((2ll * (band::kJ * b + band::kJ - 1) + 1 + g->W) * N - M, 2ll * M));
+    });
+    over(g->up_steps(), [&](int b) {
+      up(band::ceil_div((2ll * band::kRows * b + 1) * M - (1ll + g->W) * N, 2ll * N),
+         band::floor_div((2ll * (band::kRows * b + band::kRows - 1) + 1) * M + (g->W - 1ll) * N, 2ll * N));
+    });
+  } else {
+    Line dl((1ll - g->W) * N - M + 2ll * M - 1, 2ll * band::kJ * N, 2ll * M);
+    Line dh((2ll * (band::kJ - 1) + 1 + g->W) * N - M, 2ll * band::kJ * N, 2ll * M);
+    for (int b = 0; b < g->down_steps(); ++b, dl.step(), dh.step()) down(dl.q, dh.q);
+    Line ul(M - (1ll + g->W) * N + 2ll * N - 1, 2ll * band::kRows * M, 2ll * N);
+    Line uh((2ll * (band::kRows - 1) + 1) * M + (g->W - 1ll) * N, 2ll * band::kRows * M, 2ll * N);
+    for (int b = 0; b < g->up_steps(); ++b, ul.step(), uh.step()) up(ul.q, uh.q);
   }
-  if (g->ks < 4) g->ks = 4;
-  g->nq = g->M / 4;                                        // no clamping at the end while the extent is measured
-  int need = 8;
-  for (int b = 0; b < g->up_steps(); ++b) {
-    const long long j = band::ceil_div((2ll * band::kRows * b + 1) * M - (1ll + g->W) * N, 2ll * N);
-    const int q = j <= 0 ? 0 : (int)(j >> 2) & ~3;
-    const int e = band::up_quad_end(*g, b) - q;
-    if (e > need) need = e;
-  }
+  g->ks = ks;
   g->nq = (need + 7) / 8 * 8;
   return g->ks <= band::kMaxSteps && g->nq <= band::kMaxQuads && g->nq <= g->M / 4;
 }
 
 // Mh and the radices of its stages
 #define FC_MID_SHAPES(X)                                                                                          \
-  X(128, 16, 8, 1, 1) X(256, 16, 16, 1, 1) X(512, 8, 8, 8, 1) X(1024, 16, 8, 8, 1) X(2048, 16, 16, 8, 1)          \
+  X(64, 8, 8, 1, 1) X(128, 16, 8, 1, 1) X(256, 16, 16, 1, 1) X(512, 8, 8, 8, 1) X(1024, 16, 8, 8, 1) X(2048, 16, 16, 8, 1)          \
   X(4096, 16, 16, 16, 1) X(8192, 16, 8, 8, 8)
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -186,48 +212,69 @@ void fc_band_release(FcBandJob *j) { delete j; }
 // values before the transform, two planes after it, a scale per row
 static size_t unit_bytes(const FcBandJob *j) { return j->y_bytes + 2 * j->plane_bytes + align256((size_t)2 * j->d * 4); }
 
-static size_t budget(const fc_handle *h) { return h->group_bytes > ((size_t)1 << 60) ? h->group_bytes : h->group_bytes / 2 * 3; }
+// Fuller launches beat intermediates that stay in L2 (28 layers of 4 heads of 32768 tokens: 2290 / 2056 / 1977 / 1902 us with
+// 48 / 96 / 192 / 384 MB; 192 MB is where the gain no longer pays for the workspace).
+static size_t budget(const fc_handle *h) { return h->group_bytes > ((size_t)1 << 60) ? h->group_bytes : h->group_bytes * 6; }
 
 size_t fc_band_buffer_bytes(const fc_handle *h, const FcBandSizes *s, int units) {
   const size_t all = s->unit * units, most = budget(h);
   return all < most ? all : s->unit > most ? s->unit : most;
 }
 
-int fc_band_units(const fc_handle *h, const FcBandJob *j, int units, size_t buf_bytes) {
-  int nu = (int)(buf_bytes / unit_bytes(j));
-  if (nu > units) nu = units;
-  if (nu < 1) nu = 1;
-  int groups = (units + nu - 1) / nu;
-  if (groups < h->num_aux && units >= h->num_aux) groups = h->num_aux;
-  return (units + groups - 1) / groups;
-}
-
-int fc_band_ranges(const FcBandJob *j, int units) {
-  const int n = j->g.up_steps();
-  int r = (148 + units - 1) / units;
+// Blocks a unit's n steps are spread over where a launch has so many units.
+static int spread(const fc_handle *h, int n, int units) {
+  int r = units < h->num_sms ? h->num_sms / units : 1;
   if (r > n) r = n;
-  const int floor_r = (n + band::kMaxPer - 1) / band::kMaxPer;
-  if (r < floor_r) r = floor_r;
+  const int least = (n + band::kMaxPer - 1) / band::kMaxPer;
+  if (r < least) r = least;
   const int per = (n + r - 1) / r;
   return (n + per - 1) / per;
+}
+int fc_band_ranges(const fc_handle *h, const FcBandJob *j, int units) { return spread(h, j->g.up_steps(), units); }
+
+// Launch groups: of the unit counts that fit, the one whose steps spread most evenly over the SMs (a launch costs about
+// four steps besides its own).
+int fc_band_units(const fc_handle *h, const FcBandJob *j, int units, size_t buf_bytes) {
+  int most = (int)(buf_bytes / unit_bytes(j)), best = 1;
+  if (most > units) most = units;
+  long long cost = -1;
+  const int n = j->g.up_steps();
+  for (int nu = 1; nu <= most; ++nu) {
+    const int groups = (units + nu - 1) / nu, even = (units + groups - 1) / groups;
+    if (even != nu) continue;
+    const int r = fc_band_ranges(h, j, nu), per = (n + r - 1) / r, waves = (nu * r + h->num_sms - 1) / h->num_sms;
+    const long long c = (long long)groups * (waves * per + 4);
+    if (cost < 0 || c <= cost) { cost = c; best = nu; }
+  }
+  return best;
+}
+
+size_t fc_band_table_bytes(const FcBandJob *j) { return j->table_bytes; }
+long long fc_band_table_key(const FcBandJob *j) { return (long long)j->g.N + ((long long)(j->g.omega + 1) << 20) + (j->f16 ? 1ll << 40 : 0); }
+
+static band::MidTables mid_tables(const FcBandJob *j, const char *tables) {
+  const int Mh = j->g.M / 2;
+  char *m = const_cast<char *>(tables) + j->off_mid;
+  return {reinterpret_cast<float4 *>(m), reinterpret_cast<float4 *>(m) + Mh / 2,
+          reinterpret_cast<float2 *>(m + align256((size_t)Mh * 16))};
 }
 
 fc_status fc_band_tables(fc_handle *h, cudaStream_t st, const FcBandJob *j, char *tables) {
   const Geometry &g = j->g;
-  fc_status s;
-  if (j->f16) band::k_down_table<__half, 2><<<band::down_classes(g), 256, 0, st>>>(g, reinterpret_cast<__half *>(tables));
-  else band::k_down_table<__nv_bfloat16, 3><<<band::down_classes(g), 256, 0, st>>>(g, reinterpret_cast<__nv_bfloat16 *>(tables));
-  if ((s = fc_after_launch(h)) != FC_OK) return s;
-  band::k_up_table<<<band::up_classes(g), 256, 0, st>>>(g, reinterpret_cast<__half *>(tables + j->off_up));
-  if ((s = fc_after_launch(h)) != FC_OK) return s;
-  const int Mh = g.M / 2;
-  char *m = tables + j->off_mid;
-  const band::MidTables t = {reinterpret_cast<float4 *>(m), reinterpret_cast<float4 *>(m) + Mh / 2,
-                             reinterpret_cast<float2 *>(m + align256((size_t)Mh * 16))};
+  const int Mh = g.M / 2, down = band::down_classes(g) * g.ks, up = band::up_classes(g) * g.nq * 2;
+  band::MidRadices r = {};
 #define X(M_, A_, B_, C_, D_) \
-  if (Mh == M_) band::k_mid_table<band::MidShape<A_, B_, C_, D_>><<<(Mh / 2 + 63) / 64, 64, 0, st>>>(g, t);
+  if (Mh == M_) r = band::MidRadices{{A_, C_ > 1 ? B_ : 1, D_ > 1 ? C_ : 1}, D_ > 1 ? D_ : C_ > 1 ? C_ : B_};
   FC_MID_SHAPES(X)
 #undef X
+  const int tw = mid_tw_len(Mh), mid = ((tw > Mh / 2 ? tw : Mh / 2) + 255) / 256;
+  __half *um = reinterpret_cast<__half *>(tables + j->off_up);
+  if (j->f16)
+    band::k_band_tables<__half, 2><<<down + up + mid, 256, 0, st>>>(g, r, reinterpret_cast<__half *>(tables), um,
+                                                                  mid_tables(j, tables), down, up);
+  else
+    band::k_band_tables<__nv_bfloat16, 3><<<down + up + mid, 256, 0, st>>>(g, r, reinterpret_cast<__nv_bfloat16 *>(tables), um,
+                                                                         mid_tables(j, tables), down, up);
   return fc_after_launch(h);
 }
 
@@ -236,12 +283,12 @@ fc_status fc_band_bind(fc_handle *h, FcBandJob *j, const fc_kv_view *kv, const F
   EncodeTiledFn fn = encode_fn();
   if (!fn) return FC_ERR_CUDA;
   const CUtensorMapDataType dt = j->f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-  const cuuint64_t dims[3] = {(cuuint64_t)j->d, (cuuint64_t)j->H, (cuuint64_t)j->g.N};
-  const cuuint64_t str[2] = {(cuuint64_t)kv->stride_head * 2, (cuuint64_t)kv->stride_token * 2};
-  const cuuint32_t box[3] = {64, 1, (cuuint32_t)band::kSlotTok}, ones[3] = {1, 1, 1};
+  const cuuint64_t dims[4] = {64, (cuuint64_t)j->g.N, (cuuint64_t)j->d / 64, (cuuint64_t)j->H};
+  const cuuint64_t str[3] = {(cuuint64_t)kv->stride_token * 2, 128, (cuuint64_t)kv->stride_head * 2};
+  const cuuint32_t box[4] = {64, (cuuint32_t)band::kSlotTok, j->d / 64 % 2 ? 1u : 2u, 1}, ones[4] = {1, 1, 1, 1};
   for (int i = 0; i < l.layers; ++i)
     for (int v = 0; v < 2; ++v) {
-      const CUresult r = fn(v ? &j->maps.v[i] : &j->maps.k[i], dt, 3, const_cast<void *>(v ? l.v[i] : l.k[i]), dims, str, box,
+      const CUresult r = fn(v ? &j->maps.v[i] : &j->maps.k[i], dt, 4, const_cast<void *>(v ? l.v[i] : l.k[i]), dims, str, box,
                             ones, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
       if (r != CUDA_SUCCESS) return FC_ERR_INTERNAL;
@@ -249,43 +296,85 @@ fc_status fc_band_bind(fc_handle *h, FcBandJob *j, const fc_kv_view *kv, const F
   return FC_OK;
 }
 
-template <class S>
-static fc_status launch_mid(fc_handle *h, cudaStream_t st, int rows, const band::MidParams &P) {
-  fc_status s = allow_smem<band::k_mid<S>>(h->device, S::smem, 70);
-  if (s != FC_OK) return s;
-  ProfScope ps(h, FC_K_PASS2, st);
-  band::k_mid<S><<<rows / S::ROWS, S::NT, S::smem, st>>>(P);
+// A launch that may start before the kernel in front of it has ended (`early`); the kernels wait for it where they need to.
+template <class... A, class... B>
+static fc_status launch(fc_handle *h, cudaStream_t st, bool early, void (*kern)(A...), dim3 grid, int threads, size_t smem, B &&...args) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = grid;
+  lc.blockDim = dim3((unsigned)threads);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at;
+  lc.numAttrs = early ? 1 : 0;
+  if (cudaLaunchKernelEx(&lc, kern, std::forward<B>(args)...) != cudaSuccess) {
+    cudaGetLastError();
+    return FC_ERR_CUDA;
+  }
   return fc_after_launch(h);
 }
 
+template <class S>
+static fc_status launch_mid(fc_handle *h, cudaStream_t st, bool early, int rows, const band::MidParams &P) {
+  fc_status s = allow_smem<band::k_mid<S>>(h->device, S::smem, 70);
+  if (s != FC_OK) return s;
+  ProfScope ps(h, FC_K_PASS2, st);
+  return launch(h, st, early, band::k_mid<S>, dim3((unsigned)(rows / (2 * S::PAIRS))), S::NT, S::smem, P);
+}
+
+template <typename T, int NQ>
+static fc_status launch_up(fc_handle *h, cudaStream_t st, bool early, const band::Maps &maps, const band::GridMaps &grid, const Geometry &g, const band::UpParams &P, int nu) {
+  const size_t sm = band::up_smem(NQ, P.d);
+  const fc_status s = allow_smem<band::k_up<T, NQ>>(h->device, sm, cudaSharedmemCarveoutMaxShared);
+  if (s != FC_OK) return s;
+  ProfScope ps(h, FC_K_PASS3, st);
+  return launch(h, st, early, band::k_up<T, NQ>, dim3(P.ranges, nu), band::kUpThreads, sm, maps, grid, g, P);
+}
+
+static fc_status encode_grid(band::GridMaps *m, const void *hi, int rows, int M, size_t plane_bytes) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return FC_ERR_CUDA;
+  const cuuint64_t dims[3] = {(cuuint64_t)M, (cuuint64_t)rows, 2}, str[2] = {(cuuint64_t)M * 2, (cuuint64_t)plane_bytes};
+  const cuuint32_t ones[3] = {1, 1, 1};
+  for (int w = 0; w < 2; ++w) {
+    const cuuint32_t box[3] = {w ? 32u : 16u, (cuuint32_t)band::kRows, 2};
+    if (fn(w ? &m->wide : &m->narrow, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void *>(hi), dims, str, box, ones,
+           CU_TENSOR_MAP_INTERLEAVE_NONE, w ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return FC_ERR_INTERNAL;
+  }
+  return FC_OK;
+}
+
 template <typename T>
-static fc_status run_group(fc_handle *h, cudaStream_t st, const FcBandJob *j, const FcBandLaunch &l, int u0, int nu, int ranges,
-                           char *buf) {
+static fc_status run_group(fc_handle *h, cudaStream_t st, const FcBandJob *j, const FcBandLaunch &l, int u0, int nu, int cap,
+                           int ranges, bool early, char *buf) {
   const Geometry &g = j->g;
   constexpr int TERMS = std::is_same<T, __half>::value ? 2 : 3;
   fc_status s;
   float *y = reinterpret_cast<float *>(buf);
-  __half *hi = reinterpret_cast<__half *>(buf + nu * j->y_bytes), *lo = hi + nu * (j->plane_bytes / 2);
-  float *inv = reinterpret_cast<float *>(buf + nu * (j->y_bytes + 2 * j->plane_bytes));
+  // the same places for every launch of a sequence, also where the last one has fewer units
+  __half *hi = reinterpret_cast<__half *>(buf + cap * j->y_bytes), *lo = hi + cap * (j->plane_bytes / 2);
+  float *inv = reinterpret_cast<float *>(buf + cap * (j->y_bytes + 2 * j->plane_bytes));
   const int tiles = j->d / 64, pairs = (tiles + 1) / 2, n = g.down_steps();
   {
     band::DownParams P = {l.tables, y, h->status_word, j->H, j->d, u0, 0};
-    int r = (148 + nu * pairs - 1) / (nu * pairs);
-    if (r > n) r = n;
+    const int r = spread(h, n, nu * pairs);
     P.per = (n + r - 1) / r;
-    if (P.per > band::kMaxPer) P.per = band::kMaxPer;
     if ((s = allow_smem<band::k_down<T, TERMS>>(h->device, band::kDownSmem, cudaSharedmemCarveoutMaxShared)) != FC_OK) return s;
     ProfScope ps(h, FC_K_PASS1, st);
-    band::k_down<T, TERMS><<<dim3((n + P.per - 1) / P.per, pairs, nu), band::kDownThreads, band::kDownSmem, st>>>(j->maps, g, P);
-    if ((s = fc_after_launch(h)) != FC_OK) return s;
+    // never early: the caller may have put a wait for an event in front of it, and its rows may be on their way until then
+    s = launch(h, st, false, band::k_down<T, TERMS>, dim3(r, pairs, nu), band::kDownThreads, band::kDownSmem,
+               j->maps, g, P);
+    if (s != FC_OK) return s;
   }
   {
     const int Mh = g.M / 2;
-    char *m = const_cast<char *>(l.tables) + j->off_mid;
-    const band::MidParams P = {y, hi, lo, inv, {reinterpret_cast<float4 *>(m), reinterpret_cast<float4 *>(m) + Mh / 2,
-                               reinterpret_cast<float2 *>(m + align256((size_t)Mh * 16))}};
+    const band::MidParams P = {y, hi, lo, inv, mid_tables(j, l.tables)};
     s = FC_ERR_INTERNAL;
-#define X(M_, A_, B_, C_, D_) if (Mh == M_) s = launch_mid<band::MidShape<A_, B_, C_, D_>>(h, st, nu * 2 * j->d, P);
+#define X(M_, A_, B_, C_, D_) if (Mh == M_) s = launch_mid<band::MidShape<A_, B_, C_, D_>>(h, st, early, nu * 2 * j->d, P);
     FC_MID_SHAPES(X)
 #undef X
     if (s != FC_OK) return s;
@@ -293,8 +382,6 @@ static fc_status run_group(fc_handle *h, cudaStream_t st, const FcBandJob *j, co
   {
     band::UpParams P = {};
     P.table = reinterpret_cast<const __half *>(l.tables + j->off_up);
-    P.hi = hi;
-    P.lo = lo;
     P.inv = inv;
     for (int i = 0; i < l.layers; ++i) P.scores[i] = l.scores[i];
     P.part = l.part;
@@ -308,14 +395,16 @@ static fc_status run_group(fc_handle *h, cudaStream_t st, const FcBandJob *j, co
     P.u0 = u0;
     P.ranges = ranges;
     P.per = (g.up_steps() + ranges - 1) / ranges;
-    const size_t sm = band::up_smem(g.nq, j->d);
-    if ((s = allow_smem<band::k_up<T>>(h->device, sm, cudaSharedmemCarveoutMaxShared)) != FC_OK) return s;
-    ProfScope ps(h, FC_K_PASS3, st);
-    band::k_up<T><<<dim3(ranges, nu), band::kUpThreads, sm, st>>>(j->maps, g, P);
-    return fc_after_launch(h);
+    band::GridMaps grid;
+    if ((s = encode_grid(&grid, hi, nu * 2 * j->d, g.M, cap * j->plane_bytes)) != FC_OK) return s;
+    return g.nq == 8    ? launch_up<T, 8>(h, st, early, j->maps, grid, g, P, nu)
+           : g.nq == 16 ? launch_up<T, 16>(h, st, early, j->maps, grid, g, P, nu)
+                        : launch_up<T, 24>(h, st, early, j->maps, grid, g, P, nu);
   }
 }
 
-fc_status fc_band_group(fc_handle *h, cudaStream_t st, const FcBandJob *j, const FcBandLaunch &l, int u0, int nu, int ranges, char *buf) {
-  return j->f16 ? run_group<__half>(h, st, j, l, u0, nu, ranges, buf) : run_group<__nv_bfloat16>(h, st, j, l, u0, nu, ranges, buf);
+fc_status fc_band_group(fc_handle *h, cudaStream_t st, const FcBandJob *j, const FcBandLaunch &l, int u0, int nu, int cap, int ranges,
+                        bool early, char *buf) {
+  return j->f16 ? run_group<__half>(h, st, j, l, u0, nu, cap, ranges, early, buf)
+                : run_group<__nv_bfloat16>(h, st, j, l, u0, nu, cap, ranges, early, buf);
 }

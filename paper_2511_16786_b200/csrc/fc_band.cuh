@@ -29,7 +29,9 @@ constexpr int kCheb = 28;                    // terms of the expansion of H
 constexpr float kUpScale = 1024.f;           // k_up's matrix is stored times this (its low terms stay normal fp16)
 constexpr float kDownScaleF16 = 4096.f;      // k_down's fp16 matrix is stored times this
 
-struct Maps {                                // one sequence's rows in every layer of the launch
+// One sequence's rows in every layer of the launch, as [head][64 channels][token][channel]: a box is 32 tokens of a tile's
+// two 64-channel halves where both are of K or both of V (8 KB; a load costs about 80 cycles besides its bytes), else of one.
+struct Maps {
   CUtensorMap k[FC_LAYER_CHUNK], v[FC_LAYER_CHUNK];
 };
 
@@ -109,55 +111,46 @@ __device__ inline double response(const Geometry &g, double f) {          // H(f
   return x * b1 - b2 + g.cheb[0];
 }
 
-// The matrix of one step of k_down: [16-token step * 2][term * 16 + j][8 tokens], rows of 16 bytes.
+// One entry of k_down's matrix of a step: [8 tokens' chunk][term * 16 + j][8 tokens], rows of 16 bytes.
 template <typename T, int TERMS>
-__global__ void k_down_table(const __grid_constant__ Geometry g, T *__restrict__ out) {
-  const int classes = down_classes(g), b = step_of(blockIdx.x, g.down_steps(), classes);
-  const int t0 = down_start(g, b), nt = g.ks * 16;
-  T *img = out + (size_t)blockIdx.x * (down_image(g, TERMS * kJ) / 2);
-  const double step = (double)g.N / g.M, inv = (double)g.M / g.N;
-  const double scale = TERMS == 2 ? inv * kDownScaleF16 : inv;
-  for (int i = threadIdx.x; i < nt * kJ; i += blockDim.x) {
-    const int e = i & 7, j = (i >> 3) & (kJ - 1), c = i >> 7, t = t0 + c * 8 + e;
-    double v = 0.0;
-    if (t < g.N) {
-      const double x = (b * kJ + j + 0.5) * step - 0.5;
-      v = phi(g, (t - x) * inv) + phi(g, (-1.0 - t - x) * inv) + phi(g, (2.0 * g.N - 1.0 - t - x) * inv);
-      v *= scale;
-    }
+__device__ __forceinline__ void down_entry(const Geometry &g, int cls, int i, T *__restrict__ out) {
+  const int b = step_of(cls, g.down_steps(), down_classes(g));
+  const int e = i & 7, j = (i >> 3) & (kJ - 1), c = i >> 7, t = down_start(g, b) + c * 8 + e;
+  T *img = out + (size_t)cls * (down_image(g, TERMS * kJ) / 2);
+  const double inv = (double)g.M / g.N;
+  double v = 0.0;
+  if (t < g.N) {
+    const double x = (b * kJ + j + 0.5) * ((double)g.N / g.M) - 0.5;
+    v = (phi(g, (t - x) * inv) + phi(g, (-1.0 - t - x) * inv) + phi(g, (2.0 * g.N - 1.0 - t - x) * inv)) * inv;
+    if (TERMS == 2) v *= kDownScaleF16;
+  }
 #pragma unroll
-    for (int k = 0; k < TERMS; ++k) {
-      const T h = (T)(float)v;
-      img[((size_t)c * (TERMS * kJ) + k * kJ + j) * 8 + e] = h;
-      v -= (double)(float)h;
-    }
+  for (int k = 0; k < TERMS; ++k) {
+    const T h = (T)(float)v;
+    img[((size_t)c * (TERMS * kJ) + k * kJ + j) * 8 + e] = h;
+    v -= (double)(float)h;
   }
 }
 
-// The matrix of one step of k_up: [term][8 grid values][token][8].  Values are in the order the transform keeps them:
-// first (z0, z2) of ascending quads, then (z3, z1) of descending ones.
-static __global__ void k_up_table(const __grid_constant__ Geometry g, __half *__restrict__ out) {
-  const int classes = up_classes(g), b = step_of(blockIdx.x, g.up_steps(), classes);
+// One entry of k_up's matrix of a step: [term][8 grid values][token][8].  Values are in the order the transform keeps
+// them: first (z0, z2) of ascending quads, then (z3, z1) of descending ones.
+__device__ __forceinline__ void up_entry(const Geometry &g, int cls, int i, __half *__restrict__ out) {
+  const int b = step_of(cls, g.up_steps(), up_classes(g));
   const int q0 = up_quad(g, b), nk = 4 * g.nq;
-  __half *img = out + (size_t)blockIdx.x * (up_image(g) / 2);
-  const double inv = (double)g.M / g.N;
-  for (int i = threadIdx.x; i < nk * kRows; i += blockDim.x) {
-    const int e = i & 7, r = (i >> 3) & (kRows - 1), c = i >> 10, k = c * 8 + e, t = b * kRows + r;
-    const bool second = k >= 2 * g.nq;
-    const int kk = second ? k - 2 * g.nq : k;
-    const int n = second ? q0 + g.nq - 1 - (kk >> 1) : q0 + (kk >> 1);
-    const int j = 4 * n + (second ? ((kk & 1) ? 1 : 3) : 2 * (kk & 1));
-    double v = 0.0;
-    if (t < g.N) {
-      const double x = (t + 0.5) * inv - 0.5;
-      v = phi(g, x - j) + phi(g, x + 1.0 + j) + phi(g, x - (2.0 * g.M - 1.0 - j));
-      v *= (double)kUpScale;
-    }
-    const __half h = __float2half_rn((float)v);
-    const __half l = __float2half_rn((float)(v - (double)__half2float(h)));
-    img[((size_t)c * kRows + r) * 8 + e] = h;
-    img[((size_t)(nk / 8 + c) * kRows + r) * 8 + e] = l;
+  __half *img = out + (size_t)cls * (up_image(g) / 2);
+  const int e = i & 7, r = (i >> 3) & (kRows - 1), c = i >> 10, k = c * 8 + e, t = b * kRows + r;
+  const bool second = k >= 2 * g.nq;
+  const int kk = second ? k - 2 * g.nq : k;
+  const int n = second ? q0 + g.nq - 1 - (kk >> 1) : q0 + (kk >> 1);
+  const int j = 4 * n + (second ? ((kk & 1) ? 1 : 3) : 2 * (kk & 1));
+  double v = 0.0;
+  if (t < g.N) {
+    const double x = (t + 0.5) * ((double)g.M / g.N) - 0.5;
+    v = (phi(g, x - j) + phi(g, x + 1.0 + j) + phi(g, x - (2.0 * g.M - 1.0 - j))) * (double)kUpScale;
   }
+  const __half h = __float2half_rn((float)v);
+  img[((size_t)c * kRows + r) * 8 + e] = h;
+  img[((size_t)(nk / 8 + c) * kRows + r) * 8 + e] = __float2half_rn((float)(v - (double)__half2float(h)));
 }
 
 // Everything k_mid looks up.  Stage twiddles w_L^(j p), p = 1, 2, 3, 4, 8, 12, for the stages before the last, and for
@@ -170,22 +163,33 @@ struct MidTables {
 // ---------------------------------------------------------------------------------------------------- the tensor cores
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 
-// Operand descriptor: start, leading and stride byte offsets in 16-byte units, layout 0 = none, 2 = 128-byte swizzle.
-__device__ __forceinline__ unsigned long long operand(unsigned addr, unsigned lead, unsigned stride, unsigned layout) {
-  return (unsigned long long)((addr >> 4) & 0x3fffu) | ((unsigned long long)((lead >> 4) & 0x3fffu) << 16) |
-         ((unsigned long long)((stride >> 4) & 0x3fffu) << 32) | (1ull << 46) | ((unsigned long long)layout << 61);
-}
+// Operand descriptor in two words: start and leading byte offset, stride byte offset and layout (0 = none, 2 = 128-byte
+// swizzle), in 16-byte units.  Starts move by adding to the first word.
+__host__ __device__ constexpr unsigned operand_lo(unsigned lead) { return (lead >> 4) << 16; }
+__host__ __device__ constexpr unsigned operand_hi(unsigned stride, unsigned layout) { return (stride >> 4) | (1u << 14) | (layout << 29); }
 // fp32 sums of 16-bit products; A 128 x 16, B 16 x n, B and (unless a_by_rows) A with consecutive depth.
 __host__ __device__ constexpr unsigned instruction(bool f16, bool a_by_rows, int n) {
   return (1u << 4) | ((f16 ? 0u : 1u) << 7) | ((f16 ? 0u : 1u) << 10) | ((a_by_rows ? 1u : 0u) << 15) |
          ((unsigned)(n >> 3) << 17) | ((unsigned)(128 >> 4) << 24);
 }
-__device__ __forceinline__ void mma(unsigned d, unsigned long long a, unsigned long long b, unsigned idesc, bool add) {
-  asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-               ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(add ? 1u : 0u) : "memory");
+// The warp that issues runs as a whole, and one lane of it issues: descriptors are then computed once per warp, in uniform
+// registers.  (A single lane in a branch of its own took 115..134 cycles per product, several times what a product takes.)
+__device__ __forceinline__ unsigned elect() {
+  unsigned e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+  return e;
 }
-__device__ __forceinline__ void commit(unsigned long long *bar) {          // arrives once all products issued so far are done
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(smem_addr(bar)) : "memory");
+__device__ __forceinline__ void mma(unsigned lead, unsigned d, unsigned alo, unsigned ahi, unsigned blo, unsigned bhi,
+                                    unsigned idesc, unsigned add) {
+  asm volatile("{\n .reg .pred p, q;\n .reg .b64 a, b;\n setp.ne.u32 q, %0, 0;\n setp.ne.u32 p, %7, 0;\n"
+               " mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n"
+               " @q tcgen05.mma.cta_group::1.kind::f16 [%1], a, b, %6, p;\n}\n"
+               ::"r"(lead), "r"(d), "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(add) : "memory");
+}
+__device__ __forceinline__ void commit(unsigned lead, unsigned long long *bar) {  // arrives once all products so far are done
+  asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %0, 0;\n"
+               " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%1];\n}\n"
+               ::"r"(lead), "r"(smem_addr(bar)) : "memory");
 }
 __device__ __forceinline__ void tmem_alloc(unsigned *slot, unsigned cols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_addr(slot)), "r"(cols) : "memory");
@@ -216,9 +220,31 @@ __device__ __forceinline__ void load_box(void *dst, const CUtensorMap *map, int 
                ::"r"(smem_addr(dst)), "l"(reinterpret_cast<unsigned long long>(map)), "r"(c), "r"(h), "r"(t),
                  "r"(smem_addr(bar)) : "memory");
 }
+__device__ __forceinline__ void load_rows_box(void *dst, const CUtensorMap *map, int half, int head, int t, unsigned long long *bar) {
+  asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];\n"
+               ::"r"(smem_addr(dst)), "l"(reinterpret_cast<unsigned long long>(map)), "r"(0), "r"(t), "r"(half), "r"(head),
+                 "r"(smem_addr(bar)) : "memory");
+}
+// 32 tokens from t of tile `tile` (rows 128 tile .. of K's channels and then V's); the second half `second` bytes on
+__device__ __forceinline__ void load_tile(unsigned char *dst, unsigned second, const Maps &maps, int layer, int d64, int tile,
+                                          int head, int t, unsigned long long *bar) {
+  const int h = 2 * tile;
+  if ((d64 & 1) == 0) {
+    load_rows_box(dst, h >= d64 ? &maps.v[layer] : &maps.k[layer], h >= d64 ? h - d64 : h, head, t, bar);
+  } else {
+    for (int i = 0; i < 2; ++i)
+      load_rows_box(dst + i * second, h + i >= d64 ? &maps.v[layer] : &maps.k[layer], h + i >= d64 ? h + i - d64 : h + i, head, t, bar);
+  }
+}
 __device__ __forceinline__ void load_bytes(void *dst, const void *src, unsigned bytes, unsigned long long *bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
                ::"r"(smem_addr(dst)), "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(smem_addr(bar)) : "memory");
+}
+
+// 32 aligned bytes: a whole sector per lane where the lanes' rows are far apart
+__device__ __forceinline__ void store8(float *p, float a, float b, float c, float d, float e, float f, float g, float h) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n"
+               ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d), "f"(e), "f"(f), "f"(g), "f"(h) : "memory");
 }
 
 // ---------------------------------------------------------------------------------------------------- k_down
@@ -229,14 +255,18 @@ struct DownParams {
   int H, d, u0;                              // heads, channels per head, first unit (layer * H + head) of the launch
   int per;                                   // steps per block
 };
+constexpr int kStepBars = 16;                // more than the steps whose windows fit the ring
 struct DownShared {
-  unsigned long long full[kRing], empty[kRing], tfull[2], tempty[2], afull[2], aempty[2], done;
+  unsigned long long full[kRing], step[kStepBars], tfull[2], aempty[2];
   unsigned tmem;
   int start[kMaxPer + 1];                    // of the block's steps and the one after
 };
-constexpr int kDownThreads = 192;            // loads, products, and four warps that take the sums out
+// Loads; a warp per tile that issues products (one warp spent as long between its steps, in waits, as in them, 2100 cycles
+// per step of two tiles); four warps that take the sums out.
+constexpr int kDownThreads = 224;
 constexpr unsigned kDownCols = 512;
-constexpr size_t kDownSmem = 1024 + (size_t)kRing * 4 * kBoxBytes + 2 * (size_t)kMaxSteps * 2 * 48 * 16;
+constexpr unsigned kDownTable = kMaxSteps * 2 * 48 * 16;
+constexpr size_t kDownSmem = 1024 + (size_t)kRing * 4 * kBoxBytes + 2 * (size_t)kDownTable;
 
 // One block: `per` steps of 16 grid points for up to two tiles (256 rows) of one unit.  grid (ranges, tile pairs, units).
 template <typename T, int TERMS>
@@ -253,15 +283,12 @@ __global__ void __launch_bounds__(kDownThreads, 1) k_down(const __grid_constant_
   const int n = g.down_steps(), classes = down_classes(g);
   const int b0 = blockIdx.x * P.per, b1 = b0 + P.per < n ? b0 + P.per : n;
   const unsigned img = (unsigned)down_image(g, NR);
-  unsigned char *tab1 = tab + (size_t)kMaxSteps * 2 * 48 * 16;
+  unsigned char *tab1 = tab + kDownTable;
 
   if (tid == 0) {
-    for (int i = 0; i < kRing; ++i) { mbar::init(&sh.full[i], 1u); mbar::init(&sh.empty[i], 1u); }
-    for (int i = 0; i < 2; ++i) {
-      mbar::init(&sh.tfull[i], 1u); mbar::init(&sh.tempty[i], 1u);
-      mbar::init(&sh.afull[i], 1u); mbar::init(&sh.aempty[i], 4u);
-    }
-    mbar::init(&sh.done, 1u);
+    for (int i = 0; i < kRing; ++i) mbar::init(&sh.full[i], 1u);
+    for (int i = 0; i < kStepBars; ++i) mbar::init(&sh.step[i], (unsigned)nt);
+    for (int i = 0; i < 2; ++i) { mbar::init(&sh.tfull[i], 1u); mbar::init(&sh.aempty[i], 4u); }
     mbar::init_done();
   }
   if (warp == 1) tmem_alloc(&sh.tmem, kDownCols);
@@ -270,18 +297,27 @@ __global__ void __launch_bounds__(kDownThreads, 1) k_down(const __grid_constant_
   __syncthreads();
   after_sync();
   const unsigned tmem = sh.tmem;
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   if (b0 < b1) {
     const int q0 = sh.start[0] / kSlotTok;                 // ring slots are counted from here
     if (warp == 0) {
       if (lane == 0) {
         bool ok = true;
-        int q = q0, ntab = 0, cls = -1;
+        int q = q0, ntab = 0, cls = -1, past = 0, since[2] = {0, 0};
+        // the products of every step before the `n`-th of this block are done (a step's barrier is waited for in turn, so
+        // none is met a phase late)
+        auto done_before = [&](int upto) {
+          for (; past < upto && ok; ++past) ok = mbar::wait(&sh.step[past % kStepBars], (unsigned)(past / kStepBars) & 1u);
+          return ok;
+        };
+        int free_to = b0;                                        // first step whose window starts past the slot wanted
         for (int b = b0; b < b1 && ok; ++b) {
           const int c = class_of(b, n, classes);
           if (c != cls) {
             cls = c;
             const int s = ntab & 1;
-            if (ntab >= 2 && !mbar::wait(&sh.tempty[s], (unsigned)(ntab / 2 - 1) & 1u)) { ok = false; break; }
+            since[s] = b - b0;                                   // the other buffer's matrix was used until here
+            if (ntab >= 2 && !done_before(since[s ^ 1])) break;
             mbar::expect_tx(&sh.tfull[s], img);
             load_bytes(s ? tab1 : tab, static_cast<const unsigned char *>(P.table) + (size_t)c * img, img, &sh.tfull[s]);
             ++ntab;
@@ -290,14 +326,14 @@ __global__ void __launch_bounds__(kDownThreads, 1) k_down(const __grid_constant_
           const int last = (sh.start[b - b0] + 16 * g.ks - 1) / kSlotTok;
           for (; q <= last; ++q) {
             const int i = q - q0, s = i % kRing;
-            if (i >= kRing && !mbar::wait(&sh.empty[s], (unsigned)(i / kRing - 1) & 1u)) { ok = false; break; }
-            mbar::expect_tx(&sh.full[s], (unsigned)(2 * nt * kBoxBytes));
-            for (int hf = 0; hf < 2 * nt; ++hf) {
-              const int c64 = (2 * tile0 + hf) * 64;             // K's channels, then V's
-              const bool isv = c64 >= P.d;
-              load_box(smem + (size_t)(s * 4 + hf) * kBoxBytes, isv ? &maps.v[layer] : &maps.k[layer], isv ? c64 - P.d : c64,
-                       head, q * kSlotTok, &sh.full[s]);
+            if (i >= kRing) {
+              while (free_to < b && sh.start[free_to - b0] / kSlotTok <= q - kRing) ++free_to;
+              if (!done_before(free_to - b0)) break;
             }
+            mbar::expect_tx(&sh.full[s], (unsigned)(2 * nt * kBoxBytes));
+            for (int t = 0; t < nt; ++t)
+              load_tile(smem + (size_t)(s * 4 + 2 * t) * kBoxBytes, kBoxBytes, maps, layer, tiles, tile0 + t, head, q * kSlotTok,
+                        &sh.full[s]);
           }
         }
         // no load may be in flight when the block ends
@@ -307,87 +343,78 @@ __global__ void __launch_bounds__(kDownThreads, 1) k_down(const __grid_constant_
         for (int i = ntab > 2 ? ntab - 2 : 0; i < ntab; ++i) ok &= mbar::wait(&sh.tfull[i & 1], (unsigned)(i / 2) & 1u);
         if (!ok) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
       }
-    } else if (warp == 1) {
-      if (lane == 0) {
-        constexpr unsigned idesc = instruction(TERMS == 2, true, NR);
-        bool ok = true;
-        int have = q0, freed = q0, ntab = 0, cls = -1;
-        for (int b = b0; b < b1 && ok; ++b) {
-          const int start = sh.start[b - b0], last = (start + 16 * g.ks - 1) / kSlotTok, it = b - b0, buf = it & 1;
-          const int c = class_of(b, n, classes);
-          if (c != cls) {
-            cls = c;
-            if (ntab > 0) commit(&sh.tempty[(ntab - 1) & 1]);
-            if (!mbar::wait(&sh.tfull[ntab & 1], (unsigned)(ntab / 2) & 1u)) { ok = false; break; }
-            ++ntab;
-          }
-          if (it >= 2 && !mbar::wait(&sh.aempty[buf], (unsigned)(it / 2 - 1) & 1u)) { ok = false; break; }
-          for (; have <= last && ok; ++have)
-            ok = mbar::wait(&sh.full[(have - q0) % kRing], (unsigned)((have - q0) / kRing) & 1u);
-          if (!ok) break;
-          after_sync();
-          const unsigned tb = smem_addr(((ntab - 1) & 1) ? tab1 : tab);
-          // steps from the window's ends to its middle, in two sums by turns: small terms first, few roundings of large sums
-          for (int i = 0; i < g.ks; ++i) {
-            const int k = (i & 1) ? g.ks - 1 - i / 2 : i / 2;
-            const int t16 = start / 16 + k, s = (t16 / 2 - q0) % kRing;
-            const unsigned long long bd = operand(tb + (unsigned)k * (2 * NR * 16), NR * 16, 128, 0);
-            for (int t = 0; t < nt; ++t) {
-              const unsigned long long ad =
-                  operand(smem_addr(smem + (size_t)(s * 4 + 2 * t) * kBoxBytes) + (t16 & 1) * 2048, kBoxBytes, 1024, 2);
-              mma(tmem + (unsigned)(((buf * 2 + t) * 2 + ((i >> 1) & 1)) * NR), ad, bd, idesc, i >= 4 || (i & 1));
-            }
-          }
-          commit(&sh.afull[buf]);
-          const int keep = b + 1 < b1 ? sh.start[b - b0 + 1] / kSlotTok : freed;
-          for (; freed < keep; ++freed) commit(&sh.empty[(freed - q0) % kRing]);
+    } else if (warp <= 2) {
+      constexpr unsigned idesc = instruction(TERMS == 2, true, NR), ahi = operand_hi(1024, 2), bhi = operand_hi(128, 0);
+      constexpr int kGroups = 2 * kRing;                         // 16-token groups in the ring
+      const unsigned lead = elect();
+      const int tile = warp - 1;
+      const unsigned abase = ((smem_addr(smem) >> 4) | operand_lo(kBoxBytes)) + (unsigned)tile * (2 * kBoxBytes / 16), bbase = (smem_addr(tab) >> 4) | operand_lo(NR * 16);
+      bool ok = true;
+      int have = q0, ntab = 0, cls = -1, it = 0;
+      for (int b = tile < nt ? b0 : b1; b < b1 && ok; ++b) {
+        const int start = __shfl_sync(0xffffffffu, sh.start[b - b0], 0), buf = it & 1;
+        const int last = (start + 16 * g.ks - 1) / kSlotTok, c = class_of(b, n, classes);
+        if (c != cls) {
+          cls = c;
+          if (!mbar::wait_warp(&sh.tfull[ntab & 1], (unsigned)(ntab / 2) & 1u)) { ok = false; break; }
+          ++ntab;
         }
-        commit(&sh.done);                                        // nothing is left running when the block ends
-        ok &= mbar::wait(&sh.done, 0u);
-        if (!ok) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
+        if (it >= 2 && !mbar::wait_warp(&sh.aempty[buf], (unsigned)(it / 2 - 1) & 1u)) { ok = false; break; }
+        for (; have <= last && ok; ++have)
+          ok = mbar::wait_warp(&sh.full[(have - q0) % kRing], (unsigned)((have - q0) / kRing) & 1u);
+        if (!ok) break;
+        after_sync();
+        const unsigned bl = bbase + (((ntab - 1) & 1) ? kDownTable / 16 : 0u);
+        const int pos = (start / 16 - 2 * q0) % kGroups;
+        // steps from the window's ends to its middle, in two sums by turns: small terms first, few roundings of large sums
+        for (int i = 0; i < g.ks; ++i) {
+          const int k = (i & 1) ? g.ks - 1 - i / 2 : i / 2;
+          int at = pos + k;
+          if (at >= kGroups) at -= kGroups;
+          const unsigned al = abase + (unsigned)(at >> 1) * (4 * kBoxBytes / 16) + (unsigned)(at & 1) * 128u;
+          mma(lead, tmem + (unsigned)(((buf * 2 + tile) * 2 + ((i >> 1) & 1)) * NR), al, ahi, bl + (unsigned)k * (2 * NR), bhi, idesc,
+              i >= 4 || (i & 1) ? 1u : 0u);
+        }
+        commit(lead, &sh.step[it % kStepBars]);
+        ++it;
       }
+      // nothing is left running when the block ends
+      if (it > 0) ok &= mbar::wait_warp(&sh.step[(it - 1) % kStepBars], (unsigned)((it - 1) / kStepBars) & 1u);
+      if (!ok && lane == 0) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
     } else {
       const int quad = warp & 3, row = quad * 32 + lane, Mh = g.M / 2;
       const float scale = TERMS == 2 ? 1.f / kDownScaleF16 : 1.f;
       for (int b = b0; b < b1; ++b) {
         const int it = b - b0, buf = it & 1;
-        if (!mbar::wait_warp(&sh.afull[buf], (unsigned)(it / 2) & 1u)) {
+        if (!mbar::wait_warp(&sh.step[it % kStepBars], (unsigned)(it / kStepBars) & 1u)) {
           if (lane == 0) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
           break;
         }
         after_sync();
         for (int t = 0; t < nt; ++t) {
           const unsigned at = tmem + ((unsigned)quad << 21) + (unsigned)((buf * 2 + t) * 2 * NR);
-          float v[16], a[16], c[16];
-          tmem_ld16(at + (TERMS - 1) * kJ, v);
-          tmem_ld16(at + NR + (TERMS - 1) * kJ, a);
-          tmem_wait(v);
-          tmem_wait(a);
+          float v[2 * TERMS][kJ];
 #pragma unroll
-          for (int j = 0; j < kJ; ++j) v[j] += a[j];
+          for (int k = 0; k < 2 * TERMS; ++k) tmem_ld16(at + k * kJ, v[k]);
 #pragma unroll
-          for (int k = TERMS - 2; k >= 0; --k) {
-            tmem_ld16(at + k * kJ, a);
-            tmem_ld16(at + NR + k * kJ, c);
-            tmem_wait(a);
-            tmem_wait(c);
-#pragma unroll
-            for (int j = 0; j < kJ; ++j) v[j] += a[j] + c[j];
+          for (int k = 0; k < 2 * TERMS; ++k) tmem_wait(v[k]);
+          if (t + 1 == nt) {                                      // the sums have been taken out
+            before_sync();
+            __syncwarp();
+            if (lane == 0) mbar::arrive(&sh.aempty[buf]);
           }
-          if (TERMS == 2) {
+          float r[kJ];
 #pragma unroll
-            for (int j = 0; j < kJ; ++j) v[j] *= scale;
+          for (int j = 0; j < kJ; ++j) {                          // low terms first
+            r[j] = v[TERMS - 1][j] + v[2 * TERMS - 1][j];
+#pragma unroll
+            for (int k = TERMS - 2; k >= 0; --k) r[j] += v[k][j] + v[TERMS + k][j];
+            if (TERMS == 2) r[j] *= scale;
           }
           float *yr = P.y + ((size_t)blockIdx.z * 2 * P.d + (tile0 + t) * kRows + row) * g.M;
-          float4 *lo = reinterpret_cast<float4 *>(yr + 8 * b), *hi = reinterpret_cast<float4 *>(yr + 2 * (Mh - 4 - 4 * b));
-          lo[0] = make_float4(v[0], v[2], v[4], v[6]);
-          lo[1] = make_float4(v[8], v[10], v[12], v[14]);
-          hi[0] = make_float4(v[15], v[13], v[11], v[9]);
-          hi[1] = make_float4(v[7], v[5], v[3], v[1]);
+          store8(yr + 8 * b, r[0], r[2], r[4], r[6], r[8], r[10], r[12], r[14]);
+          store8(yr + 2 * (Mh - 4 - 4 * b), r[15], r[13], r[11], r[9], r[7], r[5], r[3], r[1]);
         }
-        before_sync();
-        __syncwarp();
-        if (lane == 0) mbar::arrive(&sh.aempty[buf]);
       }
     }
   }
@@ -397,15 +424,16 @@ __global__ void __launch_bounds__(kDownThreads, 1) k_down(const __grid_constant_
 }
 
 // ---------------------------------------------------------------------------------------------------- k_mid
-// One real row of M grid values as a complex transform of Mh = M/2 points, Mh = R1*R2*R3*R4, 16 points per thread.
+// Two real rows of M grid values each as a complex transform of Mh = M/2 points, Mh = R1*R2*R3*R4, 16 points of both rows per
+// thread.
 template <int R1_, int R2_, int R3_, int R4_>
 struct MidShape {
   static constexpr int R1 = R1_, R2 = R2_, R3 = R3_, R4 = R4_, Mh = R1 * R2 * R3 * R4, T = Mh / 16;
   static constexpr int RL = R4 > 1 ? R4 : R3 > 1 ? R3 : R2;         // radix of the last stage
   static constexpr int S = Mh / RL;                                  // bins of the stages before it
-  static constexpr int ROWS = T >= 256 ? 1 : 256 / T, NT = T * ROWS;
-  static constexpr int LEN = Mh + Mh / 16;                           // one entry of padding per 16: conflict-free in every stage
-  static constexpr size_t smem = (size_t)ROWS * LEN * sizeof(float2);
+  static constexpr int PAIRS = T >= 128 ? 1 : 128 / T, NT = T * PAIRS;
+  static constexpr int LEN = Mh + Mh / RL;                           // one entry of padding per RL: conflict-free in every stage
+  static constexpr size_t smem = (size_t)PAIRS * LEN * sizeof(float4);
   __host__ __device__ static constexpr int sub_of(int k0) {          // position (in units of RL) of the bins k0 + S*i
     int pos = 0, rem = S, k = k0;
     const int r[3] = {R1, R4 > 1 || R3 > 1 ? R2 : 1, R4 > 1 ? R3 : 1};
@@ -417,42 +445,44 @@ struct MidShape {
   static constexpr int tw_len = 6 * (Mh / R1 + (R3 > 1 ? R3 * R4 : 0) + (R4 > 1 ? R4 : 0));
 };
 
-template <class S>
-__global__ void k_mid_table(const __grid_constant__ Geometry g, MidTables t) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < S::Mh / 2) {
-    // pair i: bins k0 + S*l and Mh minus that; the first RL of them are the blocks that are their own partners
-    const int k0 = i >= S::RL ? i / S::RL : i < S::RL / 2 ? 0 : S::S / 2;
-    const int l = i >= S::RL ? i % S::RL : i % (S::RL / 2), k = k0 + S::S * l;
-    auto gain = [&](int m) {
-      if (m > g.omega || m >= g.M) return 0.0;
-      const double h = response(g, (double)m / (2.0 * g.M));
+struct MidRadices {                          // of the stages (1 where there is none) and of the last one
+  int r[3], last;
+};
+// Entry i of k_mid's tables: pair i of bins, and a stage twiddle.
+__device__ __forceinline__ void mid_entry(const Geometry &g, const MidRadices &m, int i, const MidTables &t) {
+  const int Mh = g.M / 2, RL = m.last, S = Mh / RL;
+  if (i < Mh / 2) {
+    // bins k0 + S*l and Mh minus that; the first RL pairs are the blocks that are their own partners
+    const int k0 = i >= RL ? i / RL : i < RL / 2 ? 0 : S / 2;
+    const int l = i >= RL ? i % RL : i % (RL / 2), k = k0 + S * l;
+    auto gain = [&](int q) {
+      if (q > g.omega || q >= g.M) return 0.0;
+      const double h = response(g, (double)q / (2.0 * g.M));
       return 1.0 / (h * h);
     };
-    const double s = 1.0 / (4.0 * S::Mh);
+    const double s = 1.0 / (4.0 * Mh);
     if (k == 0) {
-      t.gain[i] = make_float4((float)(gain(0) / (2.0 * S::Mh)), (float)(gain(S::Mh) / (2.0 * S::Mh)),
-                              (float)(gain(S::Mh / 2) * s), (float)(gain(S::Mh + S::Mh / 2) * s));
+      t.gain[i] = make_float4((float)(gain(0) / (2.0 * Mh)), (float)(gain(Mh) / (2.0 * Mh)), (float)(gain(Mh / 2) * s),
+                              (float)(gain(Mh + Mh / 2) * s));
     } else {
-      t.gain[i] = make_float4((float)(gain(k) * s), (float)(gain(g.M - k) * s), (float)(gain(S::Mh - k) * (0.5 * s)),
-                              (float)(gain(S::Mh + k) * (0.5 * s)));
+      t.gain[i] = make_float4((float)(gain(k) * s), (float)(gain(g.M - k) * s), (float)(gain(Mh - k) * (0.5 * s)),
+                              (float)(gain(Mh + k) * (0.5 * s)));
     }
     double c, sn, c4, s4;
-    const int kr = k == 0 ? S::Mh / 2 : k;                            // entry 0 serves the bin Mh/2
+    const int kr = k == 0 ? Mh / 2 : k;                               // entry 0 serves the bin Mh/2
     sincospi((double)kr / (2.0 * g.M), &sn, &c);
     sincospi(2.0 * kr / (double)g.M, &s4, &c4);
     t.rot[i] = make_float4((float)c, (float)sn, (float)c4, (float)s4);
   }
-  const int pw[6] = {1, 2, 3, 4, 8, 12};
-  int base = 0, L = S::Mh;
-  const int r[3] = {S::R1, S::R3 > 1 ? S::R2 : 1, S::R4 > 1 ? S::R3 : 1};
+  int base = 0, L = Mh;
 #pragma unroll
   for (int s = 0; s < 3; ++s) {
-    if (r[s] == 1) continue;
-    const int sub = L / r[s];
-    for (int e = i; e < 6 * sub; e += gridDim.x * blockDim.x) {
+    if (m.r[s] == 1) continue;
+    const int sub = L / m.r[s], e = i - base;
+    if (e >= 0 && e < 6 * sub) {
+      const int w = e / sub;                                          // powers 1, 2, 3, 4, 8, 12
       double c, sn;
-      sincospi(2.0 * (double)(pw[e / sub] * (e % sub)) / (double)L, &sn, &c);
+      sincospi(2.0 * (double)((w < 4 ? w + 1 : w == 4 ? 8 : 12) * (e % sub)) / (double)L, &sn, &c);
       t.tw[base + e] = make_float2((float)c, (float)-sn);
     }
     base += 6 * sub;
@@ -460,45 +490,155 @@ __global__ void k_mid_table(const __grid_constant__ Geometry g, MidTables t) {
   }
 }
 
+// All tables of a sequence in one launch: `down` + `up` + the rest of the entries, 256 per block.
+template <typename T, int TERMS>
+__global__ void __launch_bounds__(256) k_band_tables(const __grid_constant__ Geometry g, const MidRadices m, T *down, __half *up,
+                                                     MidTables mid, int down_blocks, int up_blocks) {
+  int b = blockIdx.x;
+  if (b < down_blocks) {
+    const int per = g.ks;                                             // blocks per matrix: 16 * ks * 16 entries
+    down_entry<T, TERMS>(g, b / per, (b % per) * 256 + threadIdx.x, down);
+    return;
+  }
+  b -= down_blocks;
+  if (b < up_blocks) {
+    const int per = g.nq * 2;                                         // 4 * nq * 128 entries
+    up_entry(g, b / per, (b % per) * 256 + threadIdx.x, up);
+    return;
+  }
+  mid_entry(g, m, (b - up_blocks) * 256 + threadIdx.x, mid);
+}
+
+// Both rows' values side by side: every operation is a packed one, at half the issue slots.
+struct C2 {
+  float2 re, im;
+};
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
+__device__ __forceinline__ C2 operator+(const C2 &a, const C2 &b) { return {add2(a.re, b.re), add2(a.im, b.im)}; }
+__device__ __forceinline__ C2 operator-(const C2 &a, const C2 &b) { return {sub2(a.re, b.re), sub2(a.im, b.im)}; }
+// a * w and a * conj(w), w the same for both rows or not
+__device__ __forceinline__ C2 times(const C2 &a, const C2 &w) {
+  return {fma2(a.re, w.re, neg2(mul2(a.im, w.im))), fma2(a.re, w.im, mul2(a.im, w.re))};
+}
+__device__ __forceinline__ C2 times_conj(const C2 &a, const C2 &w) {
+  return {fma2(a.re, w.re, mul2(a.im, w.im)), fma2(a.im, w.re, neg2(mul2(a.re, w.im)))};
+}
+// a + DIR*j*b and a - DIR*j*b
+template <int DIR>
+__device__ __forceinline__ void sums_j(const C2 &a, const C2 &b, C2 &plus, C2 &minus) {
+  const C2 p = {sub2(a.re, b.im), add2(a.im, b.re)}, m = {add2(a.re, b.im), sub2(a.im, b.re)};
+  plus = DIR > 0 ? p : m;
+  minus = DIR > 0 ? m : p;
+}
+// e + w*o and e - w*o, w = c + DIR*j*s, the rotation folded into the sums: w = c (1 + DIR*j*s/c), or s (c/s + DIR*j)
+template <int DIR>
+__device__ __forceinline__ void sums_w(const C2 &e, const C2 &o, float c, float s, C2 &plus, C2 &minus) {
+  const bool by_c = fabsf(c) >= fabsf(s);
+  const float f = by_c ? c : s, t = by_c ? DIR * s / c : DIR * c / s;
+  // by_c: r = o (1 + j t);  else r = DIR * j o (1 - j t)
+  const C2 r = by_c ? C2{fma2(o.im, both(-t), o.re), fma2(o.re, both(t), o.im)}
+                    : DIR > 0 ? C2{fma2(o.re, both(t), neg2(o.im)), fma2(o.im, both(t), o.re)}
+                              : C2{fma2(o.re, both(-t), o.im), fma2(o.im, both(-t), neg2(o.re))};
+  plus = {fma2(r.re, both(f), e.re), fma2(r.im, both(f), e.im)};
+  minus = {fma2(r.re, both(-f), e.re), fma2(r.im, both(-f), e.im)};
+}
+template <int DIR>
+__device__ __forceinline__ void dft4p(C2 &x0, C2 &x1, C2 &x2, C2 &x3) {
+  const C2 a = x0 + x2, b = x0 - x2, c = x1 + x3, d = x1 - x3;
+  x0 = a + c;
+  x2 = a - c;
+  sums_j<DIR>(b, d, x1, x3);
+}
+template <int DIR>
+__device__ __forceinline__ void dft8p(C2 (&x)[8]) {
+  const float h = 0.70710678118654752440f;
+  dft4p<DIR>(x[0], x[2], x[4], x[6]);
+  dft4p<DIR>(x[1], x[3], x[5], x[7]);
+  const C2 e0 = x[0], e1 = x[2], e2 = x[4], e3 = x[6], o0 = x[1], o1 = x[3], o2 = x[5], o3 = x[7];
+  x[0] = e0 + o0;
+  x[4] = e0 - o0;
+  sums_w<DIR>(e1, o1, h, h, x[1], x[5]);
+  sums_j<DIR>(e2, o2, x[2], x[6]);
+  sums_w<DIR>(e3, o3, -h, h, x[3], x[7]);
+}
+template <int R, int DIR>
+__device__ __forceinline__ void dftp(C2 (&x)[R]) {
+  if constexpr (R == 8) {
+    dft8p<DIR>(x);
+  } else {
+    static_assert(R == 16, "radix 8 or 16");
+    const float c1 = 0.92387953251128675613f, s1 = 0.38268343236508977173f, h = 0.70710678118654752440f;
+    C2 e[8], o[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) { e[i] = x[2 * i]; o[i] = x[2 * i + 1]; }
+    dft8p<DIR>(e);
+    dft8p<DIR>(o);
+    x[0] = e[0] + o[0];
+    x[8] = e[0] - o[0];
+    sums_w<DIR>(e[1], o[1], c1, s1, x[1], x[9]);
+    sums_w<DIR>(e[2], o[2], h, h, x[2], x[10]);
+    sums_w<DIR>(e[3], o[3], s1, c1, x[3], x[11]);
+    sums_j<DIR>(e[4], o[4], x[4], x[12]);
+    sums_w<DIR>(e[5], o[5], -s1, c1, x[5], x[13]);
+    sums_w<DIR>(e[6], o[6], -h, h, x[6], x[14]);
+    sums_w<DIR>(e[7], o[7], -c1, s1, x[7], x[15]);
+  }
+}
+
 // x[p] *= w^p (conjugated for the way back), w^1, 2, 3, 4, 8, 12 from the table: at most two factors each
 template <int R, bool CONJ>
-__device__ __forceinline__ void turn(float2 *x, const float2 *__restrict__ tw, int sub, int j) {
-  float2 c[4];
+__device__ __forceinline__ void turn(C2 (&x)[R], const float2 *__restrict__ tw, int sub, int j) {
+  C2 c[4];
 #pragma unroll
-  for (int p = 1; p < (R < 4 ? R : 4); ++p) {
-    c[p] = __ldg(tw + (p - 1) * sub + j);
-    if (CONJ) c[p].y = -c[p].y;
-    x[p] = cmul(x[p], c[p]);
+  for (int p = 1; p < 4; ++p) {
+    const float2 w = __ldg(tw + (p - 1) * sub + j);
+    c[p] = {both(w.x), both(w.y)};
+    x[p] = CONJ ? times_conj(x[p], c[p]) : times(x[p], c[p]);
   }
 #pragma unroll
   for (int a = 1; a < R / 4; ++a) {
-    float2 b = __ldg(tw + (2 + a) * sub + j);
-    if (CONJ) b.y = -b.y;
-    x[4 * a] = cmul(x[4 * a], b);
+    const float2 w = __ldg(tw + (2 + a) * sub + j);
+    const C2 b = {both(w.x), both(w.y)};
+    x[4 * a] = CONJ ? times_conj(x[4 * a], b) : times(x[4 * a], b);
 #pragma unroll
-    for (int p = 1; p < 4; ++p) x[4 * a + p] = cmul(x[4 * a + p], cmul(b, c[p]));
+    for (int p = 1; p < 4; ++p) {
+      const C2 bc = times(b, c[p]);
+      x[4 * a + p] = CONJ ? times_conj(x[4 * a + p], bc) : times(x[4 * a + p], bc);
+    }
   }
 }
 
 struct MidParams {
   const float *y;                            // [row][M]
-  __half *hi, *lo;                           // [tile][quad / 4][row of the tile][8]
+  __half *hi, *lo;                           // [row][M]
   float *inv;                                // [row]: minus what a stored value has to be multiplied with
   MidTables t;
 };
 
 template <class S>
-__global__ void __launch_bounds__(S::NT, S::NT == 256 ? 4 : S::NT == 512 ? 2 : 1) k_mid(const MidParams P) {
-  constexpr int Mh = S::Mh, T = S::T;
-  extern __shared__ float2 X0[];
-  __shared__ float red[S::NT / 32 > 0 ? S::NT / 32 : 1];
+__global__ void __launch_bounds__(S::NT, S::NT <= 512 ? 512 / S::NT : 1) k_mid(const MidParams P) {
+  constexpr int Mh = S::Mh, T = S::T, RL = S::RL;
+  extern __shared__ float4 X0[];
+  __shared__ float red[2][S::NT / 32];
   const int tid = threadIdx.x, t = tid % T, rl = tid / T;
-  float2 *X = X0 + rl * S::LEN;
-  const size_t row = (size_t)blockIdx.x * S::ROWS + rl;
-  auto pad = [](int pos) { return pos + (pos >> 4); };
+  float4 *X = X0 + rl * S::LEN;
+  const size_t row = 2 * ((size_t)blockIdx.x * S::PAIRS + rl);
+  auto pad = [](int pos) { return pos + pos / RL; };
+  auto get = [&](int pos) {
+    const float4 v = X[pad(pos)];
+    return C2{make_float2(v.x, v.y), make_float2(v.z, v.w)};
+  };
+  auto put = [&](int pos, const C2 &v) { X[pad(pos)] = make_float4(v.re.x, v.re.y, v.im.x, v.im.y); };
   const float2 *src = reinterpret_cast<const float2 *>(P.y) + row * Mh;
   constexpr int T2 = 6 * (Mh / S::R1), T3 = T2 + 6 * (Mh / S::R1 / S::R2);
 
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
   // one stage on the points block*L + j + sub*p
   auto forward = [&](auto radix, int L, const float2 *tw, bool first, bool last) {
     constexpr int R = decltype(radix)::value;
@@ -506,13 +646,20 @@ __global__ void __launch_bounds__(S::NT, S::NT == 256 ? 4 : S::NT == 512 ? 2 : 1
 #pragma unroll
     for (int u = 0; u < 16 / R; ++u) {
       const int i = t + T * u, blk = i / sub, j = i - blk * sub, at = blk * L + j;
-      float2 x[R];
+      C2 x[R];
 #pragma unroll
-      for (int p = 0; p < R; ++p) x[p] = first ? __ldcg(src + at + sub * p) : X[pad(at + sub * p)];
-      dft_small<R, -1>(x);
+      for (int p = 0; p < R; ++p) {
+        if (first) {
+          const float2 a = __ldcg(src + at + sub * p), b = __ldcg(src + Mh + at + sub * p);
+          x[p] = {make_float2(a.x, b.x), make_float2(a.y, b.y)};
+        } else {
+          x[p] = get(at + sub * p);
+        }
+      }
+      dftp<R, -1>(x);
       if (!last) turn<R, false>(x, tw, sub, j);
 #pragma unroll
-      for (int p = 0; p < R; ++p) X[pad(at + sub * p)] = x[p];
+      for (int p = 0; p < R; ++p) put(at + sub * p, x[p]);
     }
     __syncthreads();
   };
@@ -526,30 +673,30 @@ __global__ void __launch_bounds__(S::NT, S::NT == 256 ? 4 : S::NT == 512 ? 2 : 1
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
     const int i = t + T * u;
-    const int k0 = i >= S::RL ? i / S::RL : i < S::RL / 2 ? 0 : S::S / 2;
-    const int l = i >= S::RL ? i % S::RL : i % (S::RL / 2);
-    const int pa = pad(S::sub_of(k0) * S::RL + l);
-    const int pb = i == 0 ? pad(S::RL / 2) : k0 == 0 ? pad(S::RL - l) : pad(S::sub_of(S::S - k0) * S::RL + S::RL - 1 - l);
-    float2 a = X[pa], b = X[pb];
+    const int k0 = i >= RL ? i / RL : i < RL / 2 ? 0 : S::S / 2;
+    const int l = i >= RL ? i % RL : i % (RL / 2);
+    const int pa = S::sub_of(k0) * RL + l;
+    const int pb = i == 0 ? RL / 2 : k0 == 0 ? RL - l : S::sub_of(S::S - k0) * RL + RL - 1 - l;
+    C2 a = get(pa), b = get(pb);
     float4 gn = __ldg(P.t.gain + i);
     const float4 rt = __ldg(P.t.rot + i);
     if (i == 0) {                            // bins 0 and, by itself, Mh/2
-      const float w0 = (a.x + a.y) * gn.x, wh = (a.x - a.y) * gn.y;
-      X[pa] = make_float2(w0 + wh, w0 - wh);
+      const float2 w0 = mul2(add2(a.re, a.im), both(gn.x)), wh = mul2(sub2(a.re, a.im), both(gn.y));
+      put(pa, {add2(w0, wh), sub2(w0, wh)});
       a = b;
       gn = make_float4(gn.z, gn.w, 0.5f * gn.z, 0.5f * gn.w);
     }
-    const float2 f = make_float2(rt.x, rt.y), e = make_float2(rt.z, rt.w);   // e^(j pi k/2M), e^(2 pi j k/M)
-    const float2 s = cmul_conj(make_float2(a.x + b.x, a.y - b.y), f);
-    const float2 r = cmul_conj(cmul_conj(make_float2(a.x - b.x, a.y + b.y), f), e);
-    const float2 p = make_float2((s.x + r.y) * gn.x, (s.y - r.x) * gn.y);    // r * -j
-    const float2 q = make_float2(s.x - r.y, s.y + r.x);
-    const float uu = (q.x - q.y) * gn.z, vv = (q.x + q.y) * gn.w;
-    const float2 q2 = make_float2(uu + vv, vv - uu);
-    const float2 gs = cadd(p, q2), gd = cmul(csub(p, q2), e);
-    const float2 z = cmul(make_float2(gs.x - gd.y, gs.y + gd.x), f), y = cmul(make_float2(gs.x + gd.y, gs.y - gd.x), f);
-    if (i != 0) X[pa] = z;
-    X[pb] = i == 0 ? z : make_float2(y.x, -y.y);
+    const C2 f = {both(rt.x), both(rt.y)}, e = {both(rt.z), both(rt.w)};     // e^(j pi k/2M), e^(2 pi j k/M)
+    const C2 s = times_conj(C2{add2(a.re, b.re), sub2(a.im, b.im)}, f);
+    const C2 r = times_conj(times_conj(C2{sub2(a.re, b.re), add2(a.im, b.im)}, f), e);
+    const C2 p = {mul2(add2(s.re, r.im), both(gn.x)), mul2(sub2(s.im, r.re), both(gn.y))};          // r * -j
+    const C2 q = {sub2(s.re, r.im), add2(s.im, r.re)};
+    const float2 uu = mul2(sub2(q.re, q.im), both(gn.z)), vv = mul2(add2(q.re, q.im), both(gn.w));
+    const C2 q2 = {add2(uu, vv), sub2(vv, uu)};
+    const C2 gs = p + q2, gd = times(p - q2, e);
+    const C2 z = times(C2{sub2(gs.re, gd.im), add2(gs.im, gd.re)}, f), y = times(C2{add2(gs.re, gd.im), sub2(gs.im, gd.re)}, f);
+    if (i != 0) put(pa, z);
+    put(pb, i == 0 ? z : C2{y.re, neg2(y.im)});
   }
   __syncthreads();
 
@@ -559,13 +706,13 @@ __global__ void __launch_bounds__(S::NT, S::NT == 256 ? 4 : S::NT == 512 ? 2 : 1
 #pragma unroll
     for (int u = 0; u < 16 / R; ++u) {
       const int i = t + T * u, blk = i / sub, j = i - blk * sub, at = blk * L + j;
-      float2 x[R];
+      C2 x[R];
 #pragma unroll
-      for (int p = 0; p < R; ++p) x[p] = X[pad(at + sub * p)];
+      for (int p = 0; p < R; ++p) x[p] = get(at + sub * p);
       if (!last) turn<R, true>(x, tw, sub, j);
-      dft_small<R, +1>(x);
+      dftp<R, +1>(x);
 #pragma unroll
-      for (int p = 0; p < R; ++p) X[pad(at + sub * p)] = x[p];
+      for (int p = 0; p < R; ++p) put(at + sub * p, x[p]);
     }
     __syncthreads();
   };
@@ -575,77 +722,96 @@ __global__ void __launch_bounds__(S::NT, S::NT == 256 ? 4 : S::NT == 512 ? 2 : 1
 
   // the last stage stays in registers: points j + (Mh/R1)*p
   constexpr int R = S::R1, sub = Mh / R;
-  float2 x[16];
-  float m = 0.f;
+  C2 x[16];
+  float2 m = make_float2(0.f, 0.f);
 #pragma unroll
   for (int u = 0; u < 16 / R; ++u) {
     const int j = t + T * u;
-    float2 y[R];
+    C2 y[R];
 #pragma unroll
-    for (int p = 0; p < R; ++p) y[p] = X[pad(j + sub * p)];
+    for (int p = 0; p < R; ++p) y[p] = get(j + sub * p);
     turn<R, true>(y, P.t.tw, sub, j);
-    dft_small<R, +1>(y);
+    dftp<R, +1>(y);
 #pragma unroll
     for (int p = 0; p < R; ++p) {
       x[u * R + p] = y[p];
-      m = fmaxf(m, fmaxf(fabsf(y[p].x), fabsf(y[p].y)));
+      m.x = fmaxf(m.x, fmaxf(fabsf(y[p].re.x), fabsf(y[p].im.x)));
+      m.y = fmaxf(m.y, fmaxf(fabsf(y[p].re.y), fabsf(y[p].im.y)));
     }
   }
-  // the row's largest value decides its power of two: values below 2^15 as two fp16 terms
+  // a row's largest value decides its power of two: values below 2^15 as two fp16 terms
   constexpr int G = T < 32 ? T : 32;
 #pragma unroll
-  for (int o = G / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  for (int o = G / 2; o > 0; o >>= 1) {
+    m.x = fmaxf(m.x, __shfl_xor_sync(0xffffffffu, m.x, o));
+    m.y = fmaxf(m.y, __shfl_xor_sync(0xffffffffu, m.y, o));
+  }
   if constexpr (T > 32) {
-    if ((tid & 31) == 0) red[tid >> 5] = m;
+    if ((tid & 31) == 0) { red[0][tid >> 5] = m.x; red[1][tid >> 5] = m.y; }
     __syncthreads();
 #pragma unroll
-    for (int w = 0; w < T / 32; ++w) m = fmaxf(m, red[rl * (T / 32) + w]);
+    for (int w = 0; w < T / 32; ++w) {
+      m.x = fmaxf(m.x, red[0][rl * (T / 32) + w]);
+      m.y = fmaxf(m.y, red[1][rl * (T / 32) + w]);
+    }
   }
-  int ex = (int)((__float_as_uint(m) >> 23) & 0xffu) - 127;            // m in [2^ex, 2^(ex+1))
-  ex = ex < -100 ? -100 : ex > 126 ? 126 : ex;
-  const float sc = __uint_as_float((unsigned)(14 - ex + 127) << 23);   // 2^(14 - ex)
-  if (t == 0) P.inv[row] = -__uint_as_float((unsigned)(ex - 14 + 127) << 23) * (1.f / kUpScale);
-  const size_t base = (row / kRows) * (size_t)(Mh / 4) * kRows + row % kRows;
-  __half2 *hi = reinterpret_cast<__half2 *>(P.hi), *lo = reinterpret_cast<__half2 *>(P.lo);
+  float2 sc;
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    int ex = (int)((__float_as_uint(r ? m.y : m.x) >> 23) & 0xffu) - 127;           // largest value in [2^ex, 2^(ex+1))
+    ex = ex < -100 ? -100 : ex > 126 ? 126 : ex;
+    (r ? sc.y : sc.x) = __uint_as_float((unsigned)(14 - ex + 127) << 23);           // 2^(14 - ex)
+    if (t == 0) P.inv[row + r] = -__uint_as_float((unsigned)(ex - 14 + 127) << 23) * (1.f / kUpScale);
+  }
+  __half2 *hi = reinterpret_cast<__half2 *>(P.hi) + row * Mh, *lo = reinterpret_cast<__half2 *>(P.lo) + row * Mh;
 #pragma unroll
   for (int u = 0; u < 16 / R; ++u)
 #pragma unroll
     for (int p = 0; p < R; ++p) {
       const int n = t + T * u + sub * p;
-      const float2 v = make_float2(x[u * R + p].x * sc, x[u * R + p].y * sc);
-      const __half2 h = __floats2half2_rn(v.x, v.y);
-      const float2 hf = __half22float2(h);
-      const size_t at = (base + (size_t)(n >> 2) * kRows) * 4 + (n & 3);
-      hi[at] = h;
-      lo[at] = __floats2half2_rn(v.x - hf.x, v.y - hf.y);
+      const float2 re = mul2(x[u * R + p].re, sc), im = mul2(x[u * R + p].im, sc);
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const float2 v = r ? make_float2(re.y, im.y) : make_float2(re.x, im.x);
+        const __half2 h = __floats2half2_rn(v.x, v.y);
+        const float2 hf = __half22float2(h);
+        hi[r * Mh + n] = h;
+        lo[r * Mh + n] = __floats2half2_rn(v.x - hf.x, v.y - hf.y);
+      }
     }
 }
 
 // ---------------------------------------------------------------------------------------------------- k_up
+// The two terms of a launch's grid values, [term][row][M]: boxes of 32 or 16 values of 128 rows of both terms.
+struct GridMaps {
+  CUtensorMap wide, narrow;
+};
 struct UpParams {
-  const __half *table, *hi, *lo;
+  const __half *table;
   const float *inv;
   float *scores[FC_LAYER_CHUNK];
-  double *part, *energy;                     // [unit of the call][range][4]; energy of the first layer
+  double *part, *energy;                     // [unit of the call][step][4]; energy of the first layer
   unsigned *done;                            // [layer]
   int *status;
   long long score_stride, energy_stride;
   int H, d, u0, per, ranges;
 };
 constexpr int kUpBufs = 4;                   // sums of 128 x 128 in tensor memory
-constexpr int kXStages = 2, kYStages = 2;
-constexpr int kUpThreads = 64 + 256;         // loads, products, and eight warps: four per 64 channels of a tile
+constexpr int kYStages = 2;
+constexpr int x_stages(int nq) { return nq <= 16 ? 3 : 2; }      // as many as fit
+constexpr int kMaxX = 3;
+constexpr int kUpThreads = 64 + 256 + 32;    // grid values and matrices, products, eight warps (four per 64 channels), rows
 struct UpShared {
-  unsigned long long xfull[kXStages], xempty[kXStages], yfull[kYStages], yempty[kYStages], tfull, tempty, afull[kUpBufs],
+  unsigned long long xfull[kMaxX], xempty[kMaxX], yfull[kYStages], yempty[kYStages], tfull, tempty, afull[kUpBufs],
       aempty[kUpBufs], done;
   unsigned tmem;
   int last;
   float other[2][kRows];
-  double red[8][4];
+  double red[2][8][4];
   int quad[kMaxPer];                         // first quad of the block's steps
 };
 __host__ __device__ inline size_t up_smem(int nq, int d) {
-  return 1024 + (size_t)kXStages * 8 * kBoxBytes + (size_t)(kYStages + 1) * nq * 2048 + (size_t)2 * d * sizeof(float);
+  return 1024 + (size_t)x_stages(nq) * 8 * kBoxBytes + (size_t)(kYStages + 1) * nq * 2048 + (size_t)2 * d * sizeof(float);
 }
 
 __device__ __forceinline__ uint4 lds(unsigned addr) {
@@ -653,7 +819,6 @@ __device__ __forceinline__ uint4 lds(unsigned addr) {
   asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
   return v;
 }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 template <typename T> __device__ __forceinline__ float2 widen(unsigned v);
 template <> __device__ __forceinline__ float2 widen<__half>(unsigned v) { return __half22float2(*reinterpret_cast<const __half2 *>(&v)); }
 template <> __device__ __forceinline__ float2 widen<__nv_bfloat16>(unsigned v) {
@@ -661,13 +826,15 @@ template <> __device__ __forceinline__ float2 widen<__nv_bfloat16>(unsigned v) {
 }
 
 // One block: `per` steps of 128 tokens of one unit.  grid (ranges, units).
-template <typename T>
-__global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Maps maps, const __grid_constant__ Geometry g,
+template <typename T, int NQ>
+__global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Maps maps, const __grid_constant__ GridMaps grid,
+                                                   const __grid_constant__ Geometry g,
                                                    const __grid_constant__ UpParams P) {
+  constexpr int kXStages = x_stages(NQ);
   extern __shared__ unsigned char raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(((uintptr_t)raw + 1023) & ~(uintptr_t)1023);
   unsigned char *ys = smem + (size_t)kXStages * 8 * kBoxBytes;
-  const unsigned ybytes = (unsigned)g.nq * 2048u, run = (unsigned)g.nq * 512u;     // both terms, both runs; one run
+  constexpr unsigned ybytes = NQ * 2048u, run = NQ * 512u;                         // both terms, both runs; one run
   unsigned char *tab = ys + (size_t)kYStages * ybytes;
   float *sinv = reinterpret_cast<float *>(tab + ybytes);
   __shared__ UpShared sh;
@@ -686,96 +853,108 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Ma
   }
   if (warp == 1) tmem_alloc(&sh.tmem, 128 * kUpBufs);
   for (int i = tid; i < b1 - b0; i += kUpThreads) sh.quad[i] = up_quad(g, b0 + i);
-  for (int i = tid; i < 2 * P.d; i += kUpThreads) sinv[i] = P.inv[(size_t)blockIdx.y * 2 * P.d + i];
   before_sync();
   __syncthreads();
   after_sync();
   const unsigned tmem = sh.tmem;
-  float sum[4] = {0.f, 0.f, 0.f, 0.f};
-  double en[4] = {0.0, 0.0, 0.0, 0.0};       // hiK, totK, hiV, totV
   if (warp == 0) {
     if (lane == 0) {
       bool ok = true;
-      int ntab = 0, cls = -1, ny = 0, nx = 0;
-      for (int b = b0; b < b1 && ok; ++b) {
-        const int c = class_of(b, n, classes), q0 = sh.quad[b - b0];
-        for (int t = 0; t < tiles && ok; ++t) {
-          {
-            const int s = ny % kYStages;
-            if (ny >= kYStages && !mbar::wait(&sh.yempty[s], (unsigned)(ny / kYStages - 1) & 1u)) { ok = false; break; }
-            mbar::expect_tx(&sh.yfull[s], ybytes);
-            const size_t tile = ((size_t)blockIdx.y * tiles + t) * (size_t)(g.M / 8);
-            const size_t r1 = (tile + q0 / 4) * (kRows * 8), r2 = (tile + (g.M / 2 - q0 - g.nq) / 4) * (kRows * 8);
-            unsigned char *dst = ys + (size_t)s * ybytes;
-            load_bytes(dst, P.hi + r1, run, &sh.yfull[s]);
-            load_bytes(dst + run, P.hi + r2, run, &sh.yfull[s]);
-            load_bytes(dst + 2 * run, P.lo + r1, run, &sh.yfull[s]);
-            load_bytes(dst + 3 * run, P.lo + r2, run, &sh.yfull[s]);
-            ++ny;
-          }
-          if (c != cls) {
-            cls = c;
-            if (ntab >= 1 && !mbar::wait(&sh.tempty, (unsigned)(ntab - 1) & 1u)) { ok = false; break; }
-            mbar::expect_tx(&sh.tfull, ybytes);
-            load_bytes(tab, reinterpret_cast<const unsigned char *>(P.table) + (size_t)c * ybytes, ybytes, &sh.tfull);
-            ++ntab;
-          }
-          const int s = nx % kXStages;
-          if (nx >= kXStages && !mbar::wait(&sh.xempty[s], (unsigned)(nx / kXStages - 1) & 1u)) { ok = false; break; }
-          mbar::expect_tx(&sh.xfull[s], 8u * kBoxBytes);
-          for (int hf = 0; hf < 2; ++hf) {
-            const int c64 = (2 * t + hf) * 64;
-            const bool isv = c64 >= P.d;
-            for (int i = 0; i < 4; ++i)
-              load_box(smem + (size_t)(s * 8 + hf * 4 + i) * kBoxBytes, isv ? &maps.v[layer] : &maps.k[layer],
-                       isv ? c64 - P.d : c64, head, b * kRows + i * kSlotTok, &sh.xfull[s]);
-          }
-          ++nx;
+      int ntab = 0, cls = -1, ny = 0;
+      const int items = (b1 - b0) * tiles;
+      for (int it = 0; it < items && ok; ++it) {
+        const int b = b0 + it / tiles, t = it - (b - b0) * tiles, c = class_of(b, n, classes), q0 = sh.quad[b - b0];
+        if (c != cls) {
+          cls = c;
+          if (ntab >= 1 && !mbar::wait(&sh.tempty, (unsigned)(ntab - 1) & 1u)) { ok = false; break; }
+          mbar::expect_tx(&sh.tfull, ybytes);
+          load_bytes(tab, reinterpret_cast<const unsigned char *>(P.table) + (size_t)c * ybytes, ybytes, &sh.tfull);
+          ++ntab;
         }
+        if (it == 0) {
+          asm volatile("griddepcontrol.wait;\n" ::: "memory");
+          asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+        }
+        const int s = ny % kYStages;
+        if (ny >= kYStages && !mbar::wait(&sh.yempty[s], (unsigned)(ny / kYStages - 1) & 1u)) { ok = false; break; }
+        mbar::expect_tx(&sh.yfull[s], ybytes);
+        const int r0 = ((int)blockIdx.y * tiles + t) * kRows;
+        unsigned char *dst = ys + (size_t)s * ybytes;
+        for (int rn = 0; rn < 2; ++rn, dst += 2 * run) {       // a run: 32 values' box where there are as many, then 16
+          const int x = rn == 0 ? 2 * q0 : g.M - 2 * (q0 + NQ);
+          if (NQ >= 16) load_box(dst, &grid.wide, x, r0, 0, &sh.yfull[s]);
+          if (NQ % 16) load_box(dst + (NQ >= 16 ? 2 * kRows * 64 : 0), &grid.narrow, x + (NQ >= 16 ? 32 : 0), r0, 0, &sh.yfull[s]);
+        }
+        ++ny;
       }
-      for (int i = nx > kXStages ? nx - kXStages : 0; i < nx; ++i) ok &= mbar::wait(&sh.xfull[i % kXStages], (unsigned)(i / kXStages) & 1u);
       for (int i = ny > kYStages ? ny - kYStages : 0; i < ny; ++i) ok &= mbar::wait(&sh.yfull[i % kYStages], (unsigned)(i / kYStages) & 1u);
       if (ntab > 0) ok &= mbar::wait(&sh.tfull, (unsigned)(ntab - 1) & 1u);
       if (!ok) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
     }
-  } else if (warp == 1) {
+  } else if (warp == 10) {
     if (lane == 0) {
-      constexpr unsigned idesc = instruction(true, false, kRows);
+      // rows do not come from the kernel in front: they are on their way before it ends
       bool ok = true;
-      int ntab = 0, cls = -1, it = 0;
-      for (int b = b0; b < b1 && ok; ++b) {
-        const int c = class_of(b, n, classes);
-        for (int t = 0; t < tiles; ++t, ++it) {
-          if (c != cls) {
-            cls = c;
-            if (ntab > 0) commit(&sh.tempty);
-            if (!mbar::wait(&sh.tfull, (unsigned)ntab & 1u)) { ok = false; break; }
-            ++ntab;
-          }
-          const int s = it % kYStages, buf = it % kUpBufs;
-          if (it >= kUpBufs && !mbar::wait(&sh.aempty[buf], (unsigned)(it / kUpBufs - 1) & 1u)) { ok = false; break; }
-          if (!mbar::wait(&sh.yfull[s], (unsigned)(it / kYStages) & 1u)) { ok = false; break; }
-          after_sync();
-          const unsigned ya = smem_addr(ys) + (unsigned)s * ybytes, ta = smem_addr(tab);
-          // low times high, high times low, high times high: small terms first
-          for (int pr = 0; pr < 3; ++pr)
-            for (int k = 0; k < g.nq / 4; ++k) {
-              const unsigned off = (unsigned)k * 4096u;
-              mma(tmem + (unsigned)buf * 128u, operand(ta + (pr == 0 ? 2 * run : 0u) + off, 2048, 128, 0),
-                  operand(ya + (pr == 1 ? 2 * run : 0u) + off, 2048, 128, 0), idesc, pr + k > 0);
-            }
-          commit(&sh.yempty[s]);
-          commit(&sh.afull[buf]);
-        }
+      const int items = (b1 - b0) * tiles;
+      int nx = 0;
+      for (; nx < items; ++nx) {
+        const int s = nx % kXStages, b = b0 + nx / tiles, t = nx - (b - b0) * tiles;
+        if (nx >= kXStages && !mbar::wait(&sh.xempty[s], (unsigned)(nx / kXStages - 1) & 1u)) { ok = false; break; }
+        mbar::expect_tx(&sh.xfull[s], 8u * kBoxBytes);
+        for (int i = 0; i < 4; ++i)
+          load_tile(smem + (size_t)(s * 8 + 2 * i) * kBoxBytes, kBoxBytes, maps, layer, tiles, t, head, b * kRows + i * kSlotTok,
+                    &sh.xfull[s]);
       }
-      commit(&sh.done);
-      ok &= mbar::wait(&sh.done, 0u);
+      for (int i = nx > kXStages ? nx - kXStages : 0; i < nx; ++i) ok &= mbar::wait(&sh.xfull[i % kXStages], (unsigned)(i / kXStages) & 1u);
       if (!ok) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
     }
+  } else if (warp == 1) {
+    constexpr unsigned idesc = instruction(true, false, kRows), hi = operand_hi(128, 0);
+    constexpr unsigned wide = operand_hi(512, 4), narrow = operand_hi(256, 6);     // 64- and 32-byte swizzle
+    const unsigned lead = elect();
+    const unsigned yb = (smem_addr(ys) >> 4) | operand_lo(16), tb = (smem_addr(tab) >> 4) | operand_lo(2048);
+    bool ok = true;
+    int ntab = 0, cls = -1, it = 0;
+    for (int b = b0; b < b1 && ok; ++b) {
+      const int c = class_of(b, n, classes);
+      for (int t = 0; t < tiles; ++t, ++it) {
+        if (c != cls) {
+          cls = c;
+          if (ntab > 0) commit(lead, &sh.tempty);
+          if (!mbar::wait_warp(&sh.tfull, (unsigned)ntab & 1u)) { ok = false; break; }
+          ++ntab;
+        }
+        const int s = it % kYStages, buf = it % kUpBufs;
+        if (it >= kUpBufs && !mbar::wait_warp(&sh.aempty[buf], (unsigned)(it / kUpBufs - 1) & 1u)) { ok = false; break; }
+        if (!mbar::wait_warp(&sh.yfull[s], (unsigned)(it / kYStages) & 1u)) { ok = false; break; }
+        after_sync();
+        const unsigned ya = yb + (unsigned)s * (ybytes / 16), d = tmem + (unsigned)buf * 128u;
+        // low times high, high times low, high times high: small terms first
+#pragma unroll
+        for (int pr = 0; pr < 3; ++pr)
+#pragma unroll
+          for (int k = 0; k < NQ / 4; ++k) {
+            const int in = k % (NQ / 8), part = NQ >= 16 && in >= 2;       // step within its run, and its box
+            const bool w = NQ >= 16 && !part;
+            const unsigned off = (k / (NQ / 8)) * (2 * run) + (w ? in * 32u : part ? 2u * kRows * 64u : 0u) +
+                                 (pr == 1 ? kRows * (w ? 64u : 32u) : 0u);
+            mma(lead, d, tb + (pr == 0 ? 2 * run / 16 : 0u) + k * 256u, hi, ya + off / 16, w ? wide : narrow, idesc,
+                pr + k > 0 ? 1u : 0u);
+          }
+        commit(lead, &sh.yempty[s]);
+        commit(lead, &sh.afull[buf]);
+      }
+    }
+    commit(lead, &sh.done);
+    ok &= mbar::wait_warp(&sh.done, 0u);
+    if (!ok && lane == 0) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
   } else {
     const int quad = warp & 3, half = (warp - 2) >> 2, row = quad * 32 + lane;
     bool failed = false;
     int it = 0;
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    for (int i = tid - 64; i < 2 * P.d; i += 256) sinv[i] = __ldcg(P.inv + (size_t)blockIdx.y * 2 * P.d + i);
+    asm volatile("bar.sync 1, 256;\n" ::: "memory");
     for (int b = b0; b < b1; ++b) {
       float2 r2[2][2], x2[2][2];             // [K, V][two chains]
 #pragma unroll
@@ -787,7 +966,7 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Ma
         if (failed) continue;
         after_sync();
         const int kv = (2 * t + half) * 64 >= P.d;
-        const unsigned xr = smem_addr(smem) + (unsigned)((s * 8 + half * 4) * kBoxBytes + row * 128);
+        const unsigned xr = smem_addr(smem) + (unsigned)((s * 8 + quad * 2 + half) * kBoxBytes + lane * 128);
         const unsigned iv = smem_addr(sinv + t * kRows + half * 64);
         const unsigned at = tmem + ((unsigned)quad << 21) + (unsigned)(buf * 128 + half * 64);
         float2 rs[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, xs[2] = {rs[0], rs[0]};
@@ -797,7 +976,7 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Ma
           tmem_ld16(at + 16 * c, a);
           uint4 xv[2];
 #pragma unroll
-          for (int i = 0; i < 2; ++i) xv[i] = lds(xr + (((2 * c + i) ^ (row & 7)) << 4));
+          for (int i = 0; i < 2; ++i) xv[i] = lds(xr + (((2 * c + i) ^ (lane & 7)) << 4));
           tmem_wait(a);
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
@@ -828,37 +1007,45 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Ma
       }
       const int tok = b * kRows + row;
       const bool in = tok < g.N;
+      float sum[4];                          // hiK, totK, hiV, totV of this thread's row and channels
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         sum[2 * i] = in ? (r2[i][0].x + r2[i][0].y) + (r2[i][1].x + r2[i][1].y) : 0.f;
         sum[2 * i + 1] = in ? (x2[i][0].x + x2[i][0].y) + (x2[i][1].x + x2[i][1].y) : 0.f;
       }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) en[i] += (double)sum[i];
+      // sums of the step, so that the energies do not depend on how steps are spread over blocks: four values over the
+      // lanes at once, lane 8 i ends up with value i
+      {
+        const bool up = (lane & 16) != 0, up2 = (lane & 8) != 0;
+        double v0 = up ? (double)sum[2] : (double)sum[0], v1 = up ? (double)sum[3] : (double)sum[1];
+        v0 += __shfl_xor_sync(0xffffffffu, up ? (double)sum[0] : (double)sum[2], 16);
+        v1 += __shfl_xor_sync(0xffffffffu, up ? (double)sum[1] : (double)sum[3], 16);
+        double v = up2 ? v1 : v0;
+        v += __shfl_xor_sync(0xffffffffu, up2 ? v0 : v1, 8);
+        v += __shfl_xor_sync(0xffffffffu, v, 4);
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        if ((lane & 7) == 0) sh.red[(b - b0) & 1][warp - 2][lane >> 3] = v;
+      }
       float &o = sh.other[(b - b0) & 1][row];
       if (half == 1) o = sum[0] + sum[2];
       asm volatile("bar.sync 1, 256;\n" ::: "memory");
       if (half == 0 && in)
         P.scores[layer][(long long)head * P.score_stride + tok] = (sum[0] + sum[2] + o) * (1.f / (float)P.d);
+      if (warp == 9 && lane < 4) {
+        double v = 0.0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) v += sh.red[(b - b0) & 1][w][lane];
+        P.part[((size_t)unit * n + b) * 4 + lane] = v;
+      }
     }
     if (failed && lane == 0) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const double v = warp_sum_d(en[i]);
-      if (lane == 0) sh.red[warp - 2][i] = v;
-    }
+    __threadfence();
   }
   before_sync();
   __syncthreads();
   if (warp == 1) tmem_free(tmem, 128 * kUpBufs);
-  // energies: this block's sums, then, in the block of the layer that comes last, all of them in order
-  if (tid < 4) {
-    double v = 0.0;
-    for (int w = 0; w < 8; ++w) v += sh.red[w][tid];
-    P.part[((size_t)unit * P.ranges + blockIdx.x) * 4 + tid] = v;
-    __threadfence();
-  }
-  __syncthreads();
+  // energies: in the block of the layer that comes last, all steps' sums in order
   if (tid == 0) {
     __threadfence();
     const unsigned all = (unsigned)(P.H * P.ranges);
@@ -868,9 +1055,9 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Ma
   }
   __syncthreads();
   if (sh.last && warp < 4) {
-    const double *p = P.part + (size_t)layer * P.H * P.ranges * 4;
+    const double *p = P.part + (size_t)layer * P.H * n * 4;
     double v = 0.0;
-    for (int i = lane; i < P.H * P.ranges; i += 32) v += __ldcg(p + 4 * (size_t)i + warp);
+    for (int i = lane; i < P.H * n; i += 32) v += __ldcg(p + 4 * (size_t)i + warp);
     v = warp_sum_d(v);
     if (lane == 0) P.energy[(long long)layer * P.energy_stride + warp] = v;
   }

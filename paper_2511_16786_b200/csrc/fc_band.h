@@ -20,8 +20,11 @@ struct FcBandJob;
 FcBandJob *fc_band_plan(const fc_handle *h, const fc_kv_view *kv, int N, int omega);
 void fc_band_release(FcBandJob *j);
 int fc_band_units(const fc_handle *h, const FcBandJob *j, int units, size_t buf_bytes);   // units per launch
-int fc_band_ranges(const FcBandJob *j, int units);      // blocks a unit's rows are spread over where a launch has so many units
-// The sequence's tables, built on `st`.
+int fc_band_ranges(const fc_handle *h, const FcBandJob *j, int units);      // blocks a unit's rows are spread over where a launch has so many units
+// The sequence's tables: their size, what they depend on (the dtype, the length and the cutoff), and the launch that builds
+// them on `st`.
+size_t fc_band_table_bytes(const FcBandJob *j);
+long long fc_band_table_key(const FcBandJob *j);
 fc_status fc_band_tables(fc_handle *h, cudaStream_t st, const FcBandJob *j, char *tables);
 struct FcBandLaunch {
   const void *const *k, *const *v;     // first token of the sequence, layer by layer
@@ -34,5 +37,7 @@ struct FcBandLaunch {
 };
 // Tensor maps of the layers' rows; the launches of fc_band_group use them until the next call.
 fc_status fc_band_bind(fc_handle *h, FcBandJob *j, const fc_kv_view *kv, const FcBandLaunch &l);
-// Units [u0, u0 + nu) on `st`, intermediates at `buf`.
-fc_status fc_band_group(fc_handle *h, cudaStream_t st, const FcBandJob *j, const FcBandLaunch &l, int u0, int nu, int ranges, char *buf);
+// Units [u0, u0 + nu) on `st`, intermediates at `buf`, laid out for `cap` units.  `early`: kernels are
+// set up while the one in front ends (where the launch group has its stream to itself).
+fc_status fc_band_group(fc_handle *h, cudaStream_t st, const FcBandJob *j, const FcBandLaunch &l, int u0, int nu, int cap, int ranges,
+                        bool early, char *buf);

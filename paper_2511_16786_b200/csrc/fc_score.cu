@@ -1313,14 +1313,68 @@ fc_status score_sequence(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, co
   return FC_OK;
 }
 
-// One sequence in the kept band, for a chunk of layers.  `lp` points at the sequence's first token.
-fc_status score_band(fc_handle *h, const fc_kv_view *kv, FcBandJob *job, int nl, const fast::LayerPtrs &lp, double *energy,
-                     long long energy_stride, const ScoreLayout &L, char *wsb, const char *tables) {
+struct Jobs : std::vector<FcBandJob *> {
+  using std::vector<FcBandJob *>::vector;
+  ~Jobs() { for (FcBandJob *j : *this) fc_band_release(j); }
+};
+
+// Tables of the sequences scored in the kept band, as prepare_tables does it: the handle keeps the last few that fit a slot,
+// the others, and all while the stream is being captured, are built into the workspace.
+fc_status band_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const Jobs &band, char *spare, const char **tabs) {
+  bool cached = true, any = false, flushed = false;
+  bool used[FC_BAND_SLOTS] = {};
+  for (int b = 0; b < kv->batch; ++b) {
+    if (!band[b]) continue;
+    if (!any) {
+      any = true;
+      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+      if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { cudaGetLastError(); cap = cudaStreamCaptureStatusActive; }
+      cached = cap == cudaStreamCaptureStatusNone;
+    }
+    for (int i = 0; cached && i < FC_BAND_SLOTS; ++i)
+      if (h->band_key[i] == fc_band_table_key(band[b])) { tabs[b] = h->band_cache + i * FC_BAND_SLOT_BYTES; used[i] = true; }
+  }
+  for (int b = 0; b < kv->batch; ++b) {
+    if (!band[b] || tabs[b]) continue;
+    for (int i = 0; i < b && !tabs[b]; ++i)
+      if (band[i] && fc_band_table_key(band[i]) == fc_band_table_key(band[b])) tabs[b] = tabs[i];
+    if (tabs[b]) continue;
+    fc_status s;
+    // the tables' place may still be in use on the internal streams
+    if (!flushed && (s = fc_flush_pending(h, st)) != FC_OK) return s;
+    flushed = true;
+    int slot = -1;
+    for (int i = 0; cached && fc_band_table_bytes(band[b]) <= FC_BAND_SLOT_BYTES && i < FC_BAND_SLOTS && slot < 0; ++i) {
+      const int c = (h->band_next + i) % FC_BAND_SLOTS;
+      if (!used[c]) slot = c;
+    }
+    char *dst = spare;
+    if (slot >= 0) {
+      h->band_next = (slot + 1) % FC_BAND_SLOTS;
+      h->band_key[slot] = 0;                                   // not valid until its launch is in the stream
+      used[slot] = true;
+      dst = h->band_cache + slot * FC_BAND_SLOT_BYTES;
+    } else {
+      FcBandSizes bs;
+      fc_band_bounds(kv, kv->cu_seqlens[b + 1] - kv->cu_seqlens[b], &bs);
+      spare += bs.tables;
+    }
+    if ((s = fc_band_tables(h, st, band[b], dst)) != FC_OK) return s;
+    if (slot >= 0) h->band_key[slot] = fc_band_table_key(band[b]);
+    tabs[b] = dst;
+  }
+  return FC_OK;
+}
+
+// One sequence in the kept band, for a chunk of layers, on the internal streams or, with on_caller, on `st`.  `lp` points at
+// the sequence's first token.
+fc_status score_band(fc_handle *h, cudaStream_t st, bool on_caller, const fc_kv_view *kv, FcBandJob *job, int nl, const fast::LayerPtrs &lp,
+                     double *energy, long long energy_stride, const ScoreLayout &L, char *wsb, const char *tables) {
   const int U = nl * kv->num_heads;
-  const int nu = fc_band_units(h, job, U, L.buf_bytes);
-  const int ranges = fc_band_ranges(job, nu);
+  const int nu = fc_band_units(h, job, U, L.buf_bytes), groups = (U + nu - 1) / nu;
+  const int ranges = fc_band_ranges(h, job, nu);
   const unsigned par = h->step & 1u;               // as in score_sequence
-  if (h->step >= 2)
+  if (!on_caller && h->step >= 2)
     for (int i = 0; i < h->num_aux; ++i)
       for (int o = 0; o < h->num_aux; ++o)
         if (o != i) FC_CUDA_TRY(cudaStreamWaitEvent(h->aux[i], h->ev_done[par][o], 0));
@@ -1330,10 +1384,13 @@ fc_status score_band(fc_handle *h, const fc_kv_view *kv, FcBandJob *job, int nl,
   if (s != FC_OK) return s;
   int group = 0;
   for (int u0 = 0; u0 < U; u0 += nu, ++group) {
-    const int si = (int)((group + h->step) % (unsigned)h->num_aux);
-    s = fc_band_group(h, h->aux[si], job, l, u0, U - u0 < nu ? U - u0 : nu, ranges, wsb + L.off_buf + (size_t)si * L.buf_bytes);
+    const int si = on_caller ? 0 : (int)((group + h->step) % (unsigned)h->num_aux);
+    s = fc_band_group(h, on_caller ? st : h->aux[si], job, l, u0, U - u0 < nu ? U - u0 : nu, nu, ranges,
+                      on_caller || groups <= h->num_aux,
+                      wsb + L.off_buf + (size_t)si * L.buf_bytes);
     if (s != FC_OK) return s;
   }
+  if (on_caller) return FC_OK;
   for (int i = 0; i < h->num_aux; ++i) FC_CUDA_TRY(cudaEventRecord(h->ev_done[par][i], h->aux[i]));
   h->step++;
   h->pending_join = true;
@@ -1523,13 +1580,10 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
   const int B = kv->batch;
   const ScoreLayout L = score_layout(h, kv, num_layers);
   fc_status s;
-  bool fork = true, direct_only = true, any_fast = false, any_small = false, any_passes = false;
+  bool fork = true, direct_only = true, any_fast = false, any_small = false, any_passes = false, any_band = false;
   std::vector<PassPlan> plans(B);
   std::vector<const float4 *> tabs(B, nullptr);
-  struct Jobs : std::vector<FcBandJob *> {
-    using std::vector<FcBandJob *>::vector;
-    ~Jobs() { for (FcBandJob *j : *this) fc_band_release(j); }
-  } band(B, nullptr);
+  Jobs band(B, nullptr);
   std::vector<const char *> band_tabs(B, nullptr);
   for (int b = 0; b < B; ++b) {
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
@@ -1537,6 +1591,7 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
     if (!h->generic_only) plans[b] = plan_passes(N, kv->head_dim);
     band[b] = fc_band_plan(h, kv, N, cutoff_index(gamma, N));
     if (band[b]) {
+      any_band = true;
       plans[b].ok = true;
       plans[b].small = plans[b].pad = false;
     }
@@ -1547,19 +1602,18 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
   }
   if (any_fast && (s = prepare_tables(h, st, kv, gamma, false, reinterpret_cast<float4 *>(wsb + L.off_tab),
                                       reinterpret_cast<float2 *>(wsb + L.off_buf), tabs.data(), band.data())) != FC_OK) return s;
-  char *band_at = wsb + L.off_band;
-  for (int b = 0; b < B; ++b) {
-    if (!band[b]) continue;
-    const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
-    for (int i = 0; i < b && !band_tabs[b]; ++i)
-      if (kv->cu_seqlens[i + 1] - kv->cu_seqlens[i] == N) band_tabs[b] = band_tabs[i];
-    if (band_tabs[b]) continue;
-    // the tables' place may still be in use on the internal streams
-    if ((s = fc_flush_pending(h, st)) != FC_OK || (s = fc_band_tables(h, st, band[b], band_at)) != FC_OK) return s;
-    band_tabs[b] = band_at;
-    FcBandSizes bs;
-    fc_band_bounds(kv, N, &bs);
-    band_at += bs.tables;
+  if ((s = band_tables(h, st, kv, band, wsb + L.off_band, band_tabs.data())) != FC_OK) return s;
+  bool on_caller = any_band;                   // little enough to stay on the caller's stream: no fork, no join
+  {
+    long long steps = 0;
+    for (int b = 0; b < B; ++b) {
+      const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
+      if (band[b]) steps += (long long)((N + 127) / 128) * (num_layers < FC_LAYER_CHUNK ? num_layers : FC_LAYER_CHUNK) * kv->num_heads;
+      else if (N > 0 && !plans[b].small) on_caller = false;
+    }
+    // 128-token steps per SM; from about two on, two streams are worth their fork
+    on_caller = on_caller && steps <= 2 * h->num_sms;
+    if (on_caller && (s = fc_flush_pending(h, st)) != FC_OK) return s;
   }
   // a call that carves the workspace differently: nothing of the previous call may be in flight on the other streams
   const FcCarve carve = {wsb, L.buf_bytes, L.tot_bytes, L.hi_bytes, L.off_tot};
@@ -1573,7 +1627,7 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
   if (any_fast) h->last_carve = carve;
   for (int l0 = 0; l0 < num_layers; l0 += FC_LAYER_CHUNK) {
     const int nl = num_layers - l0 < FC_LAYER_CHUNK ? num_layers - l0 : FC_LAYER_CHUNK;
-    if (any_small && any_passes && fork) {          // the internal streams need not wait for the short sequences
+    if (any_small && any_passes && fork && !on_caller) {          // the internal streams need not wait for the short sequences
       if ((s = fork_streams(h, st)) != FC_OK) return s;
       fork = false;
     }
@@ -1601,7 +1655,7 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
         continue;
       }
       if (plans[b].small) continue;
-      if (fork) {
+      if (fork && !on_caller) {
         if ((s = fork_streams(h, st)) != FC_OK) return s;
         fork = false;
       }
@@ -1611,7 +1665,7 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
         lp.v[l] = static_cast<const T *>(layers[l0 + l].v) + (long long)start * kv->stride_token;
         lp.scores[l] = const_cast<float *>(layers[l0 + l].scores) + start;
       }
-      s = band[b] ? score_band(h, kv, band[b], nl, lp, en, 4ll * B, L, wsb, band_tabs[b])
+      s = band[b] ? score_band(h, st, on_caller, kv, band[b], nl, lp, en, 4ll * B, L, wsb, band_tabs[b])
                   : score_sequence<T>(h, st, kv, plans[b], nl, lp, gamma, en, 4ll * B, L, wsb, tabs[b]);
       if (s != FC_OK) return s;
     }
