@@ -33,10 +33,9 @@ DEFAULT_CONFIG = "cfg3"          # the 32k-token workload the target fraction is
 
 # DRAM bytes read + written per launch of the dominant kernel as an ncu capture counted them (a constant from
 # that capture, not a measurement of this run; None where no capture of the kernel and workload exists):
-# pass 2 of cfg3, 0.46 MB read + 1.94 MB written on average over 24 launches with the intermediate in the
-# persisting part of L2 (ncu --cache-control none, one pass per launch; profiles/transform_passes_ncu.md).
+# the transform of the grid values, 16 heads of 32768 tokens per launch (profiles/kept_band_ncu.md).
 NCU_TRAFFIC_BYTES = {
-    ("cfg3", "pass2"): 2.40e6,
+    ("cfg3", "pass2"): 2.61e8,
 }
 
 
@@ -115,11 +114,13 @@ def physical_gpu_index(local_rank: int) -> int:
 def step_accounting(binding, handle, cfg):
     """Algorithmic flops and HBM bytes of one step, per kernel class: what the path cannot do without (one transform of
     N points each way per complex column, whatever N is), not what the hardware or the padding of lengths that are not a
-    power of two happened to add."""
+    power of two happened to add.  16-bit sequences are scored on a grid of M points between two banded matrix products
+    (pass1 and pass3: bound by the rows they read): their pass2 is the transform of M points each way.  The step's own flops
+    stay the N-point count, so that its fraction compares across forms."""
     d, H, L = cfg.head_dim, cfg.num_heads, cfg.num_layers
     s = 4 if cfg.dtype == "f32" else 2
     acc = {k: dict(flops=0.0, bytes=0.0) for k in ("pass1", "pass2", "pass3", "select", "gather")}
-    rows = 0
+    rows, step_flops = 0, 0.0
     for N in cfg.seqlens:
         if N == 0:
             continue
@@ -127,15 +128,23 @@ def step_accounting(binding, handle, cfg):
         n1 = plan["n1"] if not plan["bluestein"] else math.sqrt(N)      # share of the outer passes
         n2 = N / n1
         cols = H * d * L                       # complex columns (K + jV) of this sequence
-        acc["pass1"]["flops"] += cols * N * 5.0 * math.log2(n1)
-        acc["pass2"]["flops"] += cols * N * (10.0 * math.log2(n2) + 8.0)
-        acc["pass3"]["flops"] += cols * N * 5.0 * math.log2(n1) + cols * N * 4.0
+        step_flops += cols * N * (10.0 * math.log2(N) + 12.0)
+        M, omega = 128, int(cfg.gamma * N)
+        while 4 * M < N or 5 * omega > 4 * M:
+            M *= 2
+        if s == 2 and N > 512 and N != 1024 and 2 * M <= N and M <= 16384:
+            acc["pass2"]["flops"] += cols * M * (10.0 * math.log2(M / 2) + 24.0)
+            acc["pass3"]["bytes"] += N * H * L * 2.0 * d * s           # K and V rows again
+        else:
+            acc["pass1"]["flops"] += cols * N * 5.0 * math.log2(n1)
+            acc["pass2"]["flops"] += cols * N * (10.0 * math.log2(n2) + 8.0)
+            acc["pass3"]["flops"] += cols * N * 5.0 * math.log2(n1) + cols * N * 4.0
         acc["pass1"]["bytes"] += N * H * L * 2.0 * d * s               # K and V rows, read once
         acc["pass3"]["bytes"] += N * H * L * 4.0                       # score write
         acc["select"]["bytes"] += N * H * L * 4.0                      # score read
         acc["gather"]["bytes"] += cfg.rho * N * H * L * (4.0 * d * s + 4.0)
         rows += N * H * L
-    return acc, rows
+    return acc, rows, step_flops
 
 
 # --------------------------------------------------------------------------- CPU baseline (oracle)
@@ -410,10 +419,9 @@ def quick_config(torch, binding, S, name, dev, peaks, alu_peak, warmup=3, steps=
     torch.cuda.synchronize(dev)
     ms = e0.elapsed_time(e1) / steps
     comp.check_device_status()
-    acc, rows = step_accounting(binding, comp.handle, cfg)
+    acc, rows, step_flops = step_accounting(binding, comp.handle, cfg)
     s = 4 if cfg.dtype == "f32" else 2
     step_bytes = rows * (2.0 * cfg.head_dim * s + 8.0 + cfg.rho * (4.0 * cfg.head_dim * s + 4.0))
-    step_flops = sum(v["flops"] for v in acc.values())
     t_bound = max(step_bytes / (peaks["hbm_gbs"] * 1e9), step_flops / (alu_peak * 1e12))
     input_gb = sum(k.numel() * k.element_size() * 2 for k in Kd) / 1e9
     comp.close()
@@ -554,7 +562,7 @@ def main():
     value = replicas.whole_job_rate(tokens, world, ms_per_step)
 
     # roofline of the dominant kernel and of the whole step
-    acc, rows = step_accounting(binding, comp.handle, cfg)
+    acc, rows, step_flops = step_accounting(binding, comp.handle, cfg)
     props = torch.cuda.get_device_properties(dev)
     # ALU peak: nominal (SMs x 128 lanes x 2 x max clock) and what a pure FMA loop sustains in this run; the
     # fractions below divide by the nominal figure (the larger of the two), the measured one is reported beside it
@@ -588,7 +596,6 @@ def main():
                 overlap_factor=sum(v["ms"] for v in shares.values()) / ms_per_step)
     s = 4 if cfg.dtype == "f32" else 2
     step_bytes = rows * (2.0 * cfg.head_dim * s + 8.0 + cfg.rho * (4.0 * cfg.head_dim * s + 4.0))
-    step_flops = sum(v["flops"] for v in acc.values())
     t_bound = max(step_bytes / (peaks["hbm_gbs"] * 1e9), step_flops / (alu_peak * 1e12))
     roof_step = dict(bound="alu" if step_flops / (alu_peak * 1e12) >= step_bytes / (peaks["hbm_gbs"] * 1e9) else "hbm",
                      t_bound_ms=1000.0 * t_bound, frac=t_bound / (ms_per_step / 1000.0),

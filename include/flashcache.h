@@ -18,7 +18,8 @@
  *   - Streams.  `stream` is a cudaStream_t passed as void*.  Results are ordered
  *     on it: work enqueued on `stream` after a call sees that call's outputs.
  *     Short sequences (powers of two up to 1024 tokens, others up to 512, where head_dim
- *     allows it) are scored by one kernel on `stream`, longer ones of up to 65536 tokens on
+ *     allows it) are scored by one kernel on `stream`, and so are longer 16-bit ones, by a few
+ *     kernels, where a call has little work; else ones of up to 65536 tokens run on
  *     the handle's internal streams (two by default), which wait for everything enqueued on
  *     `stream` before the call and which `stream` waits for before the call returns, through
  *     events; no host synchronisation is involved (see fc_set_score_overlap for the
@@ -28,8 +29,9 @@
  *     (they synchronise `stream`), fc_profile_end (waits for its events),
  *     fc_compress_host (once, to learn the row counts), the first
  *     fc_score_layer_static call on a device.  Every other call only enqueues.
- *   - Context-wide state.  While a handle scores power-of-two sequences it
- *     raises the context's persisting-L2 limit (cudaLimitPersistingL2CacheSize)
+ *   - Context-wide state.  While a handle scores long power-of-two
+ *     sequences of fp32 (or of 16 bits, with a wide cutoff) it raises the
+ *     context's persisting-L2 limit (cudaLimitPersistingL2CacheSize)
  *     to the device maximum and marks its transform workspace as a persisting
  *     access window on its internal streams; the handles of a device share the
  *     claim and the last one to let go restores the value found.  No persisting

@@ -204,11 +204,14 @@ extern "C" fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen) 
     h->tab_next = 0;
     for (int i = 0; i < FC_BAND_SLOTS; ++i) h->band_key[i] = 0;
     h->band_next = 0;
-    if (cudaMalloc(&h->band_cache, FC_BAND_SLOTS * FC_BAND_SLOT_BYTES) != cudaSuccess ||
-        cudaMalloc(&h->tab_cache, (size_t)FC_TAB_SLOTS * h->tab_slot_len * sizeof(float4)) != cudaSuccess) {
+    // kept-band tables: 2 or 4 tokens per grid point at any length, other ratios up to about 1000 or 1700 tokens
+    h->band_slot_bytes = max_seqlen <= 512 ? 0 : (size_t)(max_seqlen <= 1024 ? 640 : 1280) << 10;
+    const size_t tab_bytes = (size_t)FC_TAB_SLOTS * h->tab_slot_len * sizeof(float4);
+    if (cudaMalloc(&h->tab_cache, tab_bytes + FC_BAND_SLOTS * h->band_slot_bytes) != cudaSuccess) {
       fc_destroy(h);
       return FC_ERR_CUDA;
     }
+    h->band_cache = reinterpret_cast<char *>(h->tab_cache) + tab_bytes;
   }
   k_fill_master<<<(h->master_len + 255) / 256, 256>>>(h->master, h->master_len);
   if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
@@ -289,7 +292,6 @@ extern "C" void fc_destroy(fc_handle *h) {
   if (h->ev_inputs_free) cudaEventDestroy(h->ev_inputs_free);
   if (h->ev_outputs_done) cudaEventDestroy(h->ev_outputs_done);
   if (h->tab_cache) cudaFree(h->tab_cache);
-  if (h->band_cache) cudaFree(h->band_cache);
   if (h->master) cudaFree(h->master);
   if (h->status_word) cudaFree(h->status_word);
   if (h->done_counter) cudaFree(h->done_counter);

@@ -6,6 +6,7 @@
 #include <mutex>
 #include <new>
 #include <type_traits>
+#include <utility>
 
 namespace {
 
@@ -54,11 +55,16 @@ const double (*responses())[band::kCheb] {
 
 constexpr int kMinGrid = 128, kMaxGrid = 16384;
 
+// 16-bit rows are exact operands of the products (fp32 rows would need six of them and terms of their own).  Up to 512 tokens
+// and at 1024 one kernel does it all, and a single layer of 4 heads takes 29..33 us against 44 here (28 layers: 145 and 182
+// against 72 and 95, but a score must not depend on how many layers share a call); from 513 tokens on the three passes take
+// 41 us for one layer and 174 us for 28, this form 44 and 88.
 bool eligible(const fc_kv_view *kv, int N) {
   return kv->dtype != FC_F32 && N > 512 && N != 1024 && N <= 65536 && kv->head_dim <= 512;
 }
 
-// The coarsest grid on which the band fits: N/4 <= M <= N/2 and omega <= 0.8 M.
+// The coarsest grid on which the band fits: N/4 <= M <= N/2 and omega <= 0.8 M (a quarter more grid than the band needs: the
+// kernel's support grows without bound as that margin closes).  Where M would pass N/2 little is saved and the passes stay.
 bool make_geometry(int N, int omega, Geometry *g) {
   int M = kMinGrid;
   while (4ll * M < N || 5ll * omega > 4ll * M) M <<= 1;
@@ -212,9 +218,9 @@ void fc_band_release(FcBandJob *j) { delete j; }
 // values before the transform, two planes after it, a scale per row
 static size_t unit_bytes(const FcBandJob *j) { return j->y_bytes + 2 * j->plane_bytes + align256((size_t)2 * j->d * 4); }
 
-// Fuller launches beat intermediates that stay in L2 (28 layers of 4 heads of 32768 tokens: 2290 / 2056 / 1977 / 1902 us with
-// 48 / 96 / 192 / 384 MB; 192 MB is where the gain no longer pays for the workspace).
-static size_t budget(const fc_handle *h) { return h->group_bytes > ((size_t)1 << 60) ? h->group_bytes : h->group_bytes * 6; }
+// Fuller launches beat intermediates that stay in L2: 28 layers of 4 heads of 32768 tokens take 2290 / 2056 / 1977 / 1902 us
+// with launch groups of up to 48 / 96 / 192 / 384 MB, of 8192 tokens 569 / 520 / 518 / 492.
+static size_t budget(const fc_handle *h) { return h->group_bytes > ((size_t)1 << 60) ? h->group_bytes : h->group_bytes * 12; }
 
 size_t fc_band_buffer_bytes(const fc_handle *h, const FcBandSizes *s, int units) {
   const size_t all = s->unit * units, most = budget(h);

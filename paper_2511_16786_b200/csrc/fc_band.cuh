@@ -19,7 +19,7 @@ namespace band {
 
 constexpr int kJ = 16;                       // grid points per step of k_down
 constexpr int kSlotTok = 32;                 // tokens per ring slot of k_down and per TMA box
-constexpr int kRing = 11;                    // ring slots of k_down
+constexpr int kRing = 11;                    // ring slots of k_down: a window is at most seven, the rest are on their way
 constexpr int kMaxSteps = 12;                // 16-token steps a window of k_down may have
 constexpr int kRows = 128;                   // rows (channels of K, then of V) per tile; tokens per step of k_up
 constexpr int kBoxBytes = kSlotTok * 128;    // one box: 32 tokens x 64 channels of 2 bytes
@@ -268,6 +268,13 @@ constexpr unsigned kDownCols = 512;
 constexpr unsigned kDownTable = kMaxSteps * 2 * 48 * 16;
 constexpr size_t kDownSmem = 1024 + (size_t)kRing * 4 * kBoxBytes + 2 * (size_t)kDownTable;
 
+// What bounds it: HBM and the products alike.  A step is 64 tokens of K and V at 4 tokens per grid point, ten products of
+// 128 x 48 x 16 per tile (44 cycles each: the left operand's 4 KB at 128 bytes a cycle, a quarter cycle per column), 900
+// cycles beside 32 KB of rows.  The rows are the left operand, so that a lane of the sums is a channel and writes whole
+// sectors of its row of the grid; the three (two) terms of the matrix are columns of one product, and sums of a window go
+// to two accumulators, from the window's ends to its middle, because the tensor cores truncate when they add: the rms error
+// of a score falls from 5.9e-7 to 3.3e-7.  16 heads of 32768 tokens: 233 us with products issued by one lane, 76 us now
+// (417 MB, 5.5 TB/s).
 // One block: `per` steps of 16 grid points for up to two tiles (256 rows) of one unit.  grid (ranges, tile pairs, units).
 template <typename T, int TERMS>
 __global__ void __launch_bounds__(kDownThreads, 1) k_down(const __grid_constant__ Maps maps, const __grid_constant__ Geometry g,
@@ -620,6 +627,11 @@ struct MidParams {
   MidTables t;
 };
 
+// What bounds it: shared memory (57 % of its wavefronts), the FMA pipe (half) and issue slots (42 %) at 16 warps per SM, none
+// of them alone.  A row is transformed as half as many complex points, two rows per thread in packed arithmetic, which
+// shares the twiddles, the gains and every address: 48 M instructions for 16 heads of 32768 tokens where one row per thread
+// took 83 M; 110 us (134 us with the values stored in 16-byte pieces; one row per thread at 64 registers and 32 warps comes
+// out alike, 103 us).
 template <class S>
 __global__ void __launch_bounds__(S::NT, S::NT <= 512 ? 512 / S::NT : 1) k_mid(const MidParams P) {
   constexpr int Mh = S::Mh, T = S::T, RL = S::RL;
@@ -825,6 +837,11 @@ template <> __device__ __forceinline__ float2 widen<__nv_bfloat16>(unsigned v) {
   return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
 }
 
+// What bounds it: HBM, or L2 where a launch group fits it.  A step of 128 tokens and 128 channels is 64 KB of operands and
+// twelve products of 128 x 128 x 16 (64 cycles each); tokens are the lanes of the sums, so that a row's squares stay in one
+// thread, and the grid values are the right operand as the transform left them (64- and 32-byte swizzled boxes).  Rows, and
+// grid values with the matrices, have a loading warp each: with one for both, grid values waited for the rows before them
+// (107 us for 16 heads of 32768 tokens, 85..90 us now, 420 MB).
 // One block: `per` steps of 128 tokens of one unit.  grid (ranges, units).
 template <typename T, int NQ>
 __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Maps maps, const __grid_constant__ GridMaps grid,

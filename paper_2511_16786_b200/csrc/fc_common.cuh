@@ -15,8 +15,7 @@
 #define FC_MAX_STAGES 4
 #define FC_MAX_AUX 4     // internal streams a handle may use
 #define FC_TAB_SLOTS 8   // filter tables a handle keeps (one per sequence length, cutoff and form)
-#define FC_BAND_SLOTS 8
-#define FC_BAND_SLOT_BYTES ((size_t)1280 << 10)  // whole ratios of tokens to grid points, others up to about 1700 tokens
+#define FC_BAND_SLOTS 4  // and tables of sequences scored in the kept band
 #define FC_LAYER_CHUNK 32  // layers one launch of the scoring kernels can span (kernel-argument table)
 
 // Bits of the device status word.
@@ -79,8 +78,9 @@ struct fc_handle {
   float4 *tab_cache;
   int tab_slot_len, tab_next;
   long long tab_key[FC_TAB_SLOTS];
-  // the same for sequences scored in the kept band whose tables fit a slot (FC_BAND_SLOTS x FC_BAND_SLOT_BYTES)
+  // the same for sequences scored in the kept band whose tables fit a slot (in the allocation of tab_cache)
   char *band_cache;
+  size_t band_slot_bytes;
   int band_next;
   long long band_key[FC_BAND_SLOTS];
   // fc_compress_host (created on its first call): the stream the host-to-device copies run on, one

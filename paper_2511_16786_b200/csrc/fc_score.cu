@@ -20,6 +20,8 @@
 //   pass 2  for every k1 (with N1-k1, which holds the partner bins N-q):
 //           twiddle, DFT over n2, the filter above, inverse DFT over k2, twiddle -> B[k1][n2]
 //   pass 3  for every n2: inverse DFT over k1, |.|^2 summed over the channels -> scores
+// 16-bit sequences from 513 tokens on whose cutoff keeps at most about two fifths of the bins do not take these passes:
+// they are scored on a coarser grid between two banded matrix products (fc_band.cuh).
 // Every other length up to 65536 takes the same three passes on a longer transform with the residual written as one
 // padded convolution (fc_score_fast.cuh); the spectrum diagnostics run on the same passes.  The generic kernels of this
 // file serve the power of two 131072, spectra of short powers of two and the entry point without allocation; there,
@@ -1332,7 +1334,7 @@ fc_status band_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const
       cached = cap == cudaStreamCaptureStatusNone;
     }
     for (int i = 0; cached && i < FC_BAND_SLOTS; ++i)
-      if (h->band_key[i] == fc_band_table_key(band[b])) { tabs[b] = h->band_cache + i * FC_BAND_SLOT_BYTES; used[i] = true; }
+      if (h->band_key[i] == fc_band_table_key(band[b])) { tabs[b] = h->band_cache + i * h->band_slot_bytes; used[i] = true; }
   }
   for (int b = 0; b < kv->batch; ++b) {
     if (!band[b] || tabs[b]) continue;
@@ -1344,7 +1346,7 @@ fc_status band_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const
     if (!flushed && (s = fc_flush_pending(h, st)) != FC_OK) return s;
     flushed = true;
     int slot = -1;
-    for (int i = 0; cached && fc_band_table_bytes(band[b]) <= FC_BAND_SLOT_BYTES && i < FC_BAND_SLOTS && slot < 0; ++i) {
+    for (int i = 0; cached && fc_band_table_bytes(band[b]) <= h->band_slot_bytes && i < FC_BAND_SLOTS && slot < 0; ++i) {
       const int c = (h->band_next + i) % FC_BAND_SLOTS;
       if (!used[c]) slot = c;
     }
@@ -1353,7 +1355,7 @@ fc_status band_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const
       h->band_next = (slot + 1) % FC_BAND_SLOTS;
       h->band_key[slot] = 0;                                   // not valid until its launch is in the stream
       used[slot] = true;
-      dst = h->band_cache + slot * FC_BAND_SLOT_BYTES;
+      dst = h->band_cache + slot * h->band_slot_bytes;
     } else {
       FcBandSizes bs;
       fc_band_bounds(kv, kv->cu_seqlens[b + 1] - kv->cu_seqlens[b], &bs);

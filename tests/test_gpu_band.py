@@ -75,7 +75,7 @@ def _check(k, v, cu, gamma, scores, energy):
 # the smallest and largest sequences, every transform length, whole and broken ratios of tokens to grid points, lengths
 # around the 128-token and 16-point steps, cutoffs from none to beyond what the form takes, head widths of one to four tiles
 @pytest.mark.parametrize("N,H,d,gamma,dtype", [
-    (1024, 3, 128, 0.2, torch.bfloat16), (1025, 2, 64, 0.2, torch.float16), (1151, 1, 192, 0.15, torch.bfloat16),
+    (513, 3, 128, 0.2, torch.bfloat16), (767, 1, 64, 0.1, torch.float16), (1023, 2, 128, 0.3, torch.bfloat16), (1025, 2, 64, 0.2, torch.float16), (1151, 1, 192, 0.15, torch.bfloat16),
     (1281, 2, 128, 0.0, torch.bfloat16), (2047, 2, 128, 0.2, torch.float16), (2048, 1, 256, 0.3, torch.bfloat16),
     (2500, 2, 128, 0.39, torch.bfloat16), (3072, 2, 64, 0.25, torch.float16), (4096, 2, 128, 0.2, torch.bfloat16),
     (4097, 2, 128, 0.2, torch.bfloat16), (5119, 3, 128, 0.1, torch.float16), (8192, 2, 64, 0.2, torch.bfloat16),
@@ -107,6 +107,39 @@ def test_band_ragged_batch_strided_views_and_neighbours(fc):
     assert torch.isnan(s2[1, cu[2]:cu[3]]).all()
     s2[1, cu[2]:cu[3]] = s[1, cu[2]:cu[3]]
     assert torch.equal(s, s2)
+
+
+def test_band_heads_before_tokens(fc):
+    # [H, T, d] storage seen as [T, H, d]: the head stride is the larger one
+    k, v = _kv(1500, 3, 128, torch.float16, 7)
+    kd, vd = (x.transpose(0, 1).contiguous().cuda().transpose(0, 1) for x in (k, v))
+    s, e = _score(fc, kd, vd, [0, 1500], 0.2)
+    _check(k, v, [0, 1500], 0.2, s, e)
+
+
+def test_band_calls_agree_however_the_work_is_grouped(fc):
+    # many layers in one call (internal streams, several launch groups), one call per layer (the caller's stream), small
+    # launch groups, and a replayed capture, whose tables are built anew: the same bits
+    L, lens, H, d = 9, [2311, 1100], 2, 128
+    cu = [0] + [int(x) for x in np.cumsum(lens)]
+    K, V = zip(*(_kv(cu[-1], H, d, torch.bfloat16, 20 + l) for l in range(L)))
+    K, V = [k.cuda() for k in K], [v.cuda() for v in V]
+    ref_s, ref_e = zip(*(_score(fc, K[l], V[l], cu, 0.2) for l in range(L)))
+    for group_bytes in (None, 1 << 16):
+        comp = fc.Compressor(L, H, d, cu, torch.bfloat16, 0.2, 0.2, group_bytes=group_bytes)
+        comp.compress(K, V)
+        comp.check_device_status()
+        got = [comp.scores.clone(), comp.energy.clone()]
+        graph = comp.capture(K, V)
+        comp.scores.zero_()
+        comp.energy.zero_()
+        graph.replay()
+        comp.check_device_status()
+        for s, e in (got, [comp.scores, comp.energy]):
+            for l in range(L):
+                assert torch.equal(s[l].cpu(), ref_s[l]) and torch.equal(e[l].cpu(), ref_e[l])
+        del graph
+        comp.close()
 
 
 def test_band_scales(fc):
