@@ -53,7 +53,7 @@ const double (*responses())[band::kCheb] {
   return cheb;
 }
 
-constexpr int kMinGrid = 128, kMaxGrid = 16384;
+constexpr int kMinGrid = 256, kMaxGrid = 16384;
 
 // 16-bit rows are exact operands of the products (fp32 rows would need six of them and terms of their own).  Up to 512 tokens
 // and at 1024 one kernel does it all, and a single layer of 4 heads takes 29..33 us against 44 here (28 layers: 145 and 182
@@ -128,7 +128,7 @@ bool make_geometry(int N, int omega, Geometry *g) {
 
 // Mh and the radices of its stages
 #define FC_MID_SHAPES(X)                                                                                          \
-  X(64, 8, 8, 1, 1) X(128, 16, 8, 1, 1) X(256, 16, 16, 1, 1) X(512, 8, 8, 8, 1) X(1024, 16, 8, 8, 1) X(2048, 16, 16, 8, 1)          \
+  X(128, 16, 8, 1, 1) X(256, 16, 16, 1, 1) X(512, 8, 8, 8, 1) X(1024, 16, 8, 8, 1) X(2048, 16, 16, 8, 1)          \
   X(4096, 16, 16, 16, 1) X(8192, 16, 8, 8, 8)
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
