@@ -1591,6 +1591,8 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0) continue;
     if (!h->generic_only) plans[b] = plan_passes(N, kv->head_dim);
+    // what fc_set_score_overlap promises goes by the length, not by the form that scores it
+    if (!plans[b].ok || (plans[b].pad && !plans[b].small)) direct_only = false;
     band[b] = fc_band_plan(h, kv, N, cutoff_index(gamma, N));
     if (band[b]) {
       any_band = true;
@@ -1600,7 +1602,6 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
     any_fast = any_fast || plans[b].ok;
     any_small = any_small || plans[b].small;
     any_passes = any_passes || (plans[b].ok && !plans[b].small);
-    if (!plans[b].ok || (plans[b].pad && !plans[b].small)) direct_only = false;
   }
   if (any_fast && (s = prepare_tables(h, st, kv, gamma, false, reinterpret_cast<float4 *>(wsb + L.off_tab),
                                       reinterpret_cast<float2 *>(wsb + L.off_buf), tabs.data(), band.data())) != FC_OK) return s;

@@ -150,3 +150,34 @@ def test_band_scales(fc):
     k[:, 0, 5] = 0.0
     s, e = _score(fc, k.cuda(), v.cuda(), [0, 2048], 0.2)
     _check(k, v, [0, 2048], 0.2, s, e)
+
+
+@pytest.mark.parametrize("lens", [[1500], [2048, 1100, 300]])
+def test_band_deferred_calls_of_broken_lengths_are_complete_in_stream_order(fc, lens):
+    # fc_set_score_overlap defers the join only where every sequence is short or a power of two long: whatever the caller's
+    # stream reads after such a call is final, with enough layers that the call uses the internal streams
+    L, H, d = 28, 4, 128
+    cu = [0] + [int(x) for x in np.cumsum(lens)]
+    K, V = zip(*(_kv(cu[-1], H, d, torch.bfloat16, 40 + l) for l in range(L)))
+    K, V = [k.cuda() for k in K], [v.cuda() for v in V]
+    h = fc.fc_create(0, max(lens))
+    try:
+        ws = torch.empty(fc.fc_score_layers_workspace_bytes(h, K[0], V[0], cu, L), dtype=torch.uint8, device="cuda")
+        s = torch.empty((L, H, cu[-1]), dtype=torch.float32, device="cuda")
+        e = torch.empty((L, len(lens), 4), dtype=torch.float64, device="cuda")
+        fc.fc_score_layers(h, K, V, cu, 0.2, s, e, ws)
+        ref = s.clone(), e.clone()
+        assert fc.fc_last_device_status(h) == 0
+        fc.fc_set_score_overlap(h, True)
+        busy = torch.randn((4096, 4096), device="cuda")
+        for _ in range(5):
+            busy = torch.tanh(busy @ busy)                # the call is enqueued whole while the stream works on this
+            s.fill_(-1.0)
+            e.fill_(-1.0)
+            fc.fc_score_layers(h, K, V, cu, 0.2, s, e, ws)
+            got = s.clone(), e.clone()                    # by the caller's stream, without a joining call
+            s.fill_(-2.0)
+            assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1])
+        assert fc.fc_last_device_status(h) == 0
+    finally:
+        fc.fc_destroy(h)
