@@ -122,7 +122,7 @@ bool make_geometry(int N, int omega, Geometry *g) {
     for (int b = 0; b < g->up_steps(); ++b, ul.step(), uh.step()) up(ul.q, uh.q);
   }
   g->ks = ks;
-  g->nq = (need + 7) / 8 * 8;
+  g->nq = need <= 16 ? 16 : (need + 7) / 8 * 8;            // 16 or 24: a step of 128 tokens spans at least 44 grid points
   return g->ks <= band::kMaxSteps && g->nq <= band::kMaxQuads && g->nq <= g->M / 4;
 }
 
@@ -403,9 +403,8 @@ static fc_status run_group(fc_handle *h, cudaStream_t st, const FcBandJob *j, co
     P.per = (g.up_steps() + ranges - 1) / ranges;
     band::GridMaps grid;
     if ((s = encode_grid(&grid, hi, nu * 2 * j->d, g.M, cap * j->plane_bytes)) != FC_OK) return s;
-    return g.nq == 8    ? launch_up<T, 8>(h, st, early, j->maps, grid, g, P, nu)
-           : g.nq == 16 ? launch_up<T, 16>(h, st, early, j->maps, grid, g, P, nu)
-                        : launch_up<T, 24>(h, st, early, j->maps, grid, g, P, nu);
+    return g.nq == 16 ? launch_up<T, 16>(h, st, early, j->maps, grid, g, P, nu)
+                      : launch_up<T, 24>(h, st, early, j->maps, grid, g, P, nu);
   }
 }
 

@@ -810,7 +810,7 @@ struct UpParams {
 };
 constexpr int kUpBufs = 4;                   // sums of 128 x 128 in tensor memory
 constexpr int kYStages = 2;
-constexpr int x_stages(int nq) { return nq <= 16 ? 3 : 2; }      // as many as fit
+constexpr int x_stages(int nq) { return nq == 16 ? 3 : 2; }      // as many as fit
 constexpr int kMaxX = 3;
 constexpr int kUpThreads = 64 + 256 + 32;    // grid values and matrices, products, eight warps (four per 64 channels), rows
 struct UpShared {
@@ -897,10 +897,10 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Ma
         mbar::expect_tx(&sh.yfull[s], ybytes);
         const int r0 = ((int)blockIdx.y * tiles + t) * kRows;
         unsigned char *dst = ys + (size_t)s * ybytes;
-        for (int rn = 0; rn < 2; ++rn, dst += 2 * run) {       // a run: 32 values' box where there are as many, then 16
+        for (int rn = 0; rn < 2; ++rn, dst += 2 * run) {       // a run: a box of 32 values and, with 24 quads, one of 16
           const int x = rn == 0 ? 2 * q0 : g.M - 2 * (q0 + NQ);
-          if (NQ >= 16) load_box(dst, &grid.wide, x, r0, 0, &sh.yfull[s]);
-          if (NQ % 16) load_box(dst + (NQ >= 16 ? 2 * kRows * 64 : 0), &grid.narrow, x + (NQ >= 16 ? 32 : 0), r0, 0, &sh.yfull[s]);
+          load_box(dst, &grid.wide, x, r0, 0, &sh.yfull[s]);
+          if (NQ > 16) load_box(dst + 2 * kRows * 64, &grid.narrow, x + 32, r0, 0, &sh.yfull[s]);
         }
         ++ny;
       }
@@ -951,9 +951,9 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Ma
         for (int pr = 0; pr < 3; ++pr)
 #pragma unroll
           for (int k = 0; k < NQ / 4; ++k) {
-            const int in = k % (NQ / 8), part = NQ >= 16 && in >= 2;       // step within its run, and its box
-            const bool w = NQ >= 16 && !part;
-            const unsigned off = (k / (NQ / 8)) * (2 * run) + (w ? in * 32u : part ? 2u * kRows * 64u : 0u) +
+            const int in = k % (NQ / 8);                                   // step within its run
+            const bool w = in < 2;                                         // and its box
+            const unsigned off = (k / (NQ / 8)) * (2 * run) + (w ? in * 32u : 2u * kRows * 64u) +
                                  (pr == 1 ? kRows * (w ? 64u : 32u) : 0u);
             mma(lead, d, tb + (pr == 0 ? 2 * run / 16 : 0u) + k * 256u, hi, ya + off / 16, w ? wide : narrow, idesc,
                 pr + k > 0 ? 1u : 0u);
