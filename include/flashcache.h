@@ -211,7 +211,8 @@ size_t fc_select_workspace_bytes(const fc_handle *h, const fc_kv_view *kv);
  * omega = min(N-1, floor(gamma*N)), bins 0..omega kept (Eq. 8), transformed back
  * (Eq. 9), and every token is scored by
  *     Dev[x] = mean_c (K[x,c]-K_base[x,c])^2 + mean_c (V[x,c]-V_base[x,c])^2   (Eq. 10).
- * Arithmetic is fp32 on the stored values.
+ * Arithmetic is fp32 on the stored values.  For most 16-bit sequences of more than 512 tokens part of it is matrix products
+ * of 16-bit terms (two or three to a value) with fp32 sums, arranged so that a score is as exact as fp32 passes make it.
  * Values that are not finite: the transform of a channel mixes all tokens of its sequence, so one NaN
  * or Inf element of K or V makes every score of that (sequence, head) NaN and that sequence's energy
  * sums NaN, exactly as the definition does; other heads' scores and other sequences are unaffected.

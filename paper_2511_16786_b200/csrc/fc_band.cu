@@ -184,7 +184,7 @@ bool fc_band_bounds(const fc_kv_view *kv, int N, FcBandSizes *s) {
   // M <= N/2, windows at their largest, every step with matrices of its own
   const int M = N / 2 < kMaxGrid ? N / 2 : kMaxGrid;
   s->tables = align256((size_t)(M / band::kJ) * band::kMaxSteps * 2 * 48 * 16) +
-              align256((size_t)((N + band::kRows - 1) / band::kRows) * band::kMaxQuads * 2048) + align256((size_t)M * 32) +
+              align256((size_t)((N + band::kRows - 1) / band::kRows) * band::kMaxQuads * band::kTerms * 1024) + align256((size_t)M * 32) +
               align256((size_t)M * 6 * sizeof(float2));
   s->unit = (size_t)2 * kv->head_dim * M * 8 + align256((size_t)2 * kv->head_dim * 4) + 1024;
   s->steps = (N + band::kRows - 1) / band::kRows;
@@ -205,8 +205,7 @@ FcBandJob *fc_band_plan(const fc_handle *h, const fc_kv_view *kv, int N, int ome
   j->f16 = kv->dtype == FC_F16;
   j->H = kv->num_heads;
   j->d = kv->head_dim;
-  const int nr = band::filter_terms(j->f16) * band::kJ;
-  j->off_up = align256(band::down_classes(g) * band::down_image(g, nr));
+  j->off_up = align256(band::down_classes(g) * band::down_image(g));
   j->off_mid = j->off_up + align256(band::up_classes(g) * band::up_image(g));
   j->table_bytes = j->off_mid + align256((size_t)g.M / 2 * 16) + align256((size_t)mid_tw_len(g.M / 2) * sizeof(float2));
   j->y_bytes = (size_t)2 * j->d * g.M * sizeof(float);
@@ -276,10 +275,10 @@ fc_status fc_band_tables(fc_handle *h, cudaStream_t st, const FcBandJob *j, char
   const int tw = mid_tw_len(Mh), mid = ((tw > Mh / 2 ? tw : Mh / 2) + 255) / 256;
   __half *um = reinterpret_cast<__half *>(tables + j->off_up);
   if (j->f16)
-    band::k_band_tables<__half, 2><<<down + up + mid, 256, 0, st>>>(g, r, reinterpret_cast<__half *>(tables), um,
+    band::k_band_tables<__half><<<down + up + mid, 256, 0, st>>>(g, r, reinterpret_cast<__half *>(tables), um,
                                                                   mid_tables(j, tables), down, up);
   else
-    band::k_band_tables<__nv_bfloat16, 3><<<down + up + mid, 256, 0, st>>>(g, r, reinterpret_cast<__nv_bfloat16 *>(tables), um,
+    band::k_band_tables<__nv_bfloat16><<<down + up + mid, 256, 0, st>>>(g, r, reinterpret_cast<__nv_bfloat16 *>(tables), um,
                                                                          mid_tables(j, tables), down, up);
   return fc_after_launch(h);
 }
@@ -345,7 +344,7 @@ static fc_status encode_grid(band::GridMaps *m, const void *hi, int rows, int M,
   const cuuint64_t dims[3] = {(cuuint64_t)M, (cuuint64_t)rows, 2}, str[2] = {(cuuint64_t)M * 2, (cuuint64_t)plane_bytes};
   const cuuint32_t ones[3] = {1, 1, 1};
   for (int w = 0; w < 2; ++w) {
-    const cuuint32_t box[3] = {w ? 32u : 16u, (cuuint32_t)band::kRows, 2};
+    const cuuint32_t box[3] = {w ? 32u : 16u, (cuuint32_t)band::kRows, 1};
     if (fn(w ? &m->wide : &m->narrow, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void *>(hi), dims, str, box, ones,
            CU_TENSOR_MAP_INTERLEAVE_NONE, w ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -358,7 +357,6 @@ template <typename T>
 static fc_status run_group(fc_handle *h, cudaStream_t st, const FcBandJob *j, const FcBandLaunch &l, int u0, int nu, int cap,
                            int ranges, bool early, char *buf) {
   const Geometry &g = j->g;
-  constexpr int TERMS = std::is_same<T, __half>::value ? 2 : 3;
   fc_status s;
   float *y = reinterpret_cast<float *>(buf);
   // the same places for every launch of a sequence, also where the last one has fewer units
@@ -369,10 +367,10 @@ static fc_status run_group(fc_handle *h, cudaStream_t st, const FcBandJob *j, co
     band::DownParams P = {l.tables, y, h->status_word, j->H, j->d, u0, 0};
     const int r = spread(h, n, nu * pairs);
     P.per = (n + r - 1) / r;
-    if ((s = allow_smem<band::k_down<T, TERMS>>(h->device, band::kDownSmem, cudaSharedmemCarveoutMaxShared)) != FC_OK) return s;
+    if ((s = allow_smem<band::k_down<T>>(h->device, band::kDownSmem, cudaSharedmemCarveoutMaxShared)) != FC_OK) return s;
     ProfScope ps(h, FC_K_PASS1, st);
     // never early: the caller may have put a wait for an event in front of it, and its rows may be on their way until then
-    s = launch(h, st, false, band::k_down<T, TERMS>, dim3(r, pairs, nu), band::kDownThreads, band::kDownSmem,
+    s = launch(h, st, false, band::k_down<T>, dim3(r, pairs, nu), band::kDownThreads, band::kDownSmem,
                j->maps, g, P);
     if (s != FC_OK) return s;
   }

@@ -7,10 +7,14 @@
 //   k_up     base_t = sum_j phi((t - x_j) M/N) b_j             the transposed band, then |z_t - base_t|^2 per row
 // phi need not be flat in the band (H is divided out exactly) nor short of the theory's length; it has to suppress what
 // folds onto the band, which it does to 6e-8 of the band's own gain, i.e. to fp32 rounding.  k_down and k_up are matrix
-// products on the 5th-generation tensor cores: 16-bit K and V are exact operands, phi is a sum of three bf16 or two
-// fp16 terms and b a sum of two fp16 terms scaled per channel (24 bits each), and sums are fp32.  N is arbitrary.
+// products on the 5th-generation tensor cores: 16-bit K and V are exact operands, phi is a sum of three bf16 or fp16 terms
+// (24 and 33 bits), b a sum of two fp16 terms scaled per channel (off by at most 2^-23 of the power of two below its largest
+// neighbour), every product of at least 2^-24 of the whole is formed, and sums are fp32 (what the tensor cores cut off them is
+// dealt with at each kernel).  N is arbitrary.
 #pragma once
 #include <cuda.h>
+
+#include <type_traits>
 
 #include "fc_common.cuh"
 #include "fc_mbar.cuh"
@@ -28,6 +32,7 @@ constexpr int kMaxPer = 256;                 // steps a block of k_down or k_up 
 constexpr int kCheb = 28;                    // terms of the expansion of H
 constexpr float kUpScale = 1024.f;           // k_up's matrix is stored times this (its low terms stay normal fp16)
 constexpr float kDownScaleF16 = 4096.f;      // k_down's fp16 matrix is stored times this
+constexpr float kCutOff = 5.9604644775390625e-8f;   // 2^-24 of a sum of k_down's products is put back (see there)
 
 // One sequence's rows in every layer of the launch, as [head][64 channels][token][channel]: a box is 32 tokens of a tile's
 // two 64-channel halves where both are of K or both of V (8 KB; a load costs about 80 cycles besides its bytes), else of one.
@@ -89,9 +94,9 @@ __host__ __device__ inline int up_quad_end(const Geometry &g, int b) {
   return (int)(j >> 2) + 1;
 }
 
-__host__ __device__ inline int filter_terms(bool f16) { return f16 ? 2 : 3; }
-__host__ __device__ inline size_t down_image(const Geometry &g, int nr) { return (size_t)g.ks * 2 * nr * 16; }
-__host__ __device__ inline size_t up_image(const Geometry &g) { return (size_t)g.nq * 2048; }
+constexpr int kTerms = 3;                    // 16-bit terms of a matrix entry
+__host__ __device__ inline size_t down_image(const Geometry &g) { return (size_t)g.ks * 2 * kTerms * kJ * 16; }
+__host__ __device__ inline size_t up_image(const Geometry &g) { return (size_t)g.nq * kTerms * 1024; }
 
 // ---------------------------------------------------------------------------------------------------- tables
 __device__ inline double phi(const Geometry &g, double u) {
@@ -112,28 +117,28 @@ __device__ inline double response(const Geometry &g, double f) {          // H(f
 }
 
 // One entry of k_down's matrix of a step: [8 tokens' chunk][term * 16 + j][8 tokens], rows of 16 bytes.
-template <typename T, int TERMS>
+template <typename T>
 __device__ __forceinline__ void down_entry(const Geometry &g, int cls, int i, T *__restrict__ out) {
   const int b = step_of(cls, g.down_steps(), down_classes(g));
   const int e = i & 7, j = (i >> 3) & (kJ - 1), c = i >> 7, t = down_start(g, b) + c * 8 + e;
-  T *img = out + (size_t)cls * (down_image(g, TERMS * kJ) / 2);
+  T *img = out + (size_t)cls * (down_image(g) / 2);
   const double inv = (double)g.M / g.N;
   double v = 0.0;
   if (t < g.N) {
     const double x = (b * kJ + j + 0.5) * ((double)g.N / g.M) - 0.5;
     v = (phi(g, (t - x) * inv) + phi(g, (-1.0 - t - x) * inv) + phi(g, (2.0 * g.N - 1.0 - t - x) * inv)) * inv;
-    if (TERMS == 2) v *= kDownScaleF16;
+    if (std::is_same<T, __half>::value) v *= kDownScaleF16;
   }
 #pragma unroll
-  for (int k = 0; k < TERMS; ++k) {
+  for (int k = 0; k < kTerms; ++k) {
     const T h = (T)(float)v;
-    img[((size_t)c * (TERMS * kJ) + k * kJ + j) * 8 + e] = h;
+    img[((size_t)c * (kTerms * kJ) + k * kJ + j) * 8 + e] = h;
     v -= (double)(float)h;
   }
 }
 
 // One entry of k_up's matrix of a step: [term][8 grid values][token][8].  Values are in the order the transform keeps
-// them: first (z0, z2) of ascending quads, then (z3, z1) of descending ones.
+// them: first (z0, z2) of ascending quads, then (z3, z1) of descending ones.  The first term is a whole number (see k_up).
 __device__ __forceinline__ void up_entry(const Geometry &g, int cls, int i, __half *__restrict__ out) {
   const int b = step_of(cls, g.up_steps(), up_classes(g));
   const int q0 = up_quad(g, b), nk = 4 * g.nq;
@@ -148,9 +153,14 @@ __device__ __forceinline__ void up_entry(const Geometry &g, int cls, int i, __ha
     const double x = (t + 0.5) * ((double)g.M / g.N) - 0.5;
     v = (phi(g, x - j) + phi(g, x + 1.0 + j) + phi(g, x - (2.0 * g.M - 1.0 - j))) * (double)kUpScale;
   }
-  const __half h = __float2half_rn((float)v);
-  img[((size_t)c * kRows + r) * 8 + e] = h;
-  img[((size_t)(nk / 8 + c) * kRows + r) * 8 + e] = __float2half_rn((float)(v - (double)__half2float(h)));
+  double part = rint(v);
+#pragma unroll
+  for (int k = 0; k < kTerms; ++k) {
+    const __half h = __float2half_rn((float)part);
+    img[((size_t)(k * (nk / 8) + c) * kRows + r) * 8 + e] = h;
+    v -= (double)__half2float(h);
+    part = v;
+  }
 }
 
 // Everything k_mid looks up.  Stage twiddles w_L^(j p), p = 1, 2, 3, 4, 8, 12, for the stages before the last, and for
@@ -271,15 +281,18 @@ constexpr size_t kDownSmem = 1024 + (size_t)kRing * 4 * kBoxBytes + 2 * (size_t)
 // What bounds it: HBM and the products alike.  A step is 64 tokens of K and V at 4 tokens per grid point, ten products of
 // 128 x 48 x 16 per tile (44 cycles each: the left operand's 4 KB at 128 bytes a cycle, a quarter cycle per column), 900
 // cycles beside 32 KB of rows.  The rows are the left operand, so that a lane of the sums is a channel and writes whole
-// sectors of its row of the grid; the three (two) terms of the matrix are columns of one product, and sums of a window go
-// to two accumulators, from the window's ends to its middle, because the tensor cores truncate when they add: the rms error
-// of a score falls from 5.9e-7 to 3.3e-7.  16 heads of 32768 tokens: 233 us with products issued by one lane, 76 us now
-// (417 MB, 5.5 TB/s).
+// sectors of its row of the grid; the three terms of the matrix are columns of one product, and sums of a window go to two
+// accumulators, from the window's ends to its middle, because the tensor cores cut off, towards zero, what does not fit the
+// 24 bits of a sum: half a unit of the last place at every addition of a product of depth 16.  That mean is put back, 2^-24
+// of the sum for its last, largest additions; a model of these sums has 0.50e-6 of a score (rms, 10 % outlier rows) with one
+// accumulator, 0.31e-6 with two, 0.11e-6 with what was cut off put back.  16 heads of 32768 tokens: 233 us with products
+// issued by one lane, 75 us now (417 MB, 5.6 TB/s).
 // One block: `per` steps of 16 grid points for up to two tiles (256 rows) of one unit.  grid (ranges, tile pairs, units).
-template <typename T, int TERMS>
+template <typename T>
 __global__ void __launch_bounds__(kDownThreads, 1) k_down(const __grid_constant__ Maps maps, const __grid_constant__ Geometry g,
                                                        const DownParams P) {
-  constexpr int NR = TERMS * kJ;             // columns of one sum
+  constexpr int NR = kTerms * kJ;            // columns of one sum
+  constexpr bool kF16 = std::is_same<T, __half>::value;
   extern __shared__ unsigned char raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(((uintptr_t)raw + 1023) & ~(uintptr_t)1023);
   unsigned char *tab = smem + (size_t)kRing * 4 * kBoxBytes;
@@ -289,7 +302,7 @@ __global__ void __launch_bounds__(kDownThreads, 1) k_down(const __grid_constant_
   const int tiles = P.d / 64, tile0 = 2 * blockIdx.y, nt = tiles - tile0 < 2 ? 1 : 2;
   const int n = g.down_steps(), classes = down_classes(g);
   const int b0 = blockIdx.x * P.per, b1 = b0 + P.per < n ? b0 + P.per : n;
-  const unsigned img = (unsigned)down_image(g, NR);
+  const unsigned img = (unsigned)down_image(g);
   unsigned char *tab1 = tab + kDownTable;
 
   if (tid == 0) {
@@ -351,7 +364,7 @@ __global__ void __launch_bounds__(kDownThreads, 1) k_down(const __grid_constant_
         if (!ok) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
       }
     } else if (warp <= 2) {
-      constexpr unsigned idesc = instruction(TERMS == 2, true, NR), ahi = operand_hi(1024, 2), bhi = operand_hi(128, 0);
+      constexpr unsigned idesc = instruction(kF16, true, NR), ahi = operand_hi(1024, 2), bhi = operand_hi(128, 0);
       constexpr int kGroups = 2 * kRing;                         // 16-token groups in the ring
       const unsigned lead = elect();
       const int tile = warp - 1;
@@ -390,7 +403,7 @@ __global__ void __launch_bounds__(kDownThreads, 1) k_down(const __grid_constant_
       if (!ok && lane == 0) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
     } else {
       const int quad = warp & 3, row = quad * 32 + lane, Mh = g.M / 2;
-      const float scale = TERMS == 2 ? 1.f / kDownScaleF16 : 1.f;
+      const float scale = kF16 ? 1.f / kDownScaleF16 : 1.f;
       for (int b = b0; b < b1; ++b) {
         const int it = b - b0, buf = it & 1;
         if (!mbar::wait_warp(&sh.step[it % kStepBars], (unsigned)(it / kStepBars) & 1u)) {
@@ -400,11 +413,11 @@ __global__ void __launch_bounds__(kDownThreads, 1) k_down(const __grid_constant_
         after_sync();
         for (int t = 0; t < nt; ++t) {
           const unsigned at = tmem + ((unsigned)quad << 21) + (unsigned)((buf * 2 + t) * 2 * NR);
-          float v[2 * TERMS][kJ];
+          float v[2 * kTerms][kJ];
 #pragma unroll
-          for (int k = 0; k < 2 * TERMS; ++k) tmem_ld16(at + k * kJ, v[k]);
+          for (int k = 0; k < 2 * kTerms; ++k) tmem_ld16(at + k * kJ, v[k]);
 #pragma unroll
-          for (int k = 0; k < 2 * TERMS; ++k) tmem_wait(v[k]);
+          for (int k = 0; k < 2 * kTerms; ++k) tmem_wait(v[k]);
           if (t + 1 == nt) {                                      // the sums have been taken out
             before_sync();
             __syncwarp();
@@ -412,11 +425,12 @@ __global__ void __launch_bounds__(kDownThreads, 1) k_down(const __grid_constant_
           }
           float r[kJ];
 #pragma unroll
-          for (int j = 0; j < kJ; ++j) {                          // low terms first
-            r[j] = v[TERMS - 1][j] + v[2 * TERMS - 1][j];
-#pragma unroll
-            for (int k = TERMS - 2; k >= 0; --k) r[j] += v[k][j] + v[TERMS + k][j];
-            if (TERMS == 2) r[j] *= scale;
+          for (int j = 0; j < kJ; ++j) {                          // low terms first, and with them what was cut off
+            const float top = v[0][j] + v[kTerms][j];
+            r[j] = v[2][j] + v[kTerms + 2][j];
+            r[j] += v[1][j] + v[kTerms + 1][j];
+            r[j] = top + fmaf(top, kCutOff, r[j]);
+            if (kF16) r[j] *= scale;
           }
           float *yr = P.y + ((size_t)blockIdx.z * 2 * P.d + (tile0 + t) * kRows + row) * g.M;
           store8(yr + 8 * b, r[0], r[2], r[4], r[6], r[8], r[10], r[12], r[14]);
@@ -498,13 +512,13 @@ __device__ __forceinline__ void mid_entry(const Geometry &g, const MidRadices &m
 }
 
 // All tables of a sequence in one launch: `down` + `up` + the rest of the entries, 256 per block.
-template <typename T, int TERMS>
+template <typename T>
 __global__ void __launch_bounds__(256) k_band_tables(const __grid_constant__ Geometry g, const MidRadices m, T *down, __half *up,
                                                      MidTables mid, int down_blocks, int up_blocks) {
   int b = blockIdx.x;
   if (b < down_blocks) {
     const int per = g.ks;                                             // blocks per matrix: 16 * ks * 16 entries
-    down_entry<T, TERMS>(g, b / per, (b % per) * 256 + threadIdx.x, down);
+    down_entry<T>(g, b / per, (b % per) * 256 + threadIdx.x, down);
     return;
   }
   b -= down_blocks;
@@ -619,6 +633,23 @@ __device__ __forceinline__ void turn(C2 (&x)[R], const float2 *__restrict__ tw, 
     }
   }
 }
+
+// The largest of G adjacent lanes' values, none of them negative (a NaN counts as large)
+template <int G>
+__device__ __forceinline__ unsigned group_max(float v) {
+  unsigned u = __float_as_uint(v);
+  if constexpr (G == 32) {
+    u = __reduce_max_sync(0xffffffffu, u);
+  } else {
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) {
+      const unsigned w = __shfl_xor_sync(0xffffffffu, u, o);
+      u = u > w ? u : w;
+    }
+  }
+  return u;
+}
+__device__ __forceinline__ float unit_rounder(unsigned largest) { return __uint_as_float((largest & 0x7f800000u) + 0x06c00000u); }
 
 struct MidParams {
   const float *y;                            // [row][M]
@@ -775,6 +806,8 @@ __global__ void __launch_bounds__(S::NT, S::NT <= 512 ? 512 / S::NT : 1) k_mid(c
     (r ? sc.y : sc.x) = __uint_as_float((unsigned)(14 - ex + 127) << 23);           // 2^(14 - ex)
     if (t == 0) P.inv[row + r] = -__uint_as_float((unsigned)(ex - 14 + 127) << 23) * (1.f / kUpScale);
   }
+  // The first term of a value is a whole number of units, 2^-10 of the power of two below the largest of the 64 values
+  // (2 G complex ones' worth) that lie around it, so that k_up's sums of first terms are exact; the second is what is left.
   __half2 *hi = reinterpret_cast<__half2 *>(P.hi) + row * Mh, *lo = reinterpret_cast<__half2 *>(P.lo) + row * Mh;
 #pragma unroll
   for (int u = 0; u < 16 / R; ++u)
@@ -782,19 +815,19 @@ __global__ void __launch_bounds__(S::NT, S::NT <= 512 ? 512 / S::NT : 1) k_mid(c
     for (int p = 0; p < R; ++p) {
       const int n = t + T * u + sub * p;
       const float2 re = mul2(x[u * R + p].re, sc), im = mul2(x[u * R + p].im, sc);
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const float2 v = r ? make_float2(re.y, im.y) : make_float2(re.x, im.x);
-        const __half2 h = __floats2half2_rn(v.x, v.y);
-        const float2 hf = __half22float2(h);
-        hi[r * Mh + n] = h;
-        lo[r * Mh + n] = __floats2half2_rn(v.x - hf.x, v.y - hf.y);
-      }
+      // 1.5 * 2^13 of that power of two: adding it rounds to whole units, subtracting it leaves them
+      const float2 c = make_float2(unit_rounder(group_max<G>(fmaxf(fabsf(re.x), fabsf(im.x)))),
+                                   unit_rounder(group_max<G>(fmaxf(fabsf(re.y), fabsf(im.y)))));
+      const float2 hre = sub2(add2(re, c), c), him = sub2(add2(im, c), c), lre = sub2(re, hre), lim = sub2(im, him);
+      hi[n] = __floats2half2_rn(hre.x, him.x);
+      hi[Mh + n] = __floats2half2_rn(hre.y, him.y);
+      lo[n] = __floats2half2_rn(lre.x, lim.x);
+      lo[Mh + n] = __floats2half2_rn(lre.y, lim.y);
     }
 }
 
 // ---------------------------------------------------------------------------------------------------- k_up
-// The two terms of a launch's grid values, [term][row][M]: boxes of 32 or 16 values of 128 rows of both terms.
+// The two terms of a launch's grid values, [term][row][M]: boxes of 32 or 16 values of 128 rows of one term.
 struct GridMaps {
   CUtensorMap wide, narrow;
 };
@@ -808,14 +841,14 @@ struct UpParams {
   long long score_stride, energy_stride;
   int H, d, u0, per, ranges;
 };
-constexpr int kUpBufs = 4;                   // sums of 128 x 128 in tensor memory
-constexpr int kYStages = 2;
+constexpr int kUpBufs = 2;                   // pairs of sums of 128 x 128 in tensor memory
 constexpr int x_stages(int nq) { return nq == 16 ? 3 : 2; }      // as many as fit
 constexpr int kMaxX = 3;
+constexpr int y_stages(int nq, int term) { return term == 0 || nq == 16 ? 2 : 1; }
 constexpr int kUpThreads = 64 + 256 + 32;    // grid values and matrices, products, eight warps (four per 64 channels), rows
 struct UpShared {
-  unsigned long long xfull[kMaxX], xempty[kMaxX], yfull[kYStages], yempty[kYStages], tfull, tempty, afull[kUpBufs],
-      aempty[kUpBufs], done;
+  unsigned long long xfull[kMaxX], xempty[kMaxX], yfull[2][2], yempty[2][2], tfull[kTerms], tempty[kTerms], afull[kUpBufs],
+      aempty[kUpBufs], done;                 // y: [term][stage]
   unsigned tmem;
   int last;
   float other[2][kRows];
@@ -823,7 +856,8 @@ struct UpShared {
   int quad[kMaxPer];                         // first quad of the block's steps
 };
 __host__ __device__ inline size_t up_smem(int nq, int d) {
-  return 1024 + (size_t)x_stages(nq) * 8 * kBoxBytes + (size_t)(kYStages + 1) * nq * 2048 + (size_t)2 * d * sizeof(float);
+  return 1024 + (size_t)x_stages(nq) * 8 * kBoxBytes + (size_t)(y_stages(nq, 0) + y_stages(nq, 1) + kTerms) * nq * 1024 +
+         (size_t)2 * d * sizeof(float);
 }
 
 __device__ __forceinline__ uint4 lds(unsigned addr) {
@@ -838,22 +872,33 @@ template <> __device__ __forceinline__ float2 widen<__nv_bfloat16>(unsigned v) {
 }
 
 // What bounds it: HBM, or L2 where a launch group fits it.  A step of 128 tokens and 128 channels is 64 KB of operands and
-// twelve products of 128 x 128 x 16 (64 cycles each); tokens are the lanes of the sums, so that a row's squares stay in one
+// twenty products of 128 x 128 x 16 (64 cycles each); tokens are the lanes of the sums, so that a row's squares stay in one
 // thread, and the grid values are the right operand as the transform left them (64- and 32-byte swizzled boxes).  Rows, and
-// grid values with the matrices, have a loading warp each: with one for both, grid values waited for the rows before them
-// (107 us for 16 heads of 32768 tokens, 85..90 us now, 420 MB).
+// grid values with the matrices, have a loading warp each: with one for both, grid values waited for the rows before them.
+//
+// The tensor cores cut off what does not fit the 24 bits of a sum, so the sum that matters is one that always fits: the first
+// terms of the matrix are whole numbers of up to 11 bits, those of the grid values of up to 11 bits and a sign in units that
+// are the same for 64 values (k_mid), and a window's sum of their products stays below 2^23 such units.  All other products
+// (second terms with first ones, the matrix's third with the values' first, second with second) go to a sum of their own,
+// whose cut-off bits are 2^-10 of that size; both are added in fp32.  In a model of these sums, two terms of the matrix and
+// one sum for everything leave 0.3..0.5e-6 of a score (rms, 10 % outlier rows), this 0.7e-7, and k_mid's fp32 0.2..0.5e-6.
+//
+// A matrix comes in three parts, one per term, and products are in such an order that each part is free, and the next step's
+// on its way, well before it is needed again: lo x hi, mid x hi, mid x lo, hi x lo, hi x hi.
+//
 // One block: `per` steps of 128 tokens of one unit.  grid (ranges, units).
 template <typename T, int NQ>
 __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Maps maps, const __grid_constant__ GridMaps grid,
                                                    const __grid_constant__ Geometry g,
                                                    const __grid_constant__ UpParams P) {
-  constexpr int kXStages = x_stages(NQ);
+  constexpr int kXStages = x_stages(NQ), kHi = y_stages(NQ, 0), kLo = y_stages(NQ, 1);
   extern __shared__ unsigned char raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(((uintptr_t)raw + 1023) & ~(uintptr_t)1023);
-  unsigned char *ys = smem + (size_t)kXStages * 8 * kBoxBytes;
-  constexpr unsigned ybytes = NQ * 2048u, run = NQ * 512u;                         // both terms, both runs; one run
-  unsigned char *tab = ys + (size_t)kYStages * ybytes;
-  float *sinv = reinterpret_cast<float *>(tab + ybytes);
+  unsigned char *ys = smem + (size_t)kXStages * 8 * kBoxBytes;                     // kHi stages of first terms, kLo of second
+  constexpr unsigned ybytes = NQ * 1024u, run = NQ * 512u;                         // one term: both runs; one run
+  constexpr unsigned tbytes = NQ * 1024u;                                          // one term of a matrix
+  unsigned char *tab = ys + (size_t)(kHi + kLo) * ybytes;
+  float *sinv = reinterpret_cast<float *>(tab + kTerms * tbytes);
   __shared__ UpShared sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int unit = P.u0 + blockIdx.y, layer = unit / P.H, head = unit - layer * P.H;
@@ -862,13 +907,13 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Ma
 
   if (tid == 0) {
     for (int i = 0; i < kXStages; ++i) { mbar::init(&sh.xfull[i], 1u); mbar::init(&sh.xempty[i], 8u); }
-    for (int i = 0; i < kYStages; ++i) { mbar::init(&sh.yfull[i], 1u); mbar::init(&sh.yempty[i], 1u); }
-    mbar::init(&sh.tfull, 1u); mbar::init(&sh.tempty, 1u);
+    for (int i = 0; i < 4; ++i) { mbar::init(&sh.yfull[i >> 1][i & 1], 1u); mbar::init(&sh.yempty[i >> 1][i & 1], 1u); }
+    for (int i = 0; i < kTerms; ++i) { mbar::init(&sh.tfull[i], 1u); mbar::init(&sh.tempty[i], 1u); }
     for (int i = 0; i < kUpBufs; ++i) { mbar::init(&sh.afull[i], 1u); mbar::init(&sh.aempty[i], 8u); }
     mbar::init(&sh.done, 1u);
     mbar::init_done();
   }
-  if (warp == 1) tmem_alloc(&sh.tmem, 128 * kUpBufs);
+  if (warp == 1) tmem_alloc(&sh.tmem, 256 * kUpBufs);
   for (int i = tid; i < b1 - b0; i += kUpThreads) sh.quad[i] = up_quad(g, b0 + i);
   before_sync();
   __syncthreads();
@@ -877,35 +922,56 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Ma
   if (warp == 0) {
     if (lane == 0) {
       bool ok = true;
-      int ntab = 0, cls = -1, ny = 0;
+      int ntab[kTerms] = {}, ny[2] = {}, cls = -1;
+      auto matrix = [&](int term, int c) {
+        if (ok && ntab[term] > 0) ok = mbar::wait(&sh.tempty[term], (unsigned)(ntab[term] - 1) & 1u);
+        if (!ok) return;
+        mbar::expect_tx(&sh.tfull[term], tbytes);
+        load_bytes(tab + term * tbytes, reinterpret_cast<const unsigned char *>(P.table) + ((size_t)c * kTerms + term) * tbytes, tbytes,
+                   &sh.tfull[term]);
+        ++ntab[term];
+      };
+      auto values = [&](int term, int q0, int t) {
+        const int stages = term == 0 ? kHi : kLo, s = ny[term] % stages;
+        if (ok && ny[term] >= stages) ok = mbar::wait(&sh.yempty[term][s], (unsigned)(ny[term] / stages - 1) & 1u);
+        if (!ok) return;
+        mbar::expect_tx(&sh.yfull[term][s], ybytes);
+        const int r0 = ((int)blockIdx.y * tiles + t) * kRows;
+        unsigned char *dst = ys + (size_t)(term == 0 ? s : kHi + s) * ybytes;
+        for (int rn = 0; rn < 2; ++rn, dst += run) {           // a run: a box of 32 values and, with 24 quads, one of 16
+          const int x = rn == 0 ? 2 * q0 : g.M - 2 * (q0 + NQ);
+          load_box(dst, &grid.wide, x, r0, term, &sh.yfull[term][s]);
+          if (NQ > 16) load_box(dst + kRows * 64, &grid.narrow, x + 32, r0, term, &sh.yfull[term][s]);
+        }
+        ++ny[term];
+      };
       const int items = (b1 - b0) * tiles;
       for (int it = 0; it < items && ok; ++it) {
         const int b = b0 + it / tiles, t = it - (b - b0) * tiles, c = class_of(b, n, classes), q0 = sh.quad[b - b0];
-        if (c != cls) {
-          cls = c;
-          if (ntab >= 1 && !mbar::wait(&sh.tempty, (unsigned)(ntab - 1) & 1u)) { ok = false; break; }
-          mbar::expect_tx(&sh.tfull, ybytes);
-          load_bytes(tab, reinterpret_cast<const unsigned char *>(P.table) + (size_t)c * ybytes, ybytes, &sh.tfull);
-          ++ntab;
-        }
+        const bool fresh = c != cls;
+        cls = c;
         if (it == 0) {
+          for (int k = kTerms - 1; k >= 0; --k) matrix(k, c);
           asm volatile("griddepcontrol.wait;\n" ::: "memory");
           asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+          values(0, q0, t);
+          values(1, q0, t);
+          continue;
         }
-        const int s = ny % kYStages;
-        if (ny >= kYStages && !mbar::wait(&sh.yempty[s], (unsigned)(ny / kYStages - 1) & 1u)) { ok = false; break; }
-        mbar::expect_tx(&sh.yfull[s], ybytes);
-        const int r0 = ((int)blockIdx.y * tiles + t) * kRows;
-        unsigned char *dst = ys + (size_t)s * ybytes;
-        for (int rn = 0; rn < 2; ++rn, dst += 2 * run) {       // a run: a box of 32 values and, with 24 quads, one of 16
-          const int x = rn == 0 ? 2 * q0 : g.M - 2 * (q0 + NQ);
-          load_box(dst, &grid.wide, x, r0, 0, &sh.yfull[s]);
-          if (NQ > 16) load_box(dst + 2 * kRows * 64, &grid.narrow, x + 32, r0, 0, &sh.yfull[s]);
-        }
-        ++ny;
+        // in the order in which the places become free
+        values(0, q0, t);
+        if (fresh) { matrix(2, c); matrix(1, c); }
+        values(1, q0, t);
+        if (fresh) matrix(0, c);
       }
-      for (int i = ny > kYStages ? ny - kYStages : 0; i < ny; ++i) ok &= mbar::wait(&sh.yfull[i % kYStages], (unsigned)(i / kYStages) & 1u);
-      if (ntab > 0) ok &= mbar::wait(&sh.tfull, (unsigned)(ntab - 1) & 1u);
+      // no load may be in flight when the block ends
+      for (int k = 0; k < 2; ++k) {
+        const int stages = k == 0 ? kHi : kLo;
+        for (int i = ny[k] > stages ? ny[k] - stages : 0; i < ny[k]; ++i)
+          ok &= mbar::wait(&sh.yfull[k][i % stages], (unsigned)(i / stages) & 1u);
+      }
+      for (int k = 0; k < kTerms; ++k)
+        if (ntab[k] > 0) ok &= mbar::wait(&sh.tfull[k], (unsigned)(ntab[k] - 1) & 1u);
       if (!ok) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
     }
   } else if (warp == 10) {
@@ -931,34 +997,46 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Ma
     const unsigned lead = elect();
     const unsigned yb = (smem_addr(ys) >> 4) | operand_lo(16), tb = (smem_addr(tab) >> 4) | operand_lo(2048);
     bool ok = true;
-    int ntab = 0, cls = -1, it = 0;
+    int ntab = -1, cls = -1, it = 0;
     for (int b = b0; b < b1 && ok; ++b) {
       const int c = class_of(b, n, classes);
+      const bool leave = b + 1 < b1 && class_of(b + 1, n, classes) != c;           // another matrix after this step
       for (int t = 0; t < tiles; ++t, ++it) {
-        if (c != cls) {
-          cls = c;
-          if (ntab > 0) commit(lead, &sh.tempty);
-          if (!mbar::wait_warp(&sh.tfull, (unsigned)ntab & 1u)) { ok = false; break; }
-          ++ntab;
-        }
-        const int s = it % kYStages, buf = it % kUpBufs;
-        if (it >= kUpBufs && !mbar::wait_warp(&sh.aempty[buf], (unsigned)(it / kUpBufs - 1) & 1u)) { ok = false; break; }
-        if (!mbar::wait_warp(&sh.yfull[s], (unsigned)(it / kYStages) & 1u)) { ok = false; break; }
-        after_sync();
-        const unsigned ya = yb + (unsigned)s * (ybytes / 16), d = tmem + (unsigned)buf * 128u;
-        // low times high, high times low, high times high: small terms first
-#pragma unroll
-        for (int pr = 0; pr < 3; ++pr)
+        const bool fresh = c != cls, last = leave && t == tiles - 1;
+        if (fresh) { cls = c; ++ntab; }
+        const int sh_ = it % kHi, sl = it % kLo, buf = it % kUpBufs;
+        const unsigned yhi = yb + (unsigned)sh_ * (ybytes / 16), ylo = yb + (unsigned)(kHi + sl) * (ybytes / 16);
+        const unsigned big = tmem + (unsigned)buf * 256u, small = big + 128u;
+        auto part_here = [&](int term) { return !fresh || mbar::wait_warp(&sh.tfull[term], (unsigned)ntab & 1u); };
+        auto products = [&](unsigned d, int term, unsigned y, bool start) {
 #pragma unroll
           for (int k = 0; k < NQ / 4; ++k) {
             const int in = k % (NQ / 8);                                   // step within its run
             const bool w = in < 2;                                         // and its box
-            const unsigned off = (k / (NQ / 8)) * (2 * run) + (w ? in * 32u : 2u * kRows * 64u) +
-                                 (pr == 1 ? kRows * (w ? 64u : 32u) : 0u);
-            mma(lead, d, tb + (pr == 0 ? 2 * run / 16 : 0u) + k * 256u, hi, ya + off / 16, w ? wide : narrow, idesc,
-                pr + k > 0 ? 1u : 0u);
+            const unsigned off = (k / (NQ / 8)) * run + (w ? in * 32u : kRows * 64u);
+            mma(lead, d, tb + (unsigned)term * (tbytes / 16) + k * 256u, hi, y + off / 16, w ? wide : narrow, idesc,
+                start && k == 0 ? 0u : 1u);
           }
-        commit(lead, &sh.yempty[s]);
+        };
+        if (it >= kUpBufs && !mbar::wait_warp(&sh.aempty[buf], (unsigned)(it / kUpBufs - 1) & 1u)) { ok = false; break; }
+        if (!mbar::wait_warp(&sh.yfull[0][sh_], (unsigned)(it / kHi) & 1u) || !part_here(2)) { ok = false; break; }
+        after_sync();
+        products(small, 2, yhi, true);
+        if (last) commit(lead, &sh.tempty[2]);
+        if (!part_here(1)) { ok = false; break; }
+        after_sync();
+        products(small, 1, yhi, false);
+        if (!mbar::wait_warp(&sh.yfull[1][sl], (unsigned)(it / kLo) & 1u)) { ok = false; break; }
+        after_sync();
+        products(small, 1, ylo, false);
+        if (last) commit(lead, &sh.tempty[1]);
+        if (!part_here(0)) { ok = false; break; }
+        after_sync();
+        products(small, 0, ylo, false);
+        commit(lead, &sh.yempty[1][sl]);
+        products(big, 0, yhi, true);
+        commit(lead, &sh.yempty[0][sh_]);
+        if (last) commit(lead, &sh.tempty[0]);
         commit(lead, &sh.afull[buf]);
       }
     }
@@ -985,23 +1063,27 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Ma
         const int kv = (2 * t + half) * 64 >= P.d;
         const unsigned xr = smem_addr(smem) + (unsigned)((s * 8 + quad * 2 + half) * kBoxBytes + lane * 128);
         const unsigned iv = smem_addr(sinv + t * kRows + half * 64);
-        const unsigned at = tmem + ((unsigned)quad << 21) + (unsigned)(buf * 128 + half * 64);
+        const unsigned at = tmem + ((unsigned)quad << 21) + (unsigned)(buf * 256 + half * 64);
         float2 rs[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, xs[2] = {rs[0], rs[0]};
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          float a[16];
+          float a[16], low[16];
           tmem_ld16(at + 16 * c, a);
+          tmem_ld16(at + 128 + 16 * c, low);
           uint4 xv[2];
 #pragma unroll
           for (int i = 0; i < 2; ++i) xv[i] = lds(xr + (((2 * c + i) ^ (lane & 7)) << 4));
           tmem_wait(a);
+          tmem_wait(low);
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const uint4 sc = lds(iv + (unsigned)(4 * c + i) * 16u);
             const unsigned w0 = i & 1 ? xv[i >> 1].z : xv[i >> 1].x, w1 = i & 1 ? xv[i >> 1].w : xv[i >> 1].y;
             const float2 xa = widen<T>(w0), xb = widen<T>(w1);
-            const float2 ra = fma2(make_float2(a[4 * i], a[4 * i + 1]), make_float2(__uint_as_float(sc.x), __uint_as_float(sc.y)), xa);
-            const float2 rb = fma2(make_float2(a[4 * i + 2], a[4 * i + 3]), make_float2(__uint_as_float(sc.z), __uint_as_float(sc.w)), xb);
+            const float2 ba = add2(make_float2(a[4 * i], a[4 * i + 1]), make_float2(low[4 * i], low[4 * i + 1]));
+            const float2 bb = add2(make_float2(a[4 * i + 2], a[4 * i + 3]), make_float2(low[4 * i + 2], low[4 * i + 3]));
+            const float2 ra = fma2(ba, make_float2(__uint_as_float(sc.x), __uint_as_float(sc.y)), xa);
+            const float2 rb = fma2(bb, make_float2(__uint_as_float(sc.z), __uint_as_float(sc.w)), xb);
             rs[0] = fma2(ra, ra, rs[0]);
             rs[1] = fma2(rb, rb, rs[1]);
             xs[0] = fma2(xa, xa, xs[0]);
@@ -1061,7 +1143,7 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Ma
   }
   before_sync();
   __syncthreads();
-  if (warp == 1) tmem_free(tmem, 128 * kUpBufs);
+  if (warp == 1) tmem_free(tmem, 256 * kUpBufs);
   // energies: in the block of the layer that comes last, all steps' sums in order
   if (tid == 0) {
     __threadfence();
