@@ -845,14 +845,14 @@ constexpr int kUpBufs = 2;                   // pairs of sums of 128 x 128 in te
 constexpr int x_stages(int nq) { return nq == 16 ? 3 : 2; }      // as many as fit
 constexpr int kMaxX = 3;
 constexpr int y_stages(int nq, int term) { return term == 0 || nq == 16 ? 2 : 1; }
-constexpr int kUpThreads = 64 + 256 + 32;    // grid values and matrices, products, eight warps (four per 64 channels), rows
+// grid values and matrices, products, eight warps that take the sums out (four per 64 channels), rows, results of a step
+constexpr int kUpThreads = 64 + 256 + 32 + 32;
 struct UpShared {
   unsigned long long xfull[kMaxX], xempty[kMaxX], yfull[2][2], yempty[2][2], tfull[kTerms], tempty[kTerms], afull[kUpBufs],
-      aempty[kUpBufs], done;                 // y: [term][stage]
+      aempty[kUpBufs], rfull[2], rempty[2], done;                 // y: [term][stage]
   unsigned tmem;
   int last;
-  float other[2][kRows];
-  double red[2][8][4];
+  float4 sums[2][2][kRows];                  // of a step's rows: |residual|^2 and |z|^2 of K, of V; per 64 channels of a tile
   int quad[kMaxPer];                         // first quad of the block's steps
 };
 __host__ __device__ inline size_t up_smem(int nq, int d) {
@@ -871,8 +871,8 @@ template <> __device__ __forceinline__ float2 widen<__nv_bfloat16>(unsigned v) {
   return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
 }
 
-// What bounds it: HBM, or L2 where a launch group fits it.  A step of 128 tokens and 128 channels is 64 KB of operands and
-// twenty products of 128 x 128 x 16 (64 cycles each); tokens are the lanes of the sums, so that a row's squares stay in one
+// What bounds it: HBM, or L2 where a launch group fits it, and shared memory.  A tile of 128 tokens and 128 channels is 64 KB
+// of operands and twenty products of 128 x 128 x 16 (64 cycles each, in which they read 128 bytes a cycle, all there is); tokens are the lanes of the sums, so that a row's squares stay in one
 // thread, and the grid values are the right operand as the transform left them (64- and 32-byte swizzled boxes).  Rows, and
 // grid values with the matrices, have a loading warp each: with one for both, grid values waited for the rows before them.
 //
@@ -910,6 +910,7 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Ma
     for (int i = 0; i < 4; ++i) { mbar::init(&sh.yfull[i >> 1][i & 1], 1u); mbar::init(&sh.yempty[i >> 1][i & 1], 1u); }
     for (int i = 0; i < kTerms; ++i) { mbar::init(&sh.tfull[i], 1u); mbar::init(&sh.tempty[i], 1u); }
     for (int i = 0; i < kUpBufs; ++i) { mbar::init(&sh.afull[i], 1u); mbar::init(&sh.aempty[i], 8u); }
+    for (int i = 0; i < 2; ++i) { mbar::init(&sh.rfull[i], 8u); mbar::init(&sh.rempty[i], 1u); }
     mbar::init(&sh.done, 1u);
     mbar::init_done();
   }
@@ -991,6 +992,46 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Ma
       for (int i = nx > kXStages ? nx - kXStages : 0; i < nx; ++i) ok &= mbar::wait(&sh.xfull[i % kXStages], (unsigned)(i / kXStages) & 1u);
       if (!ok) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
     }
+  } else if (warp == 11) {
+    // scores and energies of a step, beside the next step's tiles: 1700 of 5300 cycles a step went into the fp64 sums where
+    // the warps that take the tiles out made them (16 heads of 32768 tokens 110 -> 97 us)
+    const float inv_d = 1.f / (float)P.d;
+    for (int b = b0; b < b1; ++b) {
+      const int rs = (b - b0) & 1;
+      if (!mbar::wait_warp(&sh.rfull[rs], (unsigned)((b - b0) / 2) & 1u)) {
+        if (lane == 0) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
+        break;
+      }
+      float4 lo[4], hi[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) { lo[i] = sh.sums[rs][0][32 * i + lane]; hi[i] = sh.sums[rs][1][32 * i + lane]; }
+      __syncwarp();
+      if (lane == 0) mbar::arrive(&sh.rempty[rs]);
+      double e[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int tok = b * kRows + 32 * i + lane;
+        if (tok < g.N)
+          P.scores[layer][(long long)head * P.score_stride + tok] = ((lo[i].x + lo[i].z) + (hi[i].x + hi[i].z)) * inv_d;
+        e[0] += (double)lo[i].x + (double)hi[i].x;
+        e[1] += (double)lo[i].y + (double)hi[i].y;
+        e[2] += (double)lo[i].z + (double)hi[i].z;
+        e[3] += (double)lo[i].w + (double)hi[i].w;
+      }
+      // sums of the step, so that the energies do not depend on how steps are spread over blocks: four values over the
+      // lanes at once, lane 8 i ends up with value i
+      const bool up = (lane & 16) != 0, up2 = (lane & 8) != 0;
+      double v0 = up ? e[2] : e[0], v1 = up ? e[3] : e[1];
+      v0 += __shfl_xor_sync(0xffffffffu, up ? e[0] : e[2], 16);
+      v1 += __shfl_xor_sync(0xffffffffu, up ? e[1] : e[3], 16);
+      double v = up2 ? v1 : v0;
+      v += __shfl_xor_sync(0xffffffffu, up2 ? v0 : v1, 8);
+      v += __shfl_xor_sync(0xffffffffu, v, 4);
+      v += __shfl_xor_sync(0xffffffffu, v, 2);
+      v += __shfl_xor_sync(0xffffffffu, v, 1);
+      if ((lane & 7) == 0) P.part[((size_t)unit * n + b) * 4 + (lane >> 3)] = v;
+    }
+    __threadfence();
   } else if (warp == 1) {
     constexpr unsigned idesc = instruction(true, false, kRows), hi = operand_hi(128, 0);
     constexpr unsigned wide = operand_hi(512, 4), narrow = operand_hi(256, 6);     // 64- and 32-byte swizzle
@@ -1104,42 +1145,19 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Ma
           }
         }
       }
-      const int tok = b * kRows + row;
-      const bool in = tok < g.N;
-      float sum[4];                          // hiK, totK, hiV, totV of this thread's row and channels
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        sum[2 * i] = in ? (r2[i][0].x + r2[i][0].y) + (r2[i][1].x + r2[i][1].y) : 0.f;
-        sum[2 * i + 1] = in ? (x2[i][0].x + x2[i][0].y) + (x2[i][1].x + x2[i][1].y) : 0.f;
-      }
-      // sums of the step, so that the energies do not depend on how steps are spread over blocks: four values over the
-      // lanes at once, lane 8 i ends up with value i
-      {
-        const bool up = (lane & 16) != 0, up2 = (lane & 8) != 0;
-        double v0 = up ? (double)sum[2] : (double)sum[0], v1 = up ? (double)sum[3] : (double)sum[1];
-        v0 += __shfl_xor_sync(0xffffffffu, up ? (double)sum[0] : (double)sum[2], 16);
-        v1 += __shfl_xor_sync(0xffffffffu, up ? (double)sum[1] : (double)sum[3], 16);
-        double v = up2 ? v1 : v0;
-        v += __shfl_xor_sync(0xffffffffu, up2 ? v0 : v1, 8);
-        v += __shfl_xor_sync(0xffffffffu, v, 4);
-        v += __shfl_xor_sync(0xffffffffu, v, 2);
-        v += __shfl_xor_sync(0xffffffffu, v, 1);
-        if ((lane & 7) == 0) sh.red[(b - b0) & 1][warp - 2][lane >> 3] = v;
-      }
-      float &o = sh.other[(b - b0) & 1][row];
-      if (half == 1) o = sum[0] + sum[2];
-      asm volatile("bar.sync 1, 256;\n" ::: "memory");
-      if (half == 0 && in)
-        P.scores[layer][(long long)head * P.score_stride + tok] = (sum[0] + sum[2] + o) * (1.f / (float)P.d);
-      if (warp == 9 && lane < 4) {
-        double v = 0.0;
-#pragma unroll
-        for (int w = 0; w < 8; ++w) v += sh.red[(b - b0) & 1][w][lane];
-        P.part[((size_t)unit * n + b) * 4 + lane] = v;
-      }
+      const int rs = (b - b0) & 1;
+      if (!failed && b - b0 >= 2) failed = !mbar::wait_warp(&sh.rempty[rs], (unsigned)((b - b0) / 2 - 1) & 1u);
+      if (failed) break;
+      // this thread's row and channels; rows past the end count nothing
+      const bool in = b * kRows + row < g.N;
+      sh.sums[rs][half][row] =
+          in ? make_float4((r2[0][0].x + r2[0][0].y) + (r2[0][1].x + r2[0][1].y), (x2[0][0].x + x2[0][0].y) + (x2[0][1].x + x2[0][1].y),
+                           (r2[1][0].x + r2[1][0].y) + (r2[1][1].x + r2[1][1].y), (x2[1][0].x + x2[1][0].y) + (x2[1][1].x + x2[1][1].y))
+             : make_float4(0.f, 0.f, 0.f, 0.f);
+      __syncwarp();
+      if (lane == 0) mbar::arrive(&sh.rfull[rs]);
     }
     if (failed && lane == 0) atomicOr(P.status, FC_DEV_FLAG_TIMEOUT);
-    __threadfence();
   }
   before_sync();
   __syncthreads();
