@@ -94,7 +94,8 @@ typedef struct {
  * are limited to 65536).  Allocates the twiddle table (8 bytes * 4 * next power of two of
  * max_seqlen, at least 64), room for eight filter tables (16 bytes * the power of two from 2*max_seqlen-1 up each, at
  * least 16 KiB and at most 2 MiB; lengths that are not a power of two reuse theirs from layer to layer and call to call,
- * a batch of more than eight unlike ones builds the rest in the workspace on every call) and a status word.  Returns FC_ERR_CUDA if the device cannot be
+ * a batch of more than eight unlike ones builds the rest in the workspace on every call), room for the tables of four 16-bit
+ * sequences scored on a coarser grid (640 or 1280 KiB each; none up to 512 tokens) and a status word.  Returns FC_ERR_CUDA if the device cannot be
  * used, FC_ERR_UNSUPPORTED if max_seqlen is out of range. */
 fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen);
 void fc_destroy(fc_handle *h);
@@ -188,9 +189,12 @@ fc_status fc_set_l2_persist(fc_handle *h, int32_t enabled);
  * next call by the stream that call is given (a graph launch on that stream is). */
 fc_status fc_reset_ordering(fc_handle *h);
 
-/* Target size in bytes of the transform intermediates processed per kernel group
- * (kept below the L2 capacity so they are re-read from cache, not HBM).
- * Default 32 MiB.  Affects speed only. */
+/* Target size in bytes of the transform intermediates processed per kernel group (three passes: kept below the L2 capacity so
+ * they are re-read from cache, not HBM).  Default 32 MiB.  16-bit sequences scored on a coarser grid take groups of up to four
+ * times this, which is faster than staying in cache: a scoring call's workspace holds two groups (one per internal stream),
+ * i.e. at most about 270 MB by default besides tables (28 layers of 4 heads of 32768 tokens: 272 MB in all; less where all
+ * intermediates are smaller), and up to 0.9 KB of tables per token of every distinct length that is not a power of two.
+ * Affects speed and the workspace only; set it before the workspace is queried. */
 fc_status fc_set_group_bytes(fc_handle *h, size_t bytes);
 
 /* How a sequence of length seqlen could be transformed at cutoff ratio gamma (diagnostic): out = { form, transform

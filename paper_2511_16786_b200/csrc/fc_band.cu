@@ -168,7 +168,7 @@ struct FcBandJob {
   bool f16;
   int H, d;
   size_t off_up, off_mid, table_bytes;       // k_down's matrices first
-  size_t y_bytes, plane_bytes;               // of one unit
+  size_t y_bytes;                            // grid values of one unit
   band::Maps maps;
 };
 
@@ -179,16 +179,33 @@ static int mid_tw_len(int Mh) {
   return 0;
 }
 
+// What the tables of a sequence take: k_down's matrices, k_up's, and what k_mid looks up.
+static size_t table_bytes(const Geometry &g, size_t *off_up, size_t *off_mid) {
+  *off_up = align256(band::down_classes(g) * band::down_image(g));
+  *off_mid = *off_up + align256(band::up_classes(g) * band::up_image(g));
+  return *off_mid + align256((size_t)g.M / 2 * 16) + align256((size_t)mid_tw_len(g.M / 2) * sizeof(float2));
+}
+
 bool fc_band_bounds(const fc_kv_view *kv, int N, FcBandSizes *s) {
   if (!eligible(kv, N)) return false;
-  // M <= N/2, windows at their largest, every step with matrices of its own
-  const int M = N / 2 < kMaxGrid ? N / 2 : kMaxGrid;
-  s->tables = align256((size_t)(M / band::kJ) * band::kMaxSteps * 2 * 48 * 16) +
-              align256((size_t)((N + band::kRows - 1) / band::kRows) * band::kMaxQuads * band::kTerms * 1024) + align256((size_t)M * 32) +
-              align256((size_t)M * 6 * sizeof(float2));
-  s->unit = (size_t)2 * kv->head_dim * M * 8 + align256((size_t)2 * kv->head_dim * 4) + 1024;
+  *s = FcBandSizes{};
   s->steps = (N + band::kRows - 1) / band::kRows;
-  return true;
+  // the grids make_geometry may choose (two where N is a power of two, else one), with the widest kernel's windows
+  for (int M = kMinGrid; M <= kMaxGrid && 2 * M <= N; M <<= 1) {
+    if (4ll * M < N) continue;
+    Geometry g = {};
+    g.N = N;
+    g.M = M;
+    g.same = N == 2 * M || N == 4 * M;
+    const long long span = ((band::kJ - 1ll + kKernels[kNumKernels - 1].W) * N + M - 1) / M + 16;   // tokens, from a 16th one on
+    g.ks = (int)((span + 15) / 16 < band::kMaxSteps ? (span + 15) / 16 : band::kMaxSteps);
+    g.nq = band::kMaxQuads;
+    size_t a, b;
+    const size_t tables = table_bytes(g, &a, &b), unit = (size_t)2 * kv->head_dim * M * sizeof(float) + align256((size_t)2 * kv->head_dim * 4);
+    if (tables > s->tables) s->tables = tables;
+    if (unit > s->unit) s->unit = unit;
+  }
+  return s->unit != 0;
 }
 
 bool fc_band_takes(const fc_kv_view *kv, int N, int omega) {
@@ -205,21 +222,20 @@ FcBandJob *fc_band_plan(const fc_handle *h, const fc_kv_view *kv, int N, int ome
   j->f16 = kv->dtype == FC_F16;
   j->H = kv->num_heads;
   j->d = kv->head_dim;
-  j->off_up = align256(band::down_classes(g) * band::down_image(g));
-  j->off_mid = j->off_up + align256(band::up_classes(g) * band::up_image(g));
-  j->table_bytes = j->off_mid + align256((size_t)g.M / 2 * 16) + align256((size_t)mid_tw_len(g.M / 2) * sizeof(float2));
+  j->table_bytes = table_bytes(g, &j->off_up, &j->off_mid);
   j->y_bytes = (size_t)2 * j->d * g.M * sizeof(float);
-  j->plane_bytes = (size_t)2 * j->d * g.M * sizeof(__half);
   return j;
 }
 void fc_band_release(FcBandJob *j) { delete j; }
 
-// values before the transform, two planes after it, a scale per row
-static size_t unit_bytes(const FcBandJob *j) { return j->y_bytes + 2 * j->plane_bytes + align256((size_t)2 * j->d * 4); }
+// grid values, in fp32 or (in the same place, after the transform) two fp16 terms, and a scale per row
+static size_t unit_bytes(const FcBandJob *j) { return j->y_bytes + align256((size_t)2 * j->d * 4); }
 
-// Fuller launches beat intermediates that stay in L2: 28 layers of 4 heads of 32768 tokens take 2290 / 2056 / 1977 / 1902 us
-// with launch groups of up to 48 / 96 / 192 / 384 MB, of 8192 tokens 569 / 520 / 518 / 492.
-static size_t budget(const fc_handle *h) { return h->group_bytes > ((size_t)1 << 60) ? h->group_bytes : h->group_bytes * 12; }
+// Launch groups.  Fuller launches beat intermediates that stay in L2, up to a point: 28 layers of 4 heads of 32768 tokens take
+// 2086 / 1985 / 2015 / 1951 us with groups of up to 96 / 128 / 192 / 384 MiB, of 8192 tokens 504 / 504 / 504 / 525, 32 layers
+// of 32 heads of 16384 tokens 9202 / 9050 / 9022 / 8855, and the workspace holds two of them.
+constexpr int kGroupFactor = 4;
+static size_t budget(const fc_handle *h) { return h->group_bytes > ((size_t)1 << 60) ? h->group_bytes : h->group_bytes * kGroupFactor; }
 
 size_t fc_band_buffer_bytes(const fc_handle *h, const FcBandSizes *s, int units) {
   const size_t all = s->unit * units, most = budget(h);
@@ -338,14 +354,14 @@ static fc_status launch_up(fc_handle *h, cudaStream_t st, bool early, const band
   return launch(h, st, early, band::k_up<T, NQ>, dim3(P.ranges, nu), band::kUpThreads, sm, maps, grid, g, P);
 }
 
-static fc_status encode_grid(band::GridMaps *m, const void *hi, int rows, int M, size_t plane_bytes) {
+static fc_status encode_grid(band::GridMaps *m, const void *values, int rows, int M) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return FC_ERR_CUDA;
-  const cuuint64_t dims[3] = {(cuuint64_t)M, (cuuint64_t)rows, 2}, str[2] = {(cuuint64_t)M * 2, (cuuint64_t)plane_bytes};
+  const cuuint64_t dims[3] = {(cuuint64_t)M, 2, (cuuint64_t)rows}, str[2] = {(cuuint64_t)M * 2, (cuuint64_t)M * 4};
   const cuuint32_t ones[3] = {1, 1, 1};
   for (int w = 0; w < 2; ++w) {
-    const cuuint32_t box[3] = {w ? 32u : 16u, (cuuint32_t)band::kRows, 1};
-    if (fn(w ? &m->wide : &m->narrow, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void *>(hi), dims, str, box, ones,
+    const cuuint32_t box[3] = {w ? 32u : 16u, 1, (cuuint32_t)band::kRows};
+    if (fn(w ? &m->wide : &m->narrow, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void *>(values), dims, str, box, ones,
            CU_TENSOR_MAP_INTERLEAVE_NONE, w ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return FC_ERR_INTERNAL;
@@ -359,9 +375,8 @@ static fc_status run_group(fc_handle *h, cudaStream_t st, const FcBandJob *j, co
   const Geometry &g = j->g;
   fc_status s;
   float *y = reinterpret_cast<float *>(buf);
-  // the same places for every launch of a sequence, also where the last one has fewer units
-  __half *hi = reinterpret_cast<__half *>(buf + cap * j->y_bytes), *lo = hi + cap * (j->plane_bytes / 2);
-  float *inv = reinterpret_cast<float *>(buf + cap * (j->y_bytes + 2 * j->plane_bytes));
+  // the same place for every launch of a sequence, also where the last one has fewer units
+  float *inv = reinterpret_cast<float *>(buf + cap * j->y_bytes);
   const int tiles = j->d / 64, pairs = (tiles + 1) / 2, n = g.down_steps();
   {
     band::DownParams P = {l.tables, y, h->status_word, j->H, j->d, u0, 0};
@@ -376,7 +391,7 @@ static fc_status run_group(fc_handle *h, cudaStream_t st, const FcBandJob *j, co
   }
   {
     const int Mh = g.M / 2;
-    const band::MidParams P = {y, hi, lo, inv, mid_tables(j, l.tables)};
+    const band::MidParams P = {y, inv, mid_tables(j, l.tables)};
     s = FC_ERR_INTERNAL;
 #define X(M_, A_, B_, C_, D_) if (Mh == M_) s = launch_mid<band::MidShape<A_, B_, C_, D_>>(h, st, early, nu * 2 * j->d, P);
     FC_MID_SHAPES(X)
@@ -400,7 +415,7 @@ static fc_status run_group(fc_handle *h, cudaStream_t st, const FcBandJob *j, co
     P.ranges = ranges;
     P.per = (g.up_steps() + ranges - 1) / ranges;
     band::GridMaps grid;
-    if ((s = encode_grid(&grid, hi, nu * 2 * j->d, g.M, cap * j->plane_bytes)) != FC_OK) return s;
+    if ((s = encode_grid(&grid, y, nu * 2 * j->d, g.M)) != FC_OK) return s;
     return g.nq == 16 ? launch_up<T, 16>(h, st, early, j->maps, grid, g, P, nu)
                       : launch_up<T, 24>(h, st, early, j->maps, grid, g, P, nu);
   }

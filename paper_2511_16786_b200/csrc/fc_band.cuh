@@ -652,8 +652,7 @@ __device__ __forceinline__ unsigned group_max(float v) {
 __device__ __forceinline__ float unit_rounder(unsigned largest) { return __uint_as_float((largest & 0x7f800000u) + 0x06c00000u); }
 
 struct MidParams {
-  const float *y;                            // [row][M]
-  __half *hi, *lo;                           // [row][M]
+  float *y;                                  // [row][M]; in the same place afterwards the two terms, [row][term][M]
   float *inv;                                // [row]: minus what a stored value has to be multiplied with
   MidTables t;
 };
@@ -808,7 +807,8 @@ __global__ void __launch_bounds__(S::NT, S::NT <= 512 ? 512 / S::NT : 1) k_mid(c
   }
   // The first term of a value is a whole number of units, 2^-10 of the power of two below the largest of the 64 values
   // (2 G complex ones' worth) that lie around it, so that k_up's sums of first terms are exact; the second is what is left.
-  __half2 *hi = reinterpret_cast<__half2 *>(P.hi) + row * Mh, *lo = reinterpret_cast<__half2 *>(P.lo) + row * Mh;
+  // They go where the rows came from, which this block alone has read, before it began to compute.
+  __half2 *hi = reinterpret_cast<__half2 *>(P.y) + row * 2 * Mh, *lo = hi + Mh;
 #pragma unroll
   for (int u = 0; u < 16 / R; ++u)
 #pragma unroll
@@ -820,14 +820,14 @@ __global__ void __launch_bounds__(S::NT, S::NT <= 512 ? 512 / S::NT : 1) k_mid(c
                                    unit_rounder(group_max<G>(fmaxf(fabsf(re.y), fabsf(im.y)))));
       const float2 hre = sub2(add2(re, c), c), him = sub2(add2(im, c), c), lre = sub2(re, hre), lim = sub2(im, him);
       hi[n] = __floats2half2_rn(hre.x, him.x);
-      hi[Mh + n] = __floats2half2_rn(hre.y, him.y);
+      hi[2 * Mh + n] = __floats2half2_rn(hre.y, him.y);
       lo[n] = __floats2half2_rn(lre.x, lim.x);
-      lo[Mh + n] = __floats2half2_rn(lre.y, lim.y);
+      lo[2 * Mh + n] = __floats2half2_rn(lre.y, lim.y);
     }
 }
 
 // ---------------------------------------------------------------------------------------------------- k_up
-// The two terms of a launch's grid values, [term][row][M]: boxes of 32 or 16 values of 128 rows of one term.
+// The two terms of a launch's grid values, [row][term][M]: boxes of 32 or 16 values of 128 rows of one term.
 struct GridMaps {
   CUtensorMap wide, narrow;
 };
@@ -941,8 +941,8 @@ __global__ void __launch_bounds__(kUpThreads, 1) k_up(const __grid_constant__ Ma
         unsigned char *dst = ys + (size_t)(term == 0 ? s : kHi + s) * ybytes;
         for (int rn = 0; rn < 2; ++rn, dst += run) {           // a run: a box of 32 values and, with 24 quads, one of 16
           const int x = rn == 0 ? 2 * q0 : g.M - 2 * (q0 + NQ);
-          load_box(dst, &grid.wide, x, r0, term, &sh.yfull[term][s]);
-          if (NQ > 16) load_box(dst + kRows * 64, &grid.narrow, x + 32, r0, term, &sh.yfull[term][s]);
+          load_box(dst, &grid.wide, x, term, r0, &sh.yfull[term][s]);
+          if (NQ > 16) load_box(dst + kRows * 64, &grid.narrow, x + 32, term, r0, &sh.yfull[term][s]);
         }
         ++ny[term];
       };

@@ -202,3 +202,15 @@ def test_band_single_scores_are_as_exact_as_fp32_passes(fc, N, d, gamma, dtype):
         rel = (s[h].double().numpy() - o) / o
         assert math.sqrt((rel ** 2).mean()) <= 6.2e-7
         assert abs(rel).max() <= 1e-5
+
+
+@pytest.mark.parametrize("L,H,lens,most", [(28, 4, [32768], 300e6), (28, 4, [8192], 300e6), (32, 32, [16384], 300e6), (1, 4, [2048], 20e6)])
+def test_band_workspace_is_bounded(fc, L, H, lens, most):
+    # two groups of at most four times 32 MiB and, at powers of two, a few hundred KB of tables; all intermediates where
+    # those are less: 2 streams x 4 heads x 256 channels x 1024 values of 4 bytes = 8.4 MB for one layer of 2048 tokens
+    h = fc.fc_create(0, max(lens))
+    try:
+        k = torch.empty((lens[0], H, 128), dtype=torch.bfloat16, device="cuda")
+        assert 0 < fc.fc_score_layers_workspace_bytes(h, k, k, [0, lens[0]], L) <= most
+    finally:
+        fc.fc_destroy(h)
