@@ -94,8 +94,8 @@ typedef struct {
  * are limited to 65536).  Allocates the twiddle table (8 bytes * 4 * next power of two of
  * max_seqlen, at least 64), room for eight filter tables (16 bytes * the power of two from 2*max_seqlen-1 up each, at
  * least 16 KiB and at most 2 MiB; lengths that are not a power of two reuse theirs from layer to layer and call to call,
- * a batch of more than eight unlike ones builds the rest in the workspace on every call), room for the tables of four 16-bit
- * sequences scored on a coarser grid (640 or 1280 KiB each; none up to 512 tokens) and a status word.  Returns FC_ERR_CUDA if the device cannot be
+ * a batch of more than eight unlike ones builds the rest in the workspace on every call), 2.5 or 5 MiB (from 513 and from
+ * 1025 tokens on) for the tables of up to eight 16-bit sequences scored on a coarser grid, kept in the same way, and a status word.  Returns FC_ERR_CUDA if the device cannot be
  * used, FC_ERR_UNSUPPORTED if max_seqlen is out of range. */
 fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen);
 void fc_destroy(fc_handle *h);

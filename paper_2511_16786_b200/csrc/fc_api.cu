@@ -202,16 +202,16 @@ extern "C" fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen) 
     h->tab_slot_len = m;
     for (int i = 0; i < FC_TAB_SLOTS; ++i) h->tab_key[i] = 0;
     h->tab_next = 0;
-    for (int i = 0; i < FC_BAND_SLOTS; ++i) h->band_key[i] = 0;
-    h->band_next = 0;
-    // kept-band tables: 2 or 4 tokens per grid point at any length, other ratios up to about 1000 or 1700 tokens
-    h->band_slot_bytes = max_seqlen <= 512 ? 0 : (size_t)(max_seqlen <= 1024 ? 640 : 1280) << 10;
+    for (int i = 0; i < FC_BAND_KEPT; ++i) h->band_kept[i] = {0, 0, 0, 0};
+    h->band_clock = 0;
+    // kept-band tables: 0.3 to 0.6 MB at powers of two, about 0.9 KB per token at other lengths
+    h->band_pool_bytes = max_seqlen <= 512 ? 0 : (size_t)(max_seqlen <= 1024 ? 2560 : 5120) << 10;
     const size_t tab_bytes = (size_t)FC_TAB_SLOTS * h->tab_slot_len * sizeof(float4);
-    if (cudaMalloc(&h->tab_cache, tab_bytes + FC_BAND_SLOTS * h->band_slot_bytes) != cudaSuccess) {
+    if (cudaMalloc(&h->tab_cache, tab_bytes + h->band_pool_bytes) != cudaSuccess) {
       fc_destroy(h);
       return FC_ERR_CUDA;
     }
-    h->band_cache = reinterpret_cast<char *>(h->tab_cache) + tab_bytes;
+    h->band_pool = reinterpret_cast<char *>(h->tab_cache) + tab_bytes;
   }
   k_fill_master<<<(h->master_len + 255) / 256, 256>>>(h->master, h->master_len);
   if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {

@@ -270,8 +270,46 @@ int fc_band_units(const fc_handle *h, const FcBandJob *j, int units, size_t buf_
   return best;
 }
 
-size_t fc_band_table_bytes(const FcBandJob *j) { return j->table_bytes; }
 long long fc_band_table_key(const FcBandJob *j) { return (long long)j->g.N + ((long long)(j->g.omega + 1) << 20) + (j->f16 ? 1ll << 40 : 0); }
+
+int fc_band_kept(fc_handle *h, const FcBandJob *j) {
+  for (int i = 0; i < FC_BAND_KEPT; ++i)
+    if (h->band_kept[i].key == fc_band_table_key(j)) {
+      h->band_kept[i].used = ++h->band_clock;
+      return i;
+    }
+  return -1;
+}
+
+int fc_band_place(fc_handle *h, const FcBandJob *j, const bool (&used)[FC_BAND_KEPT]) {
+  auto &kept = h->band_kept;
+  const size_t bytes = j->table_bytes;
+  size_t held = 0;
+  for (int i = 0; i < FC_BAND_KEPT; ++i)
+    if (used[i]) held += kept[i].bytes;
+  if (held + bytes > h->band_pool_bytes) return -1;
+  for (;;) {
+    int free_entry = -1, oldest = -1;
+    for (int i = 0; i < FC_BAND_KEPT; ++i) {
+      if (kept[i].key == 0 && !used[i]) free_entry = i;
+      else if (!used[i] && (oldest < 0 || (int)(kept[i].used - kept[oldest].used) < 0)) oldest = i;
+    }
+    // behind one of the tables (or first) and in nobody's way
+    for (int c = -1; free_entry >= 0 && c < FC_BAND_KEPT; ++c) {
+      if (c >= 0 && kept[c].key == 0 && !used[c]) continue;
+      const size_t off = c < 0 ? 0 : kept[c].off + kept[c].bytes;
+      bool fits = off + bytes <= h->band_pool_bytes;
+      for (int i = 0; i < FC_BAND_KEPT && fits; ++i)
+        if (kept[i].key != 0 || used[i]) fits = off + bytes <= kept[i].off || off >= kept[i].off + kept[i].bytes;
+      if (fits) {
+        kept[free_entry] = {0, off, bytes, ++h->band_clock};
+        return free_entry;
+      }
+    }
+    if (oldest < 0) return -1;
+    kept[oldest].key = 0;
+  }
+}
 
 static band::MidTables mid_tables(const FcBandJob *j, const char *tables) {
   const int Mh = j->g.M / 2;

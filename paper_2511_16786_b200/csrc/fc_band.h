@@ -23,8 +23,11 @@ int fc_band_units(const fc_handle *h, const FcBandJob *j, int units, size_t buf_
 int fc_band_ranges(const fc_handle *h, const FcBandJob *j, int units);      // blocks a unit's rows are spread over where a launch has so many units
 // The sequence's tables: their size, what they depend on (the dtype, the length and the cutoff), and the launch that builds
 // them on `st`.
-size_t fc_band_table_bytes(const FcBandJob *j);
 long long fc_band_table_key(const FcBandJob *j);
+// Tables the handle keeps: the place of the sequence's (-1: none), and a place for new ones, for which the longest unused
+// that are not in `used` make room (-1: there is none).  The caller sets the place's key once the tables are on their way.
+int fc_band_kept(fc_handle *h, const FcBandJob *j);
+int fc_band_place(fc_handle *h, const FcBandJob *j, const bool (&used)[FC_BAND_KEPT]);
 fc_status fc_band_tables(fc_handle *h, cudaStream_t st, const FcBandJob *j, char *tables);
 struct FcBandLaunch {
   const void *const *k, *const *v;     // first token of the sequence, layer by layer

@@ -15,7 +15,7 @@
 #define FC_MAX_STAGES 4
 #define FC_MAX_AUX 4     // internal streams a handle may use
 #define FC_TAB_SLOTS 8   // filter tables a handle keeps (one per sequence length, cutoff and form)
-#define FC_BAND_SLOTS 4  // and tables of sequences scored in the kept band
+#define FC_BAND_KEPT 8   // and, as long as there is room, tables of sequences scored in the kept band
 #define FC_LAYER_CHUNK 32  // layers one launch of the scoring kernels can span (kernel-argument table)
 
 // Bits of the device status word.
@@ -78,11 +78,11 @@ struct fc_handle {
   float4 *tab_cache;
   int tab_slot_len, tab_next;
   long long tab_key[FC_TAB_SLOTS];
-  // the same for sequences scored in the kept band whose tables fit a slot (in the allocation of tab_cache)
-  char *band_cache;
-  size_t band_slot_bytes;
-  int band_next;
-  long long band_key[FC_BAND_SLOTS];
+  // the same for sequences scored in the kept band, side by side in the end of tab_cache's allocation (key 0: no table)
+  char *band_pool;
+  size_t band_pool_bytes;
+  unsigned band_clock;
+  struct { long long key; size_t off, bytes; unsigned used; } band_kept[FC_BAND_KEPT];
   // fc_compress_host (created on its first call): the stream the host-to-device copies run on, one
   // event per layer (that layer's copies have landed), and the point of the previous job after
   // which the staged inputs of its arena may be overwritten

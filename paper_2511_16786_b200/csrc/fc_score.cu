@@ -1320,11 +1320,11 @@ struct Jobs : std::vector<FcBandJob *> {
   ~Jobs() { for (FcBandJob *j : *this) fc_band_release(j); }
 };
 
-// Tables of the sequences scored in the kept band, as prepare_tables does it: the handle keeps the last few that fit a slot,
-// the others, and all while the stream is being captured, are built into the workspace.
+// Tables of the sequences scored in the kept band, as prepare_tables does it: the handle keeps those of the last calls that it
+// has room for, the others, and all while the stream is being captured, are built into the workspace.
 fc_status band_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const Jobs &band, char *spare, const char **tabs) {
   bool cached = true, any = false, flushed = false;
-  bool used[FC_BAND_SLOTS] = {};
+  bool used[FC_BAND_KEPT] = {};
   for (int b = 0; b < kv->batch; ++b) {
     if (!band[b]) continue;
     if (!any) {
@@ -1333,8 +1333,8 @@ fc_status band_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const
       if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { cudaGetLastError(); cap = cudaStreamCaptureStatusActive; }
       cached = cap == cudaStreamCaptureStatusNone;
     }
-    for (int i = 0; cached && i < FC_BAND_SLOTS; ++i)
-      if (h->band_key[i] == fc_band_table_key(band[b])) { tabs[b] = h->band_cache + i * h->band_slot_bytes; used[i] = true; }
+    const int i = cached ? fc_band_kept(h, band[b]) : -1;
+    if (i >= 0) { tabs[b] = h->band_pool + h->band_kept[i].off; used[i] = true; }
   }
   for (int b = 0; b < kv->batch; ++b) {
     if (!band[b] || tabs[b]) continue;
@@ -1345,24 +1345,18 @@ fc_status band_tables(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const
     // the tables' place may still be in use on the internal streams
     if (!flushed && (s = fc_flush_pending(h, st)) != FC_OK) return s;
     flushed = true;
-    int slot = -1;
-    for (int i = 0; cached && fc_band_table_bytes(band[b]) <= h->band_slot_bytes && i < FC_BAND_SLOTS && slot < 0; ++i) {
-      const int c = (h->band_next + i) % FC_BAND_SLOTS;
-      if (!used[c]) slot = c;
-    }
+    const int place = cached ? fc_band_place(h, band[b], used) : -1;
     char *dst = spare;
-    if (slot >= 0) {
-      h->band_next = (slot + 1) % FC_BAND_SLOTS;
-      h->band_key[slot] = 0;                                   // not valid until its launch is in the stream
-      used[slot] = true;
-      dst = h->band_cache + slot * h->band_slot_bytes;
+    if (place >= 0) {
+      used[place] = true;
+      dst = h->band_pool + h->band_kept[place].off;
     } else {
       FcBandSizes bs;
       fc_band_bounds(kv, kv->cu_seqlens[b + 1] - kv->cu_seqlens[b], &bs);
       spare += bs.tables;
     }
     if ((s = fc_band_tables(h, st, band[b], dst)) != FC_OK) return s;
-    if (slot >= 0) h->band_key[slot] = fc_band_table_key(band[b]);
+    if (place >= 0) h->band_kept[place].key = fc_band_table_key(band[b]);      // valid from here on in stream order
     tabs[b] = dst;
   }
   return FC_OK;

@@ -214,3 +214,71 @@ def test_band_workspace_is_bounded(fc, L, H, lens, most):
         assert 0 < fc.fc_score_layers_workspace_bytes(h, k, k, [0, lens[0]], L) <= most
     finally:
         fc.fc_destroy(h)
+
+
+def test_band_tables_are_kept_evicted_and_rebuilt(fc):
+    # one handle over calls whose tables fill what it keeps, displace one another, do not fit at all or are more than it counts:
+    # the same bits as from a handle that has seen nothing else; one sequence (the caller's stream) and several (internal
+    # streams, deferred or not) by turns on one workspace
+    H, d = 2, 64
+    calls = [[517, 1999, 4096, 2311], [1500], [1500, 1100, 2500], [517, 1999, 4096, 2311], [3000, 2700, 4095], [2048], [2311],
+             [600, 700, 800, 900, 1000, 1100, 1200, 1300, 1400, 1700], [1100, 300, 1100], [4096, 2048], [4095], [1999, 1500]]
+    data, ref = {}, {}
+    for lens in calls:
+        cu = [0] + [int(x) for x in np.cumsum(lens)]
+        k, v = (x.cuda() for x in _kv(cu[-1], H, d, torch.float16, sum(lens)))
+        data[tuple(lens)] = (cu, k, v)
+        ref[tuple(lens)] = _score(fc, k, v, cu, 0.2)
+    h = fc.fc_create(0, 4096)
+    try:
+        ws = torch.empty(max(fc.fc_score_workspace_bytes(h, k, v, cu) for cu, k, v in data.values()), dtype=torch.uint8, device="cuda")
+        for rnd in range(4):
+            fc.fc_set_score_overlap(h, rnd % 2 == 1)
+            got = []
+            for i, lens in enumerate(calls if rnd < 2 else calls[::-1]):
+                cu, k, v = data[tuple(lens)]
+                s = torch.full((H, cu[-1]), -1.0, dtype=torch.float32, device="cuda")
+                e = torch.full((len(lens), 4), -1.0, dtype=torch.float64, device="cuda")
+                fc.fc_score_layer(h, k, v, cu, 0.2, s, e, ws)
+                got.append((lens, s, e))
+            assert fc.fc_last_device_status(h) == 0
+            for lens, s, e in got:
+                assert torch.equal(s.cpu(), ref[tuple(lens)][0]) and torch.equal(e.cpu(), ref[tuple(lens)][1]), lens
+    finally:
+        fc.fc_destroy(h)
+
+
+def test_band_more_layers_than_one_launch_spans(fc):
+    # 35 layers in one call against one call each, on a length whose work fits the caller's stream chunk by chunk and one whose does not
+    H, d, L = 1, 64, 35
+    for lens in ([640], [2500, 1030]):
+        cu = [0] + [int(x) for x in np.cumsum(lens)]
+        K, V = zip(*(_kv(cu[-1], H, d, torch.bfloat16, 70 + l) for l in range(L)))
+        K, V = [k.cuda() for k in K], [v.cuda() for v in V]
+        h = fc.fc_create(0, max(lens))
+        try:
+            ws = torch.empty(fc.fc_score_layers_workspace_bytes(h, K[0], V[0], cu, L), dtype=torch.uint8, device="cuda")
+            s = torch.empty((L, H, cu[-1]), dtype=torch.float32, device="cuda")
+            e = torch.empty((L, len(lens), 4), dtype=torch.float64, device="cuda")
+            fc.fc_score_layers(h, K, V, cu, 0.2, s, e, ws)
+            assert fc.fc_last_device_status(h) == 0
+            for l in range(L):
+                one_s, one_e = _score(fc, K[l], V[l], cu, 0.2)
+                assert torch.equal(s[l].cpu(), one_s) and torch.equal(e[l].cpu(), one_e)
+        finally:
+            fc.fc_destroy(h)
+        _check(K[34].cpu(), V[34].cpu(), cu, 0.2, s[34].cpu(), e[34].cpu())
+
+
+# wide heads: an odd number of 64-channel halves (K and V share a tile), and the widest that the form takes
+@pytest.mark.parametrize("N,H,d,dtype", [(1100, 2, 320, torch.bfloat16), (2048, 1, 448, torch.float16), (2311, 1, 512, torch.bfloat16),
+                                         (1500, 1, 576, torch.bfloat16)])
+def test_band_wide_heads(fc, N, H, d, dtype):
+    k, v = _kv(N, H, d, dtype, N + d)
+    s, e = _score(fc, k.cuda(), v.cuda(), [0, N], 0.2, repeat=2)
+    if d <= 512:
+        _check(k, v, [0, N], 0.2, s, e)
+    else:                                     # on the passes: their own tolerance
+        for h in range(H):
+            o, _ = O.score_head(k[:, h].double().numpy(), v[:, h].double().numpy(), 0.2, "fft")
+            assert np.allclose(s[h].double().numpy(), o, rtol=1e-3, atol=1e-9)
