@@ -1579,16 +1579,19 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
   bool fork = true, direct_only = true, any_fast = false, any_small = false, any_passes = false, any_band = false;
   std::vector<PassPlan> plans(B);
   std::vector<const float4 *> tabs(B, nullptr);
-  Jobs band(B, nullptr);
-  std::vector<const char *> band_tabs(B, nullptr);
+  Jobs band;                                   // of 16-bit calls only
+  std::vector<const char *> band_tabs;
+  if (kv->dtype != FC_F32) {
+    band.resize(B, nullptr);
+    band_tabs.resize(B, nullptr);
+  }
   for (int b = 0; b < B; ++b) {
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0) continue;
     if (!h->generic_only) plans[b] = plan_passes(N, kv->head_dim);
     // what fc_set_score_overlap promises goes by the length, not by the form that scores it
     if (!plans[b].ok || (plans[b].pad && !plans[b].small)) direct_only = false;
-    band[b] = fc_band_plan(h, kv, N, cutoff_index(gamma, N));
-    if (band[b]) {
+    if (kv->dtype != FC_F32 && (band[b] = fc_band_plan(h, kv, N, cutoff_index(gamma, N))) != nullptr) {
       any_band = true;
       plans[b].ok = true;
       plans[b].small = plans[b].pad = false;
@@ -1598,8 +1601,8 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
     any_passes = any_passes || (plans[b].ok && !plans[b].small);
   }
   if (any_fast && (s = prepare_tables(h, st, kv, gamma, false, reinterpret_cast<float4 *>(wsb + L.off_tab),
-                                      reinterpret_cast<float2 *>(wsb + L.off_buf), tabs.data(), band.data())) != FC_OK) return s;
-  if ((s = band_tables(h, st, kv, band, wsb + L.off_band, band_tabs.data())) != FC_OK) return s;
+                                      reinterpret_cast<float2 *>(wsb + L.off_buf), tabs.data(), any_band ? band.data() : nullptr)) != FC_OK) return s;
+  if (any_band && (s = band_tables(h, st, kv, band, wsb + L.off_band, band_tabs.data())) != FC_OK) return s;
   // A single sequence with little work (128-token steps per SM; from about two on, two streams are worth their fork) stays on
   // the caller's stream, without fork and join: one layer of 4 heads of 8192 tokens 81 -> 61 us by the host's clock.  Several
   // sequences run beside each other on the internal streams, and beside the short ones on the caller's: one layer of 4 heads
@@ -1667,7 +1670,7 @@ fc_status score_call(fc_handle *h, cudaStream_t st, const fc_kv_view *kv, const 
         lp.v[l] = static_cast<const T *>(layers[l0 + l].v) + (long long)start * kv->stride_token;
         lp.scores[l] = const_cast<float *>(layers[l0 + l].scores) + start;
       }
-      s = band[b] ? score_band(h, st, on_caller, kv, band[b], nl, lp, en, 4ll * B, L, wsb, band_tabs[b])
+      s = any_band && band[b] ? score_band(h, st, on_caller, kv, band[b], nl, lp, en, 4ll * B, L, wsb, band_tabs[b])
                   : score_sequence<T>(h, st, kv, plans[b], nl, lp, gamma, en, 4ll * B, L, wsb, tabs[b]);
       if (s != FC_OK) return s;
     }
