@@ -129,10 +129,9 @@ def step_accounting(binding, handle, cfg):
         n2 = N / n1
         cols = H * d * L                       # complex columns (K + jV) of this sequence
         step_flops += cols * N * (10.0 * math.log2(N) + 12.0)
-        M, omega = 128, int(cfg.gamma * N)
-        while 4 * M < N or 5 * omega > 4 * M:
-            M *= 2
-        if s == 2 and N > 512 and N != 1024 and 2 * M <= N and M <= 16384:
+        scored = binding.fc_scoring_form(handle, N, cfg.torch_dtype, d, cfg.gamma)
+        if scored["form"] == "band":
+            M = scored["points"]
             acc["pass2"]["flops"] += cols * M * (10.0 * math.log2(M / 2) + 24.0)
             acc["pass3"]["bytes"] += N * H * L * 2.0 * d * s           # K and V rows again
         else:

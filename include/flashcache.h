@@ -200,9 +200,15 @@ fc_status fc_set_group_bytes(fc_handle *h, size_t bytes);
 /* How a sequence of length seqlen could be transformed at cutoff ratio gamma (diagnostic): out = { form, transform
  * length, first factor N1, second factor N2 }.  Form 0, powers of two: the transform itself, as the three passes run it.
  * Forms 1 and 2, other lengths: the shortest chirp convolutions in the full-length or band form (see fc_set_chirp_band),
- * kept for callers that compare with them; the library scores such lengths by one padded convolution of at least
- * 2N - 1 points instead. */
+ * kept for callers that compare with them.  What the scoring calls run depends on the dtype as well: fc_scoring_form. */
 fc_status fc_describe_plan(const fc_handle *h, int32_t seqlen, double gamma, int32_t out[4]);
+
+/* How the scoring calls treat a sequence of seqlen tokens (diagnostic): out = { form, points }.  FC_FORM_GENERIC: column
+ * transforms of `points` through memory.  FC_FORM_SHORT: one kernel, `points` per column.  FC_FORM_DIRECT: three passes
+ * over `points` = seqlen.  FC_FORM_PADDED: three passes over a convolution of `points`.  FC_FORM_BAND: 16-bit rows, on a
+ * grid of `points` (seqlen/4 .. seqlen/2) between two banded matrix products. */
+typedef enum { FC_FORM_GENERIC = 0, FC_FORM_SHORT = 1, FC_FORM_DIRECT = 2, FC_FORM_PADDED = 3, FC_FORM_BAND = 4 } fc_form;
+fc_status fc_scoring_form(const fc_handle *h, int32_t seqlen, fc_dtype dtype, int32_t head_dim, double gamma, int32_t out[2]);
 
 /* Workspace sizes (bytes) the next two calls need for this view.  0 on bad input. */
 size_t fc_score_workspace_bytes(const fc_handle *h, const fc_kv_view *kv);

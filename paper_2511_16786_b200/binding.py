@@ -24,7 +24,7 @@ _DTYPE = {torch.float32: FC_F32, torch.float16: FC_F16, torch.bfloat16: FC_BF16}
 
 EXPORTS = (
     "fc_create", "fc_destroy", "fc_status_string", "fc_last_device_status", "fc_launch_count", "fc_selftest_bounded_wait", "fc_measure_fp32_peak", "fc_proto_dft16_stage",
-    "fc_set_group_bytes", "fc_set_chirp_band", "fc_set_internal_streams", "fc_set_l2_persist", "fc_reset_ordering", "fc_set_score_overlap", "fc_set_select_overlap", "fc_profile_begin", "fc_profile_stride", "fc_profile_end", "fc_describe_plan",
+    "fc_set_group_bytes", "fc_set_chirp_band", "fc_set_internal_streams", "fc_set_l2_persist", "fc_reset_ordering", "fc_set_score_overlap", "fc_set_select_overlap", "fc_profile_begin", "fc_profile_stride", "fc_profile_end", "fc_describe_plan", "fc_scoring_form",
     "fc_score_workspace_bytes", "fc_select_workspace_bytes",
     "fc_score_layer", "fc_allocate_budgets", "fc_select_compact", "fc_select_compact_ex",
     "fc_select_compact_layers", "fc_layer_capacity_rows", "fc_score_layers", "fc_score_layers_workspace_bytes",
@@ -132,6 +132,8 @@ def _load() -> ctypes.CDLL:
     lib.fc_profile_end.restype = c_int
     lib.fc_describe_plan.argtypes = [c_void_p, c_int32, c_double, POINTER(c_int32)]
     lib.fc_describe_plan.restype = c_int
+    lib.fc_scoring_form.argtypes = [c_void_p, c_int32, c_int32, c_int32, c_double, POINTER(c_int32)]
+    lib.fc_scoring_form.restype = c_int
     lib.fc_score_workspace_bytes.argtypes = [c_void_p, POINTER(fc_kv_view)]
     lib.fc_score_workspace_bytes.restype = c_size_t
     lib.fc_select_workspace_bytes.argtypes = [c_void_p, POINTER(fc_kv_view)]
@@ -314,6 +316,12 @@ def fc_describe_plan(handle, seqlen: int, gamma: float) -> dict:
     out = (c_int32 * 4)()
     _check(_lib.fc_describe_plan(handle, int(seqlen), float(gamma), out), "fc_describe_plan")
     return dict(bluestein=bool(out[0]), band_form=out[0] == 2, nfft=int(out[1]), n1=int(out[2]), n2=int(out[3]))
+
+
+def fc_scoring_form(handle, seqlen: int, dtype, head_dim: int, gamma: float) -> dict:
+    out = (c_int32 * 2)()
+    _check(_lib.fc_scoring_form(handle, int(seqlen), _DTYPE[dtype], int(head_dim), float(gamma), out), "fc_scoring_form")
+    return dict(form=("generic", "short", "direct", "padded", "band")[out[0]], points=int(out[1]))
 
 
 def fc_score_workspace_bytes(handle, k, v, cu_seqlens) -> int:

@@ -208,9 +208,9 @@ bool fc_band_bounds(const fc_kv_view *kv, int N, FcBandSizes *s) {
   return s->unit != 0;
 }
 
-bool fc_band_takes(const fc_kv_view *kv, int N, int omega) {
+int fc_band_grid(const fc_kv_view *kv, int N, int omega) {
   Geometry g;
-  return eligible(kv, N) && make_geometry(N, omega, &g);
+  return eligible(kv, N) && make_geometry(N, omega, &g) ? g.M : 0;
 }
 
 FcBandJob *fc_band_plan(const fc_handle *h, const fc_kv_view *kv, int N, int omega) {

@@ -11,8 +11,8 @@ bool fc_band_bounds(const fc_kv_view *kv, int N, FcBandSizes *s);
 // Intermediates of one launch group, one copy per internal stream, of a call with so many units.
 size_t fc_band_buffer_bytes(const fc_handle *h, const FcBandSizes *s, int units);
 
-// Whether a cutoff takes this form.
-bool fc_band_takes(const fc_kv_view *kv, int N, int omega);
+// The grid's points where a cutoff takes this form, 0 where it does not.
+int fc_band_grid(const fc_kv_view *kv, int N, int omega);
 
 // One sequence of a chunk of layers.
 struct FcBandJob;

@@ -903,7 +903,7 @@ void claim_persisting_l2(fc_handle *h, const fc_kv_view *kv, int num_layers, dou
     const int N = kv->cu_seqlens[b + 1] - kv->cu_seqlens[b];
     if (N == 0) continue;
     const PassPlan p = plan_passes(N, kv->head_dim);
-    if (!p.ok || p.pad || p.small || fc_band_takes(kv, N, cutoff_index(gamma, N))) continue;
+    if (!p.ok || p.pad || p.small || fc_band_grid(kv, N, cutoff_index(gamma, N)) != 0) continue;
     claim = window_fits(h, p, plan_groups(h, p, nl * kv->num_heads, kv->num_heads, kv->head_dim));
   }
   if (claim == (h->persist_on != 0)) return;
@@ -1879,6 +1879,25 @@ extern "C" fc_status fc_describe_plan(const fc_handle *h, int32_t seqlen, double
       out[3] = c.N2;
     }
   }
+  return FC_OK;
+}
+
+extern "C" fc_status fc_scoring_form(const fc_handle *h, int32_t seqlen, fc_dtype dtype, int32_t head_dim, double gamma, int32_t out[2]) {
+  if (!h || !out || seqlen < 1 || !(gamma >= 0.0 && gamma <= 1.0)) return FC_ERR_INVALID_ARG;
+  fc_kv_view kv = {};
+  const int32_t cu[2] = {0, seqlen};
+  kv.dtype = dtype;
+  kv.num_heads = 1;
+  kv.batch = 1;
+  kv.head_dim = head_dim;
+  kv.stride_token = kv.stride_head = head_dim;
+  kv.cu_seqlens = cu;
+  const fc_status s = validate_view(h, &kv, false);
+  if (s != FC_OK) return s;
+  const PassPlan p = h->generic_only ? PassPlan{} : plan_passes(seqlen, head_dim);
+  const int grid = h->generic_only ? 0 : fc_band_grid(&kv, seqlen, cutoff_index(gamma, seqlen));
+  out[0] = grid ? FC_FORM_BAND : !p.ok ? FC_FORM_GENERIC : p.small ? FC_FORM_SHORT : p.pad ? FC_FORM_PADDED : FC_FORM_DIRECT;
+  out[1] = grid ? grid : p.ok ? p.M : plan_sequence(seqlen).Nfft;
   return FC_OK;
 }
 

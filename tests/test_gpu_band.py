@@ -1,5 +1,5 @@
-"""Scoring in the kept band (16-bit inputs, cutoffs of up to about two fifths of the bins) at the edges of its windows, grids
-and dispatch rule, against the fp64 oracle."""
+"""Scoring in the kept band (16-bit inputs whose kept band a grid of a quarter to half of the tokens holds) at the edges of its
+windows, grids and dispatch rule, against the fp64 oracle."""
 import math
 
 import numpy as np
@@ -81,11 +81,34 @@ def _check(k, v, cu, gamma, scores, energy):
     (4097, 2, 128, 0.2, torch.bfloat16), (5119, 3, 128, 0.1, torch.float16), (8192, 2, 64, 0.2, torch.bfloat16),
     (10164, 2, 128, 0.2, torch.bfloat16), (16384, 1, 128, 0.3, torch.float16), (32768, 1, 128, 0.3, torch.bfloat16),
     (53602, 1, 128, 0.2, torch.float16), (65535, 1, 64, 0.2, torch.bfloat16), (65536, 1, 128, 0.2, torch.bfloat16),
-    (65536, 1, 64, 0.45, torch.bfloat16)])
+    (65536, 1, 64, 0.45, torch.bfloat16), (2200, 2, 128, 0.3, torch.bfloat16), (4200, 1, 128, 0.26, torch.float16)])
 def test_band_scores(fc, N, H, d, gamma, dtype):
     k, v = _kv(N, H, d, dtype, N)
     s, e = _score(fc, k.cuda(), v.cuda(), [0, N], gamma, repeat=3)
     _check(k, v, [0, N], gamma, s, e)
+
+
+def test_band_is_taken_where_the_rule_says(fc):
+    # 16-bit rows of 513 .. 65536 tokens, not 1024, heads of up to 512 channels, where a grid of a power of two points M holds
+    # the band (256 <= M <= 16384, N/4 <= M <= N/2, omega <= 0.8 M) and 128 tokens with the kernel's ends lie within 24 aligned quads
+    # of it, which keeps N just above 2 M with the widest kernels out (1100 tokens, 0.37)
+    h = fc.fc_create(0, 131072)
+    try:
+        form = lambda N, gamma, dtype=torch.bfloat16, d=128: tuple(fc.fc_scoring_form(h, N, dtype, d, gamma).values())
+        for N, gamma, want in [
+                (512, 0.2, ("short", 512)), (513, 0.2, ("band", 256)), (599, 0.3, ("band", 256)), (767, 0.1, ("band", 256)),
+                (1023, 0.3, ("padded", 2048)), (1024, 0.2, ("short", 1024)), (1025, 0.2, ("band", 512)), (1100, 0.37, ("padded", 2560)),
+                (1281, 0.0, ("band", 512)), (1100, 0.3, ("band", 512)), (2047, 0.2, ("band", 512)), (2048, 0.3, ("band", 1024)), (2048, 0.39, ("band", 1024)),
+                (2500, 0.39, ("padded", 5120)), (4096, 0.2, ("band", 1024)), (4097, 0.2, ("band", 2048)), (4200, 0.26, ("band", 2048)),
+                (16384, 0.3, ("band", 8192)), (32768, 0.2, ("band", 8192)), (32768, 0.45, ("direct", 32768)), (32769, 0.2, ("band", 16384)),
+                (65535, 0.2, ("band", 16384)), (65536, 0.2, ("band", 16384)), (65536, 0.45, ("direct", 65536))]:
+            assert form(N, gamma) == want, (N, gamma)
+            assert form(N, gamma, torch.float16) == want, (N, gamma)
+            assert form(N, gamma, torch.float32)[0] != "band"
+        assert form(2048, 0.2, d=512)[0] == "band" and form(2048, 0.2, d=576)[0] == "direct"
+        assert form(131072, 0.2)[0] == "generic"
+    finally:
+        fc.fc_destroy(h)
 
 
 def test_band_ragged_batch_strided_views_and_neighbours(fc):
