@@ -80,6 +80,8 @@ bool make_geometry(int N, int omega, Geometry *g) {
   g->beta = kKernels[k].beta;
   g->fc = kKernels[k].fc;
   g->fmax = kKernels[k].fmax;
+  g->up_ratio = (double)M / N;
+  g->down_ratio = (double)N / M;
   for (int i = 0; i < band::kCheb; ++i) g->cheb[i] = responses()[k][i];
   g->same = N == 2 * M || N == 4 * M;                      // 128 tokens are whole quads of the grid
   // The longest windows, over all steps or, where most are alike, over the first and last few and one between.
@@ -320,7 +322,7 @@ static band::MidTables mid_tables(const FcBandJob *j, const char *tables) {
 
 fc_status fc_band_tables(fc_handle *h, cudaStream_t st, const FcBandJob *j, char *tables) {
   const Geometry &g = j->g;
-  const int Mh = g.M / 2, down = band::down_classes(g) * g.ks, up = band::up_classes(g) * g.nq * 2;
+  const int Mh = g.M / 2, down = band::down_classes(g) * band::down_table_blocks(g), up = band::up_classes(g) * band::up_table_blocks(g);
   band::MidRadices r = {};
 #define X(M_, A_, B_, C_, D_) \
   if (Mh == M_) r = band::MidRadices{{A_, C_ > 1 ? B_ : 1, D_ > 1 ? C_ : 1}, D_ > 1 ? D_ : C_ > 1 ? C_ : B_};

@@ -49,6 +49,7 @@ struct Geometry {
   double beta, fc;                           // phi(u) = 2 fc sinc(2 fc u) exp(beta (sqrt(1 - (2u/W)^2) - 1))
   double cheb[kCheb];                        // H(f) = sum c_i T_i(2 (f/fmax)^2 - 1), f in cycles per grid point
   double fmax;
+  double up_ratio, down_ratio;               // M/N and N/M
   __host__ __device__ int down_steps() const { return M / kJ; }
   __host__ __device__ int up_steps() const { return (N + kRows - 1) / kRows; }
 };
@@ -100,8 +101,8 @@ __host__ __device__ inline size_t up_image(const Geometry &g) { return (size_t)g
 
 // ---------------------------------------------------------------------------------------------------- tables
 __device__ inline double phi(const Geometry &g, double u) {
+  if (!(2.0 * fabs(u) <= g.W)) return 0.0;   // most entries, and the images of all but the first and last few steps
   const double s = 2.0 * u / g.W, r = 1.0 - s * s;
-  if (!(r >= 0.0)) return 0.0;
   const double w = exp(g.beta * (sqrt(r) - 1.0)), a = 2.0 * g.fc * u;
   return 2.0 * g.fc * w * (fabs(a) < 1e-12 ? 1.0 : sinpi(a) / (3.14159265358979323846 * a));
 }
@@ -116,16 +117,16 @@ __device__ inline double response(const Geometry &g, double f) {          // H(f
   return x * b1 - b2 + g.cheb[0];
 }
 
-// One entry of k_down's matrix of a step: [8 tokens' chunk][term * 16 + j][8 tokens], rows of 16 bytes.
+// One entry of k_down's matrix of step b, whose window starts at `start`: [8 tokens' chunk][term * 16 + j][8 tokens], rows of
+// 16 bytes.
 template <typename T>
-__device__ __forceinline__ void down_entry(const Geometry &g, int cls, int i, T *__restrict__ out) {
-  const int b = step_of(cls, g.down_steps(), down_classes(g));
-  const int e = i & 7, j = (i >> 3) & (kJ - 1), c = i >> 7, t = down_start(g, b) + c * 8 + e;
+__device__ __forceinline__ void down_entry(const Geometry &g, int cls, int b, int start, int i, T *__restrict__ out) {
+  const int e = i & 7, j = (i >> 3) & (kJ - 1), c = i >> 7, t = start + c * 8 + e;
   T *img = out + (size_t)cls * (down_image(g) / 2);
-  const double inv = (double)g.M / g.N;
+  const double inv = g.up_ratio;
   double v = 0.0;
   if (t < g.N) {
-    const double x = (b * kJ + j + 0.5) * ((double)g.N / g.M) - 0.5;
+    const double x = (b * kJ + j + 0.5) * g.down_ratio - 0.5;
     v = (phi(g, (t - x) * inv) + phi(g, (-1.0 - t - x) * inv) + phi(g, (2.0 * g.N - 1.0 - t - x) * inv)) * inv;
     if (std::is_same<T, __half>::value) v *= kDownScaleF16;
   }
@@ -137,11 +138,10 @@ __device__ __forceinline__ void down_entry(const Geometry &g, int cls, int i, T 
   }
 }
 
-// One entry of k_up's matrix of a step: [term][8 grid values][token][8].  Values are in the order the transform keeps
+// One entry of k_up's matrix of step b, whose window starts at quad q0: [term][8 grid values][token][8].  Values are in the order the transform keeps
 // them: first (z0, z2) of ascending quads, then (z3, z1) of descending ones.  The first term is a whole number (see k_up).
-__device__ __forceinline__ void up_entry(const Geometry &g, int cls, int i, __half *__restrict__ out) {
-  const int b = step_of(cls, g.up_steps(), up_classes(g));
-  const int q0 = up_quad(g, b), nk = 4 * g.nq;
+__device__ __forceinline__ void up_entry(const Geometry &g, int cls, int b, int q0, int i, __half *__restrict__ out) {
+  const int nk = 4 * g.nq;
   __half *img = out + (size_t)cls * (up_image(g) / 2);
   const int e = i & 7, r = (i >> 3) & (kRows - 1), c = i >> 10, k = c * 8 + e, t = b * kRows + r;
   const bool second = k >= 2 * g.nq;
@@ -150,7 +150,7 @@ __device__ __forceinline__ void up_entry(const Geometry &g, int cls, int i, __ha
   const int j = 4 * n + (second ? ((kk & 1) ? 1 : 3) : 2 * (kk & 1));
   double v = 0.0;
   if (t < g.N) {
-    const double x = (t + 0.5) * ((double)g.M / g.N) - 0.5;
+    const double x = (t + 0.5) * g.up_ratio - 0.5;
     v = (phi(g, x - j) + phi(g, x + 1.0 + j) + phi(g, x - (2.0 * g.M - 1.0 - j))) * (double)kUpScale;
   }
   double part = rint(v);
@@ -511,20 +511,26 @@ __device__ __forceinline__ void mid_entry(const Geometry &g, const MidRadices &m
   }
 }
 
-// All tables of a sequence in one launch: `down` + `up` + the rest of the entries, 256 per block.
+// All tables of a sequence in one launch, 256 entries at a time: `down` blocks, then `up` blocks, then those of mid_entry.  A
+// block stays with one matrix for several rounds, since finding a window takes 64-bit divisions.
+constexpr int kDownRounds = 2, kUpRounds = 4;
+__host__ __device__ inline int down_table_blocks(const Geometry &g) { return (g.ks + kDownRounds - 1) / kDownRounds; }   // per matrix
+__host__ __device__ inline int up_table_blocks(const Geometry &g) { return g.nq * 2 / kUpRounds; }
 template <typename T>
 __global__ void __launch_bounds__(256) k_band_tables(const __grid_constant__ Geometry g, const MidRadices m, T *down, __half *up,
                                                      MidTables mid, int down_blocks, int up_blocks) {
   int b = blockIdx.x;
-  if (b < down_blocks) {
-    const int per = g.ks;                                             // blocks per matrix: 16 * ks * 16 entries
-    down_entry<T>(g, b / per, (b % per) * 256 + threadIdx.x, down);
+  if (b < down_blocks) {                                              // a matrix: ks rounds of 16 * 16 entries
+    const int per = down_table_blocks(g), cls = b / per, step = step_of(cls, g.down_steps(), down_classes(g));
+    const int start = down_start(g, step), end = (b % per + 1) * kDownRounds;
+    for (int k = end - kDownRounds; k < end && k < g.ks; ++k) down_entry<T>(g, cls, step, start, k * 256 + threadIdx.x, down);
     return;
   }
   b -= down_blocks;
-  if (b < up_blocks) {
-    const int per = g.nq * 2;                                         // 4 * nq * 128 entries
-    up_entry(g, b / per, (b % per) * 256 + threadIdx.x, up);
+  if (b < up_blocks) {                                                // 2 nq rounds
+    const int per = up_table_blocks(g), cls = b / per, step = step_of(cls, g.up_steps(), up_classes(g)), q0 = up_quad(g, step);
+#pragma unroll 1
+    for (int k = 0; k < kUpRounds; ++k) up_entry(g, cls, step, q0, ((b % per) * kUpRounds + k) * 256 + threadIdx.x, up);
     return;
   }
   mid_entry(g, m, (b - up_blocks) * 256 + threadIdx.x, mid);
