@@ -237,7 +237,11 @@ static size_t unit_bytes(const FcBandJob *j) { return j->y_bytes + align256((siz
 // 2086 / 1985 / 2015 / 1951 us with groups of up to 96 / 128 / 192 / 384 MiB, of 8192 tokens 504 / 504 / 504 / 525, 32 layers
 // of 32 heads of 16384 tokens 9202 / 9050 / 9022 / 8855, and the workspace holds two of them.
 constexpr int kGroupFactor = 4;
-static size_t budget(const fc_handle *h) { return h->group_bytes > ((size_t)1 << 60) ? h->group_bytes : h->group_bytes * kGroupFactor; }
+static size_t budget(const fc_handle *h) {
+  if (h->group_bytes > ((size_t)1 << 60)) return h->group_bytes;
+  const size_t values = h->group_bytes * kGroupFactor;
+  return values + values / 1024;             // and the scales of the rows, so that a power of two of units fits
+}
 
 size_t fc_band_buffer_bytes(const fc_handle *h, const FcBandSizes *s, int units) {
   const size_t all = s->unit * units, most = budget(h);
