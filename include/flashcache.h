@@ -18,8 +18,8 @@
  *   - Streams.  `stream` is a cudaStream_t passed as void*.  Results are ordered
  *     on it: work enqueued on `stream` after a call sees that call's outputs.
  *     Short sequences (powers of two up to 1024 tokens, others up to 512, where head_dim
- *     allows it) are scored by one kernel on `stream`, and so are longer 16-bit ones, by a few
- *     kernels, where a call has little work; else ones of up to 65536 tokens run on
+ *     allows it) are scored by one kernel on `stream`, and a single longer 16-bit one by a few
+ *     kernels on it where the call has little work; else ones of up to 65536 tokens run on
  *     the handle's internal streams (two by default), which wait for everything enqueued on
  *     `stream` before the call and which `stream` waits for before the call returns, through
  *     events; no host synchronisation is involved (see fc_set_score_overlap for the
@@ -95,7 +95,9 @@ typedef struct {
  * max_seqlen, at least 64), room for eight filter tables (16 bytes * the power of two from 2*max_seqlen-1 up each, at
  * least 16 KiB and at most 2 MiB; lengths that are not a power of two reuse theirs from layer to layer and call to call,
  * a batch of more than eight unlike ones builds the rest in the workspace on every call), 2.5 or 5 MiB (from 513 and from
- * 1025 tokens on) for the tables of up to eight 16-bit sequences scored on a coarser grid, kept in the same way, and a status word.  Returns FC_ERR_CUDA if the device cannot be
+ * 1025 tokens on) for the tables of up to eight 16-bit sequences scored on a coarser grid (at most 0.6 MB each at powers of two,
+ * else about 0.9 KB per token: those of more than 6000 tokens do not fit and are built in the workspace on every call, 15 to
+ * 60 us on the device) and a status word.  Returns FC_ERR_CUDA if the device cannot be
  * used, FC_ERR_UNSUPPORTED if max_seqlen is out of range. */
 fc_status fc_create(fc_handle **out, int device, int32_t max_seqlen);
 void fc_destroy(fc_handle *h);

@@ -13,7 +13,8 @@ namespace {
 using band::Geometry;
 
 // Kernels phi for bands up to fmax cycles per grid point: the shortest whose response folds less than 6e-8 of the band's
-// own gain onto the band while that gain varies little over it (found by scanning beta and fc; max / min, rms of max /
+// own gain onto the band while that gain varies little over it (a sinc times the "exponential of semicircle" of Barnett,
+// Magland and af Klinteberg, SIAM J. Sci. Comput. 41, 2019; found by scanning beta and fc; max / min, rms of max /
 // gain in the band, largest folded part):
 //   0.40  24  3.4  1.53  5.1e-8     0.36  20  1.8  1.15  2.5e-8     0.32  16  1.55  1.12  5.5e-8
 //   0.28  14  1.3  1.06  5.3e-8     0.25  14  1.06 1.01  5.6e-8     0.20  12  1.06  1.01  2.4e-8
@@ -56,15 +57,19 @@ const double (*responses())[band::kCheb] {
 constexpr int kMinGrid = 256, kMaxGrid = 16384;
 
 // 16-bit rows are exact operands of the products (fp32 rows would need six of them and terms of their own).  Up to 512 tokens
-// and at 1024 one kernel does it all, and a single layer of 4 heads takes 29..33 us against 44 here (28 layers: 145 and 182
-// against 72 and 95, but a score must not depend on how many layers share a call); from 513 tokens on the three passes take
-// 41 us for one layer and 174 us for 28, this form 44 and 88.
+// and at 1024 one kernel does it all, and a single layer of 4 heads takes 29..33 us there against 44 here when the form was new
+// (28 layers: 145 and 182 against 72 and 95, but a score must not depend on how many layers share a call).  One layer of 4 heads of
+// 517 / 1025 / 2048 / 4096 tokens, calls in a row: three passes 32 / 30 / 25 / 32 us, this form 23 / 29 / 29 / 31; 28 layers 150 / 277 /
+// 255 / 484 against 112 / 120 / 131 / 247.  2048 is the one length where a single layer loses, and 28 layers gain twice.
 bool eligible(const fc_kv_view *kv, int N) {
   return kv->dtype != FC_F32 && N > 512 && N != 1024 && N <= 65536 && kv->head_dim <= 512;
 }
 
-// The coarsest grid on which the band fits: N/4 <= M <= N/2 and omega <= 0.8 M (a quarter more grid than the band needs: the
-// kernel's support grows without bound as that margin closes).  Where M would pass N/2 little is saved and the passes stay.
+// The coarsest grid on which the band fits: M a power of two, N/4 <= M <= N/2 and omega <= 0.8 M (a quarter more grid than the
+// band needs: the kernel's support grows without bound as that margin closes), with windows that fit the rings (N just above 2 M
+// with the widest kernels has longer ones).  At powers of two that is a cutoff of up to two fifths, at others as little as 0.2;
+// of lengths spread evenly over their logarithm 0.83 at cutoffs of 0.2 .. 0.25, 0.53 at 0.25 .. 0.3, 0.25 at 0.3 .. 0.35 take
+// it.  Where M would pass N/2 little is saved and the passes stay.
 bool make_geometry(int N, int omega, Geometry *g) {
   int M = kMinGrid;
   while (4ll * M < N || 5ll * omega > 4ll * M) M <<= 1;
@@ -236,6 +241,7 @@ static size_t unit_bytes(const FcBandJob *j) { return j->y_bytes + align256((siz
 // Launch groups.  Fuller launches beat intermediates that stay in L2, up to a point: 28 layers of 4 heads of 32768 tokens take
 // 2086 / 1985 / 2015 / 1951 us with groups of up to 96 / 128 / 192 / 384 MiB, of 8192 tokens 504 / 504 / 504 / 525, 32 layers
 // of 32 heads of 16384 tokens 9202 / 9050 / 9022 / 8855, and the workspace holds two of them.
+// (Of the 128 MiB ones all held fifteen heads of 32768 tokens at the time, not sixteen: 2085 -> 2077 us since.)
 constexpr int kGroupFactor = 4;
 static size_t budget(const fc_handle *h) {
   if (h->group_bytes > ((size_t)1 << 60)) return h->group_bytes;

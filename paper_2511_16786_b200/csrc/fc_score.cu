@@ -20,8 +20,8 @@
 //   pass 2  for every k1 (with N1-k1, which holds the partner bins N-q):
 //           twiddle, DFT over n2, the filter above, inverse DFT over k2, twiddle -> B[k1][n2]
 //   pass 3  for every n2: inverse DFT over k1, |.|^2 summed over the channels -> scores
-// 16-bit sequences from 513 tokens on whose cutoff keeps at most about two fifths of the bins do not take these passes:
-// they are scored on a coarser grid between two banded matrix products (fc_band.cuh).
+// 16-bit sequences from 513 tokens on whose kept band fits a grid of a power of two points between a quarter and half of the
+// tokens do not take these passes: they are scored on that grid between two banded matrix products (fc_band.cuh).
 // Every other length up to 65536 takes the same three passes on a longer transform with the residual written as one
 // padded convolution (fc_score_fast.cuh); the spectrum diagnostics run on the same passes.  The generic kernels of this
 // file serve the power of two 131072, spectra of short powers of two and the entry point without allocation; there,
