@@ -33,9 +33,11 @@ DEFAULT_CONFIG = "cfg3"          # the 32k-token workload the target fraction is
 
 # DRAM bytes read + written per launch of the dominant kernel as an ncu capture counted them (a constant from
 # that capture, not a measurement of this run; None where no capture of the kernel and workload exists):
-# the transform of the grid values, 16 heads of 32768 tokens per launch (profiles/kept_band_ncu.md).
+# the transform of the grid values and the product back to tokens, 16 heads of 32768 tokens per launch
+# (profiles/kept_band_ncu.md).
 NCU_TRAFFIC_BYTES = {
-    ("cfg3", "pass2"): 2.61e8,
+    ("cfg3", "pass2"): 2.52e8,
+    ("cfg3", "pass3"): 4.30e8,
 }
 
 

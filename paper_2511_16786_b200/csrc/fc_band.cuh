@@ -665,8 +665,8 @@ struct MidParams {
 
 // What bounds it: shared memory (57 % of its wavefronts), the FMA pipe (half) and issue slots (42 %) at 16 warps per SM, none
 // of them alone.  A row is transformed as half as many complex points, two rows per thread in packed arithmetic, which
-// shares the twiddles, the gains and every address: 48 M instructions for 16 heads of 32768 tokens where one row per thread
-// took 83 M; 110 us (134 us with the values stored in 16-byte pieces; one row per thread at 64 registers and 32 warps takes
+// shares the twiddles, the gains and every address: 50 M instructions for 16 heads of 32768 tokens where one row per thread
+// took 83 M; 108 us (134 us with the values stored in 16-byte pieces; one row per thread at 64 registers and 32 warps takes
 // 103 us alone, but whole passes beside the other stream 1..5 % longer).
 template <class S>
 __global__ void __launch_bounds__(S::NT, S::NT <= 512 ? 512 / S::NT : 1) k_mid(const MidParams P) {
